@@ -1,22 +1,25 @@
-"""Builds libtokenbutler.so in-tree with nvcc for sm_100a (no JIT cache, no torch extension)."""
+"""Builds libtokenbutler.so in-tree with nvcc for sm_100a (no JIT cache, no torch extension), and beside it the
+extension module through which binding.py makes the per-step calls."""
 from __future__ import annotations
 
 import os
 import subprocess
 import sys
+import sysconfig
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libtokenbutler.so")
+CALLS = os.path.join(HERE, "_tokenbutler.so")
 SOURCES = ["tb_api.cu", "tb_cache.cu", "tb_select.cu", "tb_select_wave.cu", "tb_select_aux.cu", "tb_attention.cu", "tb_predictor.cu"]
 NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17", "-Xcompiler", "-fPIC",
               "--expt-relaxed-constexpr", "--expt-extended-lambda"]
 
 
 def _stale() -> bool:
-    if not os.path.exists(LIB):
+    if not os.path.exists(LIB) or not os.path.exists(CALLS):
         return True
-    t = os.path.getmtime(LIB)
+    t = min(os.path.getmtime(LIB), os.path.getmtime(CALLS))
     deps = [os.path.join(CSRC, f) for f in os.listdir(CSRC)] + [os.path.join(HERE, "..", "include", "tokenbutler.h")]
     return any(os.path.getmtime(d) > t for d in deps)
 
@@ -58,6 +61,12 @@ def _build_locked(verbose: bool) -> str:
     tmp = LIB + ".%d.tmp" % os.getpid()
     subprocess.check_call([nvcc, "-shared", "-o", tmp, *objs, "-gencode", "arch=compute_100a,code=sm_100a"])
     os.replace(tmp, LIB)
+    # the library is found beside the module ($ORIGIN), under the name it has there
+    tmp = CALLS + ".%d.tmp" % os.getpid()
+    subprocess.check_call([os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-fPIC", "-shared", "-I" + sysconfig.get_paths()["include"],
+                           os.path.join(CSRC, "tb_python.cpp"), "-o", tmp, "-L" + HERE, "-l:" + os.path.basename(LIB),
+                           "-Wl,-rpath,$ORIGIN"])
+    os.replace(tmp, CALLS)
     return LIB
 
 

@@ -71,3 +71,16 @@ def test_predictor_host_validation_needs_no_gpu(libpath):
     assert call(ln_weight=24) == b.TB_ERR_INVALID_ARG      # not 16-byte aligned
     assert call(model_dim=4100) == b.TB_ERR_UNSUPPORTED    # rows are read 16 bytes at a time
     assert call(n_tokens=65) == b.TB_ERR_CAPACITY
+
+
+def test_extension_module_unpacks_like_ctypes(libpath):
+    from paper_2503_07518_b200 import binding as b
+    b.lib()
+    p, s = b.select_params(4), type("Stream", (), {"cuda_stream": 0})()
+    # a null context reaches the entry point and is refused there; what cannot be unpacked raises before the call
+    assert b._calls.select_topk(None, 0, 1, (0,), 1, None, p, None, None, s) == b.TB_ERR_INVALID_ARG
+    assert b._calls.append_kv(None, 0, 1, None, list(range(100)), None, None, s) == b.TB_ERR_INVALID_ARG
+    for bad in ((None, 0, 1, None, 1, None, object(), None, None, s), (None, 0, 1, ["x"], 1, None, p, None, None, s),
+                (None, "0", 1, None, 1, None, p, None, None, s), (None, 0, 1, None, 1, None, p, None, None)):
+        with pytest.raises((TypeError, ValueError)):
+            b._calls.select_topk(*bad)
