@@ -3,18 +3,33 @@
 //     q = W2 . act(W1 . LN(h))          per decoded token h, once per producer layer,
 // the step right before the selection path: its output is the q_imp of the producer's consumer layers.
 //
-// At decode batch sizes both linears are matrix-vector products bound by reading their weights once
-// (8 MB per producer for an 8B-shaped model), so there is no tensor-core tile here: one warp per
-// output row, 16-byte loads, fp32 accumulation, every token of the call against the row while it is
-// in registers.  Two launches: hidden units (layer norm folded in; each block recomputes the few
-// tokens' statistics rather than exchanging them), then outputs written in the layout
-// tb_select_topk reads.  No context: weights and scratch belong to the caller.
+// At decode batch sizes both linears are bound by reading their weights once (8 MB per producer for an 8B-shaped
+// model) and, at a microsecond of HBM time, by the latencies around that.  Two launches: hidden units (layer norm folded
+// in), then outputs written in the layout tb_select_topk reads.  bf16: tensor-core tiles with the weights as the left
+// operand; fp32: one warp (pair) per output row, 16-byte loads, every token of the call against the row while it is in
+// registers.  No context: weights and scratch belong to the caller.
 #include <cooperative_groups.h>
+#include <type_traits>
 
 #include "tb_common.cuh"
 #include "tb_internal.h"
 
 namespace tb {
+
+#ifdef TB_PHASE_TIMING
+__device__ unsigned long long g_pred_ns[2][12][256];     // [hidden / out kernel][stamp][block], last launch
+__device__ __forceinline__ void pred_stamp(int k, int i) {
+    if (threadIdx.x == 0) {
+        unsigned long long t;
+        asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
+        const int b = blockIdx.x + gridDim.x * blockIdx.y;
+        if (b < 256) g_pred_ns[k][i][b] = t;
+    }
+}
+extern "C" int tb_debug_pred_ns(unsigned long long* out) { return (int)cudaMemcpyFromSymbol(out, g_pred_ns, sizeof(g_pred_ns)); }
+#else
+#define pred_stamp(k, i) ((void)0)
+#endif
 
 namespace {
 
@@ -209,182 +224,374 @@ __global__ void __launch_bounds__(kPredThreads) predictor_out_kernel(const T* __
     }
 }
 
-// ---- several tokens at once (bf16): both linears on the tensor cores ---------------------------------
-// With 5 or more tokens the products above re-walk a weight row once per token chunk; a tile of 16
-// tokens x 8 outputs per mma.sync.m16n8k16 reads each weight once for all of them.  The left operand
-// (normalised hidden states, resp. hidden units) is fp32: it is split into a bf16 high and low part
-// and multiplied twice, so the products keep ~16 bits of it and accumulate in fp32.
-// The 16 k-indices of an MMA step are mapped to channels so that every thread's operands are 16
-// contiguous bytes: over a run of 32 channels, thread (row gid, column pair tig) takes channels
-// 8 tig .. 8 tig + 7; the first four feed the first MMA step (k = 2 tig, 2 tig + 1, 2 tig + 8, 2 tig + 9),
-// the last four the second.  Both operands use the same mapping, so the sum over channels is unchanged.
+// ---- bf16: both linears on the tensor cores, weights as the left operand ------------------------------
+// D[32 weight rows x tokens] += W[32 x K] . X[K x tokens] with mma.sync.m16n8k16: the weights are exact in bf16, and
+// the fp32 right operand (scaled hidden states, resp. hidden units) is split into bf16 terms, one MMA each, accumulated
+// in fp32: three terms, which hold all 24 bits of it, for up to four tokens, two (16 bits) for more.  A block's work is 32 weight rows x 512 channels -- 32 KB of
+// weights, about what an SM receives in a memory latency, so that an 8B-shaped linear (8 MB) is 128 blocks that
+// request everything they need at once -- against all tokens of the call.  The tensor pipe is idle most of the time
+// and latency is what there is to save: every thread's weights are in flight before it looks at the tokens.
+// Measured, one call of a 4096 -> 512 -> 4096 predictor in a chain of them: 7.2 us with 1 token, 7.2 with 8, 11.9 with
+// 24, 31 with 64, of which 1.3 are the weights at the copy bandwidth.  (Before: 8.8 with a warp pair per hidden unit and
+// 18.7, 31.9, 61 with 16-token left tiles whose blocks each normalised every token.)  The weights go through shared
+// memory because their copies then cost no registers: with the fragments loaded straight into registers the kernels
+// spilled and ran at 11.3 us.  Two blocks must fit an SM: the output kernel's blocks sit beside the hidden kernel's and
+// have their weights before the hidden units exist, and at one block per SM only 15 of the 16 clusters start at once.
+//
+// The 16 k-indices of an MMA step are mapped to channels so that every thread's operands are 16 contiguous bytes:
+// over a run of 32 channels, thread (row gid, column pair tig) takes channels 8 tig .. 8 tig + 7; the first four feed
+// the first MMA step (k = 2 tig, 2 tig + 1, 2 tig + 8, 2 tig + 9), the last four the second.  Both operands use the
+// same mapping, so the sum over channels is unchanged.
+constexpr int kTileRows = 32;        // weight rows of a block
+constexpr int kChunk = 512;          // channels of a block's tile: 4 warps x 4 runs of 32, for each of two 16-row halves
+constexpr int kTileTokMax = 32;      // tokens staged at once; a kernel instance stages 8 * kN8 of them
+constexpr int kXPitch = kChunk * 2 + 64;   // bytes per (term, token) row: eight rows' 64-byte pieces hit all banks twice
+constexpr int kClusterK = 8;         // blocks (one cluster) that share the channels of a hidden-unit tile
+
 __device__ __forceinline__ void mma_bf16_16x8x16(float* d, uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0, uint32_t b1) {
     asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
                  : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
                  : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
 }
-// fp32 pair -> bf16x2 high parts and bf16x2 of what they leave
-__device__ __forceinline__ void split_bf16x2(float x, float y, uint32_t& hi, uint32_t& lo) {
-    const __nv_bfloat16 xh = __float2bfloat16_rn(x), yh = __float2bfloat16_rn(y);
-    const __nv_bfloat16 xl = __float2bfloat16_rn(x - __bfloat162float(xh)), yl = __float2bfloat16_rn(y - __bfloat162float(yh));
-    hi = (uint32_t)__bfloat16_as_ushort(xh) | ((uint32_t)__bfloat16_as_ushort(yh) << 16);
-    lo = (uint32_t)__bfloat16_as_ushort(xl) | ((uint32_t)__bfloat16_as_ushort(yl) << 16);
-}
-// One run of 32 channels: x0 / x1 = this thread's 8 left-operand values of rows gid / gid + 8 (zeros for
-// rows past the tokens), w = its 8 right-operand values (16 bytes of the weight row of output gid).
-__device__ __forceinline__ void mma_run32(float* acc, const float* x0, const float* x1, const uint4& w) {
-    const uint32_t wb[4] = {w.x, w.y, w.z, w.w};
+// Writes 8 consecutive values as bf16 terms, 16 bytes each, `stride` bytes apart.
+template <int kTerms>
+__device__ __forceinline__ void store_terms(unsigned char* dst, size_t stride, float* x) {
 #pragma unroll
-    for (int st = 0; st < 2; ++st) {
-        uint32_t h0, l0, h1, l1, h2, l2, h3, l3;
-        split_bf16x2(x0[4 * st], x0[4 * st + 1], h0, l0);          // row gid,     k = 2 tig, 2 tig + 1
-        split_bf16x2(x1[4 * st], x1[4 * st + 1], h1, l1);          // row gid + 8
-        split_bf16x2(x0[4 * st + 2], x0[4 * st + 3], h2, l2);      // row gid,     k = 2 tig + 8, 2 tig + 9
-        split_bf16x2(x1[4 * st + 2], x1[4 * st + 3], h3, l3);
-        mma_bf16_16x8x16(acc, h0, h1, h2, h3, wb[2 * st], wb[2 * st + 1]);
-        mma_bf16_16x8x16(acc, l0, l1, l2, l3, wb[2 * st], wb[2 * st + 1]);
+    for (int k = 0; k < kTerms; ++k) {
+        uint32_t t[4];
+#pragma unroll
+        for (int e = 0; e < 8; e += 2) {
+            const __nv_bfloat162 v = __floats2bfloat162_rn(x[e], x[e + 1]);
+            t[e / 2] = *reinterpret_cast<const uint32_t*>(&v);
+            x[e] -= __low2float(v), x[e + 1] -= __high2float(v);
+        }
+        *reinterpret_cast<uint4*>(dst + k * stride) = make_uint4(t[0], t[1], t[2], t[3]);
     }
 }
 
-constexpr int kSplitK = 4;           // thread blocks (one cluster) that share the channels of a hidden-unit tile
+// The block's weights of one chunk go to shared memory by 16-byte asynchronous copies, whole lines at a time; a warp
+// then multiplies 16 of the rows (half mt) by a quarter kq of the 512 channels.
+constexpr int kWBytes = kTileRows * kXPitch;
+// requests channels [c_begin, min(c_begin + kChunk, c_end)) of rows row0 ..; rows past the matrix repeat its last one,
+// channels past the end are zero
+__device__ __forceinline__ void request_weights(unsigned char* ws, const __nv_bfloat16* __restrict__ W, int n_rows, int pitch, int row0,
+                                                int c_begin, int c_end) {
+#pragma unroll
+    for (int i = 0; i < kTileRows * (kChunk / 8) / kPredThreads; ++i) {
+        const int e = i * kPredThreads + threadIdx.x, row = e / (kChunk / 8), v = e % (kChunk / 8), c = c_begin + v * 8;
+        unsigned char* dst = ws + row * kXPitch + v * 16;
+        if (c < c_end)
+            asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(dst)), "l"(W + (size_t)min(row0 + row, n_rows - 1) * pitch + c) : "memory");
+        else
+            *reinterpret_cast<uint4*>(dst) = make_uint4(0u, 0u, 0u, 0u);
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+}
+__device__ __forceinline__ void wait_weights() { asm volatile("cp.async.wait_group 0;" ::: "memory"); }
 
-// hidden[t][j] for 8 hidden units per cluster of kSplitK blocks: block r takes a quarter of the channels,
-// its 8 warps a run of 32 channels at a time; partial tiles are summed in rank 0's shared memory
-// (distributed shared memory, fixed order).  The layer-norm statistics of the tokens are split over
-// the cluster the same way.
-__global__ void __launch_bounds__(kPredThreads) predictor_hidden_mma_kernel(const __nv_bfloat16* __restrict__ H,
-                                                                            const __nv_bfloat16* __restrict__ ln_w,
-                                                                            const __nv_bfloat16* __restrict__ ln_b,
-                                                                            const __nv_bfloat16* __restrict__ W1,
-                                                                            float* __restrict__ hidden, int n_tok, int E, int hid,
-                                                                            float eps, int act) {
-    using EB = Elem<__nv_bfloat16>;
+// acc += W . X for kN8 groups of eight staged tokens.  A single group has two accumulators, so that the chain of
+// dependent MMAs is half as long.  kNorm: also gb += W . (column 0 = ln_w, column 1 = ln_b), whose operand gbx comes
+// straight from the parameters.
+template <int kN8>
+constexpr int kAccs = kN8 == 1 ? 2 : kN8;
+template <int kTerms, int kN8, bool kNorm>
+__device__ __forceinline__ void mma_tile(float (&acc)[kAccs<kN8>][4], const unsigned char* ws, const unsigned char* xs, float* gb,
+                                         const uint4* gbx) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, gid = lane >> 2, tig = lane & 3, mt = warp >> 2, kq = warp & 3;
+    const int off = (kq * 128 + 8 * tig) * 2;
+    const unsigned char* wa = ws + (mt * 16 + gid) * kXPitch + off;
+    const unsigned char* x0 = xs + gid * kXPitch + off;
+#pragma unroll
+    for (int r = 0; r < 4; ++r) {
+        const uint4 a = *reinterpret_cast<const uint4*>(wa + r * 64), b = *reinterpret_cast<const uint4*>(wa + 8 * kXPitch + r * 64);
+        if constexpr (kNorm) {
+            mma_bf16_16x8x16(gb, a.x, b.x, a.y, b.y, gbx[r].x, gbx[r].y);
+            mma_bf16_16x8x16(gb, a.z, b.z, a.w, b.w, gbx[r].z, gbx[r].w);
+        }
+#pragma unroll
+        for (int k = 0; k < kTerms; ++k) {
+            uint4 x[kN8];
+#pragma unroll
+            for (int n = 0; n < kN8; ++n) x[n] = *reinterpret_cast<const uint4*>(x0 + (k * kN8 + n) * 8 * kXPitch + r * 64);
+#pragma unroll
+            for (int n = 0; n < kN8; ++n) mma_bf16_16x8x16(acc[n], a.x, b.x, a.y, b.y, x[n].x, x[n].y);
+#pragma unroll
+            for (int n = 0; n < kN8; ++n) mma_bf16_16x8x16(acc[kN8 == 1 ? 1 : n], a.z, b.z, a.w, b.w, x[n].z, x[n].w);
+        }
+    }
+}
+// The four channel quarters' accumulators, [quarter][row][token]
+template <int kN8>
+using TileSums = float[4][kTileRows][kN8 * 8 + 1];
+template <int kN8>
+__device__ __forceinline__ void put_sums(TileSums<kN8>& s, float (&acc)[kAccs<kN8>][4]) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, gid = lane >> 2, tig = lane & 3, row = (warp >> 2) * 16 + gid;
+    if constexpr (kN8 == 1) acc[0][0] += acc[1][0], acc[0][1] += acc[1][1], acc[0][2] += acc[1][2], acc[0][3] += acc[1][3];
+#pragma unroll
+    for (int n = 0; n < kN8; ++n) {
+        s[warp & 3][row][n * 8 + 2 * tig] = acc[n][0], s[warp & 3][row][n * 8 + 2 * tig + 1] = acc[n][1];
+        s[warp & 3][row + 8][n * 8 + 2 * tig] = acc[n][2], s[warp & 3][row + 8][n * 8 + 2 * tig + 1] = acc[n][3];
+    }
+}
+template <int kN8>
+__device__ __forceinline__ float get_sum(const TileSums<kN8>& s, int row, int tok) { return (s[0][row][tok] + s[1][row][tok]) + (s[2][row][tok] + s[3][row][tok]); }
+
+// hidden[t][j] = act( sum_c W1[j][c] * ((h[t][c] - mean_t) * rstd_t * ln_w[c] + ln_b[c]) ), fp32 or (two terms) as
+// bf16 [term][t][j], for 32 hidden units per cluster of eight blocks, an eighth of the channels each.  No block waits for a token's statistics: with a shift s of
+// its own (the token's mean over the block's first channels) block b computes
+//     P = sum_c w ln_w (h - s),   G = sum_c w ln_w,   B = sum_c w ln_b
+// and the shifted sums of h and h^2 over its channels; behind one exchange through distributed shared memory
+//     sum = rstd * sum_b (P_b - (mean - s_b) G_b) + sum_b B_b
+// where mean - s_b is small against the spread, so nothing cancels.  Blocks are summed in rank order.
+template <int kTerms, int kN8>
+__global__ void __launch_bounds__(kPredThreads, 2) predictor_hidden_tile_kernel(const __nv_bfloat16* __restrict__ H,
+                                                                                const __nv_bfloat16* __restrict__ ln_w,
+                                                                                const __nv_bfloat16* __restrict__ ln_b,
+                                                                                const __nv_bfloat16* __restrict__ W1,
+                                                                                float* __restrict__ hidden, int n_tok, int E, int hid,
+                                                                                float eps, int act) {
     namespace cg = cooperative_groups;
+    using EB = Elem<__nv_bfloat16>;
     cg::cluster_group cluster = cg::this_cluster();
     const int rank = (int)cluster.block_rank();        // == blockIdx.x
-    pdl_launch_dependents();
-    __shared__ float s_mean[kPredMaxTokens], s_rstd[kPredMaxTokens];
-    __shared__ float s_acc[kSplitK][kPredWarps][16][8];   // rank 0 receives every block's per-warp tiles
+    constexpr int kRows = kTileRows / kClusterK;       // hidden units this block finishes
+    constexpr int kTileTok = kN8 * 8, kOwn = kN8;      // tokens of a group; of those, the ones a warp looks after
+    constexpr size_t kTermStride = (size_t)kTileTok * kXPitch;
+    extern __shared__ __align__(128) unsigned char ws[];   // weights [32 rows][kXPitch], then states [term][token][kXPitch]
+    unsigned char* xs = ws + kWBytes;
+    __shared__ TileSums<kN8> s_sum;
+    __shared__ float2 s_gb[4][kTileRows];              // (G, B) of the block's rows, per channel quarter
+    // from every block of the cluster (a buffer per token group): P and (G, B) of this block's rows, and every token's
+    // (shift, shifted sum, shifted sum of squares)
+    __shared__ float s_p[2][kClusterK][kRows][kTileTok];
+    __shared__ float2 s_gb_all[kClusterK][kRows];
+    __shared__ float4 s_stat[2][kClusterK][kTileTok];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, gid = lane >> 2, tig = lane & 3;
-    // statistics of tokens rank*8+warp, +32, ...: shifted one-pass sums, sixteen 16-byte loads in flight
-    for (int t = rank * kPredWarps + warp; t < n_tok; t += kSplitK * kPredWarps) {
-        const uint4* h4 = reinterpret_cast<const uint4*>(H + (size_t)t * E);
-        const float shift = __bfloat162float(H[(size_t)t * E]);
-        float f[8], s1 = 0.f, s2 = 0.f;
-#pragma unroll 4
-        for (int v = lane; v < E / 8; v += 32) {
-            EB::unpack16(__ldg(h4 + v), f);
+    const int j0 = blockIdx.y * kTileRows;
+    const int span = (((E + 31) / 32 + kClusterK - 1) / kClusterK) * 32;     // channels of a block
+    const int c_begin = min(E, rank * span), c_end = min(E, c_begin + span);
+    const int n_chunk = (span + kChunk - 1) / kChunk;
+    const uint4 zero = make_uint4(0u, 0u, 0u, 0u);
+    pred_stamp(0, 0);
+    // The states may come from the predecessor, and so may the weights: wait, then let the output kernel get ready.
+    pdl_wait();
+    pdl_launch_dependents();
+    pred_stamp(0, 1);
+
+    for (int t0 = 0, group = 0; t0 < n_tok; t0 += kTileTok, ++group) {
+        const int n_here = min(kTileTok, n_tok - t0);
+        float acc[kAccs<kN8>][4] = {}, gb[4] = {};
+        float shift[kOwn], s1[kOwn], s2[kOwn];
 #pragma unroll
-            for (int e = 0; e < 8; ++e) {
-                const float d = f[e] - shift;
-                s1 += d, s2 = fmaf(d, d, s2);
+        for (int i = 0; i < kOwn; ++i) shift[i] = s1[i] = s2[i] = 0.f;
+        for (int kc = 0; kc < n_chunk; ++kc) {
+            const int c0 = c_begin + kc * kChunk;
+            if (n_chunk > 1 || group == 0) {
+                if (kc + group) __syncthreads();       // the previous chunk's operands have been read
+                request_weights(ws, W1, hid, E, j0, c0, c_end);
             }
-        }
-        s1 = warp_sum(s1), s2 = warp_sum(s2);
-        if (lane < kSplitK) {                          // lane r tells block r
-            const float m = s1 / (float)E;
-            *cluster.map_shared_rank(&s_mean[t], lane) = shift + m;
-            *cluster.map_shared_rank(&s_rstd[t], lane) = rsqrtf(fmaxf(s2 / (float)E - m * m, 0.f) + eps);
-        }
-    }
-    cluster.sync();
-    const int j0 = blockIdx.y * 8;                     // the cluster's hidden units; hid is a multiple of 8
-    const __nv_bfloat16* wrow = W1 + (size_t)(j0 + gid) * E;
-    const int n_runs = E / 32, runs_per_block = (n_runs + kSplitK - 1) / kSplitK;
-    const int r_begin = rank * runs_per_block, r_end = min(n_runs, r_begin + runs_per_block);
-    float(*acc0)[kPredWarps][16][8] = cluster.map_shared_rank(s_acc, 0);
-    for (int t0 = 0; t0 < n_tok; t0 += 16) {
-        const int ta = t0 + gid, tb_ = t0 + gid + 8;
-        const bool va = ta < n_tok, vb = tb_ < n_tok;
-        const float ma = va ? s_mean[ta] : 0.f, ra = va ? s_rstd[ta] : 0.f, mb = vb ? s_mean[tb_] : 0.f, rb = vb ? s_rstd[tb_] : 0.f;
-        float acc[4] = {0.f, 0.f, 0.f, 0.f};
-        for (int r0 = r_begin + warp; r0 < r_end; r0 += 2 * kPredWarps) {       // two runs' loads in flight
-            uint4 wv[2], gv[2], bv[2], hav[2], hbv[2];
+            // A warp looks after tokens warp, warp + 8, ... of the group, a lane after channels 8 lane .. + 7 and
+            // 256 + 8 lane .. + 7 of the chunk.
+            uint4 hv[kOwn][2], gv[2];
 #pragma unroll
-            for (int i = 0; i < 2; ++i) {
-                const int r = r0 + i * kPredWarps;
-                const int c = min(r, r_end - 1) * 32 + 8 * tig;
-                wv[i] = __ldg(reinterpret_cast<const uint4*>(wrow + c));
-                gv[i] = __ldg(reinterpret_cast<const uint4*>(ln_w + c));
-                bv[i] = __ldg(reinterpret_cast<const uint4*>(ln_b + c));
-                hav[i] = va ? __ldg(reinterpret_cast<const uint4*>(H + (size_t)ta * E + c)) : make_uint4(0u, 0u, 0u, 0u);
-                hbv[i] = vb ? __ldg(reinterpret_cast<const uint4*>(H + (size_t)tb_ * E + c)) : make_uint4(0u, 0u, 0u, 0u);
-            }
+            for (int i = 0; i < kOwn; ++i)
 #pragma unroll
-            for (int i = 0; i < 2; ++i) {
-                if (r0 + i * kPredWarps >= r_end) break;   // warp-uniform
-                float g[8], b[8], ha[8], hb[8];
-                EB::unpack16(gv[i], g), EB::unpack16(bv[i], b), EB::unpack16(hav[i], ha), EB::unpack16(hbv[i], hb);
-#pragma unroll
-                for (int e = 0; e < 8; ++e) {
-                    ha[e] = va ? fmaf((ha[e] - ma) * ra, g[e], b[e]) : 0.f;
-                    hb[e] = vb ? fmaf((hb[e] - mb) * rb, g[e], b[e]) : 0.f;
+                for (int v = 0; v < 2; ++v) {
+                    const int tl = i * kPredWarps + warp, c = c0 + v * 256 + lane * 8;
+                    hv[i][v] = tl < n_here && c < c_end ? __ldg(reinterpret_cast<const uint4*>(H + (size_t)(t0 + tl) * E + c)) : zero;
                 }
-                mma_run32(acc, ha, hb, wv[i]);
+#pragma unroll
+            for (int v = 0; v < 2; ++v) {
+                const int c = c0 + v * 256 + lane * 8;
+                gv[v] = c < c_end ? __ldg(reinterpret_cast<const uint4*>(ln_w + c)) : zero;
+            }
+            // right operand of the G, B product: column 0 = layer-norm weights, column 1 = biases
+            uint4 gbx[4];
+            if (group == 0) {
+                const __nv_bfloat16* src = gid == 0 ? ln_w : ln_b;
+#pragma unroll
+                for (int r = 0; r < 4; ++r) {
+                    const int c = c0 + ((warp & 3) * 4 + r) * 32 + 8 * tig;
+                    gbx[r] = gid < 2 && c < c_end ? __ldg(reinterpret_cast<const uint4*>(src + c)) : zero;
+                }
+            }
+            if (kc == 0) {
+                const int n = min(kChunk, c_end - c0);
+#pragma unroll
+                for (int i = 0; i < kOwn; ++i) {
+                    float f[8];
+                    EB::unpack16(hv[i][0], f);
+                    shift[i] = ((f[0] + f[1]) + (f[2] + f[3])) + ((f[4] + f[5]) + (f[6] + f[7]));
+                    EB::unpack16(hv[i][1], f);
+                    shift[i] += ((f[0] + f[1]) + (f[2] + f[3])) + ((f[4] + f[5]) + (f[6] + f[7]));
+                }
+#pragma unroll
+                for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+                    for (int i = 0; i < kOwn; ++i) shift[i] += __shfl_xor_sync(0xffffffffu, shift[i], o);
+#pragma unroll
+                for (int i = 0; i < kOwn; ++i) shift[i] = n > 0 ? shift[i] / (float)n : 0.f;
+            }
+#pragma unroll
+            for (int i = 0; i < kOwn; ++i) {
+                const int tl = i * kPredWarps + warp;
+#pragma unroll
+                for (int v = 0; v < 2; ++v) {
+                    const bool in = c0 + v * 256 + lane * 8 < c_end;
+                    float h[8], g[8];
+                    EB::unpack16(hv[i][v], h), EB::unpack16(gv[v], g);
+#pragma unroll
+                    for (int e = 0; e < 8; ++e) {
+                        const float d = in ? h[e] - shift[i] : 0.f;      // (tokens past the end: all zero)
+                        s1[i] += d, s2[i] = fmaf(d, d, s2[i]);
+                        h[e] = d * g[e];
+                    }
+                    store_terms<kTerms>(xs + (size_t)tl * kXPitch + (v * 256 + lane * 8) * 2, kTermStride, h);
+                }
+            }
+            pred_stamp(0, 7);
+            wait_weights();
+            __syncthreads();
+            pred_stamp(0, 2);
+            if (group == 0) mma_tile<kTerms, kN8, true>(acc, ws, xs, gb, gbx);
+            else mma_tile<kTerms, kN8, false>(acc, ws, xs, nullptr, nullptr);
+        }
+        put_sums<kN8>(s_sum, acc);
+        if (group == 0 && tig == 0) {
+            s_gb[warp & 3][(warp >> 2) * 16 + gid] = make_float2(gb[0], gb[1]);
+            s_gb[warp & 3][(warp >> 2) * 16 + gid + 8] = make_float2(gb[2], gb[3]);
+        }
+        __syncthreads();
+        pred_stamp(0, 3);
+        for (int e = tid; e < kTileRows * kTileTok; e += kPredThreads) {
+            const int row = e / kTileTok, tok = e % kTileTok;
+            if (tok < n_here) *cluster.map_shared_rank(&s_p[group & 1][rank][row % kRows][tok], row / kRows) = get_sum<kN8>(s_sum, row, tok);
+        }
+        if (group == 0 && tid < kTileRows) {
+            const float2 a = s_gb[0][tid], b = s_gb[1][tid], c = s_gb[2][tid], d = s_gb[3][tid];
+            *cluster.map_shared_rank(&s_gb_all[rank][tid % kRows], tid / kRows) = make_float2((a.x + b.x) + (c.x + d.x), (a.y + b.y) + (c.y + d.y));
+        }
+#pragma unroll
+        for (int i = 0; i < kOwn; ++i) {
+            const int tl = i * kPredWarps + warp;
+            if (tl >= n_here) break;                   // warp-uniform
+            const float a = warp_sum(s1[i]), b = warp_sum(s2[i]);
+            if (lane < kClusterK) *cluster.map_shared_rank(&s_stat[group & 1][rank][tl], lane) = make_float4(shift[i], a, b, 0.f);   // lane r tells block r
+        }
+        pred_stamp(0, 4);
+        cluster.sync();
+        pred_stamp(0, 5);
+        if (tid < kRows * kTileTok) {
+            const int row = tid / kTileTok, tok = tid % kTileTok, j = j0 + rank * kRows + row;
+            if (tok < n_here && j < hid) {
+                float4 st[kClusterK];
+                float mean = 0.f;
+#pragma unroll
+                for (int r = 0; r < kClusterK; ++r) {
+                    st[r] = s_stat[group & 1][r][tok];
+                    const float n = (float)max(0, min(span, E - r * span));
+                    mean += fmaf(n, st[r].x, st[r].y);
+                }
+                mean /= (float)E;
+                float var = 0.f, sum = 0.f, bias = 0.f;
+#pragma unroll
+                for (int r = 0; r < kClusterK; ++r) {
+                    // sum of (h - mean)^2 = sum of (d - u)^2 with d = h - shift, u = mean - shift
+                    const float n = (float)max(0, min(span, E - r * span)), u = mean - st[r].x;
+                    const float2 w = s_gb_all[r][row];
+                    var += fmaf(u, fmaf(n, u, -2.f * st[r].y), st[r].z);
+                    sum += fmaf(-u, w.x, s_p[group & 1][r][row][tok]);
+                    bias += w.y;
+                }
+                const float rstd = rsqrtf(fmaxf(var / (float)E, 0.f) + eps);
+                const float x = activate(fmaf(rstd, sum, bias), act);
+                if constexpr (kTerms == 2) {           // two terms take the room of the fp32 value: split here, once
+                    __nv_bfloat16* term = reinterpret_cast<__nv_bfloat16*>(hidden) + (size_t)(t0 + tok) * hid + j;
+                    const __nv_bfloat16 hi = __float2bfloat16_rn(x);
+                    term[0] = hi, term[(size_t)n_tok * hid] = __float2bfloat16_rn(x - __bfloat162float(hi));
+                } else {
+                    hidden[(size_t)(t0 + tok) * hid + j] = x;
+                }
             }
         }
-        // acc: rows gid (acc[0..1]) and gid + 8 (acc[2..3]), units 2 tig, 2 tig + 1 -> rank 0
-        acc0[rank][warp][gid][2 * tig] = acc[0], acc0[rank][warp][gid][2 * tig + 1] = acc[1];
-        acc0[rank][warp][gid + 8][2 * tig] = acc[2], acc0[rank][warp][gid + 8][2 * tig + 1] = acc[3];
-        cluster.sync();
-        if (rank == 0 && tid < 128) {
-            const int row = tid >> 3, col = tid & 7;
-            float a = 0.f;
-#pragma unroll
-            for (int r = 0; r < kSplitK; ++r)
-#pragma unroll
-                for (int w = 0; w < kPredWarps; ++w) a += s_acc[r][w][row][col];
-            if (t0 + row < n_tok) hidden[(size_t)(t0 + row) * hid + j0 + col] = activate(a, act);
-        }
-        cluster.sync();                                // rank 0 has read the tiles before the next round overwrites them
+        pred_stamp(0, 6);
     }
 }
 
-// q_imp for 8 output rows per half block: a block's 8 warps are 2 output tiles x 4 quarters of the row.
-__global__ void __launch_bounds__(kPredThreads) predictor_out_mma_kernel(const __nv_bfloat16* __restrict__ W2, const float* __restrict__ hidden,
-                                                                         float* __restrict__ q_imp, int n_tok, int hid, int n_out,
-                                                                         int per_slot) {
-    __shared__ float s_acc[2][4][16][8];
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, gid = lane >> 2, tig = lane & 3;
-    const int tile = warp >> 2, quarter = warp & 3;
-    const int o0 = (blockIdx.x * 2 + tile) * 8;        // n_out is a multiple of 8
-    const bool live = o0 < n_out;
-    const __nv_bfloat16* wrow = W2 + (size_t)(live ? o0 + gid : 0) * hid;
-    const int n_runs = hid / 32, runs_per_q = (n_runs + 3) / 4;
-    const int r_begin = quarter * runs_per_q, r_end = min(n_runs, r_begin + runs_per_q);
-    // the weights of this warp's first two runs do not depend on the hidden units: fetch them, then wait
-    uint4 wpre[2];
-#pragma unroll
-    for (int i = 0; i < 2; ++i) wpre[i] = __ldg(reinterpret_cast<const uint4*>(wrow + min(r_begin + i, max(n_runs - 1, 0)) * 32 + 8 * tig));
-    pdl_wait();                                        // the hidden units come from the previous kernel
-    for (int t0 = 0; t0 < n_tok; t0 += 16) {
-        const int ta = t0 + gid, tb_ = t0 + gid + 8;
-        const bool va = ta < n_tok, vb = tb_ < n_tok;
-        float acc[4] = {0.f, 0.f, 0.f, 0.f};
-        for (int r = r_begin; r < r_end; ++r) {
-            const int c = r * 32 + 8 * tig;
-            const uint4 wv = r - r_begin < 2 ? wpre[r - r_begin] : __ldg(reinterpret_cast<const uint4*>(wrow + c));
-            float ha[8], hb[8];
-#pragma unroll
-            for (int e = 0; e < 8; e += 4) {
-                const float4 xa = va ? __ldcg(reinterpret_cast<const float4*>(hidden + (size_t)ta * hid + c + e)) : make_float4(0.f, 0.f, 0.f, 0.f);
-                const float4 xb = vb ? __ldcg(reinterpret_cast<const float4*>(hidden + (size_t)tb_ * hid + c + e)) : make_float4(0.f, 0.f, 0.f, 0.f);
-                ha[e] = xa.x, ha[e + 1] = xa.y, ha[e + 2] = xa.z, ha[e + 3] = xa.w;
-                hb[e] = xb.x, hb[e + 1] = xb.y, hb[e + 2] = xb.z, hb[e + 3] = xb.w;
+// q_imp for 32 output rows per block, all hidden units.
+template <int kTerms, int kN8>
+__global__ void __launch_bounds__(kPredThreads, 2) predictor_out_tile_kernel(const __nv_bfloat16* __restrict__ W2, const float* __restrict__ hidden,
+                                                                          float* __restrict__ q_imp, int n_tok, int hid, int n_out,
+                                                                          int per_slot) {
+    extern __shared__ __align__(128) unsigned char ws[];   // weights [32 rows][kXPitch], then hidden units [term][token][kXPitch]
+    unsigned char* xs = ws + kWBytes;
+    constexpr int kTileTok = kN8 * 8;
+    constexpr size_t kTermStride = (size_t)kTileTok * kXPitch;
+    __shared__ TileSums<kN8> s_sum;
+    const int tid = threadIdx.x;
+    const int o0 = blockIdx.x * kTileRows, n_chunk = (hid + kChunk - 1) / kChunk;
+    // the weights do not depend on the hidden units (and the predecessor, which computes those, started after
+    // everything before it): fetch them, then wait
+    pred_stamp(1, 0);
+    request_weights(ws, W2, n_out, hid, o0, 0, hid);
+    pdl_wait();
+    pdl_launch_dependents();
+    pred_stamp(1, 1);
+    for (int t0 = 0; t0 < n_tok; t0 += kTileTok) {
+        const int n_here = min(kTileTok, n_tok - t0);
+        float acc[kAccs<kN8>][4] = {};
+        for (int kc = 0; kc < n_chunk; ++kc) {
+            if (n_chunk > 1 && t0 + kc) {
+                __syncthreads();                       // the previous chunk's operands have been read
+                request_weights(ws, W2, n_out, hid, o0, kc * kChunk, hid);
             }
-            mma_run32(acc, ha, hb, wv);
+            constexpr int kVec = kChunk / 8, kStep = kPredThreads / kVec;      // 8 values at a time, four tokens per round
+            const int c = kc * kChunk + tid % kVec * 8;
+            if constexpr (kTerms == 2) {               // the hidden-unit kernel has split them
+                if (t0 + kc) __syncthreads();          // the previous operands have been read
+#pragma unroll
+                for (int i = 0; i < kTerms * kTileTok / kStep; ++i) {
+                    const int row = i * kStep + tid / kVec, tl = row % kTileTok;
+                    unsigned char* dst = xs + row * kXPitch + tid % kVec * 16;
+                    if (tl < n_here && c < hid)
+                        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(dst)),
+                                     "l"(reinterpret_cast<const __nv_bfloat16*>(hidden) + ((size_t)(row / kTileTok) * n_tok + t0 + tl) * hid + c)
+                                     : "memory");
+                    else
+                        *reinterpret_cast<uint4*>(dst) = make_uint4(0u, 0u, 0u, 0u);
+                }
+                asm volatile("cp.async.commit_group;" ::: "memory");
+            } else {
+                float4 x[kTileTok / kStep][2];
+#pragma unroll
+                for (int i = 0; i < kTileTok / kStep; ++i) {
+                    const int tl = i * kStep + tid / kVec;
+                    const bool in = tl < n_here && c < hid;
+                    const float4* src = reinterpret_cast<const float4*>(hidden + (size_t)(t0 + tl) * hid + c);
+                    x[i][0] = in ? __ldcg(src) : make_float4(0.f, 0.f, 0.f, 0.f);
+                    x[i][1] = in ? __ldcg(src + 1) : make_float4(0.f, 0.f, 0.f, 0.f);
+                }
+                if (kc) __syncthreads();
+#pragma unroll
+                for (int i = 0; i < kTileTok / kStep; ++i) {
+                    float v[8] = {x[i][0].x, x[i][0].y, x[i][0].z, x[i][0].w, x[i][1].x, x[i][1].y, x[i][1].z, x[i][1].w};
+                    store_terms<kTerms>(xs + (size_t)(i * kStep + tid / kVec) * kXPitch + tid % kVec * 16, kTermStride, v);
+                }
+            }
+            wait_weights();
+            __syncthreads();
+            pred_stamp(1, 3);
+            mma_tile<kTerms, kN8, false>(acc, ws, xs, nullptr, nullptr);
         }
-        s_acc[tile][quarter][gid][2 * tig] = acc[0], s_acc[tile][quarter][gid][2 * tig + 1] = acc[1];
-        s_acc[tile][quarter][gid + 8][2 * tig] = acc[2], s_acc[tile][quarter][gid + 8][2 * tig + 1] = acc[3];
+        put_sums<kN8>(s_sum, acc);
         __syncthreads();
-        {
-            const int tl = tid >> 7, row = (tid >> 3) & 15, col = tid & 7;   // 256 threads = 2 tiles x 16 rows x 8 columns
-            const int t = t0 + row, o = (blockIdx.x * 2 + tl) * 8 + col;
-            const float a = s_acc[tl][0][row][col] + s_acc[tl][1][row][col] + s_acc[tl][2][row][col] + s_acc[tl][3][row][col];
-            if (t < n_tok && o < n_out) q_imp[((size_t)(o / per_slot) * n_tok + t) * per_slot + o % per_slot] = a;
+        pred_stamp(1, 4);
+        for (int e = tid; e < kTileRows * kTileTok; e += kPredThreads) {
+            const int row = e % kTileRows, tok = e / kTileRows, o = o0 + row;
+            if (tok < n_here && o < n_out) q_imp[((size_t)(o / per_slot) * n_tok + t0 + tok) * per_slot + o % per_slot] = get_sum<kN8>(s_sum, row, tok);
         }
-        __syncthreads();
     }
+    pred_stamp(1, 5);
 }
 
 }  // namespace
@@ -409,46 +616,54 @@ extern "C" tb_status tb_predict_importance_queries(const tb_predictor* p, const 
     const long long n_out = (long long)p->n_slots * p->n_q_heads * p->imp_dim;
     if (n_out > (1ll << 24)) return TB_ERR_UNSUPPORTED;
     cudaStream_t s = (cudaStream_t)stream;
-    const int g1 = (p->hidden_dim + kPredWarps / 2 - 1) / (kPredWarps / 2), g2 = (int)((n_out + kPredWarps - 1) / kPredWarps);
+    const int per_slot = p->n_q_heads * p->imp_dim, n_out_i = (int)n_out;
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(g2, 1, 1), cfg.blockDim = dim3(kPredThreads, 1, 1), cfg.stream = s;
-    int stage_tok = (int)(48 * 1024 / (p->hidden_dim * sizeof(float))) / kTokChunk * kTokChunk;   // hidden_dim <= 1536 gives >= 8
-    stage_tok = stage_tok > kStageTok ? kStageTok : stage_tok < kTokChunk ? kTokChunk : stage_tok;
-    cfg.dynamicSmemBytes = (size_t)stage_tok * p->hidden_dim * sizeof(float);
-    cudaLaunchAttribute attr[1];
+    cfg.blockDim = dim3(kPredThreads, 1, 1), cfg.stream = s;
+    cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;   // see pdl_wait()
     attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr, cfg.numAttrs = 1;
-    const int per_slot = p->n_q_heads * p->imp_dim, n_out_i = (int)n_out;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = kClusterK, attr[1].val.clusterDim.y = 1, attr[1].val.clusterDim.z = 1;
+    cfg.attrs = attr;
     cudaError_t e;
-    if (p->dtype == TB_BF16 && n_tokens >= 5 && p->model_dim % 32 == 0 && p->hidden_dim % 32 == 0 && n_out % 8 == 0) {
-        // several tokens: tensor-core tiles of 16 tokens x 8 outputs
-        {
-            cudaLaunchConfig_t c1 = {};
-            c1.gridDim = dim3(kSplitK, p->hidden_dim / 8, 1), c1.blockDim = dim3(kPredThreads, 1, 1), c1.stream = s;
-            cudaLaunchAttribute a1[1];
-            a1[0].id = cudaLaunchAttributeClusterDimension;
-            a1[0].val.clusterDim.x = kSplitK, a1[0].val.clusterDim.y = 1, a1[0].val.clusterDim.z = 1;
-            c1.attrs = a1, c1.numAttrs = 1;
-            if (cudaLaunchKernelEx(&c1, predictor_hidden_mma_kernel, (const __nv_bfloat16*)hidden_dev, (const __nv_bfloat16*)p->ln_weight,
-                                   (const __nv_bfloat16*)p->ln_bias, (const __nv_bfloat16*)p->w1, scratch_dev, (int)n_tokens,
-                                   (int)p->model_dim, (int)p->hidden_dim, p->ln_eps, (int)p->activation) != cudaSuccess)
-                return TB_ERR_CUDA;
-        }
-        cfg.gridDim = dim3((unsigned)((n_out / 8 + 1) / 2), 1, 1);
-        cfg.dynamicSmemBytes = 0;
-        e = cudaLaunchKernelEx(&cfg, predictor_out_mma_kernel, (const __nv_bfloat16*)p->w2, (const float*)scratch_dev, q_imp_dev,
-                               (int)n_tokens, (int)p->hidden_dim, n_out_i, per_slot);
-    } else if (p->dtype == TB_BF16) {
-        predictor_hidden_kernel<__nv_bfloat16><<<g1, kPredThreads, 0, s>>>(
-            (const __nv_bfloat16*)hidden_dev, (const __nv_bfloat16*)p->ln_weight, (const __nv_bfloat16*)p->ln_bias,
-            (const __nv_bfloat16*)p->w1, scratch_dev, n_tokens, p->model_dim, p->hidden_dim, p->ln_eps, p->activation);
-        e = cudaLaunchKernelEx(&cfg, predictor_out_kernel<__nv_bfloat16>, (const __nv_bfloat16*)p->w2, (const float*)scratch_dev,
-                               q_imp_dev, (int)n_tokens, (int)p->hidden_dim, n_out_i, per_slot, stage_tok);
+    if (p->dtype == TB_BF16) {
+        // eights of tokens staged at once: all of the call's, or equal shares of at most 32
+        auto launch = [&](auto terms, auto eights) {
+            constexpr int kTerms = decltype(terms)::value, kN8 = decltype(eights)::value;
+            constexpr int smem = kWBytes + kTerms * kN8 * 8 * kXPitch;
+            static unsigned char seen[64];
+            if (first_use_on_this_device(seen)) {
+                cudaError_t r = cudaFuncSetAttribute(predictor_hidden_tile_kernel<kTerms, kN8>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+                if (r == cudaSuccess) r = cudaFuncSetAttribute(predictor_out_tile_kernel<kTerms, kN8>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+                if (r != cudaSuccess) return r;
+            }
+            cfg.dynamicSmemBytes = smem;
+            cfg.gridDim = dim3(kClusterK, (p->hidden_dim + kTileRows - 1) / kTileRows, 1), cfg.numAttrs = 2;
+            cudaError_t r = cudaLaunchKernelEx(&cfg, predictor_hidden_tile_kernel<kTerms, kN8>, (const __nv_bfloat16*)hidden_dev,
+                                               (const __nv_bfloat16*)p->ln_weight, (const __nv_bfloat16*)p->ln_bias,
+                                               (const __nv_bfloat16*)p->w1, scratch_dev, (int)n_tokens, (int)p->model_dim,
+                                               (int)p->hidden_dim, p->ln_eps, (int)p->activation);
+            if (r != cudaSuccess) return r;
+            cfg.gridDim = dim3((unsigned)((n_out + kTileRows - 1) / kTileRows), 1, 1), cfg.numAttrs = 1;
+            return cudaLaunchKernelEx(&cfg, predictor_out_tile_kernel<kTerms, kN8>, (const __nv_bfloat16*)p->w2, (const float*)scratch_dev,
+                                      q_imp_dev, (int)n_tokens, (int)p->hidden_dim, n_out_i, per_slot);
+        };
+        const int groups = (n_tokens + kTileTokMax - 1) / kTileTokMax, n8 = ((n_tokens + groups - 1) / groups + 7) / 8;
+        using std::integral_constant;
+        if (n_tokens < 5) e = launch(integral_constant<int, 3>{}, integral_constant<int, 1>{});
+        else if (n8 == 1) e = launch(integral_constant<int, 2>{}, integral_constant<int, 1>{});
+        else if (n8 == 2) e = launch(integral_constant<int, 2>{}, integral_constant<int, 2>{});
+        else if (n8 == 3) e = launch(integral_constant<int, 2>{}, integral_constant<int, 3>{});
+        else e = launch(integral_constant<int, 2>{}, integral_constant<int, 4>{});
     } else {
+        const int g1 = (p->hidden_dim + kPredWarps / 2 - 1) / (kPredWarps / 2), g2 = (int)((n_out + kPredWarps - 1) / kPredWarps);
+        int stage_tok = (int)(48 * 1024 / (p->hidden_dim * sizeof(float))) / kTokChunk * kTokChunk;   // hidden_dim <= 1536 gives >= 8
+        stage_tok = stage_tok > kStageTok ? kStageTok : stage_tok < kTokChunk ? kTokChunk : stage_tok;
         predictor_hidden_kernel<float><<<g1, kPredThreads, 0, s>>>((const float*)hidden_dev, (const float*)p->ln_weight,
                                                                    (const float*)p->ln_bias, (const float*)p->w1, scratch_dev, n_tokens,
                                                                    p->model_dim, p->hidden_dim, p->ln_eps, p->activation);
+        cfg.gridDim = dim3(g2, 1, 1), cfg.numAttrs = 1;
+        cfg.dynamicSmemBytes = (size_t)stage_tok * p->hidden_dim * sizeof(float);
         e = cudaLaunchKernelEx(&cfg, predictor_out_kernel<float>, (const float*)p->w2, (const float*)scratch_dev, q_imp_dev,
                                (int)n_tokens, (int)p->hidden_dim, n_out_i, per_slot, stage_tok);
     }

@@ -493,6 +493,25 @@ def test_predictor_forward_matches_oracle(H, act):
         assert np.abs(got - want).max() <= 2e-4, np.abs(got - want).max()
 
 
+@pytest.mark.parametrize("tokens", [1, 4, 5, 8, 9, 16, 17, 24, 25, 32, 33, 48, 64])
+def test_predictor_tile_edges(H, tokens):
+    """The bf16 tiles at every number of staged token groups, with channel counts that leave a block a partial chunk,
+    several chunks or nothing, and row counts off the 32-row tile.  |error| <= 4e-5 on outputs of magnitude ~2: both
+    left operands are rounded to at least 16 bits, 2^-17 of sums whose terms' norm is ~2, plus fp32 accumulation."""
+    import torch
+    for E, hid, slots, heads, dp in ((4096, 512, 4, 8, 32), (72, 8, 1, 1, 16), (4872, 1032, 3, 3, 32), (8192, 264, 1, 8, 16)):
+        w = wl.workload(2, batch=tokens, n_q_heads=heads, n_kv_heads=1, imp_dim=dp)
+        Hs, ln_w, ln_b, W1, W2 = wl.gen_predictor(w, 1, model_dim=E, hidden_dim=hid, slots=slots)
+        ref = H.orc.predict_queries(Hs, ln_w, ln_b, W1, W2, w.dtype)
+        dev = [H.to_dev(a, w.dtype) for a in (Hs, ln_w, ln_b, W1, W2)]
+        scratch = torch.full((tokens * hid,), float("nan"), dtype=torch.float32, device="cuda")
+        q = torch.full((slots, tokens, heads, dp), float("nan"), dtype=torch.float32, device="cuda")
+        assert tb().predict_importance_queries(*dev, w.dtype, heads, slots, dp, scratch, q) == tb().TB_OK
+        torch.cuda.synchronize()
+        want = ref.reshape(tokens, slots, heads, dp).transpose(1, 0, 2, 3)
+        assert np.abs(q.cpu().numpy() - want).max() <= 4e-5, (E, hid, np.abs(q.cpu().numpy() - want).max())
+
+
 def test_predictor_output_feeds_selection(H):
     """The predictor's output block is the q_imp argument of tb_select_topk for its consumer layers:
     selecting with it on the GPU equals selecting with the oracle's queries in the oracle."""
