@@ -8,53 +8,64 @@ namespace tb {
 
 struct AppendTable {
     int tok_off[kMaxLaunchSeq + 1];  // prefix sums of n_new over the listed sequences
+    int blk_off[kMaxLaunchSeq + 1];  // and of the blocks that copy them
 };
 
-// One thread per 16-byte chunk of a (token, head) K|V row pair.
+// A block belongs to one (layer, sequence); a warp moves 512 contiguous bytes of the cache at a time (a bf16 K|V row
+// pair, or half an fp32 one), kAppendUnroll of them in flight: a copy of 16 bytes per thread and no division per
+// element.  Bound by DRAM bandwidth for prompts and by the launch for a decode token.  32K tokens x 8 heads, one layer
+// (268 MB moved): 70 us with one 16-byte copy in flight per thread, 44 (6.1 TB/s) with eight.
 // The last block to finish advances the device length counters (read by every block of this launch at
 // its start, so they may only change once all have arrived).
+constexpr int kAppendThreads = 256;
+constexpr int kAppendUnroll = 8;
 template <typename T>
-__global__ void append_kernel(Geom gm, UnitTable ut, AppendTable at, int total_new, const T* __restrict__ k_new,
-                              const T* __restrict__ v_new, T* __restrict__ kv, int32_t* __restrict__ len_dev,
-                              uint32_t* __restrict__ counter, int32_t* __restrict__ status, T* __restrict__ res_rows,
-                              int res_sinks, int res_window) {
-    constexpr int kPer16 = Elem<T>::kPer16;
-    const int chunks_per_row = gm.D / kPer16;          // 16-byte chunks in one K (or V) row
-    const int chunks_per_pair = 2 * chunks_per_row;
+__global__ void __launch_bounds__(kAppendThreads) append_kernel(Geom gm, UnitTable ut, AppendTable at, int total_new,
+                                                                const T* __restrict__ k_new, const T* __restrict__ v_new,
+                                                                T* __restrict__ kv, int32_t* __restrict__ len_dev,
+                                                                uint32_t* __restrict__ counter, int32_t* __restrict__ status,
+                                                                T* __restrict__ res_rows, int res_sinks, int res_window) {
+    constexpr int kPer16 = Elem<T>::kPer16, D = 128;
+    constexpr int kRowChunks = D / kPer16, kPieces = 2 * kRowChunks / 32;      // 16-byte chunks of a row, 512-byte pieces of a pair
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int ll = blockIdx.y;
-    const long long work = (long long)total_new * gm.Hkv * chunks_per_pair;
+    int s = 0;
+    for (int step = kMaxLaunchSeq / 2; step > 0; step >>= 1)       // the last sequence that starts at or before this block
+        if (s + step < ut.n_seq && at.blk_off[s + step] <= (int)blockIdx.x) s += step;
+    const int n_s = at.tok_off[s + 1] - at.tok_off[s];
     // Launched as a programmatic dependent (a decode step appends right after the previous layer's
     // attention): resident early, but the new rows may come from the predecessor and the cache rows
     // written here may still be read by it, so wait first; the successor may then get ready.
     pdl_wait();
     pdl_launch_dependents();
-    for (long long w = (long long)blockIdx.x * blockDim.x + threadIdx.x; w < work; w += (long long)gridDim.x * blockDim.x) {
-        int chunk = (int)(w % chunks_per_pair);
-        long long th = w / chunks_per_pair;
-        int h = (int)(th % gm.Hkv);
-        int tok = (int)(th / gm.Hkv);                  // index into the concatenated new tokens
-        int s = 0;
-        while (s + 1 < ut.n_seq && at.tok_off[s + 1] <= tok) ++s;
-        const int base = unit_len(gm, ut, ll, s);
-        if (base + (at.tok_off[s + 1] - at.tok_off[s]) > gm.max_seq_len) continue;   // only a replayed graph gets here (reported below)
-        int pos = base + (tok - at.tok_off[s]);
-        int is_v = chunk >= chunks_per_row;
-        int c16 = is_v ? chunk - chunks_per_row : chunk;
-        const T* src = (is_v ? v_new : k_new) + (((size_t)ll * total_new + tok) * gm.Hkv + h) * gm.D;
-        size_t row = (((size_t)(ut.layer_begin + ll) * gm.max_batch + ut.seq_id[s]) * gm.Hkv + h) * gm.max_seq_len + pos;
-        T* dst = kv + row * 2 * gm.D + (size_t)is_v * gm.D;
-        const uint4 val = reinterpret_cast<const uint4*>(src)[c16];
-        reinterpret_cast<uint4*>(dst)[c16] = val;
-        if (res_rows) {
-            // resident copies (offloaded KV): the first res_sinks tokens, and a ring of the res_window most recent
-            const int n_s = at.tok_off[s + 1] - at.tok_off[s];
-            int slot = -1;
-            if (pos < res_sinks) slot = pos;
-            else if (res_window > 0 && pos >= base + n_s - res_window) slot = res_sinks + pos % res_window;
-            if (slot >= 0) {
-                const size_t unit = ((size_t)(ut.layer_begin + ll) * gm.max_batch + ut.seq_id[s]) * gm.Hkv + h;
-                T* rdst = res_rows + (unit * (size_t)(res_sinks + res_window) + slot) * 2 * gm.D + (size_t)is_v * gm.D;
-                reinterpret_cast<uint4*>(rdst)[c16] = val;
+    const int base = unit_len(gm, ut, ll, s);
+    const unsigned n_piece = (unsigned)n_s * gm.Hkv * kPieces;
+    const unsigned first = (blockIdx.x - at.blk_off[s]) * (kAppendThreads / 32 * kAppendUnroll) + warp;
+    if (base + n_s <= gm.max_seq_len && first < n_piece) {        // (beyond the capacity: only a replayed graph gets here, reported below)
+        const size_t unit0 = ((size_t)(ut.layer_begin + ll) * gm.max_batch + ut.seq_id[s]) * gm.Hkv;
+        const size_t src0 = ((size_t)ll * total_new + at.tok_off[s]) * gm.Hkv;
+        const unsigned hkv = gm.Hkv;
+        uint4 val[kAppendUnroll];
+#pragma unroll
+        for (int i = 0; i < kAppendUnroll; ++i) {
+            const unsigned p = first + i * (kAppendThreads / 32), pair = p / kPieces;   // pair = (token, head), as in the source
+            const unsigned chunk = p % kPieces * 32 + lane;
+            const T* src = (chunk >= kRowChunks ? v_new : k_new) + (src0 + pair) * D;
+            if (p < n_piece) val[i] = __ldcs(reinterpret_cast<const uint4*>(src) + (chunk & (kRowChunks - 1)));
+        }
+#pragma unroll
+        for (int i = 0; i < kAppendUnroll; ++i) {
+            const unsigned p = first + i * (kAppendThreads / 32), pair = p / kPieces, tok = pair / hkv, h = pair - tok * hkv;
+            const unsigned chunk = p % kPieces * 32 + lane;
+            if (p >= n_piece) break;                   // warp-uniform
+            const int pos = base + (int)tok;
+            reinterpret_cast<uint4*>(kv + ((unit0 + h) * gm.max_seq_len + pos) * 2 * D)[chunk] = val[i];
+            if (res_rows) {
+                // resident copies (offloaded KV): the first res_sinks tokens, and a ring of the res_window most recent
+                int slot = -1;
+                if (pos < res_sinks) slot = pos;
+                else if (res_window > 0 && pos >= base + n_s - res_window) slot = res_sinks + pos % res_window;
+                if (slot >= 0) reinterpret_cast<uint4*>(res_rows + ((unit0 + h) * (size_t)(res_sinks + res_window) + slot) * 2 * D)[chunk] = val[i];
             }
         }
     }
@@ -73,17 +84,18 @@ __global__ void append_kernel(Geom gm, UnitTable ut, AppendTable at, int total_n
 
 cudaError_t launch_append(const tb_ctx* c, const UnitTable& ut, const int* n_new, const int* tok_off, int total_new,
                           const void* k, const void* v, cudaStream_t s) {
-    (void)n_new;
     AppendTable at;
     for (int i = 0; i <= ut.n_seq; ++i) at.tok_off[i] = tok_off[i];
     const Geom& gm = c->geom;
-    int es = gm.dtype == TB_BF16 ? 2 : 4;
-    long long work = (long long)total_new * gm.Hkv * (2 * gm.D * es / 16);
-    int threads = 256;
-    long long blocks = (work + threads - 1) / threads;
-    if (blocks > 148 * 16) blocks = 148 * 16;
+    constexpr int per_block = kAppendThreads / 32 * kAppendUnroll;
+    at.blk_off[0] = 0;
+    for (int i = 0; i < ut.n_seq; ++i) {
+        const long long pieces = (long long)n_new[i] * gm.Hkv * (gm.dtype == TB_BF16 ? 1 : 2);
+        at.blk_off[i + 1] = at.blk_off[i] + (int)((pieces + per_block - 1) / per_block);
+    }
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)blocks, ut.layer_count, 1), cfg.blockDim = dim3(threads, 1, 1), cfg.dynamicSmemBytes = 0, cfg.stream = s;
+    cfg.gridDim = dim3((unsigned)at.blk_off[ut.n_seq], ut.layer_count, 1);
+    cfg.blockDim = dim3(kAppendThreads, 1, 1), cfg.dynamicSmemBytes = 0, cfg.stream = s;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;   // see pdl_wait()
     attr[0].val.programmaticStreamSerializationAllowed = 1;
@@ -161,17 +173,23 @@ __device__ __forceinline__ void project_finish(const Geom& gm, const UnitTable& 
     }
 }
 
-constexpr int kProjTokens = 32;   // tokens per block
-constexpr int kProjThreads = 128; // 4 threads per token, each owning dp/4 outputs
+// fp32 storage: CUDA-core tiles of 64 tokens x d' outputs, 8 outputs of DP / 16 tokens per thread, so that the FMA
+// units and not the shared-memory reads bound it (per four channels and token: a 16-byte read of K and, shared by the
+// thread's tokens, eight of W for 32 FMAs).  K rows arrive by 16-byte cp.async; four blocks per SM hide their latency.
+// 32K tokens x 8 heads x 2 layers (335 MB): 329 us with one token and d' / 4 outputs per thread, 162 like this.
+constexpr int kProjTokens = 64;   // tokens per block
+constexpr int kProjThreads = 128;
 
-template <typename T, int DP>
-__global__ void __launch_bounds__(kProjThreads) project_kernel(Geom gm, UnitTable ut, ProjectTable pt, const T* __restrict__ kv,
-                                                               const T* __restrict__ Wall, T* __restrict__ kimp,
-                                                               int32_t* __restrict__ len_proj_dev, uint32_t* __restrict__ counter) {
+template <int DP>
+__global__ void __launch_bounds__(kProjThreads, 4) project_kernel(Geom gm, UnitTable ut, ProjectTable pt, const float* __restrict__ kv,
+                                                                  const float* __restrict__ Wall, float* __restrict__ kimp,
+                                                                  int32_t* __restrict__ len_proj_dev, uint32_t* __restrict__ counter) {
     constexpr int D = 128;
-    constexpr int JPT = DP / 4;                       // outputs per thread
-    __shared__ float Ws[D * DP];
-    __shared__ float Ks[kProjTokens][D + 1];
+    constexpr int kPitch = D + 4;                     // floats per K row: eight rows' 16-byte pieces hit all banks once
+    constexpr int OG = DP / 8, TG = kProjThreads / OG, TPT = kProjTokens / TG;   // output groups, token groups, tokens per thread
+    extern __shared__ __align__(128) unsigned char smem[];
+    float* Ws = reinterpret_cast<float*>(smem);       // [channel][DP]
+    float* Ks = Ws + D * DP;                          // [token][kPitch]
 
     const int ll = blockIdx.z / ut.n_seq, s = blockIdx.z % ut.n_seq, h = blockIdx.y;
     const int layer = ut.layer_begin + ll;
@@ -182,38 +200,54 @@ __global__ void __launch_bounds__(kProjThreads) project_kernel(Geom gm, UnitTabl
 
     // One key stream per KV head, or (one list per layer) a single stream that sums the heads'
     // projections: K_imp[t] = sum_h K[t][h] . W[h], heads in ascending order on one fp32 chain.
-    const int n_sum = gm.Hkv / gm.Hi;
+    const int n_sum = nt ? gm.Hkv / gm.Hi : 0;
     const size_t pair = (size_t)layer * gm.max_batch + ut.seq_id[s];
-    const int t = threadIdx.x / 4, jq = threadIdx.x % 4;
-    float acc[JPT];
+    const int og = threadIdx.x % OG, tg = threadIdx.x / OG;
+    float acc[TPT][8];
 #pragma unroll
-    for (int j = 0; j < JPT; ++j) acc[j] = 0.f;
+    for (int i = 0; i < TPT; ++i)
+#pragma unroll
+        for (int j = 0; j < 8; ++j) acc[i][j] = 0.f;
     for (int hs = 0; hs < n_sum; ++hs) {
         const int hk = h * n_sum + hs;
-        const T* W = Wall + ((size_t)layer * gm.Hkv + hk) * D * DP;
-        if (hs) __syncthreads();
-        for (int i = threadIdx.x; i < D * DP; i += kProjThreads) Ws[i] = Elem<T>::to_f32(W[i]);
-        if (nt == 0) break;
-        const size_t krow0 = (pair * gm.Hkv + hk) * gm.max_seq_len + t0;
-        for (int i = threadIdx.x; i < nt * D; i += kProjThreads) {
-            int tt = i / D, ch = i % D;
-            Ks[tt][ch] = Elem<T>::to_f32(kv[(krow0 + tt) * 2 * D + ch]);
-        }
-        __syncthreads();
-        if (t < nt) {
+        const float* W = Wall + ((size_t)layer * gm.Hkv + hk) * D * DP;
+        const float* K = kv + ((pair * gm.Hkv + hk) * gm.max_seq_len + t0) * 2 * D;
+        if (hs) __syncthreads();                      // the previous head's tiles are consumed
+        for (int i = threadIdx.x; i < D * DP / 4; i += kProjThreads)
+            asm volatile("cp.async.ca.shared.global [%0], [%1], 16;" ::"r"(smem_u32(Ws + i * 4)), "l"(W + i * 4) : "memory");
 #pragma unroll 4
-            for (int ch = 0; ch < D; ++ch) {
-                float kx = Ks[t][ch];
-#pragma unroll
-                for (int j = 0; j < JPT; ++j) acc[j] = fmaf(kx, Ws[ch * DP + jq * JPT + j], acc[j]);
-            }
+        for (int i = threadIdx.x; i < nt * (D / 4); i += kProjThreads) {
+            const int t = i / (D / 4), c = i % (D / 4) * 4;
+            asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(Ks + t * kPitch + c)), "l"(K + (size_t)t * 2 * D + c) : "memory");
         }
-    }
-    if (t < nt) {
-        const size_t row0 = (pair * gm.Hi + h) * gm.max_seq_len + t0;
-        T* dst = kimp + (row0 + t) * DP + jq * JPT;
+        asm volatile("cp.async.commit_group;\ncp.async.wait_group 0;" ::: "memory");
+        __syncthreads();
+        if (tg < nt)                                  // (rows past the range hold whatever: their results are not stored)
+#pragma unroll 2
+            for (int c = 0; c < D; c += 4) {
+                float4 k[TPT];
 #pragma unroll
-        for (int j = 0; j < JPT; ++j) dst[j] = Elem<T>::from_f32(acc[j]);
+                for (int i = 0; i < TPT; ++i) k[i] = *reinterpret_cast<const float4*>(Ks + (tg + i * TG) * kPitch + c);
+#pragma unroll
+                for (int e = 0; e < 4; ++e) {
+                    const float4 w0 = *reinterpret_cast<const float4*>(Ws + (c + e) * DP + og * 8), w1 = *reinterpret_cast<const float4*>(Ws + (c + e) * DP + og * 8 + 4);
+                    const float w[8] = {w0.x, w0.y, w0.z, w0.w, w1.x, w1.y, w1.z, w1.w};
+#pragma unroll
+                    for (int i = 0; i < TPT; ++i) {
+                        const float kx = e == 0 ? k[i].x : e == 1 ? k[i].y : e == 2 ? k[i].z : k[i].w;
+#pragma unroll
+                        for (int j = 0; j < 8; ++j) acc[i][j] = fmaf(kx, w[j], acc[i][j]);
+                    }
+                }
+            }
+    }
+#pragma unroll
+    for (int i = 0; i < TPT; ++i) {
+        const int t = tg + i * TG;
+        if (t >= nt) break;
+        float* dst = kimp + ((pair * gm.Hi + h) * gm.max_seq_len + t0 + t) * DP + og * 8;
+        *reinterpret_cast<float4*>(dst) = make_float4(acc[i][0], acc[i][1], acc[i][2], acc[i][3]);
+        *reinterpret_cast<float4*>(dst + 4) = make_float4(acc[i][4], acc[i][5], acc[i][6], acc[i][7]);
     }
     project_finish(gm, ut, pt, len_proj_dev, counter);
 }
@@ -366,11 +400,17 @@ cudaError_t launch_project(const tb_ctx* c, const UnitTable& ut, const int* pos_
         return cudaGetLastError();
     }
     dim3 grid((max_range + kProjTokens - 1) / kProjTokens, gm.Hi, ut.layer_count * ut.n_seq);
-#define TB_PROJ(T, DP) \
-    project_kernel<T, DP><<<grid, kProjThreads, 0, s>>>(gm, ut, pt, (const T*)c->kv, (const T*)c->st.W, (T*)c->kimp, c->st.len_proj, c->st.misc_counter + 1)
-    if (gm.dp == 32) TB_PROJ(float, 32); else TB_PROJ(float, 16);
-#undef TB_PROJ
-    return cudaGetLastError();
+    auto launch = [&](auto kernel, unsigned char (&seen)[64]) {
+        const int smem = (128 * gm.dp + kProjTokens * (128 + 4)) * 4;
+        if (first_use_on_this_device(seen)) {
+            cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+            if (e != cudaSuccess) return e;
+        }
+        kernel<<<grid, kProjThreads, smem, s>>>(gm, ut, pt, (const float*)c->kv, (const float*)c->st.W, (float*)c->kimp, c->st.len_proj, c->st.misc_counter + 1);
+        return cudaGetLastError();
+    };
+    static unsigned char seen32[64], seen16[64];
+    return gm.dp == 32 ? launch(project_kernel<32>, seen32) : launch(project_kernel<16>, seen16);
 }
 
 }  // namespace tb
