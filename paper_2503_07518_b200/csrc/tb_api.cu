@@ -441,8 +441,18 @@ tb_status tb_select_topk(tb_ctx* c, int32_t lb, int32_t lc, const int32_t* seq_i
             UnitTable ut;
             fill_table(c, &ut, l0, n, seqs, n_seq);
             const size_t unit_off = (size_t)(l0 - lb) * n_seq * c->geom.Hl;
+            bool finished = false;                       // the selection kernel has done neighbours and the caller's copy too
             if (refresh) {
+                int max_cand = 0;
+                for (int i = 0; i < n * n_seq; ++i) {
+                    int lo, hi;
+                    cand_range(ut.len[i], p->sinks, p->recent, &lo, &hi);
+                    if (hi - lo > max_cand) max_cand = hi - lo;
+                }
+                finished = select_small_takes(c, ut, max_cand, p->radius > 0 || idx_out || cnt_out);
                 SelectArgs a;
+                a.radius = p->radius, a.nmode = p->nmode;
+                a.idx_copy = idx_out ? idx_out + unit_off * c->geom.idx_cap : nullptr, a.cnt_copy = cnt_out ? cnt_out + unit_off : nullptr;
                 a.q_imp = q_imp + (size_t)(l0 - lb) * n_seq * c->geom.Hl * c->geom.gl * c->cfg.imp_dim;
                 a.budget = p->budget, a.sinks = p->sinks, a.recent = p->recent, a.reduce = reduce;
                 if (p->radius == 0) {
@@ -450,10 +460,11 @@ tb_status tb_select_topk(tb_ctx* c, int32_t lb, int32_t lc, const int32_t* seq_i
                 } else {
                     a.idx_dst = c->wk.sel_idx, a.cnt_dst = c->wk.sel_cnt, a.dst_is_state = 0, a.idx_stride = c->wk.sel_stride;
                 }
-                cudaError_t e = launch_select(c, ut, a, (cudaStream_t)stream, dry);
+                cudaError_t e = finished ? launch_select_small(c, ut, a, max_cand, (cudaStream_t)stream, dry)
+                                         : launch_select(c, ut, a, (cudaStream_t)stream, dry);
                 if (e != cudaSuccess) return dry ? TB_ERR_UNSUPPORTED : TB_ERR_CUDA;
                 if (!dry) c->last_list_write = (long long)c->launches, c->launches++;
-                if (p->radius > 0) {
+                if (p->radius > 0 && !finished) {
                     NeighborArgs na;
                     na.idx_src = c->wk.sel_idx, na.cnt_src = c->wk.sel_cnt, na.src_stride = c->wk.sel_stride;
                     na.radius = p->radius, na.nmode = p->nmode, na.sinks = p->sinks, na.recent = p->recent;
@@ -466,7 +477,7 @@ tb_status tb_select_topk(tb_ctx* c, int32_t lb, int32_t lc, const int32_t* seq_i
                     c->last_list_write = (long long)c->launches, c->launches++;
                 }
             }
-            if (!dry && (idx_out || cnt_out)) {
+            if (!dry && (idx_out || cnt_out) && !finished) {
                 if (launch_copy_lists(c, ut, idx_out ? idx_out + unit_off * c->geom.idx_cap : nullptr,
                                       cnt_out ? cnt_out + unit_off : nullptr, (cudaStream_t)stream) != cudaSuccess)
                     return TB_ERR_CUDA;

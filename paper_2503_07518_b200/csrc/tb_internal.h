@@ -54,6 +54,11 @@ struct SelectArgs {
     int idx_stride;
     int budget, sinks, recent;
     int reduce;           // tb_group_reduce: TB_GROUP_SUM or TB_GROUP_MAX
+    // Read by the kernels that finish a list themselves (neighbours, the caller's copy); the others are followed by
+    // the neighbour and copy kernels.
+    int radius, nmode;
+    int32_t* idx_copy;    // [layer_count][n_seq][Hl][idx_cap] or NULL
+    int32_t* cnt_copy;
 };
 
 struct NeighborArgs {
@@ -197,6 +202,10 @@ cudaError_t launch_score(const tb_ctx* c, const UnitTable& ut, const float* q_im
 cudaError_t launch_select(const tb_ctx* c, const UnitTable& ut, const SelectArgs& a, cudaStream_t s, bool dry = false);
 // one block per problem; launch_select hands over to it when a launch holds at least two problems per SM
 cudaError_t launch_select_wave(const tb_ctx* c, const UnitTable& ut, const SelectArgs& a, cudaStream_t s, bool dry = false);
+// small problems: one block each, neighbours and the caller's copy of the list included; whether a launch whose longest
+// problem has max_cand candidates is its kind (more: neighbours or copies are wanted)
+bool select_small_takes(const tb_ctx* c, const UnitTable& ut, int max_cand, bool more);
+cudaError_t launch_select_small(const tb_ctx* c, const UnitTable& ut, const SelectArgs& a, int max_cand, cudaStream_t s, bool dry = false);
 // few, long problems: a cluster per problem on parked keys
 cudaError_t launch_select_cw(const tb_ctx* c, const UnitTable& ut, const SelectArgs& a, cudaStream_t s, bool dry = false);
 cudaError_t launch_neighbors(const tb_ctx* c, const UnitTable& ut, const NeighborArgs& a, cudaStream_t s, bool dry = false);

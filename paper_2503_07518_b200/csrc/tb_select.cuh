@@ -2,6 +2,8 @@
 // and the fused kernel produce bit-identical scores) and the launch-unit decoding.
 #pragma once
 
+#include <type_traits>
+
 #include "tb_common.cuh"
 #include "tb_internal.h"
 
@@ -129,6 +131,227 @@ __device__ __forceinline__ void check_candidates_projected(const Geom& gm, const
         const size_t pair = (size_t)(ut.layer_begin + ll) * gm.max_batch + ut.seq_id[s];
         if (ut.len_proj_dev[pair] < hi) atomicExch(status, kStatusUnprojected);
     }
+}
+
+// ---- bf16 rows straight into tensor-core fragments ------------------------------------------------------
+//
+// Over a 64-byte row (32 dimensions) thread tig of a row's four takes 16 contiguous bytes, so a warp's 16-byte load is
+// eight whole rows, and with the query's dimensions permuted the same way the four 4-byte words are the A operand of two
+// m16n8k16 steps (8 bytes and one step for 16 dimensions).  No shared memory, no barrier; every warp keeps kU groups of 32
+// rows in flight.   D[16 rows x 8] += K[16 x 16] . Q[16 x 8], fp32 accumulators; Q is split into three bf16 terms that hold
+// all 24 bits of the fp32 query, lowest term first, so every product is exact and only the fp32 sums round (against fp64:
+// rms error 1.4e-8 of sum |q k|, where the FMA chains above have 2.0e-8).  TB_GROUP_SUM: all eight columns hold the summed
+// query and a lane keeps the value that belongs to its row; TB_GROUP_MAX: column = head, a row's score is the largest over
+// the columns.  A row's score depends only on its bytes, never on where it sits.
+constexpr int kQueryFrags = 3 * 2 * 32;   // a query's B fragments: terms x steps x lanes
+
+__device__ __forceinline__ void mma_16816(float (&d)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0, uint32_t b1) {
+    asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
+                 : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
+                 : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
+}
+
+template <int DP, int RED>
+struct FragScorer {
+    static constexpr int kSteps = DP / 16, kTerms = 3, kRowBytes = DP * 2;
+    typedef typename std::conditional<DP == 32, uint4, uint2>::type Piece;    // a thread's quarter of a row
+    const uint2* frag;                                 // this lane's B fragments, [term][step][lane], in shared memory
+    // Called by all threads of the block with the queries staged and visible; `frags` holds kQueryFrags entries.
+    __device__ __forceinline__ void load_staged(const float* qs, int g, uint2* frags) {
+        const int lane = threadIdx.x & 31, st = threadIdx.x >> 5, gid = lane >> 2, tig = lane & 3;
+        frag = frags + lane;
+        if (st < kSteps) {
+            uint32_t b[kTerms][2];
+#pragma unroll
+            for (int half = 0; half < 2; ++half) {
+                const int k = tig * (DP / 4) + st * 4 + half * 2;             // the dimensions of word 2 st + half of the piece
+                float x, y;
+                if constexpr (RED == TB_GROUP_SUM) {
+                    x = y = 0.f;
+                    for (int u = 0; u < g; ++u) {      // in head order
+                        const float2 v = *reinterpret_cast<const float2*>(qs + u * DP + k);
+                        x += v.x, y += v.y;
+                    }
+                } else {
+                    const float2 v = *reinterpret_cast<const float2*>(qs + min(gid, g - 1) * DP + k);
+                    x = v.x, y = v.y;
+                }
+#pragma unroll
+                for (int t = 0; t < kTerms; ++t) {
+                    const __nv_bfloat162 v = __floats2bfloat162_rn(x, y);
+                    b[t][half] = *reinterpret_cast<const uint32_t*>(&v);
+                    x -= __low2float(v), y -= __high2float(v);
+                }
+            }
+#pragma unroll
+            for (int t = 0; t < kTerms; ++t) frags[(t * kSteps + st) * 32 + lane] = make_uint2(b[t][0], b[t][1]);
+        }
+        __syncthreads();
+    }
+    // v[m]: this thread's piece of row 8 m + gid of the 32; returns the score of the row this lane looks after (my_row)
+    __device__ __forceinline__ float score(const Piece (&v)[4], int row0, int& my_row) const {
+        const int lane = threadIdx.x & 31, gid = lane >> 2, tig = lane & 3;
+        float d[2][4];
+#pragma unroll
+        for (int m = 0; m < 2; ++m) d[m][0] = d[m][1] = d[m][2] = d[m][3] = 0.f;
+#pragma unroll
+        for (int t = kTerms - 1; t >= 0; --t) {
+            const uint2 b0 = frag[t * kSteps * 32];
+            mma_16816(d[0], v[0].x, v[1].x, v[0].y, v[1].y, b0.x, b0.y);
+            mma_16816(d[1], v[2].x, v[3].x, v[2].y, v[3].y, b0.x, b0.y);
+            if constexpr (DP == 32) {
+                const uint2 b1 = frag[(t * kSteps + 1) * 32];
+                mma_16816(d[0], v[0].z, v[1].z, v[0].w, v[1].w, b1.x, b1.y);
+                mma_16816(d[1], v[2].z, v[3].z, v[2].w, v[3].w, b1.x, b1.y);
+            }
+        }
+        // lane (gid, tig) takes row gid + 8 tig: accumulator 0 / 2 of the first 16 rows, then of the second
+        my_row = row0 + gid + 8 * tig;
+        float r[4] = {d[0][0], d[0][2], d[1][0], d[1][2]};
+        if constexpr (RED == TB_GROUP_MAX) {
+            r[0] = fmaxf(r[0], d[0][1]), r[1] = fmaxf(r[1], d[0][3]), r[2] = fmaxf(r[2], d[1][1]), r[3] = fmaxf(r[3], d[1][3]);
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                r[i] = fmaxf(r[i], __shfl_xor_sync(0xffffffffu, r[i], 1));
+                r[i] = fmaxf(r[i], __shfl_xor_sync(0xffffffffu, r[i], 2));
+            }
+        }
+        const float lo = tig & 1 ? r[1] : r[0], hi = tig & 1 ? r[3] : r[2];
+        return tig & 2 ? hi : lo;
+    }
+    // rows at `rows` (the first of the 32), n of them exist
+    __device__ __forceinline__ static void load(Piece (&v)[4], const unsigned char* rows, int n) {
+        const int lane = threadIdx.x & 31, gid = lane >> 2, tig = lane & 3;
+        const unsigned char* p = rows + gid * kRowBytes + tig * (kRowBytes / 4);
+#pragma unroll
+        for (int m = 0; m < 4; ++m)
+            if (8 * m + gid < n) v[m] = __ldcg(reinterpret_cast<const Piece*>(p + 8 * m * kRowBytes));
+    }
+};
+
+// The bf16 stream of a block: rows [0, n) from `rows`, in groups of 32 dealt to the warps in turn, kU groups per warp in
+// flight.
+template <int DP, int RED, int kU>
+struct RowStream {
+    typedef FragScorer<DP, RED> Scorer;
+    typename Scorer::Piece v[kU][4];
+    const unsigned char* rows;
+    int n, warp, n_warps;
+    __device__ __forceinline__ void load(int u, int g) {
+        if (g * 32 < n) Scorer::load(v[u], rows + (size_t)g * 32 * Scorer::kRowBytes, n - g * 32);
+    }
+    __device__ __forceinline__ void start(const unsigned char* rows_, int n_) {
+        rows = rows_, n = n_, warp = threadIdx.x >> 5, n_warps = blockDim.x >> 5;
+#pragma unroll
+        for (int u = 0; u < kU; ++u) {
+#pragma unroll
+            for (int m = 0; m < 4; ++m) v[u][m] = {};
+            load(u, u * n_warps + warp);
+        }
+    }
+    // consume(slot, score) for every row
+    template <typename F>
+    __device__ __forceinline__ void run(const Scorer& scorer, F&& consume) {
+        for (int g0 = warp; g0 * 32 < n; g0 += kU * n_warps) {
+#pragma unroll
+            for (int u = 0; u < kU; ++u) {
+                const int g = g0 + u * n_warps;
+                if (g * 32 >= n) break;                // warp-uniform
+                int slot;
+                const float sc = scorer.score(v[u], g * 32, slot);
+                load(u, g + kU * n_warps);
+                if (slot < n) consume(slot, sc);
+            }
+        }
+    }
+};
+
+// ---- from a bitmask of the candidates to the list -------------------------------------------------------
+// Bit i of `mask` = candidate i (token lo + i) is selected; n_bits candidates, bits past them zero.
+
+// Neighbour fetching on the mask (paper Sec. 3.4): `out` (as many words as mask, in other memory) = the selection with
+// its neighbours, clipped to the candidates.  DILATE: every position within `radius`.  CLUSTER: every run of consecutive
+// positions [a, b] gets radius * (b - a + 1) extra positions just outside, the larger half after b.  All threads call
+// it, with `mask` complete and visible; `out` is visible to all on return.
+template <int kThreads>
+__device__ __forceinline__ void expand_mask(const uint32_t* mask, uint32_t* out, int n_bits, int radius, int nmode) {
+    const int n_words = (n_bits + 31) / 32;
+    const uint32_t last = n_bits & 31 ? (1u << (n_bits & 31)) - 1u : 0xffffffffu;
+    if (nmode == TB_NEIGHBOR_DILATE) {
+        for (int w = threadIdx.x; w < n_words; w += kThreads) {
+            uint32_t m = mask[w];
+            for (int d = 1; d <= radius; ++d) {        // bits d positions up and down
+                const int wd = d >> 5, sh = d & 31;
+                const uint32_t lo1 = w - wd >= 0 ? mask[w - wd] : 0u, lo2 = w - wd - 1 >= 0 ? mask[w - wd - 1] : 0u;
+                const uint32_t hi1 = w + wd < n_words ? mask[w + wd] : 0u, hi2 = w + wd + 1 < n_words ? mask[w + wd + 1] : 0u;
+                m |= __funnelshift_l(lo2, lo1, sh) | __funnelshift_r(hi1, hi2, sh);
+            }
+            out[w] = w == n_words - 1 ? m & last : m;
+        }
+        __syncthreads();
+        return;
+    }
+    for (int w = threadIdx.x; w < n_words; w += kThreads) out[w] = mask[w];
+    __syncthreads();
+    auto mark = [&](long long from, long long to) {    // positions [from, to), clipped
+        for (int x = (int)max(0ll, from); x < (int)min((long long)n_bits, to); ++x) atomicOr(&out[x >> 5], 1u << (x & 31));
+    };
+    for (int w = threadIdx.x; w < n_words; w += kThreads) {
+        const uint32_t m = mask[w];
+        uint32_t starts = m & ~((m << 1) | (w ? mask[w - 1] >> 31 : 0u));
+        while (starts) {
+            const int a = w * 32 + __ffs(starts) - 1;
+            starts &= starts - 1;
+            int e = a;                                 // first position behind the run
+            while (e < n_words * 32) {
+                const int sh = e & 31;
+                const uint32_t rest = ~mask[e >> 5] >> sh;
+                if (rest) { e += __ffs(rest) - 1; break; }
+                e += 32 - sh;
+            }
+            e = min(e, n_bits);
+            const long long n = (long long)radius * (e - a);
+            mark(e, e + (n + 1) / 2), mark(a - n / 2, a);
+        }
+    }
+    __syncthreads();
+}
+
+// Writes the ascending list of a mask: its first `limit` positions, as tokens, to dst and (unless null) to copy.
+// Returns the number of bits.  A thread owns a run of 16-bit half words; `slots` holds kThreads / 32 ints.
+template <int kThreads>
+__device__ __forceinline__ int write_mask_list(const uint32_t* mask, int n_bits, int lo, int limit, int32_t* __restrict__ dst,
+                                               int32_t* __restrict__ copy, int* slots) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const uint16_t* mask16 = reinterpret_cast<const uint16_t*>(mask);
+    const int n_half = (n_bits + 15) / 16;
+    const int per = (n_half + kThreads - 1) / kThreads;
+    const int w0 = min(n_half, (int)threadIdx.x * per), w1 = min(n_half, w0 + per);
+    int cnt = 0;
+    for (int w = w0; w < w1; ++w) cnt += __popc((uint32_t)mask16[w]);
+    const int incl = warp_incl_scan(cnt, lane);
+    if (lane == 31) slots[warp] = incl;
+    __syncthreads();
+    int o = incl - cnt, total = 0;
+#pragma unroll
+    for (int w = 0; w < kThreads / 32; ++w) {
+        const int x = slots[w];
+        total += x;
+        o += w < warp ? x : 0;
+    }
+    for (int w = w0; w < w1; ++w) {
+        uint32_t bits = mask16[w];
+        while (bits) {
+            const int t = lo + w * 16 + __ffs(bits) - 1;
+            bits &= bits - 1;
+            if (o < limit) {
+                dst[o] = t;
+                if (copy) copy[o] = t;
+            }
+            ++o;
+        }
+    }
+    return total;
 }
 
 }  // namespace tb

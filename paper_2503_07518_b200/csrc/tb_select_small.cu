@@ -1,0 +1,366 @@
+// Selection of small problems: scoring, exact top-B, neighbour fetching and the copy of the list for the caller, one
+// block per (layer, sequence, list), one launch (paper Sec. 3.4, Sec. 4 "Token Selection Policy").
+//
+// A problem of a few thousand candidates is 32 to 512 KB of projected keys: one SM takes it in within 1 to 6 us, and
+// what a launch costs beyond that is latency.  So everything stays inside one block of 512 threads:
+//   stream   bf16 rows straight into tensor-core fragments (see RowStream), fp32 rows through 2-D TMA tiles of 256 rows, all
+//            requested at once when they fit; the order-preserving key goes to shared memory, score sums stay in registers
+//   digit    mean and deviation of all the scores place 2046 equal slices of score across mean +- 4.5 deviations (one
+//            barrier), an open bin on either side; bins are monotone in the score whatever the moments say, so the
+//            selection never depends on them, only how few keys share the threshold's bin does (a handful)
+//   finish   histogram, threshold bin, bitmask, the bin's keys ranked pairwise (equal scores by position), neighbours
+//            on the bitmask, list
+// A crowded threshold bin (massive ties, a few huge outliers) goes through the key's own digits instead (11 + 11 + 10).
+//
+// The launch is a programmatic dependent: no clusters, so an early start cannot misplace anything.
+#include "tb_select.cuh"
+
+namespace tb {
+
+namespace {
+
+constexpr int kThreads = 512;
+constexpr int kWarps = kThreads / 32;
+constexpr int kHalf = 256;          // rows of a tile = threads that score it
+constexpr int kMaxCand = 8192;      // one bitmask half word per thread
+constexpr int kBins = 2048;
+constexpr int kMaxRank = kThreads;  // keys of the threshold bin that are ranked pairwise
+
+struct __align__(16) SmallSmem {
+    int hist[kBins];
+    uint32_t mask[kMaxCand / 32], mask_out[kMaxCand / 32];
+    uint2 cand[kMaxRank];           // (key, candidate) of the threshold bin
+    float qs[kMaxGroup * 32];       // the list's importance queries
+    uint2 frags[kQueryFrags];       // ... as tensor-core operands
+    uint64_t full[kMaxCand / kHalf];
+    float part[kWarps][2];
+    int slots[kWarps];
+    int bin, krem, count, n_cand;
+};
+
+__device__ __forceinline__ float key_score(uint32_t key) { return __uint_as_float(key & 0x80000000u ? key & 0x7fffffffu : ~key); }
+
+// The bin that holds the k-th largest of the histogrammed keys: all threads get it, with k' = k - keys in higher bins
+// and the bin's population.  1 <= k <= total.
+__device__ __forceinline__ void find_bin(SmallSmem* sm, int nbins, int k, int& bin, int& krem, int& count) {
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    int b[4] = {0, 0, 0, 0};
+    if (tid * 4 < nbins) {
+        const int4 x = reinterpret_cast<const int4*>(sm->hist)[tid];
+        b[0] = x.x, b[1] = x.y, b[2] = x.z, b[3] = x.w;
+    }
+    const int mine = (b[0] + b[1]) + (b[2] + b[3]);
+    const int incl = warp_incl_scan(mine, lane);
+    if (lane == 31) sm->slots[warp] = incl;
+    __syncthreads();
+    int below = incl - mine, total = 0;
+#pragma unroll
+    for (int w = 0; w < kWarps; ++w) {
+        const int x = sm->slots[w];
+        total += x;
+        below += w < warp ? x : 0;
+    }
+    int run = total - below - mine;                    // keys in bins above this thread's
+    if (run < k && k <= run + mine) {                  // exactly one thread
+#pragma unroll
+        for (int i = 3; i >= 0; --i) {
+            if (run < k && k <= run + b[i]) sm->bin = tid * 4 + i, sm->krem = k - run, sm->count = b[i];
+            run += b[i];
+        }
+    }
+    __syncthreads();
+    bin = sm->bin, krem = sm->krem, count = sm->count;
+}
+
+struct NoStream {
+    __device__ __forceinline__ void start(const unsigned char*, int) {}
+};
+
+// bf16 rows: kU groups of 32 rows in flight per warp (see RowStream); fp32 rows (kU = 0): through a ring of n_stages tiles
+template <typename T, int DP, int RED, int kU>
+__global__ void __launch_bounds__(kThreads, kU == 2 ? 2 : 1) select_small_kernel(const __grid_constant__ CUtensorMap tmap,
+                                                                                 const unsigned char* __restrict__ kimp, Geom gm, UnitTable ut,
+                                                                                 SelectArgs a, int n_stages, int max_tiles, uint32_t wait_limit,
+                                                                                 int32_t* __restrict__ state_idx, int32_t* __restrict__ state_cnt,
+                                                                                 int32_t* __restrict__ status) {
+    constexpr int RB = DP * Elem<T>::kBytes, NCH = RB / 16;
+    constexpr uint32_t kTileBytes = kHalf * RB;
+    constexpr bool kDirect = kU > 0;
+    extern __shared__ unsigned char smem_raw[];
+    unsigned char* ring = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);   // swizzled boxes start on the swizzle period
+    uint32_t* keys = reinterpret_cast<uint32_t*>(ring + n_stages * kTileBytes);          // max_tiles * 256
+    SmallSmem* sm = reinterpret_cast<SmallSmem*>(keys + max_tiles * kHalf);
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+
+    // What needs nothing from the predecessor runs beside its tail.
+    if (tid == 0) sm->n_cand = 0;
+    if (!kDirect && tid == 0) prefetch_tmap(&tmap);
+    if (!kDirect && tid < n_stages) mbar_init(&sm->full[tid], 1), fence_mbar_init();
+    reinterpret_cast<int4*>(sm->hist)[tid] = make_int4(0, 0, 0, 0);
+    int ll, s, h;
+    decode_unit(gm, ut, blockIdx.x, ll, s, h);
+    const size_t cu = list_unit(gm, ut, ll, s, h);
+    int32_t* idx_dst = state_idx + cu * gm.idx_cap;
+    int32_t* idx_copy = a.idx_copy ? a.idx_copy + (size_t)blockIdx.x * gm.idx_cap : nullptr;
+    int32_t* cnt_copy = a.cnt_copy ? a.cnt_copy + blockIdx.x : nullptr;
+    pdl_wait();
+    pdl_launch_dependents();                           // (waits for this grid's completion before it reads a list)
+
+    const int L = unit_len(gm, ut, ll, s);
+    const int lo = min(a.sinks, L), hi = max(lo, L - a.recent), ncand = hi - lo;
+    const int k = min(a.budget, ncand);
+    check_candidates_projected(gm, ut, ll, s, hi, status);
+    if (k <= 0 || k == ncand) {                        // nothing to rank: none, or all (neighbours add nothing then)
+        for (int i = tid; i < k; i += kThreads) {
+            idx_dst[i] = lo + i;
+            if (idx_copy) idx_copy[i] = lo + i;
+        }
+        if (tid == 0) {
+            state_cnt[cu] = max(k, 0);
+            if (cnt_copy) *cnt_copy = max(k, 0);
+        }
+        return;
+    }
+    const int n_tiles = (ncand + kHalf - 1) / kHalf;   // <= max_tiles
+    const long long row0 = (long long)key_unit(gm, ut, ll, s, h) * gm.max_seq_len + lo;
+    auto request = [&](int t) {                        // tile t, into its stage
+        uint64_t* bar = &sm->full[t % n_stages];
+        mbar_arrive_expect_tx(bar, kTileBytes);
+        tma_load_2d(ring + t % n_stages * kTileBytes, &tmap, 0, (int)(row0 + (long long)t * kHalf), bar);
+    };
+    if (!kDirect && tid == 0)
+        for (int t = 0; t < min(n_stages, n_tiles); ++t) request(t);
+    if (tid < gm.gl * DP) sm->qs[tid] = a.q_imp[query_row(gm, ut, ll, s, h) * DP + tid];
+    typename std::conditional<kDirect, RowStream<DP, RED, kDirect ? kU : 1>, NoStream>::type rs;
+    rs.start(kimp + row0 * RB, ncand);
+    __syncthreads();
+
+    // ---- stream ------------------------------------------------------------------------------------
+    float s1 = 0.f, s2 = 0.f;
+    auto keep = [&](int slot, float sc) {
+        keys[slot] = order_key(sc);
+        s1 += sc, s2 = fmaf(sc, sc, s2);
+    };
+    if constexpr (kDirect) {
+        FragScorer<DP, RED> scorer;
+        scorer.load_staged(sm->qs, gm.gl, sm->frags);
+        rs.run(scorer, keep);
+    } else {
+        // The two halves of the block take tiles in turn; the number of stages is even when stages are used again, so that
+        // a stage belongs to one half (its barrier's phases are then waited for in order).  A wait that runs out
+        // (wait_limit polls; a correct run never gets there) makes its half request nothing further, score what it never
+        // received as the lowest key and go on; the other half's waits are bounded the same way, so every copy in flight
+        // has landed or been waited for in full before the block ends.
+        GroupScorer<T, DP, RED> scorer;
+        scorer.load_staged(sm->qs, gm.gl);
+        const int half = tid / kHalf, r = tid % kHalf;
+        bool dead = false;
+        for (int t = half; t < n_tiles; t += 2) {
+            const int st = t % n_stages, slot = t * kHalf + r;
+            const bool ok = mbar_wait(&sm->full[st], (t / n_stages) & 1, wait_limit);
+            dead |= !ok;
+            const unsigned char* tile = ring + st * kTileBytes;
+            if (slot < ncand && ok) {
+                const uint32_t off = r * RB;
+                keep(slot, scorer.score([&](int c) {
+                    uint32_t o = off + c * 16;
+                    o ^= ((o >> 7) & (NCH - 1)) << 4;  // TMA swizzle of 16-byte chunks (mode = row size)
+                    return *reinterpret_cast<const uint4*>(tile + o);
+                }));
+            } else if (slot < ncand) {
+                keys[slot] = 0u;
+            }
+            if (t + n_stages < n_tiles) {              // uniform per half
+                if (half == 0) asm volatile("bar.sync 1, %0;" ::"n"(kHalf) : "memory");   // the half has read the stage
+                else asm volatile("bar.sync 2, %0;" ::"n"(kHalf) : "memory");
+                if (r == 0 && !dead) {
+                    fence_proxy_async();
+                    request(t + n_stages);
+                }
+            }
+        }
+        if (dead && lane == 0) atomicExch(status, kStatusTimeout);
+    }
+    s1 = warp_sum(s1), s2 = warp_sum(s2);
+    if (lane == 0) sm->part[warp][0] = s1, sm->part[warp][1] = s2;
+    __syncthreads();
+
+    // ---- digit and histogram --------------------------------------------------------------------------
+    float m1 = 0.f, m2 = 0.f;
+#pragma unroll
+    for (int w = 0; w < kWarps; ++w) m1 += sm->part[w][0], m2 += sm->part[w][1];
+    m1 /= (float)ncand, m2 = m2 / (float)ncand - m1 * m1;
+    const float dev = sqrtf(fmaxf(m2, 0.f));
+    const float base = m1 - 4.5f * dev, scale = dev > 0.f ? (float)(kBins - 2) / (9.f * dev) : 0.f;
+    auto bin_of = [&](uint32_t key) { return (int)fminf(fmaxf((key_score(key) - base) * scale + 1.f, 0.f), (float)(kBins - 1)); };
+    for (int i = tid; i < ncand; i += kThreads) atomicAdd(&sm->hist[bin_of(keys[i])], 1);
+    __syncthreads();
+    int bin, kr, bc;
+    find_bin(sm, kBins, k, bin, kr, bc);
+
+    const uint4* keys4 = reinterpret_cast<const uint4*>(keys);
+    // verdict(key): 2 = selected, 1 = to be ranked among its equals-so-far, 0 = not.  Lane l of a warp holds slots
+    // 4 l .. 4 l + 3 of a group: its verdicts are a nibble of the bitmask, eight lanes make a word.
+    auto classify = [&](auto verdict, bool whole) {
+        for (int v = tid; v < n_tiles * (kHalf / 4); v += kThreads) {
+            const uint4 x = keys4[v];
+            const uint32_t kk[4] = {x.x, x.y, x.z, x.w};
+            uint32_t word = 0u, rank = 0u;
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                const int w = v * 4 + e < ncand ? verdict(kk[e]) : 0;
+                word |= (uint32_t)(w == 2 || (whole && w == 1)) << e;
+                rank |= (uint32_t)(w == 1 && !whole) << e;
+            }
+            word <<= 4 * (lane & 7);
+            word |= __shfl_xor_sync(0xffffffffu, word, 1);
+            word |= __shfl_xor_sync(0xffffffffu, word, 2);
+            word |= __shfl_xor_sync(0xffffffffu, word, 4);
+            if ((lane & 7) == 0) sm->mask[v >> 3] = word;
+            while (rank) {
+                const int e = __ffs(rank) - 1;
+                rank &= rank - 1;
+                sm->cand[atomicAdd(&sm->n_cand, 1)] = make_uint2(keys[v * 4 + e], (uint32_t)(v * 4 + e));
+            }
+        }
+        __syncthreads();
+    };
+    if (bc == kr || bc <= kMaxRank) {
+        classify([&](uint32_t key) { const int b = bin_of(key); return b > bin ? 2 : b == bin ? 1 : 0; }, bc == kr);
+        if (bc != kr) {
+            if (tid < bc) {                            // rank: larger key first, equal keys by position
+                const uint2 it = sm->cand[tid];
+                int before = 0;
+#pragma unroll 4
+                for (int j = 0; j < bc; ++j) {
+                    const uint2 o = sm->cand[j];
+                    before += (o.x > it.x) | ((o.x == it.x) & (o.y < it.y));
+                }
+                if (before < kr) atomicOr(&sm->mask[it.y >> 5], 1u << (it.y & 31));
+            }
+            __syncthreads();
+        }
+    } else {
+        // The key's own digits.  What is left at the end are equal keys: the first ones in position order are taken.
+        uint32_t prefix = 0;
+        int low_bits = 32;
+        kr = k;
+#pragma unroll 1
+        for (int pass = 0; pass < 3; ++pass) {
+            const int bits = pass == 2 ? 10 : 11, shift = low_bits - bits;
+            reinterpret_cast<int4*>(sm->hist)[tid] = make_int4(0, 0, 0, 0);
+            __syncthreads();
+            for (int i = tid; i < ncand; i += kThreads) {
+                const uint32_t key = keys[i];
+                if (pass == 0 || (key >> low_bits) == prefix) atomicAdd(&sm->hist[(key >> shift) & ((1 << bits) - 1)], 1);
+            }
+            __syncthreads();
+            find_bin(sm, 1 << bits, kr, bin, kr, bc);
+            prefix = (prefix << bits) | (uint32_t)bin, low_bits = shift;
+        }
+        classify([&](uint32_t key) { return key > prefix ? 2 : 0; }, false);
+        // the equal keys' bits, then as many of them as are wanted, lowest positions first
+        const int n_words = n_tiles * (kHalf / 32);    // <= 256 < kThreads
+        uint32_t eq = 0u;
+        if (tid < n_words)
+            for (int e = 0; e < 32; ++e) eq |= (uint32_t)(tid * 32 + e < ncand && keys[tid * 32 + e] == prefix) << e;
+        const int n_eq = __popc(eq), incl = warp_incl_scan(n_eq, lane);
+        if (lane == 31) sm->slots[warp] = incl;
+        __syncthreads();
+        int before = incl - n_eq;
+        for (int w = 0; w < warp; ++w) before += sm->slots[w];
+        uint32_t take = 0u;
+        while (eq && before < kr) take |= eq & (0u - eq), eq &= eq - 1, ++before;
+        if (take) sm->mask[tid] |= take;
+        __syncthreads();
+    }
+
+    // ---- neighbours and list -----------------------------------------------------------------------------
+    const uint32_t* mask = sm->mask;
+    if (a.radius > 0) {
+        expand_mask<kThreads>(sm->mask, sm->mask_out, ncand, a.radius, a.nmode);
+        mask = sm->mask_out;
+    }
+    const int total = write_mask_list<kThreads>(mask, ncand, lo, gm.idx_cap, idx_dst, idx_copy, sm->slots);
+    if (tid == 0) {
+        state_cnt[cu] = total;
+        if (cnt_copy) *cnt_copy = total;
+    }
+}
+
+size_t small_smem(int n_stages, int n_tiles, int tile_bytes) {
+    return 1024 + (size_t)n_stages * tile_bytes + (size_t)n_tiles * kHalf * 4 + sizeof(SmallSmem);
+}
+
+}  // namespace
+
+// Launches of up to two blocks per SM.  Measured against the cluster kernel and the one-block-per-problem kernel, us per
+// launch at 32 dimensions, bf16 (this / the other): 32 problems of 1000 candidates 5.7 / 7.0, 2000 6.9 / 10.4, 4000 9.3 / 9.5,
+// 6000 level (its clusters bring four times the SMs to few problems; at 16 dimensions 8000 candidates 12.2 / 10.5);
+// 96 problems of 2000 7.5 / 10.2, 8000 16.1 / 21.8; 192 problems of 800 8.3 / 8.7, 2000 level, 4000 18.5 / 19.0, 8000 31.7 / 28.9;
+// 288 of 2000 12.1 / 16.1; 384 problems, a second wave: level or worse.  Neighbours and the caller's copy come for next to
+// nothing here and cost two more launches there (96 problems of 3000 with both: 8.3 / 18.4).
+bool select_small_takes(const tb_ctx* c, const UnitTable& ut, int max_cand, bool more) {
+    if (c->drop_tile >= 0) return false;               // wait diagnostics: see select_kernel
+    const int n_units = ut.layer_count * ut.n_seq * c->geom.Hl;
+    const bool few = 3 * n_units <= c->sm_count, alone = n_units <= c->sm_count;
+    return n_units <= 2 * c->sm_count && max_cand <= (more || (alone && !few) ? kMaxCand : kMaxCand / 2);
+}
+
+cudaError_t launch_select_small(const tb_ctx* c, const UnitTable& ut, const SelectArgs& a, int max_cand, cudaStream_t s, bool dry) {
+    if (dry) return cudaSuccess;
+    const Geom& gm = c->geom;
+    const int n_units = ut.layer_count * ut.n_seq * gm.Hl;
+    const int tile_bytes = kHalf * gm.dp * (gm.dtype == TB_BF16 ? 2 : 4);
+    const int n_tiles = max_cand > kHalf ? (max_cand + kHalf - 1) / kHalf : 1;
+    const uint32_t wait_limit = c->wait_poll_limit > 0 ? (uint32_t)c->wait_poll_limit : kWaitPollLimit;
+
+    // fp32: all tiles in flight at once if an SM's share of shared memory holds them, all of it when every block has an SM
+    // to itself, half otherwise.
+    const bool direct = gm.dtype == TB_BF16, alone = n_units <= c->sm_count;
+    const size_t room = (alone ? 226 : 112) * 1024;
+    int n_stages = direct ? 0 : n_tiles;
+    if (small_smem(n_stages, n_tiles, tile_bytes) > room) {
+        n_stages &= ~1;                                // even: see the stream loop
+        while (n_stages > 2 && small_smem(n_stages, n_tiles, tile_bytes) > room) n_stages -= 2;
+    }
+
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(n_units, 1, 1), cfg.blockDim = dim3(kThreads, 1, 1), cfg.stream = s;
+    cfg.dynamicSmemBytes = small_smem(n_stages, n_tiles, tile_bytes);
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;   // see pdl_wait()
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr, cfg.numAttrs = 1;
+    auto launch = [&](auto kernel, unsigned char (&seen)[64]) {
+        if (first_use_on_this_device(seen)) {
+            cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
+            if (e != cudaSuccess) return e;
+        }
+        return cudaLaunchKernelEx(&cfg, kernel, c->kimp_map, (const unsigned char*)c->kimp, gm, ut, a, n_stages, n_tiles, wait_limit,
+                                  c->st.idx, c->st.cnt, c->st.status);
+    };
+    // a block alone on its SM keeps four groups of rows in flight per warp, two blocks two each (their registers)
+#define TB_SMALL(T, DP, RED, U)                                        \
+    do {                                                               \
+        static unsigned char seen[64];                                 \
+        return launch(select_small_kernel<T, DP, RED, U>, seen);       \
+    } while (0)
+#define TB_SMALL_U(DP, RED)                                            \
+    do {                                                               \
+        if (direct && alone) TB_SMALL(__nv_bfloat16, DP, RED, 4);      \
+        if (direct) TB_SMALL(__nv_bfloat16, DP, RED, 2);               \
+        TB_SMALL(float, DP, RED, 0);                                   \
+    } while (0)
+    const bool max = a.reduce == TB_GROUP_MAX;
+    if (gm.dp == 32) {
+        if (max) TB_SMALL_U(32, TB_GROUP_MAX);
+        TB_SMALL_U(32, TB_GROUP_SUM);
+    }
+    if (max) TB_SMALL_U(16, TB_GROUP_MAX);
+    TB_SMALL_U(16, TB_GROUP_SUM);
+#undef TB_SMALL_U
+#undef TB_SMALL
+}
+
+}  // namespace tb

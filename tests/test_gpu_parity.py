@@ -653,3 +653,28 @@ def test_long_problem_cluster_kernel_unusual_distributions(H):
     expo = r.integers(-100, 101, size=(2, L))
     sign = r.choice([-1.0, 1.0], size=(2, L))
     _crafted_scores_case(H, (sign * np.exp2(expo)).astype(np.float32), budget=9000)
+
+
+@pytest.mark.parametrize("cfg,dp", [(2, 32), (2, 16), (1, 32), (1, 16)])
+@pytest.mark.parametrize("L,budget,sinks,recent", [(20, 1, 3, 2), (31, 7, 0, 0), (33, 32, 0, 0), (257, 100, 1, 0), (2055, 513, 4, 64), (4113, 2, 0, 17),
+                                                   (8192, 700, 0, 0)])
+def test_small_selection_kernel_edges(H, cfg, dp, L, budget, sinks, recent):
+    """One-block selection: sizes around the 32-row groups, the 256-row tiles and the largest it takes, both reductions and
+    neighbour rules, with the caller's copy checked against the stored list through the attention that follows."""
+    for radius, nmode, reduce in ((0, 0, 0), (1, 0, 1), (3, 1, 0), (40, 0, 0)):
+        w = wl.workload(cfg, n_layers=1, n_q_heads=4, n_kv_heads=2, imp_dim=dp, batch=2, lengths=[L, max(1, L - 5)], budget=budget, sinks=sinks,
+                        recent=recent, radius=radius, nmode=nmode, outlier_channels=0)
+        full_pipeline_check(H, H.Case(w), tb().select_params(budget, sinks, recent, radius, nmode, reduce=reduce))
+
+
+def test_small_selection_kernel_unusual_distributions(H):
+    """Crowded threshold bins (ties, one huge outlier, sums that overflow) and more problems than SMs (two blocks per SM)."""
+    r = np.random.Generator(np.random.PCG64(78))
+    for n_seq, L in ((2, 5003), (40, 1500)):
+        shape = (n_seq, 4, L)
+        _crafted_batch_case(H, np.full(shape, -3.5, np.float32), budget=300, sinks=3, recent=5)
+        _crafted_batch_case(H, r.integers(0, 3, size=shape).astype(np.float32), budget=900)
+        _crafted_batch_case(H, (r.choice([-1.0, 1.0], size=shape) * np.exp2(r.integers(-100, 101, size=shape))).astype(np.float32), budget=333)
+        x = _bf16_exact(r.standard_normal(shape))
+        x[:, :, 7] = 1e6
+        _crafted_batch_case(H, _bf16_exact(x), budget=200)
