@@ -17,7 +17,6 @@ namespace tb {
 
 constexpr int kAttnThreads = 128;
 constexpr int kAttnWarps = kAttnThreads / 32;
-constexpr int kRowsPerIter = 4;
 constexpr int kAttnMaxCluster = 16;      // splits that can be merged inside a thread-block cluster (16 is non-portable)
 constexpr float kLog2e = 1.4426950408889634f;
 constexpr float kLn2 = 0.6931471805599453f;
@@ -40,20 +39,7 @@ struct RowMap {
     }
     __device__ __forceinline__ int sink_ref(int t) const { return res_ref(t); }
     __device__ __forceinline__ int window_ref(int t) const { return res_ref(t); }
-    __device__ __forceinline__ int token(int r, bool& bad) const {
-        bad = false;
-        if (dense) return r;
-        if (r < n_sink) return sink_ref(r);
-        r -= n_sink;
-        if (r < n_list) {
-            if (kSources && use_imp) return (kRowSrcImportant << kRowSrcShift) | r;
-            int t = list[r];
-            if (t < 0 || t >= L) { bad = true; return 0; }
-            return t;
-        }
-        return window_ref(w_begin + (r - n_list));
-    }
-    // the same with a bad list entry reported as -1 (nothing else depends on the loaded value)
+    // a bad list entry is reported as -1 (nothing else depends on the loaded value)
     __device__ __forceinline__ int token_or_neg(int r) const {
         if (dense) return r;
         if (r < n_sink) return sink_ref(r);
@@ -88,7 +74,7 @@ struct AttnUnit {
 
 // Publishes one split's (m, l, o) per query head and lets the last block to arrive for the
 // (sequence, KV head) merge all splits in split order:  M = max m_j;  l = sum l_j 2^(m_j-M);
-// out = sum o_j 2^(m_j-M) / l;  lse = (M + log2 l) ln 2.  Called by all 128 threads; thread = channel.
+// out = sum o_j 2^(m_j-M) / l;  lse = (M + log2 l) ln 2.  Called by all 128 threads.
 struct SplitSink {
     float* part_o;
     float* part_ml;
@@ -98,12 +84,7 @@ struct SplitSink {
     size_t hq0;        // first query head of this (layer, sequence, KV head) in the launch
     int lu, split, nsplit;
 
-    __device__ __forceinline__ void publish(int u, float M, float lsum, float o) const {
-        const size_t pq = (hq0 + u) * kMaxSplits + split;
-        part_o[pq * 128 + threadIdx.x] = o;
-        if (threadIdx.x == 0) part_ml[pq * 2] = M, part_ml[pq * 2 + 1] = lsum;
-    }
-    // the same, for a thread that holds channel `ch` of head u / the head's statistics
+    // by the thread that holds channel `ch` of head u / the head's statistics
     __device__ __forceinline__ void publish_at(int u, int ch, float o) const { part_o[((hq0 + u) * kMaxSplits + split) * 128 + ch] = o; }
     __device__ __forceinline__ void publish_stat(int u, float M, float lsum) const {
         const size_t pq = (hq0 + u) * kMaxSplits + split;
@@ -161,176 +142,22 @@ struct SplitSink {
     }
 };
 
-template <typename T>
-struct RowVec;   // the 4 channels of a 128-channel row that one lane owns
-template <>
-struct RowVec<float> {
-    float4 v;
-    __device__ __forceinline__ void load(const float* row, int lane) { v = __ldg(reinterpret_cast<const float4*>(row) + lane); }
-    __device__ __forceinline__ void get(float* f) const { f[0] = v.x, f[1] = v.y, f[2] = v.z, f[3] = v.w; }
-};
-template <>
-struct RowVec<__nv_bfloat16> {
-    uint2 v;
-    __device__ __forceinline__ void load(const __nv_bfloat16* row, int lane) { v = __ldg(reinterpret_cast<const uint2*>(row) + lane); }
-    __device__ __forceinline__ void get(float* f) const { f[0] = bf16_lo(v.x), f[1] = bf16_hi(v.x), f[2] = bf16_lo(v.y), f[3] = bf16_hi(v.y); }
-};
-
-template <typename T, int G>
-__global__ void __launch_bounds__(kAttnThreads) attn_kernel(Geom gm, UnitTable ut, AttnArgs a, const T* __restrict__ kv,
-                                                            const int32_t* __restrict__ state_idx, const int32_t* __restrict__ state_cnt,
-                                                            float* __restrict__ part_o, float* __restrict__ part_ml,
-                                                            uint32_t* __restrict__ counters, int32_t* __restrict__ status) {
-    constexpr int D = 128;
-    __shared__ float sh_o[kAttnWarps][G][D];
-    __shared__ float sh_m[kAttnWarps][G], sh_l[kAttnWarps][G];
-    __shared__ int sh_last;
-
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int split = blockIdx.x, h = blockIdx.y;
-    const int ll = blockIdx.z / ut.n_seq, s = blockIdx.z % ut.n_seq;
-    const int L = unit_len(gm, ut, ll, s);
-    const int g = gm.ga;
-    const AttnUnit au(gm, ut, ll, s, h);
-    const int lu = au.lu;
-
-    RowMap<true> rm;
-    rm.L = L, rm.dense = a.dense;
-    rm.res_sinks = a.res_rows ? a.res_sinks : 0, rm.res_window = a.res_rows ? a.res_window : 0;
-    rm.use_imp = a.imp_rows != nullptr && a.idx == nullptr;
-    rm.n_sink = a.dense ? 0 : min(a.sinks, L);
-    rm.w_begin = a.dense ? 0 : max(rm.n_sink, L - a.recent);
-    int n_list = 0;
-    if (!a.dense) {
-        const int known = a.known_cnt[ll * ut.n_seq + s];
-        n_list = a.idx ? a.cnt[au.list_l] : (known >= 0 ? known : state_cnt[au.list_c]);
-        n_list = max(0, min(n_list, gm.idx_cap));
-    }
-    rm.n_list = n_list;
-    rm.list = a.idx ? a.idx + (size_t)au.list_l * gm.idx_cap : state_idx + au.list_c * gm.idx_cap;
-    const int n_rows = a.dense ? L : rm.n_sink + n_list + (L - rm.w_begin);
-
-    const int r_begin = (int)((long long)n_rows * split / a.nsplit);
-    const int r_end = (int)((long long)n_rows * (split + 1) / a.nsplit);
-    const int per_warp = (r_end - r_begin + kAttnWarps - 1) / kAttnWarps;
-    const int wb = min(r_end, r_begin + warp * per_warp), we = min(r_end, wb + per_warp);
-
-    // this lane's 4 channels of each query head, pre-scaled so that logits are in base-2 units
-    const float qscale = a.sm_scale * kLog2e;
-    float q[G][4];
-    const T* qbase = reinterpret_cast<const T*>(a.q) + ((size_t)(ll * ut.n_seq + s) * gm.Hq + h * g) * D;
-#pragma unroll
-    for (int u = 0; u < G; ++u) {
-        if (u < g) {
-            RowVec<T> rv;
-            rv.load(qbase + u * D, lane);
-            rv.get(q[u]);
-        } else {
-            q[u][0] = q[u][1] = q[u][2] = q[u][3] = 0.f;
-        }
-    }
-
-    float m[G], l[G], acc[G][4];
-#pragma unroll
-    for (int u = 0; u < G; ++u) {
-        m[u] = -INFINITY, l[u] = 0.f;
-        acc[u][0] = acc[u][1] = acc[u][2] = acc[u][3] = 0.f;
-    }
-
-    // the unit's rows in the cache and in the optional copies, indexed by a row reference's source
-    const T* src_base[3] = {kv + au.kv_c * gm.max_seq_len * 2 * D,
-                            reinterpret_cast<const T*>(a.res_rows) + au.kv_c * (size_t)(a.res_sinks + a.res_window) * 2 * D,
-                            reinterpret_cast<const T*>(a.imp_rows) + au.list_c * (size_t)gm.idx_cap * 2 * D};
-    bool any_bad = false;
-    for (int r0 = wb; r0 < we; r0 += kRowsPerIter) {
-        RowVec<T> kr[kRowsPerIter], vr[kRowsPerIter];
-        bool valid[kRowsPerIter];
-#pragma unroll
-        for (int i = 0; i < kRowsPerIter; ++i) {
-            bool bad = false;
-            valid[i] = r0 + i < we;
-            int t = valid[i] ? rm.token(r0 + i, bad) : 0;
-            if (bad) valid[i] = false, any_bad = true;
-            const int which = t >> kRowSrcShift;
-            const T* row = (which == 0 ? src_base[0] : which == 1 ? src_base[1] : src_base[2]) + (size_t)(t & kRowIdxMask) * 2 * D;
-            kr[i].load(row, lane);
-            vr[i].load(row + D, lane);
-        }
-        float x[kRowsPerIter][G];
-#pragma unroll
-        for (int i = 0; i < kRowsPerIter; ++i) {
-            float kf[4];
-            kr[i].get(kf);
-#pragma unroll
-            for (int u = 0; u < G; ++u) {
-                float p = q[u][0] * kf[0];
-                p = fmaf(q[u][1], kf[1], p);
-                p = fmaf(q[u][2], kf[2], p);
-                p = fmaf(q[u][3], kf[3], p);
-                p = warp_sum(p);
-                x[i][u] = valid[i] ? p * qscale : -INFINITY;
-            }
-        }
-#pragma unroll
-        for (int u = 0; u < G; ++u) {
-            float mn = m[u];
-#pragma unroll
-            for (int i = 0; i < kRowsPerIter; ++i) mn = fmaxf(mn, x[i][u]);
-            const float ms = mn == -INFINITY ? 0.f : mn;
-            const float corr = exp2f(m[u] - ms);
-            m[u] = mn;
-            l[u] *= corr;
-            acc[u][0] *= corr, acc[u][1] *= corr, acc[u][2] *= corr, acc[u][3] *= corr;
-#pragma unroll
-            for (int i = 0; i < kRowsPerIter; ++i) {
-                const float p = exp2f(x[i][u] - ms);
-                float vf[4];
-                vr[i].get(vf);
-                l[u] += p;
-                acc[u][0] = fmaf(p, vf[0], acc[u][0]);
-                acc[u][1] = fmaf(p, vf[1], acc[u][1]);
-                acc[u][2] = fmaf(p, vf[2], acc[u][2]);
-                acc[u][3] = fmaf(p, vf[3], acc[u][3]);
-            }
-        }
-    }
-    if (any_bad && lane == 0) atomicExch(status, kStatusBadIndex);
-
-    // ---- combine the block's warps (fixed order) and publish the split's partial ------------------
-#pragma unroll
-    for (int u = 0; u < G; ++u) {
-        if (lane == 0) sh_m[warp][u] = m[u], sh_l[warp][u] = l[u];
-        *reinterpret_cast<float4*>(&sh_o[warp][u][lane * 4]) = make_float4(acc[u][0], acc[u][1], acc[u][2], acc[u][3]);
-    }
-    __syncthreads();
-    SplitSink sink{part_o, part_ml, counters, a.out, a.lse, (size_t)(ll * ut.n_seq + s) * gm.Hq + h * g, lu, split, a.nsplit};
-    for (int u = 0; u < g; ++u) {
-        float M = -INFINITY;
-#pragma unroll
-        for (int w = 0; w < kAttnWarps; ++w) M = fmaxf(M, sh_m[w][u]);
-        const float Ms = M == -INFINITY ? 0.f : M;
-        float lsum = 0.f, o = 0.f;
-#pragma unroll
-        for (int w = 0; w < kAttnWarps; ++w) {
-            const float e = exp2f(sh_m[w][u] - Ms);
-            lsum += sh_l[w][u] * e;
-            o += sh_o[w][u][tid] * e;
-        }
-        sink.publish(u, M, lsum, o);
-    }
-    sink.merge_if_last(g, &sh_last);
-}
-
 // ---------------------------------------------------------------------------------------------------
-// bf16 path: tensor-core tiles of (16 gathered tokens) x (query heads padded to 8).
+// Each warp owns a ring of 8 KB shared-memory stages of gathered K|V row pairs, copied by the whole warp with 16-byte
+// cp.async.
 //
-// Each warp owns a ring of shared-memory stages; a stage holds 16 gathered K|V row pairs (512 B each,
-// copied by the whole warp with 16-byte cp.async) at a 512-byte pitch with the 16-byte chunks of a row
+// bf16: tensor-core tiles of (16 gathered tokens) x (query heads padded to 8).  A stage holds 16 row pairs (512 B each)
+// at a 512-byte pitch with the 16-byte chunks of a row
 // permuted by the row number, so that ldmatrix reads are bank-conflict free.  S = K Q^T (tokens x heads) and O^T += V^T P^T (channels x heads) run on
 // mma.sync m16n8k16 (bf16 in, fp32 accumulate) with the GQA group's heads as the N = 8 columns --
 // the one place where batch x group makes the contraction a real dense tile; P is split into a bf16
 // high and low part (two MMAs) so that the probabilities keep ~16 bits, and reaches the B operand
 // through movmatrix transposes.  24 MMAs per 16 tokens.
+//
+// fp32: FMA (a tolerance of 1e-5 rules out TF32).  A stage holds 8 row pairs (1 KB each).  Eight lanes share a row (16
+// channels each, 128 contiguous bytes per access), so a warp works on four rows at a time and a dot product costs three
+// shuffles; the four lane groups keep an online softmax each and are merged once, at the end.  3276 rows x 8 KV heads, four
+// query heads each (27 MB): 20.7 us with a warp per row and no overlap between launches, 13.6 like this.
 
 #ifdef TB_PHASE_TIMING
 __device__ unsigned long long g_attn_phase_ns[2][16];
@@ -364,7 +191,7 @@ extern "C" int tb_debug_attn_blocks_ns(unsigned long long* out) {
 #define attn_stamp(i) ((void)0)
 #endif
 
-constexpr int kTileTok = 16;
+constexpr int kTileTok = 16;                          // rows of a stage (fp32: 8)
 // A stage holds 16 K|V rows at a pitch of 512 bytes; the 16-byte chunk c of row i sits at chunk
 // c ^ (i & 7), so the eight rows of an ldmatrix tile hit eight different bank groups without padding.
 // Every 128-byte line of a source row therefore lands in one 128-byte line of shared memory and the
@@ -396,6 +223,148 @@ __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
     return *reinterpret_cast<uint32_t*>(&v);
 }
 
+// The fp32 warp's rows: tiles of 8 rows from its stages, each row shared by eight lanes; leaves the warp's accumulators and
+// statistics parked at the start of `my_stage` in the layout described at the kernel's merge.  tokens_of / issue_token /
+// commit: the kernel's gather.
+template <int G, int kStages, typename Tokens, typename Issue, typename Commit>
+__device__ __forceinline__ void f32_rows(const float* __restrict__ qbase, int g, float qscale, unsigned char* my_stage, int wb, int we,
+                                         int n_tiles, uint32_t bad_bits, bool& any_bad, Tokens tokens_of, Issue issue_token, Commit commit) {
+    constexpr int kTok = 8, D = 128;
+    const int lane = threadIdx.x & 31, r4 = lane >> 3, c8 = lane & 7;
+    // Channels of a lane: chunks j * 8 + c8 (j = 0..3) of four.  Up to four heads' queries sit in registers, eight are read
+    // again per tile (L1 hits).
+    float4 q[G <= 4 ? G : 1][4];
+    if constexpr (G <= 4) {
+#pragma unroll
+        for (int u = 0; u < G; ++u)
+#pragma unroll
+            for (int j = 0; j < 4; ++j)
+                q[u][j] = u < g ? __ldg(reinterpret_cast<const float4*>(qbase + u * D) + j * 8 + c8) : make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+    float m[G], l[G];
+    float4 acc[G][4];
+#pragma unroll
+    for (int u = 0; u < G; ++u) {
+        m[u] = -INFINITY, l[u] = 0.f;
+#pragma unroll
+        for (int j = 0; j < 4; ++j) acc[u][j] = make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+    for (int tile = 0; tile < n_tiles; ++tile) {
+        const int r0 = wb + tile * kTok;
+        const bool in_range = lane < kTok && r0 + lane < we;
+        const bool bad = in_range && (bad_bits & 1u);
+        any_bad |= bad;
+        bad_bits >>= 1;
+        const unsigned vmask = __ballot_sync(0xffffffffu, in_range && !bad);
+        asm volatile("cp.async.wait_group %0;" ::"n"(kStages - 1) : "memory");
+        __syncwarp();                                  // every lane's copies of this tile are visible to the warp
+        const float4* rows = reinterpret_cast<const float4*>(my_stage + tile % kStages * kStageBytes);
+        float x[2][G];                                 // rows r4 and 4 + r4
+#pragma unroll
+        for (int i = 0; i < 2; ++i) {
+            const float4* k4 = rows + (i * 4 + r4) * 64 + c8;
+            float4 k[4];
+#pragma unroll
+            for (int j = 0; j < 4; ++j) k[j] = k4[j * 8];
+#pragma unroll
+            for (int u = 0; u < G; ++u) {
+                float d = 0.f;
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    float4 qv;
+                    if constexpr (G <= 4) qv = q[u][j];
+                    else qv = __ldg(reinterpret_cast<const float4*>(qbase + min(u, g - 1) * D) + j * 8 + c8);
+                    d = fmaf(qv.x, k[j].x, d), d = fmaf(qv.y, k[j].y, d), d = fmaf(qv.z, k[j].z, d), d = fmaf(qv.w, k[j].w, d);
+                }
+                x[i][u] = d;
+            }
+        }
+#pragma unroll
+        for (int off = 1; off < 8; off <<= 1)
+#pragma unroll
+            for (int i = 0; i < 2; ++i)
+#pragma unroll
+                for (int u = 0; u < G; ++u) x[i][u] += __shfl_xor_sync(0xffffffffu, x[i][u], off);
+        const bool v0 = (vmask >> r4) & 1u, v1 = (vmask >> (4 + r4)) & 1u;
+        bool moved = false;
+        float corr[G];
+#pragma unroll
+        for (int u = 0; u < G; ++u) {
+            x[0][u] = v0 ? x[0][u] * qscale : -INFINITY, x[1][u] = v1 ? x[1][u] * qscale : -INFINITY;
+            const float mn = fmaxf(m[u], fmaxf(x[0][u], x[1][u])), ms = mn == -INFINITY ? 0.f : mn;
+            corr[u] = exp2f(m[u] - ms);
+            moved |= mn != m[u];
+            m[u] = mn;
+            x[0][u] = exp2f(x[0][u] - ms), x[1][u] = exp2f(x[1][u] - ms);
+            l[u] = fmaf(l[u], corr[u], x[0][u] + x[1][u]);
+        }
+        if (__any_sync(0xffffffffu, moved)) {
+#pragma unroll
+            for (int u = 0; u < G; ++u)
+#pragma unroll
+                for (int j = 0; j < 4; ++j) acc[u][j].x *= corr[u], acc[u][j].y *= corr[u], acc[u][j].z *= corr[u], acc[u][j].w *= corr[u];
+        }
+#pragma unroll
+        for (int i = 0; i < 2; ++i) {
+            const float4* v4 = rows + (i * 4 + r4) * 64 + 32 + c8;
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                const float4 v = v4[j * 8];
+#pragma unroll
+                for (int u = 0; u < G; ++u) {
+                    acc[u][j].x = fmaf(x[i][u], v.x, acc[u][j].x), acc[u][j].y = fmaf(x[i][u], v.y, acc[u][j].y);
+                    acc[u][j].z = fmaf(x[i][u], v.z, acc[u][j].z), acc[u][j].w = fmaf(x[i][u], v.w, acc[u][j].w);
+                }
+            }
+        }
+        __syncwarp();                                  // the warp is done reading this stage
+        if (tile + kStages < n_tiles) {
+            const int t = tokens_of(tile + kStages);
+            bad_bits |= (uint32_t)(t < 0) << (kStages - 1);
+            issue_token(tile + kStages, max(t, 0));
+        }
+        commit();
+    }
+    asm volatile("cp.async.wait_group 0;" ::: "memory");
+    // the four lane groups' softmaxes become one
+#pragma unroll
+    for (int u = 0; u < G; ++u) {
+        float M = m[u];
+        M = fmaxf(M, __shfl_xor_sync(0xffffffffu, M, 8)), M = fmaxf(M, __shfl_xor_sync(0xffffffffu, M, 16));
+        const float e = exp2f(m[u] - (M == -INFINITY ? 0.f : M));
+        m[u] = M, l[u] *= e;
+        l[u] += __shfl_xor_sync(0xffffffffu, l[u], 8), l[u] += __shfl_xor_sync(0xffffffffu, l[u], 16);
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            float v[4] = {acc[u][j].x * e, acc[u][j].y * e, acc[u][j].z * e, acc[u][j].w * e};
+#pragma unroll
+            for (int i = 0; i < 4; ++i) v[i] += __shfl_xor_sync(0xffffffffu, v[i], 8), v[i] += __shfl_xor_sync(0xffffffffu, v[i], 16);
+            acc[u][j] = make_float4(v[0], v[1], v[2], v[3]);
+        }
+    }
+    __syncwarp();
+    // lane group r4 parks chunk j = r4 of its channels (selected, not indexed: the accumulators stay in registers)
+    float* park = reinterpret_cast<float*>(my_stage);
+#pragma unroll
+    for (int u = 0; u < G; ++u) {
+        const float4 v = r4 == 0 ? acc[u][0] : r4 == 1 ? acc[u][1] : r4 == 2 ? acc[u][2] : acc[u][3];
+        const float w[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+            const int ch = (r4 * 8 + c8) * 4 + e, in = ch & 15;
+            park[(((ch >> 4) * 32 + (in & 7) * 4 + (u >> 1)) << 2) + (u & 1) + 2 * (in >> 3)] = w[e];
+        }
+    }
+    float4 stat = make_float4(-INFINITY, 0.f, -INFINITY, 0.f);     // heads 2 (lane & 3), 2 (lane & 3) + 1
+#pragma unroll
+    for (int u = 0; u < G; ++u)
+        if ((lane & 3) == u >> 1) {
+            if (u & 1) stat.z = m[u], stat.w = l[u];
+            else stat.x = m[u], stat.y = l[u];
+        }
+    reinterpret_cast<float4*>(my_stage)[8 * 32 + lane] = stat;
+}
+
 // Shared memory behind the warps' stages for the merge inside a cluster of C blocks: the accumulator slices this
 // block owns from every block ([slices per owner][C][32 lanes] float4) and every block's (m, l) ([C][4] float4).
 static inline size_t cluster_merge_bytes(int C) { return (size_t)((8 + C - 1) / C) * C * 32 * 16 + (size_t)C * 4 * 16; }
@@ -407,13 +376,17 @@ static inline size_t cluster_merge_bytes(int C) { return (size_t)((8 + C - 1) / 
 // go through the global workspace and the last block to arrive merges them (NW must be 4 then).
 // kSources: the resident sink / window copies or the Important buffer are bound and a row reference names
 // its source; without them (the usual case) the gather carries no trace of the option.
-template <int NW, int kMmaStages, bool kSources = false>
-__global__ void __launch_bounds__(NW * 32) attn_mma_kernel(Geom gm, UnitTable ut, AttnArgs a, const __nv_bfloat16* __restrict__ kv,
+// FG: 0 = bf16 storage; else fp32 storage with up to FG query heads per unit.
+template <int NW, int kMmaStages, bool kSources = false, int FG = 0>
+__global__ void __launch_bounds__(NW * 32) attn_mma_kernel(Geom gm, UnitTable ut, AttnArgs a, const void* __restrict__ kv,
                                                            const int32_t* __restrict__ state_idx,
                                                            const int32_t* __restrict__ state_cnt, float* __restrict__ part_o,
                                                            float* __restrict__ part_ml, uint32_t* __restrict__ counters,
                                                            int32_t* __restrict__ status) {
     constexpr int D = 128;
+    constexpr bool kF32 = FG > 0;
+    constexpr int kTok = kF32 ? 8 : kTileTok;          // rows of a stage
+    constexpr int kRowBytes = 2 * D * (kF32 ? 4 : 2);  // a K|V row pair
     extern __shared__ __align__(128) unsigned char smem_dyn[];
     __shared__ int sh_last;
 
@@ -462,36 +435,36 @@ __global__ void __launch_bounds__(NW * 32) attn_mma_kernel(Geom gm, UnitTable ut
     const bool small = n_rows < (1 << 24);             // nsplit <= 32
     const int r_begin = small ? (int)((unsigned)n_rows * (unsigned)split / (unsigned)a.nsplit) : (int)((long long)n_rows * split / a.nsplit);
     const int r_end = small ? (int)((unsigned)n_rows * (unsigned)(split + 1) / (unsigned)a.nsplit) : (int)((long long)n_rows * (split + 1) / a.nsplit);
-    const int tiles_all = (r_end - r_begin + kTileTok - 1) / kTileTok;
+    const int tiles_all = (r_end - r_begin + kTok - 1) / kTok;
     // dealt evenly: no warp gets more than one tile above another (a tile beyond a warp's stages waits for
     // a stage to drain and then for its rows, a whole memory latency)
     const int tiles_lo = tiles_all / NW, tiles_rem = tiles_all % NW;
-    const int wb = min(r_end, r_begin + (warp * tiles_lo + min(warp, tiles_rem)) * kTileTok);
-    const int we = min(r_end, wb + (tiles_lo + (warp < tiles_rem ? 1 : 0)) * kTileTok);
-    const int n_tiles = (we - wb + kTileTok - 1) / kTileTok;
+    const int wb = min(r_end, r_begin + (warp * tiles_lo + min(warp, tiles_rem)) * kTok);
+    const int we = min(r_end, wb + (tiles_lo + (warp < tiles_rem ? 1 : 0)) * kTok);
+    const int n_tiles = (we - wb + kTok - 1) / kTok;
 
     unsigned char* my_stage = smem_dyn + (size_t)warp * kMmaStages * kStageBytes;
-    // the unit's rows in the cache and in the optional copies (see RowMap), 512 bytes per K|V row pair
-    const unsigned char* kv_unit = reinterpret_cast<const unsigned char*>(kv) + au.kv_c * gm.max_seq_len * 2 * D * 2;
-    const unsigned char* res_unit = reinterpret_cast<const unsigned char*>(a.res_rows) + au.kv_c * (size_t)(a.res_sinks + a.res_window) * 2 * D * 2;
-    const unsigned char* imp_unit = reinterpret_cast<const unsigned char*>(a.imp_rows) + au.list_c * (size_t)gm.idx_cap * 2 * D * 2;
+    // the unit's rows in the cache and in the optional copies (see RowMap)
+    const unsigned char* kv_unit = reinterpret_cast<const unsigned char*>(kv) + au.kv_c * gm.max_seq_len * kRowBytes;
+    const unsigned char* res_unit = reinterpret_cast<const unsigned char*>(a.res_rows) + au.kv_c * (size_t)(a.res_sinks + a.res_window) * kRowBytes;
+    const unsigned char* imp_unit = reinterpret_cast<const unsigned char*>(a.imp_rows) + au.list_c * (size_t)gm.idx_cap * kRowBytes;
 
     if (!waited) {
         pdl_wait();
         pdl_launch_dependents();
     }
     bool any_bad = false;
-    // Gather of one tile: the whole warp copies each 512-byte K|V row with one 16-byte cp.async per
-    // lane (one warp instruction per row; the per-row TMA bulk copies this replaces queued up at the
+    // Gather of one tile: the whole warp copies each K|V row with one 16-byte cp.async per
+    // lane and 512 bytes (one warp instruction per row; the per-row TMA bulk copies this replaces queued up at the
     // SM's single TMA port and took ~2 us to issue).  Rows past the end of the warp's range repeat
     // its last row (their probabilities are masked to zero), so a stage always holds finite numbers.
     // Every tile slot commits exactly one group, empty or not, so "all but the newest
     // kMmaStages-1 groups are complete" always means "the tile about to be used has landed".
     const uint32_t stage_u32 = smem_u32(my_stage);
-    auto issue_token = [&](int tile, int t) {     // t: lane i < 16 holds the token of row i
+    auto issue_token = [&](int tile, int t) {     // t: lane i < kTok holds the token of row i
         const uint32_t dst = stage_u32 + (tile % kMmaStages) * kStageBytes;
 #pragma unroll
-        for (int i = 0; i < kTileTok; ++i) {
+        for (int i = 0; i < kTok; ++i) {
             const int ti = __shfl_sync(0xffffffffu, t, i);
             const unsigned char* src = kv_unit;
             int row = ti;
@@ -500,20 +473,26 @@ __global__ void __launch_bounds__(NW * 32) attn_mma_kernel(Geom gm, UnitTable ut
                 src = which == 0 ? kv_unit : which == 1 ? res_unit : imp_unit;
                 row = ti & kRowIdxMask;
             }
-            asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst + i * kRowPitch + ((lane ^ (i & 7)) << 4)),
-                         "l"(src + lane * 16 + (size_t)row * 512) : "memory");
+            const unsigned char* from = src + lane * 16 + (size_t)row * kRowBytes;
+            if constexpr (kF32) {
+#pragma unroll
+                for (int half = 0; half < 2; ++half)
+                    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst + i * kRowBytes + half * 512 + lane * 16), "l"(from + half * 512) : "memory");
+            } else {
+                asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst + i * kRowPitch + ((lane ^ (i & 7)) << 4)), "l"(from) : "memory");
+            }
         }
     };
     auto commit = [&]() { asm volatile("cp.async.commit_group;" ::: "memory"); };
     attn_stamp(1);
-    // Lane i < 16 keeps, one bit per tile from the current one on, whether its row of that tile is a
+    // Lane i < kTok keeps, one bit per tile from the current one on, whether its row of that tile is a
     // bad list entry (outside the cached tokens): known when the tile's rows are issued, used when
     // the tile is consumed.  (Reading the entry a second time at consumption, as an earlier version did,
     // cost 5-8% of the kernel; fetching the entries one tile ahead of their issue cost 4% on
     // bandwidth-saturated launches and is not done.)
     uint32_t bad_bits = 0;
     auto tokens_of = [&](int tile) {                // -1 = bad entry
-        return (tile < n_tiles && lane < kTileTok) ? rm.token_or_neg(min(wb + tile * kTileTok + lane, we - 1)) : 0;
+        return (tile < n_tiles && lane < kTok) ? rm.token_or_neg(min(wb + tile * kTok + lane, we - 1)) : 0;
     };
     {   // the first tiles' list entries are fetched together (one memory round trip), then their rows
         int tok[kMmaStages];
@@ -530,196 +509,7 @@ __global__ void __launch_bounds__(NW * 32) attn_mma_kernel(Geom gm, UnitTable ut
 
     if (a.early_ok) pdl_wait();                        // the queries are this call's input
     attn_stamp(7);
-    // Q^T as the B operand of S = K Q^T: k = channels, n = query heads (gid; heads >= g are zero padding)
-    uint32_t qb[8][2];
-    {
-        const __nv_bfloat16* qbase = reinterpret_cast<const __nv_bfloat16*>(a.q) + ((size_t)(ll * ut.n_seq + s) * gm.Hq + h * g) * D;
-#pragma unroll
-        for (int ks = 0; ks < 8; ++ks) {
-            qb[ks][0] = qb[ks][1] = 0u;
-            if (gid < g) {
-                qb[ks][0] = __ldg(reinterpret_cast<const uint32_t*>(qbase + gid * D + ks * 16 + tig * 2));
-                qb[ks][1] = __ldg(reinterpret_cast<const uint32_t*>(qbase + gid * D + ks * 16 + 8 + tig * 2));
-            }
-        }
-    }
     const float qscale = a.sm_scale * kLog2e;
-#ifdef TB_PHASE_TIMING
-    if (qb[7][1] == 0x7fc1dead) any_bad = true;            // the stamp below waits for the queries
-    attn_stamp(8);
-#endif
-
-    // O^T accumulators: 8 tiles of (16 channels x 8 heads); this thread: channels mt*16 + gid (+8),
-    // heads 2*tig and 2*tig+1 -- the same two heads as its columns of S.
-    float o[8][4];
-#pragma unroll
-    for (int i = 0; i < 8; ++i) o[i][0] = o[i][1] = o[i][2] = o[i][3] = 0.f;
-    float m_run[2] = {-INFINITY, -INFINITY}, l_run[2] = {0.f, 0.f};   // heads 2*tig, 2*tig+1; l over this thread's tokens
-
-    // per-lane ldmatrix row addresses inside a stage
-    const int mi = lane >> 3, r8 = lane & 7;
-    // row offset + swizzled chunk: chunk 2 ks + (mi >> 1) of the K half, 16 + 2 mt + (mi & 1) of the V half,
-    // each xor (row & 7) = r8; the k-step / channel-tile part is xored in at the use
-    const uint32_t k_row_off = ((mi & 1) * 8 + r8) * kRowPitch, k_swz = (uint32_t)((mi >> 1) ^ r8) << 4;        // ^ ks * 32   (A of S = K Q^T)
-    const uint32_t v_row_off = ((mi >> 1) * 8 + r8) * kRowPitch + 256, v_swz = (uint32_t)((mi & 1) ^ r8) << 4;  // ^ mt * 32   (A of O^T = V^T P^T)
-
-    // A warp whose rows all fit its stages (two or three tiles: the latency-bound launches, where a block holds a
-    // few hundred rows) takes its first two tiles as one 32-token tile: the two S = K Q^T chains interleave, there
-    // is one softmax update instead of two, and every O^T accumulator gets four MMAs behind two loads.  One tile
-    // at a time is a chain of ~1500 dependent cycles per tile with nothing to overlap it in the warp.
-    int tile_first = 0;
-    if (n_tiles >= 2 && n_tiles <= kMmaStages) {
-        const bool inA = lane < kTileTok && wb + lane < we, inB = lane < kTileTok && wb + kTileTok + lane < we;
-        const bool badA = inA && (bad_bits & 1u), badB = inB && (bad_bits & 2u);
-        any_bad |= badA | badB;
-        bad_bits >>= 2;
-        const unsigned vmA = __ballot_sync(0xffffffffu, inA && !badA), vmB = __ballot_sync(0xffffffffu, inB && !badB);
-        asm volatile("cp.async.wait_group %0;" ::"n"(kMmaStages - 2) : "memory");
-        __syncwarp();
-        attn_stamp(3);
-        const uint32_t sA = stage_u32, sB = stage_u32 + kStageBytes;
-        float ca[4] = {0.f, 0.f, 0.f, 0.f}, cb[4] = {0.f, 0.f, 0.f, 0.f};
-#pragma unroll
-        for (int ks = 0; ks < 8; ++ks) {
-            uint32_t a0, a1, a2, a3, b0, b1, b2, b3;
-            ldmatrix_x4(sA + k_row_off + ((ks * 32) ^ k_swz), a0, a1, a2, a3);
-            ldmatrix_x4(sB + k_row_off + ((ks * 32) ^ k_swz), b0, b1, b2, b3);
-            mma_bf16(ca, a0, a1, a2, a3, qb[ks][0], qb[ks][1]);
-            mma_bf16(cb, b0, b1, b2, b3, qb[ks][0], qb[ks][1]);
-        }
-        const bool vA0 = (vmA >> gid) & 1u, vA1 = (vmA >> (gid + 8)) & 1u, vB0 = (vmB >> gid) & 1u, vB1 = (vmB >> (gid + 8)) & 1u;
-        float x[8];
-        x[0] = vA0 ? ca[0] * qscale : -INFINITY, x[1] = vA0 ? ca[1] * qscale : -INFINITY;
-        x[2] = vA1 ? ca[2] * qscale : -INFINITY, x[3] = vA1 ? ca[3] * qscale : -INFINITY;
-        x[4] = vB0 ? cb[0] * qscale : -INFINITY, x[5] = vB0 ? cb[1] * qscale : -INFINITY;
-        x[6] = vB1 ? cb[2] * qscale : -INFINITY, x[7] = vB1 ? cb[3] * qscale : -INFINITY;
-        float tmax[2] = {fmaxf(fmaxf(x[0], x[2]), fmaxf(x[4], x[6])), fmaxf(fmaxf(x[1], x[3]), fmaxf(x[5], x[7]))};
-#pragma unroll
-        for (int off = 4; off < 32; off <<= 1) {
-            tmax[0] = fmaxf(tmax[0], __shfl_xor_sync(0xffffffffu, tmax[0], off));
-            tmax[1] = fmaxf(tmax[1], __shfl_xor_sync(0xffffffffu, tmax[1], off));
-        }
-        // these are the warp's first rows: nothing accumulated yet to rescale
-        m_run[0] = tmax[0], m_run[1] = tmax[1];
-        const float ms0 = tmax[0] == -INFINITY ? 0.f : tmax[0], ms1 = tmax[1] == -INFINITY ? 0.f : tmax[1];
-        float p[8];
-#pragma unroll
-        for (int i = 0; i < 8; ++i) p[i] = exp2f(x[i] - ((i & 1) ? ms1 : ms0));
-        l_run[0] = (p[0] + p[2]) + (p[4] + p[6]);
-        l_run[1] = (p[1] + p[3]) + (p[5] + p[7]);
-        float ph[8], pl[8];
-#pragma unroll
-        for (int i = 0; i < 8; ++i) {
-            ph[i] = __bfloat162float(__float2bfloat16_rn(p[i]));
-            pl[i] = p[i] - ph[i];
-        }
-        const uint32_t hA0 = movmatrix_trans(pack_bf16(ph[0], ph[1])), hA1 = movmatrix_trans(pack_bf16(ph[2], ph[3]));
-        const uint32_t lA0 = movmatrix_trans(pack_bf16(pl[0], pl[1])), lA1 = movmatrix_trans(pack_bf16(pl[2], pl[3]));
-        const uint32_t hB0 = movmatrix_trans(pack_bf16(ph[4], ph[5])), hB1 = movmatrix_trans(pack_bf16(ph[6], ph[7]));
-        const uint32_t lB0 = movmatrix_trans(pack_bf16(pl[4], pl[5])), lB1 = movmatrix_trans(pack_bf16(pl[6], pl[7]));
-#pragma unroll
-        for (int mt = 0; mt < 8; ++mt) {
-            uint32_t a0, a1, a2, a3, b0, b1, b2, b3;
-            ldmatrix_x4_trans(sA + v_row_off + ((mt * 32) ^ v_swz), a0, a1, a2, a3);
-            ldmatrix_x4_trans(sB + v_row_off + ((mt * 32) ^ v_swz), b0, b1, b2, b3);
-            mma_bf16(o[mt], a0, a1, a2, a3, hA0, hA1);
-            mma_bf16(o[mt], a0, a1, a2, a3, lA0, lA1);
-            mma_bf16(o[mt], b0, b1, b2, b3, hB0, hB1);
-            mma_bf16(o[mt], b0, b1, b2, b3, lB0, lB1);
-        }
-        __syncwarp();
-        commit(), commit();                            // the two tile slots' groups of the loop below
-        tile_first = 2;
-    }
-    for (int tile = tile_first; tile < n_tiles; ++tile) {
-        const int st = tile % kMmaStages;
-        const int r0 = wb + tile * kTileTok;
-        // validity of the tile's 16 rows (past-the-end and out-of-range list entries are masked)
-        const bool in_range = lane < kTileTok && r0 + lane < we;
-        const bool bad = in_range && (bad_bits & 1u);
-        any_bad |= bad;
-        bad_bits >>= 1;
-        const unsigned vmask = __ballot_sync(0xffffffffu, in_range && !bad);
-        asm volatile("cp.async.wait_group %0;" ::"n"(kMmaStages - 1) : "memory");
-        __syncwarp();                                  // every lane's copies of this tile are visible to the warp
-        if (tile == 0) attn_stamp(3);
-        const uint32_t sb = stage_u32 + st * kStageBytes;
-
-        // S[token][head]: this thread holds tokens gid (c0,c1) and gid+8 (c2,c3), heads 2*tig, 2*tig+1
-        float sc[4] = {0.f, 0.f, 0.f, 0.f};
-#pragma unroll
-        for (int ks = 0; ks < 8; ++ks) {
-            uint32_t a0, a1, a2, a3;
-            ldmatrix_x4(sb + k_row_off + ((ks * 32) ^ k_swz), a0, a1, a2, a3);
-            mma_bf16(sc, a0, a1, a2, a3, qb[ks][0], qb[ks][1]);
-        }
-#ifdef TB_PHASE_TIMING
-        if (tile == 0) { if (sc[0] == 1.2345e33f) any_bad = true; attn_stamp(9); }
-#endif
-        const bool v0 = (vmask >> gid) & 1u, v1 = (vmask >> (gid + 8)) & 1u;
-        float x[4];
-        x[0] = v0 ? sc[0] * qscale : -INFINITY, x[1] = v0 ? sc[1] * qscale : -INFINITY;
-        x[2] = v1 ? sc[2] * qscale : -INFINITY, x[3] = v1 ? sc[3] * qscale : -INFINITY;
-        float tmax[2] = {fmaxf(x[0], x[2]), fmaxf(x[1], x[3])};
-#pragma unroll
-        for (int off = 4; off < 32; off <<= 1) {       // over the 8 token rows held by lanes with the same tig
-            tmax[0] = fmaxf(tmax[0], __shfl_xor_sync(0xffffffffu, tmax[0], off));
-            tmax[1] = fmaxf(tmax[1], __shfl_xor_sync(0xffffffffu, tmax[1], off));
-        }
-        float corr[2], ms[2];
-#pragma unroll
-        for (int e = 0; e < 2; ++e) {
-            const float m_new = fmaxf(m_run[e], tmax[e]);
-            ms[e] = m_new == -INFINITY ? 0.f : m_new;
-            corr[e] = exp2f(m_run[e] - ms[e]);
-            m_run[e] = m_new;
-        }
-        float p[4];
-        p[0] = exp2f(x[0] - ms[0]), p[1] = exp2f(x[1] - ms[1]), p[2] = exp2f(x[2] - ms[0]), p[3] = exp2f(x[3] - ms[1]);
-        l_run[0] = l_run[0] * corr[0] + p[0] + p[2];
-        l_run[1] = l_run[1] * corr[1] + p[1] + p[3];
-        if (__any_sync(0xffffffffu, corr[0] != 1.f || corr[1] != 1.f)) {
-#pragma unroll
-            for (int i = 0; i < 8; ++i) o[i][0] *= corr[0], o[i][1] *= corr[1], o[i][2] *= corr[0], o[i][3] *= corr[1];
-        }
-        // P = P_hi + P_lo in bf16, transposed into the B operand (k = tokens, n = heads)
-        float ph[4], pl[4];
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            ph[i] = __bfloat162float(__float2bfloat16_rn(p[i]));
-            pl[i] = p[i] - ph[i];
-        }
-        const uint32_t bh0 = movmatrix_trans(pack_bf16(ph[0], ph[1])), bh1 = movmatrix_trans(pack_bf16(ph[2], ph[3]));
-        const uint32_t bl0 = movmatrix_trans(pack_bf16(pl[0], pl[1])), bl1 = movmatrix_trans(pack_bf16(pl[2], pl[3]));
-#pragma unroll
-        for (int mt = 0; mt < 8; ++mt) {
-            uint32_t a0, a1, a2, a3;
-            ldmatrix_x4_trans(sb + v_row_off + ((mt * 32) ^ v_swz), a0, a1, a2, a3);
-            mma_bf16(o[mt], a0, a1, a2, a3, bh0, bh1);
-            mma_bf16(o[mt], a0, a1, a2, a3, bl0, bl1);
-        }
-#ifdef TB_PHASE_TIMING
-        if (tile == 0) { if (o[7][3] == 1.2345e33f) any_bad = true; attn_stamp(10); }
-#endif
-        __syncwarp();                                  // the warp is done reading this stage
-        if (tile + kMmaStages < n_tiles) {
-            const int t = tokens_of(tile + kMmaStages);
-            bad_bits |= (uint32_t)(t < 0) << (kMmaStages - 1);         // bit k is tile + 1 + k now
-            issue_token(tile + kMmaStages, max(t, 0));
-        }
-        commit();
-    }
-    asm volatile("cp.async.wait_group 0;" ::: "memory");
-    if (any_bad && lane < kTileTok) atomicExch(status, kStatusBadIndex);
-
-    // ---- the warps' results become the block's, the blocks' the problem's -------------------------------
-    attn_stamp(4);
-#pragma unroll
-    for (int off = 4; off < 32; off <<= 1) {
-        l_run[0] += __shfl_xor_sync(0xffffffffu, l_run[0], off);
-        l_run[1] += __shfl_xor_sync(0xffffffffu, l_run[1], off);
-    }
-    __syncwarp();
     const size_t hq0 = (size_t)(ll * ut.n_seq + s) * gm.Hq + h * g;
     // Every warp parks its accumulators in its own (drained) stages, lane by lane in the MMA layout -- float4
     // number mt * 32 + lane is accumulator tile mt (16 channels) of that lane, number 256 + lane its (m, l) of
@@ -729,12 +519,204 @@ __global__ void __launch_bounds__(NW * 32) attn_mma_kernel(Geom gm, UnitTable ut
     // (Measured alternatives, all within 0.03 us per launch of this one: a binary tree over the warps with a
     // named barrier per pair; two barriers with the weights computed once.  Parking only the lanes of real heads
     // when the group has at most four -- half the shared-memory traffic, 16 shuffles -- was 0.5 us slower.)
-    {
-        float4* tbuf = reinterpret_cast<float4*>(my_stage);
+    // (bf16 and fp32 work differs up to here; from the parked accumulators on they are the same.)
+    float4* tbuf = reinterpret_cast<float4*>(my_stage);
+    if constexpr (kF32) {
+        f32_rows<FG, kMmaStages>(reinterpret_cast<const float*>(a.q) + hq0 * D, g, qscale, my_stage, wb, we, n_tiles, bad_bits, any_bad, tokens_of, issue_token, commit);
+    } else {
+        // Q^T as the B operand of S = K Q^T: k = channels, n = query heads (gid; heads >= g are zero padding)
+        uint32_t qb[8][2];
+        {
+            const __nv_bfloat16* qbase = reinterpret_cast<const __nv_bfloat16*>(a.q) + ((size_t)(ll * ut.n_seq + s) * gm.Hq + h * g) * D;
+#pragma unroll
+            for (int ks = 0; ks < 8; ++ks) {
+                qb[ks][0] = qb[ks][1] = 0u;
+                if (gid < g) {
+                    qb[ks][0] = __ldg(reinterpret_cast<const uint32_t*>(qbase + gid * D + ks * 16 + tig * 2));
+                    qb[ks][1] = __ldg(reinterpret_cast<const uint32_t*>(qbase + gid * D + ks * 16 + 8 + tig * 2));
+                }
+            }
+        }
+#ifdef TB_PHASE_TIMING
+        if (qb[7][1] == 0x7fc1dead) any_bad = true;            // the stamp below waits for the queries
+        attn_stamp(8);
+#endif
+
+        // O^T accumulators: 8 tiles of (16 channels x 8 heads); this thread: channels mt*16 + gid (+8),
+        // heads 2*tig and 2*tig+1 -- the same two heads as its columns of S.
+        float o[8][4];
+#pragma unroll
+        for (int i = 0; i < 8; ++i) o[i][0] = o[i][1] = o[i][2] = o[i][3] = 0.f;
+        float m_run[2] = {-INFINITY, -INFINITY}, l_run[2] = {0.f, 0.f};   // heads 2*tig, 2*tig+1; l over this thread's tokens
+
+        // per-lane ldmatrix row addresses inside a stage
+        const int mi = lane >> 3, r8 = lane & 7;
+        // row offset + swizzled chunk: chunk 2 ks + (mi >> 1) of the K half, 16 + 2 mt + (mi & 1) of the V half,
+        // each xor (row & 7) = r8; the k-step / channel-tile part is xored in at the use
+        const uint32_t k_row_off = ((mi & 1) * 8 + r8) * kRowPitch, k_swz = (uint32_t)((mi >> 1) ^ r8) << 4;        // ^ ks * 32   (A of S = K Q^T)
+        const uint32_t v_row_off = ((mi >> 1) * 8 + r8) * kRowPitch + 256, v_swz = (uint32_t)((mi & 1) ^ r8) << 4;  // ^ mt * 32   (A of O^T = V^T P^T)
+
+        // A warp whose rows all fit its stages (two or three tiles: the latency-bound launches, where a block holds a
+        // few hundred rows) takes its first two tiles as one 32-token tile: the two S = K Q^T chains interleave, there
+        // is one softmax update instead of two, and every O^T accumulator gets four MMAs behind two loads.  One tile
+        // at a time is a chain of ~1500 dependent cycles per tile with nothing to overlap it in the warp.
+        int tile_first = 0;
+        if (n_tiles >= 2 && n_tiles <= kMmaStages) {
+            const bool inA = lane < kTileTok && wb + lane < we, inB = lane < kTileTok && wb + kTileTok + lane < we;
+            const bool badA = inA && (bad_bits & 1u), badB = inB && (bad_bits & 2u);
+            any_bad |= badA | badB;
+            bad_bits >>= 2;
+            const unsigned vmA = __ballot_sync(0xffffffffu, inA && !badA), vmB = __ballot_sync(0xffffffffu, inB && !badB);
+            asm volatile("cp.async.wait_group %0;" ::"n"(kMmaStages - 2) : "memory");
+            __syncwarp();
+            attn_stamp(3);
+            const uint32_t sA = stage_u32, sB = stage_u32 + kStageBytes;
+            float ca[4] = {0.f, 0.f, 0.f, 0.f}, cb[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+            for (int ks = 0; ks < 8; ++ks) {
+                uint32_t a0, a1, a2, a3, b0, b1, b2, b3;
+                ldmatrix_x4(sA + k_row_off + ((ks * 32) ^ k_swz), a0, a1, a2, a3);
+                ldmatrix_x4(sB + k_row_off + ((ks * 32) ^ k_swz), b0, b1, b2, b3);
+                mma_bf16(ca, a0, a1, a2, a3, qb[ks][0], qb[ks][1]);
+                mma_bf16(cb, b0, b1, b2, b3, qb[ks][0], qb[ks][1]);
+            }
+            const bool vA0 = (vmA >> gid) & 1u, vA1 = (vmA >> (gid + 8)) & 1u, vB0 = (vmB >> gid) & 1u, vB1 = (vmB >> (gid + 8)) & 1u;
+            float x[8];
+            x[0] = vA0 ? ca[0] * qscale : -INFINITY, x[1] = vA0 ? ca[1] * qscale : -INFINITY;
+            x[2] = vA1 ? ca[2] * qscale : -INFINITY, x[3] = vA1 ? ca[3] * qscale : -INFINITY;
+            x[4] = vB0 ? cb[0] * qscale : -INFINITY, x[5] = vB0 ? cb[1] * qscale : -INFINITY;
+            x[6] = vB1 ? cb[2] * qscale : -INFINITY, x[7] = vB1 ? cb[3] * qscale : -INFINITY;
+            float tmax[2] = {fmaxf(fmaxf(x[0], x[2]), fmaxf(x[4], x[6])), fmaxf(fmaxf(x[1], x[3]), fmaxf(x[5], x[7]))};
+#pragma unroll
+            for (int off = 4; off < 32; off <<= 1) {
+                tmax[0] = fmaxf(tmax[0], __shfl_xor_sync(0xffffffffu, tmax[0], off));
+                tmax[1] = fmaxf(tmax[1], __shfl_xor_sync(0xffffffffu, tmax[1], off));
+            }
+            // these are the warp's first rows: nothing accumulated yet to rescale
+            m_run[0] = tmax[0], m_run[1] = tmax[1];
+            const float ms0 = tmax[0] == -INFINITY ? 0.f : tmax[0], ms1 = tmax[1] == -INFINITY ? 0.f : tmax[1];
+            float p[8];
+#pragma unroll
+            for (int i = 0; i < 8; ++i) p[i] = exp2f(x[i] - ((i & 1) ? ms1 : ms0));
+            l_run[0] = (p[0] + p[2]) + (p[4] + p[6]);
+            l_run[1] = (p[1] + p[3]) + (p[5] + p[7]);
+            float ph[8], pl[8];
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+                ph[i] = __bfloat162float(__float2bfloat16_rn(p[i]));
+                pl[i] = p[i] - ph[i];
+            }
+            const uint32_t hA0 = movmatrix_trans(pack_bf16(ph[0], ph[1])), hA1 = movmatrix_trans(pack_bf16(ph[2], ph[3]));
+            const uint32_t lA0 = movmatrix_trans(pack_bf16(pl[0], pl[1])), lA1 = movmatrix_trans(pack_bf16(pl[2], pl[3]));
+            const uint32_t hB0 = movmatrix_trans(pack_bf16(ph[4], ph[5])), hB1 = movmatrix_trans(pack_bf16(ph[6], ph[7]));
+            const uint32_t lB0 = movmatrix_trans(pack_bf16(pl[4], pl[5])), lB1 = movmatrix_trans(pack_bf16(pl[6], pl[7]));
+#pragma unroll
+            for (int mt = 0; mt < 8; ++mt) {
+                uint32_t a0, a1, a2, a3, b0, b1, b2, b3;
+                ldmatrix_x4_trans(sA + v_row_off + ((mt * 32) ^ v_swz), a0, a1, a2, a3);
+                ldmatrix_x4_trans(sB + v_row_off + ((mt * 32) ^ v_swz), b0, b1, b2, b3);
+                mma_bf16(o[mt], a0, a1, a2, a3, hA0, hA1);
+                mma_bf16(o[mt], a0, a1, a2, a3, lA0, lA1);
+                mma_bf16(o[mt], b0, b1, b2, b3, hB0, hB1);
+                mma_bf16(o[mt], b0, b1, b2, b3, lB0, lB1);
+            }
+            __syncwarp();
+            commit(), commit();                            // the two tile slots' groups of the loop below
+            tile_first = 2;
+        }
+        for (int tile = tile_first; tile < n_tiles; ++tile) {
+            const int st = tile % kMmaStages;
+            const int r0 = wb + tile * kTileTok;
+            // validity of the tile's 16 rows (past-the-end and out-of-range list entries are masked)
+            const bool in_range = lane < kTileTok && r0 + lane < we;
+            const bool bad = in_range && (bad_bits & 1u);
+            any_bad |= bad;
+            bad_bits >>= 1;
+            const unsigned vmask = __ballot_sync(0xffffffffu, in_range && !bad);
+            asm volatile("cp.async.wait_group %0;" ::"n"(kMmaStages - 1) : "memory");
+            __syncwarp();                                  // every lane's copies of this tile are visible to the warp
+            if (tile == 0) attn_stamp(3);
+            const uint32_t sb = stage_u32 + st * kStageBytes;
+
+            // S[token][head]: this thread holds tokens gid (c0,c1) and gid+8 (c2,c3), heads 2*tig, 2*tig+1
+            float sc[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+            for (int ks = 0; ks < 8; ++ks) {
+                uint32_t a0, a1, a2, a3;
+                ldmatrix_x4(sb + k_row_off + ((ks * 32) ^ k_swz), a0, a1, a2, a3);
+                mma_bf16(sc, a0, a1, a2, a3, qb[ks][0], qb[ks][1]);
+            }
+#ifdef TB_PHASE_TIMING
+            if (tile == 0) { if (sc[0] == 1.2345e33f) any_bad = true; attn_stamp(9); }
+#endif
+            const bool v0 = (vmask >> gid) & 1u, v1 = (vmask >> (gid + 8)) & 1u;
+            float x[4];
+            x[0] = v0 ? sc[0] * qscale : -INFINITY, x[1] = v0 ? sc[1] * qscale : -INFINITY;
+            x[2] = v1 ? sc[2] * qscale : -INFINITY, x[3] = v1 ? sc[3] * qscale : -INFINITY;
+            float tmax[2] = {fmaxf(x[0], x[2]), fmaxf(x[1], x[3])};
+#pragma unroll
+            for (int off = 4; off < 32; off <<= 1) {       // over the 8 token rows held by lanes with the same tig
+                tmax[0] = fmaxf(tmax[0], __shfl_xor_sync(0xffffffffu, tmax[0], off));
+                tmax[1] = fmaxf(tmax[1], __shfl_xor_sync(0xffffffffu, tmax[1], off));
+            }
+            float corr[2], ms[2];
+#pragma unroll
+            for (int e = 0; e < 2; ++e) {
+                const float m_new = fmaxf(m_run[e], tmax[e]);
+                ms[e] = m_new == -INFINITY ? 0.f : m_new;
+                corr[e] = exp2f(m_run[e] - ms[e]);
+                m_run[e] = m_new;
+            }
+            float p[4];
+            p[0] = exp2f(x[0] - ms[0]), p[1] = exp2f(x[1] - ms[1]), p[2] = exp2f(x[2] - ms[0]), p[3] = exp2f(x[3] - ms[1]);
+            l_run[0] = l_run[0] * corr[0] + p[0] + p[2];
+            l_run[1] = l_run[1] * corr[1] + p[1] + p[3];
+            if (__any_sync(0xffffffffu, corr[0] != 1.f || corr[1] != 1.f)) {
+#pragma unroll
+                for (int i = 0; i < 8; ++i) o[i][0] *= corr[0], o[i][1] *= corr[1], o[i][2] *= corr[0], o[i][3] *= corr[1];
+            }
+            // P = P_hi + P_lo in bf16, transposed into the B operand (k = tokens, n = heads)
+            float ph[4], pl[4];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                ph[i] = __bfloat162float(__float2bfloat16_rn(p[i]));
+                pl[i] = p[i] - ph[i];
+            }
+            const uint32_t bh0 = movmatrix_trans(pack_bf16(ph[0], ph[1])), bh1 = movmatrix_trans(pack_bf16(ph[2], ph[3]));
+            const uint32_t bl0 = movmatrix_trans(pack_bf16(pl[0], pl[1])), bl1 = movmatrix_trans(pack_bf16(pl[2], pl[3]));
+#pragma unroll
+            for (int mt = 0; mt < 8; ++mt) {
+                uint32_t a0, a1, a2, a3;
+                ldmatrix_x4_trans(sb + v_row_off + ((mt * 32) ^ v_swz), a0, a1, a2, a3);
+                mma_bf16(o[mt], a0, a1, a2, a3, bh0, bh1);
+                mma_bf16(o[mt], a0, a1, a2, a3, bl0, bl1);
+            }
+#ifdef TB_PHASE_TIMING
+            if (tile == 0) { if (o[7][3] == 1.2345e33f) any_bad = true; attn_stamp(10); }
+#endif
+            __syncwarp();                                  // the warp is done reading this stage
+            if (tile + kMmaStages < n_tiles) {
+                const int t = tokens_of(tile + kMmaStages);
+                bad_bits |= (uint32_t)(t < 0) << (kMmaStages - 1);         // bit k is tile + 1 + k now
+                issue_token(tile + kMmaStages, max(t, 0));
+            }
+            commit();
+        }
+        asm volatile("cp.async.wait_group 0;" ::: "memory");
+        attn_stamp(4);
+#pragma unroll
+        for (int off = 4; off < 32; off <<= 1) {
+            l_run[0] += __shfl_xor_sync(0xffffffffu, l_run[0], off);
+            l_run[1] += __shfl_xor_sync(0xffffffffu, l_run[1], off);
+        }
+        __syncwarp();
 #pragma unroll
         for (int mt = 0; mt < 8; ++mt) tbuf[mt * 32 + lane] = make_float4(o[mt][0], o[mt][1], o[mt][2], o[mt][3]);
         tbuf[8 * 32 + lane] = make_float4(m_run[0], l_run[0], m_run[1], l_run[1]);
     }
+    if (any_bad && lane < kTok) atomicExch(status, kStatusBadIndex);
+
+    // ---- the warps' results become the block's, the blocks' the problem's -------------------------------
     __syncthreads();
     auto warp_buf = [&](int w) { return reinterpret_cast<const float4*>(smem_dyn + (size_t)w * kMmaStages * kStageBytes); };
     // block result of slot (mt, ln): acc = (head 2tg ch, head 2tg+1 ch, head 2tg ch+8, head 2tg+1 ch+8), ch = mt*16 + ln/4
@@ -883,7 +865,9 @@ cudaError_t launch_attention(const tb_ctx* c, const UnitTable& ut, const AttnArg
     const int units = ut.layer_count * ut.n_seq * gm.Ha;
     a.cluster_merge = 0;
     int nw = kAttnWarps;
-    if (gm.dtype == TB_BF16) {
+    const bool f32 = gm.dtype != TB_BF16;
+    const int tok = f32 ? 8 : kTileTok;               // rows of a stage
+    {
         static unsigned char seen[64];
         int* max_active = const_cast<tb_ctx*>(c)->attn_max_active;
         if (first_use_on_this_device(seen)) {
@@ -897,6 +881,13 @@ cudaError_t launch_attention(const tb_ctx* c, const UnitTable& ut, const AttnArg
             prepare(attn_mma_kernel<8, 2, false>, 220, true), prepare(attn_mma_kernel<8, 2, true>, 220, true);
             prepare(attn_mma_kernel<8, 3, false>, 220, true), prepare(attn_mma_kernel<8, 3, true>, 220, true);
             prepare(attn_mma_kernel<12, 2, false>, 224, false), prepare(attn_mma_kernel<12, 2, true>, 224, false);
+            auto prepare_f32 = [&](auto group) {
+                constexpr int G = decltype(group)::value;
+                prepare(attn_mma_kernel<4, 2, true, G>, 113, true), prepare(attn_mma_kernel<8, 2, true, G>, 220, true);
+                prepare(attn_mma_kernel<8, 3, true, G>, 220, true);
+            };
+            prepare_f32(std::integral_constant<int, 1>{}), prepare_f32(std::integral_constant<int, 2>{});
+            prepare_f32(std::integral_constant<int, 4>{}), prepare_f32(std::integral_constant<int, 8>{});
             if (e != cudaSuccess) return e;
             (void)cudaGetLastError();
         }
@@ -925,7 +916,7 @@ cudaError_t launch_attention(const tb_ctx* c, const UnitTable& ut, const AttnArg
         // for every problem at once; the splits merge inside the cluster.  Many problems: 4-warp
         // blocks, two per SM, clusters of up to 8; splits beyond that go through the global workspace.
         int n = 0;
-        const int by_rows = max_rows / (8 * kTileTok) < 1 ? 1 : max_rows / (8 * kTileTok);
+        const int by_rows = max_rows / (8 * tok) < 1 ? 1 : max_rows / (8 * tok);
 #ifdef TB_FORCE_ATTN_CLUSTER
         n = TB_FORCE_ATTN_CLUSTER;
 #else
@@ -940,33 +931,21 @@ cudaError_t launch_attention(const tb_ctx* c, const UnitTable& ut, const AttnArg
         for (int cand = 16; cand >= 1 && !n; cand = cand > 8 ? cand - 2 : cand - 1)
             if (cand <= by_rows && units * cand <= c->sm_count && (cand <= 8 || clusters_that_fit(cand) >= units)) n = cand;
 #endif
-        if (n && max_rows / n <= 1024) {
+        if (n && max_rows / n <= 64 * tok) {
             a.nsplit = n, nw = 8, a.cluster_merge = 1;
             // more than two tiles per warp would leave the third waiting for a free stage: 12 warps
             // per block when their rings and the merge area still fit the SM
             const int rows_per_block = (max_rows + n - 1) / n;
-            if (rows_per_block > 8 * 2 * kTileTok && 12 * 2 * kStageBytes + cluster_merge_bytes(n) <= 224 * 1024) nw = 12;
+            if (!f32 && rows_per_block > 8 * 2 * kTileTok && 12 * 2 * kStageBytes + cluster_merge_bytes(n) <= 224 * 1024) nw = 12;
         } else {
             a.nsplit = pick_nsplit(c, units, max_rows);
             // clusters only when the whole launch is resident at once: in multi-wave launches the
             // co-scheduling constraint costs more than the global merge (measured on the batch-8 workload)
             if (a.nsplit <= 8 && units * a.nsplit <= 2 * c->sm_count) a.cluster_merge = 1;
         }
-    } else {
-        a.nsplit = pick_nsplit(c, units, max_rows);
     }
     dim3 grid(a.nsplit, gm.Ha, ut.layer_count * ut.n_seq);
-#define TB_ATTN(T, G)                                                                                                   \
-    attn_kernel<T, G><<<grid, kAttnThreads, 0, s>>>(gm, ut, a, (const T*)c->kv, c->st.idx, c->st.cnt, c->wk.part_o,     \
-                                                   c->wk.part_ml, c->st.attn_counter, c->st.status)
-#define TB_ATTN_G(T)                                  \
-    do {                                              \
-        if (gm.ga == 1) TB_ATTN(T, 1);                \
-        else if (gm.ga == 2) TB_ATTN(T, 2);           \
-        else if (gm.ga <= 4) TB_ATTN(T, 4);           \
-        else TB_ATTN(T, 8);                           \
-    } while (0)
-    if (gm.dtype == TB_BF16) {
+    {
         const size_t merge_bytes = a.cluster_merge ? cluster_merge_bytes(a.nsplit) : 0;
         // three stages per warp when the 8-warp block still fits the SM with them
         const int nst = (nw == 8 && 8 * 3 * kStageBytes + merge_bytes <= 220 * 1024 && a.nsplit <= 8) ? 3 : 2;
@@ -990,24 +969,28 @@ cudaError_t launch_attention(const tb_ctx* c, const UnitTable& ut, const AttnArg
         attr[1].val.programmaticStreamSerializationAllowed = 1;
         cfg.attrs = attr;
         cfg.numAttrs = 2;
-        const __nv_bfloat16* kvp = (const __nv_bfloat16*)c->kv;
+        auto launch = [&](auto kernel) {
+            return cudaLaunchKernelEx(&cfg, kernel, gm, ut, a, (const void*)c->kv, (const int32_t*)c->st.idx, (const int32_t*)c->st.cnt, c->wk.part_o,
+                                      c->wk.part_ml, c->st.attn_counter, c->st.status);
+        };
+        if (f32) {
+            auto launch_f32 = [&](auto group) {
+                constexpr int G = decltype(group)::value;
+                return nw == 4 ? launch(attn_mma_kernel<4, 2, true, G>) : nst == 3 ? launch(attn_mma_kernel<8, 3, true, G>) : launch(attn_mma_kernel<8, 2, true, G>);
+            };
+            if (gm.ga == 1) return launch_f32(std::integral_constant<int, 1>{});
+            if (gm.ga == 2) return launch_f32(std::integral_constant<int, 2>{});
+            if (gm.ga <= 4) return launch_f32(std::integral_constant<int, 4>{});
+            return launch_f32(std::integral_constant<int, 8>{});
+        }
         const bool sources = a.res_rows != nullptr || a.imp_rows != nullptr;
-#define TB_MMA(NW_, ST_)                                                                                                          \
-    (sources ? cudaLaunchKernelEx(&cfg, attn_mma_kernel<NW_, ST_, true>, gm, ut, a, kvp, (const int32_t*)c->st.idx,               \
-                                  (const int32_t*)c->st.cnt, c->wk.part_o, c->wk.part_ml, c->st.attn_counter, c->st.status)       \
-             : cudaLaunchKernelEx(&cfg, attn_mma_kernel<NW_, ST_, false>, gm, ut, a, kvp, (const int32_t*)c->st.idx,              \
-                                  (const int32_t*)c->st.cnt, c->wk.part_o, c->wk.part_ml, c->st.attn_counter, c->st.status))
+#define TB_MMA(NW_, ST_) (sources ? launch(attn_mma_kernel<NW_, ST_, true>) : launch(attn_mma_kernel<NW_, ST_, false>))
         if (nw == 12) return TB_MMA(12, 2);
         if (nw == 8 && nst == 3) return TB_MMA(8, 3);
         if (nw == 8) return TB_MMA(8, 2);
         return TB_MMA(4, 2);
 #undef TB_MMA
-    } else {
-        TB_ATTN_G(float);
     }
-#undef TB_ATTN_G
-#undef TB_ATTN
-    return cudaGetLastError();
 }
 
 }  // namespace tb
@@ -1047,7 +1030,9 @@ tb_status static_scratch_for_current_device(unsigned char** out, int* sm_count) 
         if (cudaGetSymbolAddress(&p, g_static_scratch) != cudaSuccess || !p) return TB_ERR_CUDA;
         int sms = 0;
         if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return TB_ERR_CUDA;
-        if (cudaFuncSetAttribute(tb::attn_mma_kernel<4, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, 113 * 1024) != cudaSuccess)
+        const auto prepare = [](auto kernel) { return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 113 * 1024) == cudaSuccess; };
+        if (!prepare(tb::attn_mma_kernel<4, 2>) || !prepare(tb::attn_mma_kernel<4, 2, true, 1>) || !prepare(tb::attn_mma_kernel<4, 2, true, 2>) ||
+            !prepare(tb::attn_mma_kernel<4, 2, true, 4>) || !prepare(tb::attn_mma_kernel<4, 2, true, 8>))
             return TB_ERR_CUDA;
         g_sm_count[dev] = sms;
         g_scratch_addr[dev] = static_cast<unsigned char*>(p);
@@ -1141,14 +1126,14 @@ extern "C" tb_status tb_sparse_decode_attention_static(const void* kv_dev, int32
     if (cudaMemsetAsync(counters, 0, kStaticCounters, s) != cudaSuccess) return TB_ERR_CUDA;
     dim3 grid(a.nsplit, n_kv_heads, n_seq);
     // the stored-list arguments of the kernels are never read here (caller lists or dense)
-    if (kv_dtype == TB_BF16) {
-        attn_mma_kernel<4, 2><<<grid, kAttnThreads, kAttnWarps * 2 * kStageBytes, s>>>(
-            gm, ut, a, (const __nv_bfloat16*)kv_dev, nullptr, nullptr, part_o, part_ml, counters, status);
-    } else {
-#define TB_ATTN_S(G) attn_kernel<float, G><<<grid, kAttnThreads, 0, s>>>(gm, ut, a, (const float*)kv_dev, nullptr, nullptr, part_o, part_ml, counters, status)
-        if (gm.ga == 1) TB_ATTN_S(1); else if (gm.ga == 2) TB_ATTN_S(2); else if (gm.ga <= 4) TB_ATTN_S(4); else TB_ATTN_S(8);
-#undef TB_ATTN_S
-    }
+    const auto launch = [&](auto kernel) {
+        kernel<<<grid, kAttnThreads, kAttnWarps * 2 * kStageBytes, s>>>(gm, ut, a, kv_dev, nullptr, nullptr, part_o, part_ml, counters, status);
+    };
+    if (kv_dtype == TB_BF16) launch(attn_mma_kernel<4, 2>);
+    else if (gm.ga == 1) launch(attn_mma_kernel<4, 2, true, 1>);
+    else if (gm.ga == 2) launch(attn_mma_kernel<4, 2, true, 2>);
+    else if (gm.ga <= 4) launch(attn_mma_kernel<4, 2, true, 4>);
+    else launch(attn_mma_kernel<4, 2, true, 8>);
     return cudaGetLastError() == cudaSuccess ? TB_OK : TB_ERR_CUDA;
 }
 

@@ -678,3 +678,13 @@ def test_small_selection_kernel_unusual_distributions(H):
         x = _bf16_exact(r.standard_normal(shape))
         x[:, :, 7] = 1e6
         _crafted_batch_case(H, _bf16_exact(x), budget=200)
+
+
+@pytest.mark.parametrize("heads", [1, 2, 3, 4, 7, 8])
+@pytest.mark.parametrize("budget", [1, 7, 64, 130, 600, 2500])
+def test_fp32_attention_shapes(H, heads, budget):
+    """fp32 tiles of 8 rows: every group-size instance, rows that leave partial tiles, one block and clusters, few problems
+    and (dense, in the same context) many splits."""
+    w = wl.workload(1, n_layers=1, n_q_heads=2 * heads, n_kv_heads=2, batch=2, lengths=[budget + 300, max(60, budget // 2)], budget=budget, sinks=3,
+                    recent=5)
+    full_pipeline_check(H, H.Case(w), tb().select_params(budget, 3, 5), dense_too=True)
