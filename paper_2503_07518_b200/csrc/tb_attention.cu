@@ -74,7 +74,7 @@ struct AttnUnit {
 
 // Publishes one split's (m, l, o) per query head and lets the last block to arrive for the
 // (sequence, KV head) merge all splits in split order:  M = max m_j;  l = sum l_j 2^(m_j-M);
-// out = sum o_j 2^(m_j-M) / l;  lse = (M + log2 l) ln 2.  Called by all 128 threads.
+// out = sum o_j 2^(m_j-M) / l;  lse = (M + log2 l) ln 2.  Called by all threads of the block.
 struct SplitSink {
     float* part_o;
     float* part_ml;
@@ -90,6 +90,7 @@ struct SplitSink {
         const size_t pq = (hq0 + u) * kMaxSplits + split;
         part_ml[pq * 2] = M, part_ml[pq * 2 + 1] = lsum;
     }
+    template <int kThreads>
     __device__ __forceinline__ void merge_if_last(int g, int* sh_last) const {
         const int tid = threadIdx.x;
         __threadfence();
@@ -105,7 +106,7 @@ struct SplitSink {
         // all (head, split) statistics in one round trip, then weights, then 16-byte wide sums
         __shared__ float mm[kMaxGroup][kMaxSplits], lw[kMaxGroup][kMaxSplits], w[kMaxGroup][kMaxSplits];
         __shared__ float Lsum[kMaxGroup];
-        for (int i = tid; i < g * nsplit; i += kAttnThreads) {
+        for (int i = tid; i < g * nsplit; i += kThreads) {
             const int u = i / nsplit, j = i % nsplit;
             const size_t pq = (hq0 + u) * kMaxSplits + j;
             mm[u][j] = __ldcg(&part_ml[pq * 2]);
@@ -126,7 +127,7 @@ struct SplitSink {
             if (lse) lse[hq0 + tid] = (M + log2f(lsum)) * kLn2;
         }
         __syncthreads();
-        for (int item = tid; item < g * 32; item += kAttnThreads) {
+        for (int item = tid; item < g * 32; item += kThreads) {
             const int u = item >> 5, c4 = item & 31;
             const float4* src = reinterpret_cast<const float4*>(part_o + (hq0 + u) * kMaxSplits * 128) + c4;
             float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -373,7 +374,7 @@ static inline size_t cluster_merge_bytes(int C) { return (size_t)((8 + C - 1) / 
 // cluster (one block per split): the warps of a block fold their results through shared memory, the blocks exchange
 // channel slices of theirs through distributed shared memory, one cluster barrier, and every block merges
 // and writes the slices it owns -- no partials in global memory, no last-block round trips.  Without it (more splits than a cluster holds) the splits
-// go through the global workspace and the last block to arrive merges them (NW must be 4 then).
+// go through the global workspace and the last block to arrive merges them.
 // kSources: the resident sink / window copies or the Important buffer are bound and a row reference names
 // its source; without them (the usual case) the gather carries no trace of the option.
 // FG: 0 = bf16 storage; else fp32 storage with up to FG query heads per unit.
@@ -816,7 +817,7 @@ __global__ void __launch_bounds__(NW * 32) attn_mma_kernel(Geom gm, UnitTable ut
             else if (C <= 9) owner_merge(std::integral_constant<int, 9>{});
             else owner_merge(std::integral_constant<int, kAttnMaxCluster>{});
         }
-    } else if constexpr (NW == kAttnWarps) {
+    } else {
         // splits through the global workspace, merged by the last block to arrive
         SplitSink sink{part_o, part_ml, counters, a.out, a.lse, hq0, lu, split, a.nsplit};
         for (int slot = tid; slot < 256; slot += NW * 32) {
@@ -832,7 +833,7 @@ __global__ void __launch_bounds__(NW * 32) attn_mma_kernel(Geom gm, UnitTable ut
                 if (mt == 0 && ln < 4) sink.publish_stat(u0 + 1, stat.z, stat.w);
             }
         }
-        sink.merge_if_last(g, &sh_last);
+        sink.merge_if_last<NW * 32>(g, &sh_last);
     }
     attn_stamp(6);
 }
@@ -880,7 +881,7 @@ cudaError_t launch_attention(const tb_ctx* c, const UnitTable& ut, const AttnArg
             prepare(attn_mma_kernel<4, 2, false>, 113, true), prepare(attn_mma_kernel<4, 2, true>, 113, true);
             prepare(attn_mma_kernel<8, 2, false>, 220, true), prepare(attn_mma_kernel<8, 2, true>, 220, true);
             prepare(attn_mma_kernel<8, 3, false>, 220, true), prepare(attn_mma_kernel<8, 3, true>, 220, true);
-            prepare(attn_mma_kernel<12, 2, false>, 224, false), prepare(attn_mma_kernel<12, 2, true>, 224, false);
+            prepare(attn_mma_kernel<12, 2, false>, 220, true), prepare(attn_mma_kernel<12, 2, true>, 220, true);
             auto prepare_f32 = [&](auto group) {
                 constexpr int G = decltype(group)::value;
                 prepare(attn_mma_kernel<4, 2, true, G>, 113, true), prepare(attn_mma_kernel<8, 2, true, G>, 220, true);
@@ -911,34 +912,57 @@ cudaError_t launch_attention(const tb_ctx* c, const UnitTable& ut, const AttnArg
             }
             return max_active[csize];
         };
-        // Few problems (one layer of a small batch): blocks of 8 warps, one per SM, and the largest
-        // cluster (up to 16 blocks, sizes above 8 are non-portable) that the device can keep resident
-        // for every problem at once; the splits merge inside the cluster.  Many problems: 4-warp
-        // blocks, two per SM, clusters of up to 8; splits beyond that go through the global workspace.
+        // Up to a block per SM: C blocks per problem, one cluster, merged inside it.  Measured over 4 to 192 problems of 64
+        // to 20480 rows, 4, 8 and 12 warps, every cluster size and the global merge (figures: bf16, us per launch in a chain
+        // of layers):
+        //  - a launch that takes at most half of the SMs leaves the other half to the next layer's blocks, which fetch their
+        //    lists and first rows meanwhile: small blocks then (8 problems of 640 rows: 3.2 with 4 blocks each; 32 of 320: 3.2
+        //    with 2, 4.0 with 3);
+        //  - what does not fit there takes blocks of two tiles per warp, 384 rows with 12 warps, or more, as far as 128
+        //    blocks go (32 problems of 640 rows: 3.9 with 2 x 12 warps, 5.2 with 4 x 8; 24 of 1280: 5.3 with 4 blocks each, 8.9
+        //    with 6; 96 of 2560: 23.1 with one, 38.8 with 3 x 4 warps and the global merge; 16 of 15000: 23 with 6, 25 with 18
+        //    x 4 warps and the global merge);
+        //  - clusters of 3, 7 and 8 pack badly into the SMs of a GPC (3 is taken where the choice is 2), pairs fit everywhere; 9 fits when it takes half of the chip (non-portable:
+        //    asked for);
+        //  - the global merge is left with what has too few problems for its rows (4 problems of 20480 rows: 12.6 with 32
+        //    blocks of 8 warps each, 15.3 with a cluster of 9), very long rows on a chip that clusters leave a third empty (96
+        //    of 10240: 76.6 with 3 x 4 warps, 82.0 with one block of 12), and more problems than SMs.
+        const int half = c->sm_count / 2, most = c->sm_count - c->sm_count / 8;
+        const int small_block = f32 ? 64 : 256, large_block = f32 ? 192 : 384;
+        auto allowed = [&](int C) { return C <= 2 || (C >= 4 && C <= 6) || (C == 9 && units * 9 <= half && clusters_that_fit(9) >= units); };
+        auto largest = [&](int want, int blocks) {         // the largest size up to `want` that keeps the launch within `blocks`
+            int C = want < 9 ? want : 9;
+            while (C > 1 && (units * C > (C == 2 && blocks == most ? c->sm_count : blocks) || !(allowed(C) || (C == 3 && blocks == most)))) --C;
+            return C;
+        };
         int n = 0;
-        const int by_rows = max_rows / (8 * tok) < 1 ? 1 : max_rows / (8 * tok);
+        if (units <= c->sm_count) {
+            int want = (max_rows + small_block - 1) / small_block, least = (max_rows + large_block - 1) / large_block;
+            if (max_rows > 1536) want = least = 9;
+            else if (want > 6) want = 6;
+            if (want == 3) want = 4;
+            if (least == 3 && 4 * units <= most) least = 4;
+            n = largest(want, half);
+            if (n < want && n < least) n = largest(least, most);
+        }
 #ifdef TB_FORCE_ATTN_CLUSTER
         n = TB_FORCE_ATTN_CLUSTER;
-#else
-        // First choice: a launch that takes at most half of the SMs, so that the next layer's blocks
-        // (programmatic dependent launch) can fetch their lists and first rows on free SMs while this
-        // layer still computes (config 2, 8 problems: clusters of 9 run at 7.36 us per layer, the largest
-        // that fits, 10, at 7.86, 8 at 8.65).  Otherwise the largest cluster that fits once.
-        {
-            const int cand = c->sm_count / (2 * units);
-            if (cand >= 6 && cand <= 16 && cand <= by_rows && clusters_that_fit(cand) >= units) n = cand;
-        }
-        for (int cand = 16; cand >= 1 && !n; cand = cand > 8 ? cand - 2 : cand - 1)
-            if (cand <= by_rows && units * cand <= c->sm_count && (cand <= 8 || clusters_that_fit(cand) >= units)) n = cand;
 #endif
-        if (n && max_rows / n <= 64 * tok) {
-            a.nsplit = n, nw = 8, a.cluster_merge = 1;
-            // more than two tiles per warp would leave the third waiting for a free stage: 12 warps
-            // per block when their rings and the merge area still fit the SM
-            const int rows_per_block = (max_rows + n - 1) / n;
-            if (!f32 && rows_per_block > 8 * 2 * kTileTok && 12 * 2 * kStageBytes + cluster_merge_bytes(n) <= 224 * 1024) nw = 12;
+        const int rows_per_block = n ? (max_rows + n - 1) / n : 0;
+        // fp32 rows keep an SM's warps busier: 4-warp blocks, two per SM, when they fill more of the chip
+        const int n4 = f32 && units <= c->sm_count ? 2 * most / units : 0;
+        if (n && n4 <= 8 && rows_per_block > large_block && 10 * n4 > 23 * n) {
+            a.nsplit = n4, a.cluster_merge = 1;
+        } else if (n && !(units * n < (f32 ? half : 48) && rows_per_block > (f32 ? 700 : 1536)) && !(units * n < most && rows_per_block > 8192)) {
+            a.nsplit = n, a.cluster_merge = 1;
+            nw = rows_per_block <= (f32 ? 64 : 112) ? 4 : rows_per_block <= 256 || f32 ? 8 : 12;
         } else {
             a.nsplit = pick_nsplit(c, units, max_rows);
+            // few problems, one block of 8 warps per SM: as many rows in flight as two of 4, half the partials to merge
+            if (a.nsplit > 16) {
+                nw = 8;
+                if (f32) a.nsplit = c->sm_count / units < kMaxSplits ? c->sm_count / units : kMaxSplits;
+            }
             // clusters only when the whole launch is resident at once: in multi-wave launches the
             // co-scheduling constraint costs more than the global merge (measured on the batch-8 workload)
             if (a.nsplit <= 8 && units * a.nsplit <= 2 * c->sm_count) a.cluster_merge = 1;
