@@ -449,7 +449,8 @@ tb_status tb_select_topk(tb_ctx* c, int32_t lb, int32_t lc, const int32_t* seq_i
                     cand_range(ut.len[i], p->sinks, p->recent, &lo, &hi);
                     if (hi - lo > max_cand) max_cand = hi - lo;
                 }
-                finished = select_small_takes(c, ut, max_cand, p->radius > 0 || idx_out || cnt_out);
+                const bool small = select_small_takes(c, ut, max_cand, p->radius > 0 || idx_out || cnt_out);
+                finished = small;
                 SelectArgs a;
                 a.radius = p->radius, a.nmode = p->nmode;
                 a.idx_copy = idx_out ? idx_out + unit_off * c->geom.idx_cap : nullptr, a.cnt_copy = cnt_out ? cnt_out + unit_off : nullptr;
@@ -460,8 +461,9 @@ tb_status tb_select_topk(tb_ctx* c, int32_t lb, int32_t lc, const int32_t* seq_i
                 } else {
                     a.idx_dst = c->wk.sel_idx, a.cnt_dst = c->wk.sel_cnt, a.dst_is_state = 0, a.idx_stride = c->wk.sel_stride;
                 }
-                cudaError_t e = finished ? launch_select_small(c, ut, a, max_cand, (cudaStream_t)stream, dry)
-                                         : launch_select(c, ut, a, (cudaStream_t)stream, dry);
+                if (small) a.dst_is_state = 1, a.idx_stride = c->geom.idx_cap;
+                cudaError_t e = small ? launch_select_small(c, ut, a, max_cand, (cudaStream_t)stream, dry)
+                                      : launch_select(c, ut, a, (cudaStream_t)stream, dry, &finished);
                 if (e != cudaSuccess) return dry ? TB_ERR_UNSUPPORTED : TB_ERR_CUDA;
                 if (!dry) c->last_list_write = (long long)c->launches, c->launches++;
                 if (p->radius > 0 && !finished) {

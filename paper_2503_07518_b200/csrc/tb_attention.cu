@@ -867,7 +867,6 @@ cudaError_t launch_attention(const tb_ctx* c, const UnitTable& ut, const AttnArg
     a.cluster_merge = 0;
     int nw = kAttnWarps;
     const bool f32 = gm.dtype != TB_BF16;
-    const int tok = f32 ? 8 : kTileTok;               // rows of a stage
     {
         static unsigned char seen[64];
         int* max_active = const_cast<tb_ctx*>(c)->attn_max_active;

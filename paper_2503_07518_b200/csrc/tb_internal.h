@@ -199,9 +199,12 @@ cudaError_t launch_score(const tb_ctx* c, const UnitTable& ut, const float* q_im
                          cudaStream_t s);
 // `dry`: work out the launch configuration and report whether it exists, launch nothing, change nothing
 // (the entry points check every chunk of a call this way before the first real launch)
-cudaError_t launch_select(const tb_ctx* c, const UnitTable& ut, const SelectArgs& a, cudaStream_t s, bool dry = false);
+// *finished: the launch fetches neighbours and fills the caller's copies itself
+cudaError_t launch_select(const tb_ctx* c, const UnitTable& ut, const SelectArgs& a, cudaStream_t s, bool dry, bool* finished);
 // one block per problem; launch_select hands over to it when a launch holds at least two problems per SM
-cudaError_t launch_select_wave(const tb_ctx* c, const UnitTable& ut, const SelectArgs& a, cudaStream_t s, bool dry = false);
+cudaError_t launch_select_wave(const tb_ctx* c, const UnitTable& ut, const SelectArgs& a, cudaStream_t s, bool dry, bool* finished);
+// several lists per key stream (bf16, one list per query head): a cluster per stream
+cudaError_t launch_select_shared(const tb_ctx* c, const UnitTable& ut, const SelectArgs& a, cudaStream_t s, bool dry, bool* finished);
 // small problems: one block each, neighbours and the caller's copy of the list included; whether a launch whose longest
 // problem has max_cand candidates is its kind (more: neighbours or copies are wanted)
 bool select_small_takes(const tb_ctx* c, const UnitTable& ut, int max_cand, bool more);

@@ -703,7 +703,8 @@ static int select_stage_count(int tiles_per_cta, int tile_bytes) {
     return n;
 }
 
-cudaError_t launch_select(const tb_ctx* c, const UnitTable& ut, const SelectArgs& a, cudaStream_t s, bool dry) {
+cudaError_t launch_select(const tb_ctx* c, const UnitTable& ut, const SelectArgs& a, cudaStream_t s, bool dry, bool* finished) {
+    *finished = false;
     const Geom& gm = c->geom;
     const int n_units = ut.layer_count * ut.n_seq * gm.Hl;
     int max_cand = 0;
@@ -716,7 +717,9 @@ cudaError_t launch_select(const tb_ctx* c, const UnitTable& ut, const SelectArgs
     // cluster kernel takes.
     const bool to_wave = 2 * n_units >= 3 * c->sm_count || max_cand > kCwLimit, to_cw = max_cand > kCwFrom && max_cand <= kCwLimit;
     if (c->drop_tile >= 0 && (to_wave || to_cw)) return cudaErrorInvalidConfiguration;   // wait diagnostics: single-block launches of this kernel only
-    if (to_wave) return launch_select_wave(c, ut, a, s, dry);
+    // Lists that share a key stream read it once.
+    if (gm.dtype == TB_BF16 && gm.Hl > gm.Hi && c->drop_tile < 0) return launch_select_shared(c, ut, a, s, dry, finished);
+    if (to_wave) return launch_select_wave(c, ut, a, s, dry, finished);
     // Long problems (beyond ~48K candidates) go to the cluster kernel that parks the keys in memory and
     // keeps 2 bytes per row on chip: two blocks per SM where this one, with 4 bytes per row, has room for
     // one (128K tokens: 70.1 -> 59.1 us per launch; at 32K the two are level, below that this one wins).

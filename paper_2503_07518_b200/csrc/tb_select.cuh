@@ -188,10 +188,8 @@ struct FragScorer {
         }
         __syncthreads();
     }
-    // v[m]: this thread's piece of row 8 m + gid of the 32; returns the score of the row this lane looks after (my_row)
-    __device__ __forceinline__ float score(const Piece (&v)[4], int row0, int& my_row) const {
-        const int lane = threadIdx.x & 31, gid = lane >> 2, tig = lane & 3;
-        float d[2][4];
+    // v[m]: this thread's piece of row 8 m + gid of the 32; d[m][2 i + e]: row 16 m + 8 i + gid, column 2 tig + e
+    __device__ __forceinline__ void columns(const Piece (&v)[4], float (&d)[2][4]) const {
 #pragma unroll
         for (int m = 0; m < 2; ++m) d[m][0] = d[m][1] = d[m][2] = d[m][3] = 0.f;
 #pragma unroll
@@ -205,6 +203,12 @@ struct FragScorer {
                 mma_16816(d[1], v[2].z, v[3].z, v[2].w, v[3].w, b1.x, b1.y);
             }
         }
+    }
+    // returns the score of the row this lane looks after (my_row)
+    __device__ __forceinline__ float score(const Piece (&v)[4], int row0, int& my_row) const {
+        const int lane = threadIdx.x & 31, gid = lane >> 2, tig = lane & 3;
+        float d[2][4];
+        columns(v, d);
         // lane (gid, tig) takes row gid + 8 tig: accumulator 0 / 2 of the first 16 rows, then of the second
         my_row = row0 + gid + 8 * tig;
         float r[4] = {d[0][0], d[0][2], d[1][0], d[1][2]};
@@ -252,15 +256,23 @@ struct RowStream {
     // consume(slot, score) for every row
     template <typename F>
     __device__ __forceinline__ void run(const Scorer& scorer, F&& consume) {
+        run_groups([&](const typename Scorer::Piece (&piece)[4], int row0) {
+            int slot;
+            const float sc = scorer.score(piece, row0, slot);
+            return [=, &consume] { if (slot < n) consume(slot, sc); };
+        });
+    }
+    // f(pieces, first row) for every group of 32; what it returns is called once the group's successor has been requested
+    template <typename F>
+    __device__ __forceinline__ void run_groups(F&& f) {
         for (int g0 = warp; g0 * 32 < n; g0 += kU * n_warps) {
 #pragma unroll
             for (int u = 0; u < kU; ++u) {
                 const int g = g0 + u * n_warps;
                 if (g * 32 >= n) break;                // warp-uniform
-                int slot;
-                const float sc = scorer.score(v[u], g * 32, slot);
+                auto rest = f(v[u], g * 32);
                 load(u, g + kU * n_warps);
-                if (slot < n) consume(slot, sc);
+                rest();
             }
         }
     }
@@ -317,6 +329,36 @@ __device__ __forceinline__ void expand_mask(const uint32_t* mask, uint32_t* out,
     __syncthreads();
 }
 
+// Where a list goes: the context's (or the neighbour kernel's input), and the caller's copy.
+struct ListOut {
+    int32_t* idx;
+    int32_t* cnt;
+    int32_t* idx_copy;
+    int32_t* cnt_copy;
+    int radius, nmode, cap;
+    __device__ __forceinline__ ListOut(const Geom& gm, const SelectArgs& a, size_t state_row, int launch_row, int32_t* state_idx, int32_t* state_cnt) {
+        const size_t row = a.dst_is_state ? state_row : (size_t)launch_row;
+        idx = (a.dst_is_state ? state_idx : a.idx_dst) + row * a.idx_stride;
+        cnt = (a.dst_is_state ? state_cnt : a.cnt_dst) + row;
+        idx_copy = a.idx_copy ? a.idx_copy + (size_t)launch_row * gm.idx_cap : nullptr;
+        cnt_copy = a.cnt_copy ? a.cnt_copy + launch_row : nullptr;
+        radius = a.radius, nmode = a.nmode, cap = a.idx_stride;
+    }
+    __device__ __forceinline__ void count(int n) const {   // one thread
+        *cnt = n;
+        if (cnt_copy) *cnt_copy = n;
+    }
+    // every candidate (neighbours add nothing), or none
+    template <int kThreads>
+    __device__ __forceinline__ void all(int lo, int n) const {
+        for (int i = threadIdx.x; i < n; i += kThreads) {
+            idx[i] = lo + i;
+            if (idx_copy) idx_copy[i] = lo + i;
+        }
+        if (threadIdx.x == 0) count(max(n, 0));
+    }
+};
+
 // Writes the ascending list of a mask: its first `limit` positions, as tokens, to dst and (unless null) to copy.
 // Returns the number of bits.  A thread owns a run of 16-bit half words; `slots` holds kThreads / 32 ints.
 template <int kThreads>
@@ -352,6 +394,17 @@ __device__ __forceinline__ int write_mask_list(const uint32_t* mask, int n_bits,
         }
     }
     return total;
+}
+
+// From the mask to the finished list; `other` = room for a second mask (radius > 0 only).  All threads, mask visible.
+template <int kThreads>
+__device__ __forceinline__ void finish_mask_list(const uint32_t* mask, uint32_t* other, int n_bits, int lo, const ListOut& out, int* slots) {
+    if (out.radius > 0) {
+        expand_mask<kThreads>(mask, other, n_bits, out.radius, out.nmode);
+        mask = other;
+    }
+    const int total = write_mask_list<kThreads>(mask, n_bits, lo, out.cap, out.idx, out.idx_copy, slots);
+    if (threadIdx.x == 0) out.count(total);
 }
 
 }  // namespace tb

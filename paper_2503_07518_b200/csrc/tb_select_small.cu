@@ -100,9 +100,7 @@ __global__ void __launch_bounds__(kThreads, kU == 2 ? 2 : 1) select_small_kernel
     int ll, s, h;
     decode_unit(gm, ut, blockIdx.x, ll, s, h);
     const size_t cu = list_unit(gm, ut, ll, s, h);
-    int32_t* idx_dst = state_idx + cu * gm.idx_cap;
-    int32_t* idx_copy = a.idx_copy ? a.idx_copy + (size_t)blockIdx.x * gm.idx_cap : nullptr;
-    int32_t* cnt_copy = a.cnt_copy ? a.cnt_copy + blockIdx.x : nullptr;
+    const ListOut out(gm, a, cu, blockIdx.x, state_idx, state_cnt);
     pdl_wait();
     pdl_launch_dependents();                           // (waits for this grid's completion before it reads a list)
 
@@ -111,14 +109,7 @@ __global__ void __launch_bounds__(kThreads, kU == 2 ? 2 : 1) select_small_kernel
     const int k = min(a.budget, ncand);
     check_candidates_projected(gm, ut, ll, s, hi, status);
     if (k <= 0 || k == ncand) {                        // nothing to rank: none, or all (neighbours add nothing then)
-        for (int i = tid; i < k; i += kThreads) {
-            idx_dst[i] = lo + i;
-            if (idx_copy) idx_copy[i] = lo + i;
-        }
-        if (tid == 0) {
-            state_cnt[cu] = max(k, 0);
-            if (cnt_copy) *cnt_copy = max(k, 0);
-        }
+        out.all<kThreads>(lo, k);
         return;
     }
     const int n_tiles = (ncand + kHalf - 1) / kHalf;   // <= max_tiles
@@ -276,16 +267,7 @@ __global__ void __launch_bounds__(kThreads, kU == 2 ? 2 : 1) select_small_kernel
     }
 
     // ---- neighbours and list -----------------------------------------------------------------------------
-    const uint32_t* mask = sm->mask;
-    if (a.radius > 0) {
-        expand_mask<kThreads>(sm->mask, sm->mask_out, ncand, a.radius, a.nmode);
-        mask = sm->mask_out;
-    }
-    const int total = write_mask_list<kThreads>(mask, ncand, lo, gm.idx_cap, idx_dst, idx_copy, sm->slots);
-    if (tid == 0) {
-        state_cnt[cu] = total;
-        if (cnt_copy) *cnt_copy = total;
-    }
+    finish_mask_list<kThreads>(sm->mask, sm->mask_out, ncand, lo, out, sm->slots);
 }
 
 size_t small_smem(int n_stages, int n_tiles, int tile_bytes) {

@@ -169,8 +169,7 @@ __device__ __forceinline__ void wave_find_digit(const int* hist, int k, WaveSmem
 // written nothing, when they do not fit (a crowded threshold bin): the caller then takes the general
 // path.  All threads call it and all get the same answer.
 __device__ __forceinline__ bool wave_finish_mask(int* hist, WaveSmem* sm, const Digit dg, const uint32_t* __restrict__ keys,
-                                                 unsigned char* scratch, int scratch_bytes, int ncand, int k, int lo,
-                                                 int32_t* __restrict__ idx_dst, int32_t* __restrict__ cnt_dst) {
+                                                 unsigned char* scratch, int scratch_bytes, int ncand, int k, int lo, const ListOut& out) {
     const int tid = threadIdx.x, lane = tid & 31;
 #ifdef TB_PHASE_TIMING
     unsigned long long tf0 = wave_now();
@@ -311,23 +310,8 @@ __device__ __forceinline__ bool wave_finish_mask(int* hist, WaveSmem* sm, const 
     }
 
     FIN_MARK(2);
-    // ascending list from the mask: each thread owns a run of words
-    const int per = (n_words + kThreads - 1) / kThreads;
-    const int w0 = min(n_words, tid * per), w1 = min(n_words, w0 + per);
-    int cnt = 0;
-    for (int w = w0; w < w1; ++w) cnt += __popc(mask[w]);
-    int total;
-    int o = wave_excl_scan(cnt, sm->warp_a, total);
-    for (int w = w0; w < w1; ++w) {
-        uint32_t bits = mask[w];
-        while (bits) {
-            const int b = __ffs(bits) - 1;
-            bits &= bits - 1;
-            if (o < k) idx_dst[o] = lo + w * 32 + b;
-            ++o;
-        }
-    }
-    if (tid == 0) *cnt_dst = k;
+    // (the list of the bin's keys is done with: neighbours are fetched into its place; the launcher has made room)
+    finish_mask_list<kThreads>(mask, reinterpret_cast<uint32_t*>(scratch + mask_bytes), ncand, lo, out, sm->warp_a);
     FIN_MARK(3);
     return true;
 }
@@ -458,6 +442,30 @@ __device__ __forceinline__ void wave_general(int* hist, WaveSmem* sm, const uint
 
 }
 
+// The general path, then what is left to do with the list it wrote: neighbours (on a bitmask in `scratch`) and the copy.
+__device__ __forceinline__ void wave_general_finish(int* hist, WaveSmem* sm, const uint32_t* __restrict__ keys_unit, unsigned char* scratch,
+                                                    int scratch_bytes, int ncand, int k, int lo, const ListOut& out) {
+    wave_general(hist, sm, keys_unit, reinterpret_cast<uint4*>(scratch), scratch_bytes / 16, ncand, k, lo, out.idx, out.cnt);
+    if (out.radius == 0 && !out.idx_copy && !out.cnt_copy) return;
+    __syncthreads();                                   // the block sees its own list
+    if (out.radius > 0) {
+        const int n_words = (ncand + 31) / 32;
+        uint32_t* mask = reinterpret_cast<uint32_t*>(scratch);
+        for (int i = threadIdx.x; i < n_words; i += kThreads) mask[i] = 0u;
+        __syncthreads();
+        for (int i = threadIdx.x; i < k; i += kThreads) {
+            const int p = out.idx[i] - lo;
+            atomicOr(&mask[p >> 5], 1u << (p & 31));
+        }
+        __syncthreads();
+        finish_mask_list<kThreads>(mask, mask + ((n_words + 3) & ~3), ncand, lo, out, sm->warp_a);
+        return;
+    }
+    for (int i = threadIdx.x; i < k; i += kThreads)
+        if (out.idx_copy) out.idx_copy[i] = out.idx[i];
+    if (threadIdx.x == 0) out.count(k);
+}
+
 template <typename T, int DP, int RED>
 __global__ void __launch_bounds__(kThreads, 4)
     select_wave_kernel(const __grid_constant__ CUtensorMap tmap, const unsigned char* __restrict__ kimp, Geom gm, UnitTable ut,
@@ -473,11 +481,7 @@ __global__ void __launch_bounds__(kThreads, 4)
     unsigned char* stage_base = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
     int* hist = reinterpret_cast<int*>(stage_base + n_stages * kTileBytes);       // one digit at a time
     WaveSmem* sm = reinterpret_cast<WaveSmem*>(hist + kDigitBins);
-    // The ring is idle once the rows are streamed; it then caches the problem's keys (as many as fit).
-    uint4* key_cache = reinterpret_cast<uint4*>(stage_base);
-    const int cache_vecs = n_stages * (int)kTileBytes / 16;                      // 16-byte vectors of 4 keys
-
-    const int tid = threadIdx.x, lane = tid & 31;
+    const int tid = threadIdx.x;
     const int pair = order.pair[blockIdx.x / gm.Hl], h = blockIdx.x % gm.Hl;
     const int ll = pair / ut.n_seq, s = pair % ut.n_seq;
     const int L = unit_len(gm, ut, ll, s);
@@ -487,17 +491,9 @@ __global__ void __launch_bounds__(kThreads, 4)
     const int k = min(a.budget, ncand);
     check_candidates_projected(gm, ut, ll, s, hi, status);
     const size_t cu = list_unit(gm, ut, ll, s, h);
-    const size_t dst_row = a.dst_is_state ? cu : (size_t)pair * gm.Hl + h;
-    int32_t* idx_dst = (a.dst_is_state ? state_idx : a.idx_dst) + dst_row * a.idx_stride;
-    int32_t* cnt_dst = (a.dst_is_state ? state_cnt : a.cnt_dst) + dst_row;
-
-    if (k <= 0) {
-        if (tid == 0) *cnt_dst = 0;
-        return;
-    }
-    if (k == ncand) {                                  // budget covers every candidate: no ranking needed
-        for (int i = tid; i < ncand; i += kThreads) idx_dst[i] = lo + i;
-        if (tid == 0) *cnt_dst = k;
+    const ListOut out(gm, a, cu, pair * gm.Hl + h, state_idx, state_cnt);
+    if (k <= 0 || k == ncand) {                        // nothing, or everything: no ranking needed
+        out.all<kThreads>(lo, k);
         return;
     }
 
@@ -618,11 +614,8 @@ __global__ void __launch_bounds__(kThreads, 4)
     wave_stamp(2);
 
     // ---- finish -----------------------------------------------------------------------------------
-    if (wave_finish_mask(hist, sm, dg, keys_unit, stage_base, n_stages * (int)kTileBytes, ncand, k, lo, idx_dst, cnt_dst)) {
-        wave_stamp(3);
-        return;
-    }
-    wave_general(hist, sm, keys_unit, key_cache, cache_vecs, ncand, k, lo, idx_dst, cnt_dst);
+    if (!wave_finish_mask(hist, sm, dg, keys_unit, stage_base, n_stages * (int)kTileBytes, ncand, k, lo, out))
+        wave_general_finish(hist, sm, keys_unit, stage_base, n_stages * (int)kTileBytes, ncand, k, lo, out);
     wave_stamp(3);
 }
 
@@ -634,16 +627,230 @@ extern "C" int tb_debug_fin_blk(unsigned long long* out) { return (int)cudaMemcp
 extern "C" int tb_debug_wave_ns(unsigned long long* out) { return (int)cudaMemcpyFromSymbol(out, g_wave_ns, sizeof(g_wave_ns)); }
 #endif
 
-cudaError_t launch_select_wave(const tb_ctx* c, const UnitTable& ut, const SelectArgs& a, cudaStream_t s, bool dry) {
-    const Geom& gm = c->geom;
-    const int n_pairs = ut.layer_count * ut.n_seq, n_units = n_pairs * gm.Hl;
-    WaveOrder order;
-    int cand[kMaxLaunchUnits];
+// ===================================================================================================
+// Lists that share a key stream (one list per query head: the g heads of a group rank the same projected keys by g
+// queries; bf16).  A cluster of g blocks per stream: block r streams an g-th of the rows once and scores them for all g
+// lists -- the tensor-core columns are the heads (see FragScorer) --, parks g keys per row and counts g histograms; behind
+// one cluster barrier it sums the blocks' histograms of list r and finishes that list like the kernel above.
+constexpr int kSharedU = 4;         // groups of 32 rows in flight per warp
+
+struct __align__(16) SharedSmem {
+    WaveSmem w;                     // (its queries are unused)
+    float qs[kMaxGroup * 32];
+    uint2 frags[kQueryFrags];
+    uint32_t sample[kMaxGroup][kSampleRows];
+    uint32_t s_lo[kMaxGroup], s_hi[kMaxGroup];
+    Digit digit[kMaxGroup];
+    alignas(16) unsigned char rows[kSampleRows * 64];
+};
+
+template <int DP>
+__global__ void __launch_bounds__(kThreads, 2)
+    select_shared_kernel(const unsigned char* __restrict__ kimp, Geom gm, UnitTable ut, WaveOrder order, SelectArgs a, int scratch_bytes, int keep_in_l2,
+                         int32_t* __restrict__ state_idx, int32_t* __restrict__ state_cnt, int32_t* __restrict__ status, uint32_t* __restrict__ keys_g) {
+    typedef RowStream<DP, TB_GROUP_MAX, kSharedU> Stream;
+    constexpr int RB = DP * 2;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    int* hist = reinterpret_cast<int*>(smem_raw);                                 // [g][kDigitBins]
+    const int g = gm.Hl / gm.Hi;                       // lists per stream = blocks per cluster
+    SharedSmem* sm = reinterpret_cast<SharedSmem*>(hist + g * kDigitBins);
+    unsigned char* scratch = reinterpret_cast<unsigned char*>(sm + 1);
+    const int tid = threadIdx.x, lane = tid & 31, gid = lane >> 2, tig = lane & 3;
+    const int pair = order.pair[blockIdx.x / gm.Hl], h = blockIdx.x % gm.Hl, rank = h % g;
+    const int ll = pair / ut.n_seq, s = pair % ut.n_seq;
+    const int L = unit_len(gm, ut, ll, s), lo = min(a.sinks, L), hi = max(lo, L - a.recent), ncand = hi - lo, k = min(a.budget, ncand);
+    check_candidates_projected(gm, ut, ll, s, hi, status);
+    const size_t cu = list_unit(gm, ut, ll, s, h);
+    const ListOut out(gm, a, cu, pair * gm.Hl + h, state_idx, state_cnt);
+    if (k <= 0 || k == ncand) {                        // uniform over the cluster
+        out.all<kThreads>(lo, k);
+        return;
+    }
+    const unsigned char* stream = kimp + ((size_t)key_unit(gm, ut, ll, s, h) * gm.max_seq_len + lo) * RB;
+    const int span = ((ncand + g * 32 - 1) / (g * 32)) * 32, slot0 = min(ncand, rank * span), n_local = min(span, ncand - slot0);
+    const size_t key_pitch = (gm.max_seq_len + 255) & ~255;
+    uint32_t* keys0 = keys_g + (cu - rank) * key_pitch;                           // the group's rows of parked keys
+    const uint64_t keep_policy = keep_in_l2 ? l2_policy_evict_last() : l2_policy_evict_first();
+
+    const bool sampled = ncand >= kMinSampled;
+    {
+        const float* q = a.q_imp + query_row(gm, ut, ll, s, h - rank) * DP;       // one query per list, consecutive
+        if (tid < g * DP) sm->qs[tid] = __ldg(q + tid);
+        if (sampled)
+            for (int c = tid; c < kSampleRows * RB / 16; c += kThreads) {
+                const int row = (int)((long long)(c / (RB / 16)) * ncand / kSampleRows);
+                reinterpret_cast<uint4*>(sm->rows)[c] = __ldg(reinterpret_cast<const uint4*>(stream + (size_t)row * RB) + c % (RB / 16));
+            }
+    }
+    Stream rs;
+    rs.start(stream + (size_t)slot0 * RB, n_local);
+    for (int i = tid; i < g * kDigitBins; i += kThreads) hist[i] = 0;
+    __syncthreads();
+    typename Stream::Scorer scorer;
+    scorer.load_staged(sm->qs, g, sm->frags);
+
+    // ---- every list's first digit, from the same 64 rows in every block (see the kernel above) ---------------
+    if (sampled) {
+        for (int i = tid; i < g * kSampleRows; i += kThreads) {
+            const int u = i / kSampleRows, r = i % kSampleRows;
+            float acc = 0.f;
+#pragma unroll 4
+            for (int c = 0; c < DP; c += 2) {
+                const uint32_t w = *reinterpret_cast<const uint32_t*>(sm->rows + r * RB + c * 2);
+                acc = fmaf(sm->qs[u * DP + c], bf16_lo(w), acc), acc = fmaf(sm->qs[u * DP + c + 1], bf16_hi(w), acc);
+            }
+            sm->sample[u][r] = order_key(acc);
+        }
+        __syncthreads();
+        for (int i = tid; i < g * kSampleRows; i += kThreads) {
+            const int u = i / kSampleRows, me = i % kSampleRows;
+            const uint32_t mine = sm->sample[u][me];
+            int r = 0;
+#pragma unroll 8
+            for (int j = 0; j < kSampleRows; ++j) {
+                const uint32_t x = sm->sample[u][j];
+                r += (x > mine) | ((x == mine) & (j < me));
+            }
+            const float p = (float)k / (float)ncand, mean = p * kSampleRows, sd = sqrtf(mean * (1.f - p));
+            if (r == max(0, (int)floorf(mean - 6.f * sd) - 3)) sm->s_hi[u] = mine;
+            if (r == min(kSampleRows - 1, (int)ceilf(mean + 6.f * sd) + 3)) sm->s_lo[u] = mine;
+        }
+        __syncthreads();
+    }
+    if (tid < g) {
+        Digit dg = {0u, 21};
+        if (sampled) {
+            const uint32_t s_lo = sm->s_lo[tid], width = sm->s_hi[tid] - s_lo;
+            uint32_t range = width + (width >> 1);     // room above the highest bracketing sample
+            if (range < width) range = 0xffffffffu;
+            dg.base = s_lo, dg.shift = 0;
+            while ((range >> dg.shift) >= 2046u) ++dg.shift;
+        }
+        sm->digit[tid] = dg;
+    }
+    __syncthreads();
+
+    // ---- stream: this lane looks after lists 2 tig and 2 tig + 1 -----------------------------------------------
+    {
+        Digit dg[2];
+        uint32_t* keys[2];
+        int* bins[2];
+#pragma unroll
+        for (int e = 0; e < 2; ++e) {
+            const int u = min(2 * tig + e, g - 1);
+            dg[e] = sm->digit[u], keys[e] = keys0 + u * key_pitch + slot0, bins[e] = hist + u * kDigitBins;
+        }
+        rs.run_groups([&](const typename Stream::Scorer::Piece (&v)[4], int row0) {
+            struct { float d[2][4]; } x;
+            scorer.columns(v, x.d);
+            return [&, x, row0] {
+#pragma unroll
+                for (int m = 0; m < 2; ++m)
+#pragma unroll
+                    for (int i = 0; i < 2; ++i) {
+                        const int slot = row0 + 16 * m + 8 * i + gid;
+#pragma unroll
+                        for (int e = 0; e < 2; ++e)
+                            if (2 * tig + e < g && slot < n_local) {
+                                const uint32_t key = order_key(x.d[m][2 * i + e]);
+                                st_global_hint(keys[e] + slot, key, keep_policy);
+                                hist_add(&bins[e][dg[e].bin(key)]);
+                            }
+                    }
+            };
+        });
+    }
+    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+
+    // ---- list `rank`: its histogram from the cluster, then the usual finish ---------------------------------------
+    int* mine = hist + rank * kDigitBins;              // (read by this block only)
+    {
+        int4 sum[2] = {make_int4(0, 0, 0, 0), make_int4(0, 0, 0, 0)};
+        for (int r = 0; r < g; ++r) {
+            uint64_t peer;
+            asm volatile("mapa.u64 %0, %1, %2;" : "=l"(peer) : "l"(reinterpret_cast<uint64_t>(mine + tid * 8)), "r"((rank + r) % g));
+#pragma unroll
+            for (int j = 0; j < 2; ++j) {
+                const int4 x = reinterpret_cast<const int4*>(peer)[j];
+                sum[j].x += x.x, sum[j].y += x.y, sum[j].z += x.z, sum[j].w += x.w;
+            }
+        }
+        reinterpret_cast<int4*>(mine)[tid * 2] = sum[0], reinterpret_cast<int4*>(mine)[tid * 2 + 1] = sum[1];
+    }
+    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");          // the peers' histograms have been read
+    __syncthreads();
+    const uint32_t* keys_unit = keys0 + rank * key_pitch;
+    const Digit dg = sm->digit[rank];
+    if (!wave_finish_mask(mine, &sm->w, dg, keys_unit, scratch, scratch_bytes, ncand, k, lo, out))
+        wave_general_finish(mine, &sm->w, keys_unit, scratch, scratch_bytes, ncand, k, lo, out);
+    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");            // this block's histograms stay until they have been read
+}
+
+namespace {
+
+// The pairs of a launch, longest first, and their candidates; returns the most.
+int longest_first(const UnitTable& ut, const SelectArgs& a, WaveOrder& order, int (&cand)[kMaxLaunchUnits]) {
+    const int n_pairs = ut.layer_count * ut.n_seq;
     for (int i = 0; i < n_pairs; ++i) {
         const int L = ut.len[i], lo = a.sinks < L ? a.sinks : L, hi = L - a.recent > lo ? L - a.recent : lo;
         cand[i] = hi - lo, order.pair[i] = (uint16_t)i;
     }
     std::stable_sort(order.pair, order.pair + n_pairs, [&](uint16_t x, uint16_t y) { return cand[x] > cand[y]; });
+    return cand[order.pair[0]];
+}
+
+// The arguments of a launch that can fetch neighbours (`room` bytes on chip for two bitmasks) and copy the lists itself, or
+// that leaves both to the kernels after it.
+SelectArgs finishing_args(const tb_ctx* c, const SelectArgs& a_in, int max_cand, size_t room, bool* finished) {
+    SelectArgs a = a_in;
+    *finished = a.radius == 0 || (size_t)(max_cand + 255) / 256 * 64 <= room;
+    if (*finished) a.dst_is_state = 1, a.idx_dst = a.cnt_dst = nullptr, a.idx_stride = c->geom.idx_cap;
+    else a.radius = 0, a.idx_copy = a.cnt_copy = nullptr;
+    return a;
+}
+
+}  // namespace
+
+cudaError_t launch_select_shared(const tb_ctx* c, const UnitTable& ut, const SelectArgs& a_in, cudaStream_t s, bool dry, bool* finished) {
+    const Geom& gm = c->geom;
+    const int n_pairs = ut.layer_count * ut.n_seq, n_units = n_pairs * gm.Hl, g = gm.Hl / gm.Hi;
+    WaveOrder order;
+    int cand[kMaxLaunchUnits];
+    const int max_cand = longest_first(ut, a_in, order, cand);
+    // scratch: two bitmasks or one and the keys set aside, within half an SM where that is enough
+    const size_t fixed = (size_t)g * kDigitBins * sizeof(int) + sizeof(SharedSmem);
+    size_t scratch = (size_t)(max_cand + 255) / 256 * 64 + 8192;
+    if (scratch < 24 * 1024) scratch = 24 * 1024;
+    if (fixed + scratch > 220 * 1024) scratch = 220 * 1024 - fixed;
+    const SelectArgs a = finishing_args(c, a_in, max_cand, scratch, finished);
+    double parked = 0;
+    for (int i = 0; i < n_pairs; ++i) parked += 4.0 * cand[i] * gm.Hl;
+    const int keep_in_l2 = parked <= 96e6;
+    if (dry) return cudaSuccess;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(n_units, 1, 1), cfg.blockDim = dim3(kThreads, 1, 1), cfg.dynamicSmemBytes = fixed + scratch, cfg.stream = s;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = g, attr[0].val.clusterDim.y = 1, attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr, cfg.numAttrs = 1;
+    auto launch = [&](auto kernel, unsigned char (&seen)[64]) {
+        if (first_use_on_this_device(seen)) {
+            cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 224 * 1024);
+            if (e != cudaSuccess) return e;
+        }
+        return cudaLaunchKernelEx(&cfg, kernel, (const unsigned char*)c->kimp, gm, ut, order, a, (int)scratch, keep_in_l2, c->st.idx, c->st.cnt, c->st.status,
+                                  c->wk.sel_keys);
+    };
+    static unsigned char seen32[64], seen16[64];
+    return gm.dp == 32 ? launch(select_shared_kernel<32>, seen32) : launch(select_shared_kernel<16>, seen16);
+}
+
+cudaError_t launch_select_wave(const tb_ctx* c, const UnitTable& ut, const SelectArgs& a_in, cudaStream_t s, bool dry, bool* finished) {
+    const Geom& gm = c->geom;
+    const int n_pairs = ut.layer_count * ut.n_seq, n_units = n_pairs * gm.Hl;
+    WaveOrder order;
+    int cand[kMaxLaunchUnits];
+    const int max_cand = longest_first(ut, a_in, order, cand);
     const int tile_bytes = kRows * gm.dp * (gm.dtype == TB_BF16 ? 2 : 4);
     // Ring depth: the SM's shared memory split among the blocks it will hold (four when the launch has
     // that many per SM: 32 KB rings, 128 KB in flight; fewer blocks get deeper rings).
@@ -654,6 +861,7 @@ cudaError_t launch_select_wave(const tb_ctx* c, const UnitTable& ut, const Selec
     if (n_stages > kStagesMax) n_stages = kStagesMax;
     if (n_stages < 2) n_stages = 2;
     const size_t smem = fixed + (size_t)n_stages * tile_bytes;
+    const SelectArgs a = finishing_args(c, a_in, max_cand, (size_t)n_stages * tile_bytes, finished);
     // 4 bytes of key per candidate: ask L2 to keep them only while a launch's worth fits comfortably
     double parked = 0;
     for (int i = 0; i < n_pairs; ++i) parked += 4.0 * cand[i] * gm.Hl;

@@ -100,3 +100,28 @@ def test_scope_argument_checks(H):
     kvh, qh, lay = sizes_of(0), sizes_of(1), sizes_of(2)
     assert kvh[0] == qh[0] == lay[0] and kvh[1] == qh[1] == 8 * lay[1]
     assert qh[2] > kvh[2] > lay[2]
+
+
+@pytest.mark.parametrize("q_heads,kv_heads,dp", [(4, 2, 32), (8, 2, 16), (7, 1, 32), (8, 1, 32), (3, 1, 16)])
+def test_lists_that_share_a_key_stream(H, q_heads, kv_heads, dp):
+    """Per-query-head lists beyond the one-block kernel: shares of the stream that end off a 32-row group, a sequence short
+    enough to be unsampled beside a long one, both neighbour rules, and thresholds in crowded bins (massive ties)."""
+    for lengths, budget, sinks, recent, radius, nmode in (([9001, 700], 300, 2, 5, 0, 0), ([12345, 8300], 1000, 0, 0, 1, 1), ([40007], 5, 0, 16, 2, 0)):
+        w = wl.workload(2, n_layers=1, n_q_heads=q_heads, n_kv_heads=kv_heads, imp_dim=dp, batch=len(lengths), lengths=lengths, budget=budget,
+                        sinks=sinks, recent=recent, radius=radius, nmode=nmode)
+        case = H.Case(w, list_scope=tb().TB_SCOPE_Q_HEAD)
+        p = tb().select_params(budget, sinks, recent, radius, nmode)
+        full_pipeline_check(H, case, p)
+        _, qi = H.queries(w)
+        for ties in (np.zeros_like(qi), np.where(np.arange(dp) == 0, np.float32(1), np.float32(0)) * np.ones_like(qi)):
+            if ties.any():                             # few distinct scores: the first channel of every key is 0, 1 or 2
+                for b, L in enumerate(lengths):
+                    v = (np.arange(L) * 7919 % 3).astype(np.float32)
+                    case.Kimp[0][b][:, :L, 0] = wl.to_storage(v, w.dtype)
+                    case.ctx.kimp[0, b, :, :L] = H.to_dev(case.Kimp[0][b][:, :L], w.dtype)
+            lists = H.gpu_select(case, ties, p)
+            assert case.ctx.get_status() == 0
+            for b in range(w.batch):
+                for h in range(q_heads):
+                    _, full, _ = case.oracle_select(0, b, h, ties[0, b], p)
+                    assert np.array_equal(lists[0][b][h], full)
