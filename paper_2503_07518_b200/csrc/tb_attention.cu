@@ -817,7 +817,7 @@ __global__ void __launch_bounds__(NW * 32) attn_mma_kernel(Geom gm, UnitTable ut
             else if (C <= 9) owner_merge(std::integral_constant<int, 9>{});
             else owner_merge(std::integral_constant<int, kAttnMaxCluster>{});
         }
-    } else {
+    } else if constexpr (NW != 12) {                     // (12-warp blocks always merge in their cluster: its code alone costs them 0.9%)
         // splits through the global workspace, merged by the last block to arrive
         SplitSink sink{part_o, part_ml, counters, a.out, a.lse, hq0, lu, split, a.nsplit};
         for (int slot = tid; slot < 256; slot += NW * 32) {

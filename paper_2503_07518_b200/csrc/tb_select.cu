@@ -308,6 +308,7 @@ __global__ void __launch_bounds__(kSelThreads) select_kernel(const __grid_consta
     // depends on the sample, never the result.  Called by all threads, once, when the sample rows have
     // had time to arrive: the keys scored before that are counted then (`done_tiles` of them per thread).
     SampledDigit dg = {0u, 22};
+    DigitCounter counter;
     auto place_digit = [&](int done_tiles) {
         asm volatile("cp.async.wait_group 0;" ::: "memory");
         __syncthreads();
@@ -346,7 +347,7 @@ __global__ void __launch_bounds__(kSelThreads) select_kernel(const __grid_consta
         while ((range >> dg.shift) >= (uint32_t)(kFastBins - 2)) ++dg.shift;
         for (int i = 0; i < done_tiles; ++i) {
             const int slot = i * kTileRows + tid;
-            if (slot < n_local) smem_add(&hist[dg.bin(keys[slot])], 1);   // this thread's own earlier keys
+            if (slot < n_local) counter.add(hist, dg.bin(keys[slot]));   // this thread's own earlier keys
         }
     };
     // the tile before which the digit is placed: late enough for the sample to have landed without a wait
@@ -375,7 +376,7 @@ __global__ void __launch_bounds__(kSelThreads) select_kernel(const __grid_consta
             }
             keys[slot] = key;
             if (!sampled) smem_add(&hist[key >> 21], 1);
-            else if (i >= place_at) smem_add(&hist[dg.bin(key)], 1);
+            else if (i >= place_at) counter.add(hist, dg.bin(key));
         }
         if (__syncthreads_or(!ok)) dead = true;        // all reads of this stage are done; uniform verdict on the wait
         if (!dead && i + n_stages < my_tiles) {
@@ -391,10 +392,9 @@ __global__ void __launch_bounds__(kSelThreads) select_kernel(const __grid_consta
         if (++st == n_stages) st = 0, phase ^= 1u;
     }
     if (dead && tid == 0) atomicExch(status, kStatusTimeout);
-    if (place_at == my_tiles) {                        // a short share: the digit is placed after its last tile
-        place_digit(my_tiles);
-        __syncthreads();                               // the histogram is read next
-    }
+    if (place_at == my_tiles) place_digit(my_tiles);   // a short share: the digit is placed after its last tile
+    counter.flush(hist);
+    __syncthreads();                                   // the histogram is read next
     phase_stamp(2);
 
     uint32_t prefix = 0;          // general path: digits fixed so far (value of key >> low_bits)
@@ -713,16 +713,21 @@ cudaError_t launch_select(const tb_ctx* c, const UnitTable& ut, const SelectArgs
         if (hi - lo > max_cand) max_cand = hi - lo;
     }
     // Many problems (one and a half per SM or more; measured crossover between 32 and 256 on 148 SMs)
-    // fill the GPU by themselves: one block each, no clusters.  So do problems beyond what the parked-key
-    // cluster kernel takes.
-    const bool to_wave = 2 * n_units >= 3 * c->sm_count || max_cand > kCwLimit, to_cw = max_cand > kCwFrom && max_cand <= kCwLimit;
+    // fill the GPU by themselves: one block each, no clusters.  So do more problems than SMs as long as they are short (160
+    // of 9500 candidates: 34.3 us against 36.7 in clusters, 192 of 16000: 47.6 / 54.5), and problems beyond what the
+    // parked-key cluster kernel takes.
+    // Long problems go to the cluster kernel that parks the keys in memory and keeps 2 bytes per row on chip: two blocks per
+    // SM where this one, with 4 bytes per row, has room for one.  Where the line lies depends on the blocks per problem that
+    // leaves it: eight to four (128K tokens: 70.1 -> 59.1 us per launch; at 32K the two are level), two (128 problems of
+    // 32000: 49.3 against 56.7; of 16000 32.4 / 30.3); three and one place badly (96 of 64000: 106 / 89, 160: 154 / 141).
+    const int cw_blocks = 2 * c->sm_count / n_units;
+    const int cw_from = cw_blocks >= 4 ? kCwFrom : cw_blocks == 2 ? 20 * 1024 : 2 * kCwFrom;
+    const bool to_wave = 2 * n_units >= 3 * c->sm_count || (n_units > c->sm_count && max_cand <= 20 * 1024) || max_cand > kCwLimit;
+    const bool to_cw = max_cand > cw_from && max_cand <= kCwLimit;
     if (c->drop_tile >= 0 && (to_wave || to_cw)) return cudaErrorInvalidConfiguration;   // wait diagnostics: single-block launches of this kernel only
     // Lists that share a key stream read it once.
     if (gm.dtype == TB_BF16 && gm.Hl > gm.Hi && c->drop_tile < 0) return launch_select_shared(c, ut, a, s, dry, finished);
     if (to_wave) return launch_select_wave(c, ut, a, s, dry, finished);
-    // Long problems (beyond ~48K candidates) go to the cluster kernel that parks the keys in memory and
-    // keeps 2 bytes per row on chip: two blocks per SM where this one, with 4 bytes per row, has room for
-    // one (128K tokens: 70.1 -> 59.1 us per launch; at 32K the two are level, below that this one wins).
     if (to_cw) return launch_select_cw(c, ut, a, s, dry);
     const int n_tiles = (max_cand + kTileRows - 1) / kTileRows;
     // Cluster size: enough blocks to cover the GPU about twice, at least 4 tiles per block, and a

@@ -278,6 +278,22 @@ struct RowStream {
     }
 };
 
+// Counts digits in a shared-memory histogram.  Nine keys in ten lie below a sampled bracket, in bin 0: added one by one to
+// the same address they would cost a pass of the shared-memory pipe each (measured: 11 per instruction of 16 keys, half of
+// a kernel's time), so that bin is counted in a register and added once, by flush().
+struct DigitCounter {
+    int below = 0;
+    __device__ __forceinline__ void add(int* hist, int bin) {
+        if (bin == 0) ++below;
+        else asm volatile("red.shared.add.s32 [%0], 1;" ::"r"(smem_u32(hist + bin)) : "memory");
+    }
+    __device__ __forceinline__ void flush(int* hist) {   // whole warps; followed by a barrier
+        below = warp_sum_int(below);
+        if ((threadIdx.x & 31) == 0 && below) atomicAdd(hist, below);
+        below = 0;
+    }
+};
+
 // ---- from a bitmask of the candidates to the list -------------------------------------------------------
 // Bit i of `mask` = candidate i (token lo + i) is selected; n_bits candidates, bits past them zero.
 

@@ -575,6 +575,7 @@ __global__ void __launch_bounds__(kThreads, 4)
     // further tile, still waits -- bounded -- for those in flight, gives the rows it never received the
     // lowest key and finishes normally; the status word tells the caller that this call's lists are void.
     bool dead = false;
+    DigitCounter counter;
     int issued = min(n_stages, n_tiles);               // tiles whose copy has been requested
     int st = 0;
     uint32_t phase = 0;
@@ -595,7 +596,7 @@ __global__ void __launch_bounds__(kThreads, 4)
                 key = order_key(sc);
             }
             st_global_hint(keys_unit + slot, key, keep_policy);
-            hist_add(&hist[dg.bin(key)]);
+            counter.add(hist, dg.bin(key));
         }
         if (__syncthreads_or(!ok)) dead = true;        // all reads of this stage are done; uniform verdict on the wait
         if (!dead && i + n_stages < n_tiles) {
@@ -610,6 +611,7 @@ __global__ void __launch_bounds__(kThreads, 4)
         if (++st == n_stages) st = 0, phase ^= 1u;
     }
     if (dead && tid == 0) atomicExch(status, kStatusTimeout);
+    counter.flush(hist);
     __syncthreads();                                   // histogram complete, own keys visible to the block
     wave_stamp(2);
 
@@ -730,35 +732,49 @@ __global__ void __launch_bounds__(kThreads, 2)
     }
     __syncthreads();
 
-    // ---- stream: this lane looks after lists 2 tig and 2 tig + 1 -----------------------------------------------
+    // ---- stream: a lane's accumulators are lists 2 tig and 2 tig + 1.  With up to four lists the lanes tig >= 2 have none of
+    // their own and take half of the rows of the lanes tig - 2 (the second 16 of a group).
     {
+        const bool halves = g <= 4;
+        const int u0 = 2 * (halves ? tig & 1 : tig);
         Digit dg[2];
         uint32_t* keys[2];
         int* bins[2];
+        DigitCounter counter[2];
 #pragma unroll
         for (int e = 0; e < 2; ++e) {
-            const int u = min(2 * tig + e, g - 1);
+            const int u = min(u0 + e, g - 1);
             dg[e] = sm->digit[u], keys[e] = keys0 + u * key_pitch + slot0, bins[e] = hist + u * kDigitBins;
         }
+        auto take = [&](int slot, int e, float score) {
+            if (u0 + e < g && slot < n_local) {
+                const uint32_t key = order_key(score);
+                st_global_hint(keys[e] + slot, key, keep_policy);
+                counter[e].add(bins[e], dg[e].bin(key));
+            }
+        };
         rs.run_groups([&](const typename Stream::Scorer::Piece (&v)[4], int row0) {
             struct { float d[2][4]; } x;
             scorer.columns(v, x.d);
             return [&, x, row0] {
+                if (halves) {
+                    const int base = row0 + 16 * (tig >> 1) + gid;
 #pragma unroll
-                for (int m = 0; m < 2; ++m)
-#pragma unroll
-                    for (int i = 0; i < 2; ++i) {
-                        const int slot = row0 + 16 * m + 8 * i + gid;
-#pragma unroll
-                        for (int e = 0; e < 2; ++e)
-                            if (2 * tig + e < g && slot < n_local) {
-                                const uint32_t key = order_key(x.d[m][2 * i + e]);
-                                st_global_hint(keys[e] + slot, key, keep_policy);
-                                hist_add(&bins[e][dg[e].bin(key)]);
-                            }
+                    for (int j = 0; j < 4; ++j) {
+                        const float other = __shfl_sync(0xffffffffu, x.d[1][j], lane & ~2);
+                        take(base + 8 * (j >> 1), j & 1, tig < 2 ? x.d[0][j] : other);
                     }
+                } else {
+#pragma unroll
+                    for (int m = 0; m < 2; ++m)
+#pragma unroll
+                        for (int j = 0; j < 4; ++j) take(row0 + 16 * m + 8 * (j >> 1) + gid, j & 1, x.d[m][j]);
+                }
             };
         });
+#pragma unroll
+        for (int e = 0; e < 2; ++e)                    // (lanes of a warp count for different lists)
+            if (u0 + e < g && counter[e].below) atomicAdd(bins[e], counter[e].below);
     }
     asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
 
@@ -1034,6 +1050,7 @@ __global__ void __launch_bounds__(kThreads, 2)
     GroupScorer<T, DP, RED> scorer;
     scorer.load_staged(sm->qs, gm.gl);
     Digit dg = {0u, 21};
+    DigitCounter counter;
     // identical in every block of the cluster: same rows, same arithmetic.  Called by all threads, once.
     auto place_digit = [&](int done_tiles) {
         if (tid < kSampleRows) sm->sample[tid] = order_key(scorer.score([&](int c) { return srow[c]; }));
@@ -1078,7 +1095,7 @@ __global__ void __launch_bounds__(kThreads, 2)
             const int slot = i * kRows + tid;
             if (i < done_tiles && slot < n_local) {
                 const uint16_t b = (uint16_t)dg.bin(kk[i]);
-                hist_add(&hist[b]);
+                counter.add(hist, b);
                 bins[slot] = b;
             }
         }
@@ -1116,7 +1133,7 @@ __global__ void __launch_bounds__(kThreads, 2)
 #endif
             if (placed) {
                 b = (uint16_t)dg.bin(key);
-                hist_add(&hist[b]);
+                counter.add(hist, b);
             }
         }
         bins[slot] = b;
@@ -1134,6 +1151,7 @@ __global__ void __launch_bounds__(kThreads, 2)
     }
     if (dead && tid == 0) atomicExch(status, kStatusTimeout);
     if (place_at == my_tiles) place_digit(my_tiles);   // a short share: the digit is placed after its last tile
+    counter.flush(hist);
     __syncthreads();
     CW_MARK(2);
 #ifdef TB_PHASE_TIMING
