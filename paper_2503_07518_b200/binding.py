@@ -161,9 +161,8 @@ def predict_importance_queries(hidden, ln_weight, ln_bias, w1, w2, dtype, n_q_he
     returns its status code."""
     if _calls is None:
         lib()
-    n_tokens, model_dim = hidden.shape
-    return _calls.predict_importance_queries(dtype, model_dim, w1.shape[0], n_q_heads, n_slots, imp_dim, activation, ln_eps, ln_weight,
-                                             ln_bias, w1, w2, hidden, n_tokens, scratch, q_imp, stream)
+    return _calls.predict_importance_queries(dtype, n_q_heads, n_slots, imp_dim, activation, ln_eps, ln_weight, ln_bias, w1, w2, hidden,
+                                             scratch, q_imp, stream)
 
 
 class Context:

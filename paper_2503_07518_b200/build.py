@@ -43,6 +43,15 @@ def build(force: bool = False, verbose: bool = False) -> str:
 
 def _build_locked(verbose: bool) -> str:
     nvcc = os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")
+    import torch
+    cxx = os.environ.get("CXX", "g++")
+    torch_dir = os.path.dirname(torch.__file__)
+    calls_obj = os.path.join(CSRC, "tb_python.o")
+    calls = subprocess.Popen([cxx, "-O2", "-std=c++17", "-fPIC", "-D_GLIBCXX_USE_CXX11_ABI=%d" % torch._C._GLIBCXX_USE_CXX11_ABI,
+                              "-I" + sysconfig.get_paths()["include"], "-I" + os.path.join(torch_dir, "include"),
+                              "-I" + os.path.join(torch_dir, "include", "torch", "csrc", "api", "include"),
+                              "-I" + os.path.join(os.path.dirname(os.path.dirname(nvcc)), "include"), "-c", os.path.join(CSRC, "tb_python.cpp"),
+                              "-o", calls_obj], stdout=subprocess.PIPE, stderr=subprocess.STDOUT, text=True)
     objs = []
     procs = []
     for src in SOURCES:
@@ -61,11 +70,14 @@ def _build_locked(verbose: bool) -> str:
     tmp = LIB + ".%d.tmp" % os.getpid()
     subprocess.check_call([nvcc, "-shared", "-o", tmp, *objs, "-gencode", "arch=compute_100a,code=sm_100a"])
     os.replace(tmp, LIB)
-    # the library is found beside the module ($ORIGIN), under the name it has there
+    out, _ = calls.communicate()
+    if calls.returncode:
+        sys.stderr.write(out)
+        raise RuntimeError("compiling tb_python.cpp failed")
+    # the library is found beside the module ($ORIGIN), under the name it has there; torch's are loaded when it is imported
     tmp = CALLS + ".%d.tmp" % os.getpid()
-    subprocess.check_call([os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-fPIC", "-shared", "-I" + sysconfig.get_paths()["include"],
-                           os.path.join(CSRC, "tb_python.cpp"), "-o", tmp, "-L" + HERE, "-l:" + os.path.basename(LIB),
-                           "-Wl,-rpath,$ORIGIN"])
+    subprocess.check_call([cxx, "-shared", calls_obj, "-o", tmp, "-L" + HERE, "-l:" + os.path.basename(LIB), "-L" + os.path.join(torch_dir, "lib"),
+                           "-lc10", "-lc10_cuda", "-ltorch_cpu", "-ltorch_python", "-Wl,-rpath,$ORIGIN"])
     os.replace(tmp, CALLS)
     return LIB
 
