@@ -1,5 +1,5 @@
-// Pieces shared by the selection kernels: the scoring arithmetic (one definition, so the standalone
-// and the fused kernel produce bit-identical scores) and the launch-unit decoding.
+// Pieces shared by the selection kernels: the scoring arithmetic (FMA chains; bf16 rows also on the tensor
+// cores, with exact products and fp32 sums in another order), launch-unit decoding, neighbours and lists.
 #pragma once
 
 #include <type_traits>
