@@ -24,6 +24,7 @@ constexpr int kWarps = kThreads / 32;
 constexpr int kHalf = 256;          // rows of a tile = threads that score it
 constexpr int kMaxCand = 8192;      // one bitmask half word per thread
 constexpr int kBins = 2048;
+constexpr int kMaxShare = 4;        // blocks that stream one problem
 constexpr int kMaxRank = kThreads;  // keys of the threshold bin that are ranked pairwise
 
 struct __align__(16) SmallSmem {
@@ -33,7 +34,7 @@ struct __align__(16) SmallSmem {
     float qs[kMaxGroup * 32];       // the list's importance queries
     uint2 frags[kQueryFrags];       // ... as tensor-core operands
     uint64_t full[kMaxCand / kHalf];
-    float part[kWarps][2];
+    float part[kMaxShare * kWarps][2];   // per block of the cluster and warp: sums of scores and of their squares
     int slots[kWarps];
     int bin, krem, count, n_cand;
 };
@@ -76,11 +77,13 @@ struct NoStream {
     __device__ __forceinline__ void start(const unsigned char*, int) {}
 };
 
-// bf16 rows: kU groups of 32 rows in flight per warp (see RowStream); fp32 rows (kU = 0): through a ring of n_stages tiles
-template <typename T, int DP, int RED, int kU>
+// bf16 rows: kU groups of 32 rows in flight per warp (see RowStream); fp32 rows (kU = 0): through a ring of n_stages tiles.
+// kShared: a cluster of blocks per problem streams it, block r the r-th run of share_tiles tiles, with keys and sums going
+// to block 0's shared memory; behind one cluster barrier block 0 finishes alone.
+template <typename T, int DP, int RED, int kU, bool kShared>
 __global__ void __launch_bounds__(kThreads, kU == 2 ? 2 : 1) select_small_kernel(const __grid_constant__ CUtensorMap tmap,
                                                                                  const unsigned char* __restrict__ kimp, Geom gm, UnitTable ut,
-                                                                                 SelectArgs a, int n_stages, int max_tiles, uint32_t wait_limit,
+                                                                                 SelectArgs a, int n_stages, int max_tiles, int share_tiles, uint32_t wait_limit,
                                                                                  int32_t* __restrict__ state_idx, int32_t* __restrict__ state_cnt,
                                                                                  int32_t* __restrict__ status) {
     constexpr int RB = DP * Elem<T>::kBytes, NCH = RB / 16;
@@ -92,44 +95,64 @@ __global__ void __launch_bounds__(kThreads, kU == 2 ? 2 : 1) select_small_kernel
     SmallSmem* sm = reinterpret_cast<SmallSmem*>(keys + max_tiles * kHalf);
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
 
+    uint32_t C = 1, rank = 0;
+    if constexpr (kShared) {
+        asm volatile("mov.u32 %0, %%cluster_nctaid.x;" : "=r"(C));
+        asm volatile("mov.u32 %0, %%cluster_ctaid.x;" : "=r"(rank));
+        asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");      // (waited for before the first remote store)
+    }
+    const int unit = blockIdx.x / C;
     // What needs nothing from the predecessor runs beside its tail.
     if (tid == 0) sm->n_cand = 0;
     if (!kDirect && tid == 0) prefetch_tmap(&tmap);
     if (!kDirect && tid < n_stages) mbar_init(&sm->full[tid], 1), fence_mbar_init();
     reinterpret_cast<int4*>(sm->hist)[tid] = make_int4(0, 0, 0, 0);
     int ll, s, h;
-    decode_unit(gm, ut, blockIdx.x, ll, s, h);
+    decode_unit(gm, ut, unit, ll, s, h);
     const size_t cu = list_unit(gm, ut, ll, s, h);
-    const ListOut out(gm, a, cu, blockIdx.x, state_idx, state_cnt);
+    const ListOut out(gm, a, cu, unit, state_idx, state_cnt);
     pdl_wait();
     pdl_launch_dependents();                           // (waits for this grid's completion before it reads a list)
 
+    if constexpr (kShared) asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");    // every block of the cluster runs
     const int L = unit_len(gm, ut, ll, s);
     const int lo = min(a.sinks, L), hi = max(lo, L - a.recent), ncand = hi - lo;
     const int k = min(a.budget, ncand);
     check_candidates_projected(gm, ut, ll, s, hi, status);
     if (k <= 0 || k == ncand) {                        // nothing to rank: none, or all (neighbours add nothing then)
-        out.all<kThreads>(lo, k);
+        if (rank == 0) out.all<kThreads>(lo, k);
         return;
     }
     const int n_tiles = (ncand + kHalf - 1) / kHalf;   // <= max_tiles
-    const long long row0 = (long long)key_unit(gm, ut, ll, s, h) * gm.max_seq_len + lo;
+    // this block's rows: candidates slot0 .. slot0 + n_local - 1
+    const int slot0 = min(ncand, (int)rank * share_tiles * kHalf), n_local = min(ncand - slot0, share_tiles * kHalf);
+    const int my_tiles = (n_local + kHalf - 1) / kHalf;
+    const long long row0 = (long long)key_unit(gm, ut, ll, s, h) * gm.max_seq_len + lo + slot0;
     auto request = [&](int t) {                        // tile t, into its stage
         uint64_t* bar = &sm->full[t % n_stages];
         mbar_arrive_expect_tx(bar, kTileBytes);
         tma_load_2d(ring + t % n_stages * kTileBytes, &tmap, 0, (int)(row0 + (long long)t * kHalf), bar);
     };
     if (!kDirect && tid == 0)
-        for (int t = 0; t < min(n_stages, n_tiles); ++t) request(t);
+        for (int t = 0; t < min(n_stages, my_tiles); ++t) request(t);
     if (tid < gm.gl * DP) sm->qs[tid] = a.q_imp[query_row(gm, ut, ll, s, h) * DP + tid];
     typename std::conditional<kDirect, RowStream<DP, RED, kDirect ? kU : 1>, NoStream>::type rs;
-    rs.start(kimp + row0 * RB, ncand);
+    rs.start(kimp + row0 * RB, n_local);
     __syncthreads();
 
     // ---- stream ------------------------------------------------------------------------------------
     float s1 = 0.f, s2 = 0.f;
+    uint32_t keys0 = smem_u32(keys + slot0), part0 = smem_u32(&sm->part[rank * kWarps + warp]);
+    if constexpr (kShared) {                           // the same places in block 0
+        asm volatile("mapa.shared::cluster.u32 %0, %0, 0;" : "+r"(keys0));
+        asm volatile("mapa.shared::cluster.u32 %0, %0, 0;" : "+r"(part0));
+    }
+    auto put_key = [&](int slot, uint32_t key) {
+        if constexpr (kShared) asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(keys0 + slot * 4), "r"(key) : "memory");
+        else keys[slot] = key;
+    };
     auto keep = [&](int slot, float sc) {
-        keys[slot] = order_key(sc);
+        put_key(slot, order_key(sc));
         s1 += sc, s2 = fmaf(sc, sc, s2);
     };
     if constexpr (kDirect) {
@@ -146,22 +169,22 @@ __global__ void __launch_bounds__(kThreads, kU == 2 ? 2 : 1) select_small_kernel
         scorer.load_staged(sm->qs, gm.gl);
         const int half = tid / kHalf, r = tid % kHalf;
         bool dead = false;
-        for (int t = half; t < n_tiles; t += 2) {
+        for (int t = half; t < my_tiles; t += 2) {
             const int st = t % n_stages, slot = t * kHalf + r;
             const bool ok = mbar_wait(&sm->full[st], (t / n_stages) & 1, wait_limit);
             dead |= !ok;
             const unsigned char* tile = ring + st * kTileBytes;
-            if (slot < ncand && ok) {
+            if (slot < n_local && ok) {
                 const uint32_t off = r * RB;
                 keep(slot, scorer.score([&](int c) {
                     uint32_t o = off + c * 16;
                     o ^= ((o >> 7) & (NCH - 1)) << 4;  // TMA swizzle of 16-byte chunks (mode = row size)
                     return *reinterpret_cast<const uint4*>(tile + o);
                 }));
-            } else if (slot < ncand) {
-                keys[slot] = 0u;
+            } else if (slot < n_local) {
+                put_key(slot, 0u);
             }
-            if (t + n_stages < n_tiles) {              // uniform per half
+            if (t + n_stages < my_tiles) {             // uniform per half
                 if (half == 0) asm volatile("bar.sync 1, %0;" ::"n"(kHalf) : "memory");   // the half has read the stage
                 else asm volatile("bar.sync 2, %0;" ::"n"(kHalf) : "memory");
                 if (r == 0 && !dead) {
@@ -173,13 +196,23 @@ __global__ void __launch_bounds__(kThreads, kU == 2 ? 2 : 1) select_small_kernel
         if (dead && lane == 0) atomicExch(status, kStatusTimeout);
     }
     s1 = warp_sum(s1), s2 = warp_sum(s2);
-    if (lane == 0) sm->part[warp][0] = s1, sm->part[warp][1] = s2;
-    __syncthreads();
+    if constexpr (kShared) {
+        if (lane == 0) {
+            asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(part0), "f"(s1) : "memory");
+            asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(part0 + 4), "f"(s2) : "memory");
+        }
+        asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+        if (rank != 0) return;                         // nothing reads this block's shared memory
+    } else {
+        if (lane == 0) sm->part[warp][0] = s1, sm->part[warp][1] = s2;
+        __syncthreads();
+    }
 
     // ---- digit and histogram --------------------------------------------------------------------------
     float m1 = 0.f, m2 = 0.f;
+    for (int r = 0; r < (int)C; ++r)
 #pragma unroll
-    for (int w = 0; w < kWarps; ++w) m1 += sm->part[w][0], m2 += sm->part[w][1];
+        for (int w = 0; w < kWarps; ++w) m1 += sm->part[r * kWarps + w][0], m2 += sm->part[r * kWarps + w][1];
     m1 /= (float)ncand, m2 = m2 / (float)ncand - m1 * m1;
     const float dev = sqrtf(fmaxf(m2, 0.f));
     const float base = m1 - 4.5f * dev, scale = dev > 0.f ? (float)(kBins - 2) / (9.f * dev) : 0.f;
@@ -285,8 +318,8 @@ size_t small_smem(int n_stages, int n_tiles, int tile_bytes) {
 bool select_small_takes(const tb_ctx* c, const UnitTable& ut, int max_cand, bool more) {
     if (c->drop_tile >= 0) return false;               // wait diagnostics: see select_kernel
     const int n_units = ut.layer_count * ut.n_seq * c->geom.Hl;
-    const bool few = 3 * n_units <= c->sm_count, alone = n_units <= c->sm_count;
-    return n_units <= 2 * c->sm_count && max_cand <= (more || (alone && !few) ? kMaxCand : kMaxCand / 2);
+    const bool alone = n_units <= c->sm_count;
+    return n_units <= 2 * c->sm_count && max_cand <= (more || alone ? kMaxCand : kMaxCand / 2);
 }
 
 cudaError_t launch_select_small(const tb_ctx* c, const UnitTable& ut, const SelectArgs& a, int max_cand, cudaStream_t s, bool dry) {
@@ -301,38 +334,46 @@ cudaError_t launch_select_small(const tb_ctx* c, const UnitTable& ut, const Sele
     // to itself, half otherwise.
     const bool direct = gm.dtype == TB_BF16, alone = n_units <= c->sm_count;
     const size_t room = (alone ? 226 : 112) * 1024;
-    int n_stages = direct ? 0 : n_tiles;
+    // Blocks per problem: as many as leave each at least 1024 rows and fit the SMs (a block takes in 45 to 55 bytes per clock).
+    int C = 1;
+    while (2 * C <= kMaxShare && 2 * C * n_units <= c->sm_count && n_tiles >= 2 * C * 4) C *= 2;
+    const int share_tiles = (n_tiles + C - 1) / C;
+    int n_stages = direct ? 0 : share_tiles;
     if (small_smem(n_stages, n_tiles, tile_bytes) > room) {
         n_stages &= ~1;                                // even: see the stream loop
         while (n_stages > 2 && small_smem(n_stages, n_tiles, tile_bytes) > room) n_stages -= 2;
     }
 
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(n_units, 1, 1), cfg.blockDim = dim3(kThreads, 1, 1), cfg.stream = s;
+    cfg.gridDim = dim3(n_units * C, 1, 1), cfg.blockDim = dim3(kThreads, 1, 1), cfg.stream = s;
     cfg.dynamicSmemBytes = small_smem(n_stages, n_tiles, tile_bytes);
-    cudaLaunchAttribute attr[1];
+    cudaLaunchAttribute attr[2];
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = C, attr[1].val.clusterDim.y = 1, attr[1].val.clusterDim.z = 1;
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;   // see pdl_wait()
     attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr, cfg.numAttrs = 1;
+    cfg.attrs = attr, cfg.numAttrs = C > 1 ? 2 : 1;
     auto launch = [&](auto kernel, unsigned char (&seen)[64]) {
         if (first_use_on_this_device(seen)) {
             cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
             if (e != cudaSuccess) return e;
         }
-        return cudaLaunchKernelEx(&cfg, kernel, c->kimp_map, (const unsigned char*)c->kimp, gm, ut, a, n_stages, n_tiles, wait_limit,
+        return cudaLaunchKernelEx(&cfg, kernel, c->kimp_map, (const unsigned char*)c->kimp, gm, ut, a, n_stages, n_tiles, share_tiles, wait_limit,
                                   c->st.idx, c->st.cnt, c->st.status);
     };
     // a block alone on its SM keeps four groups of rows in flight per warp, two blocks two each (their registers)
-#define TB_SMALL(T, DP, RED, U)                                        \
+#define TB_SMALL(T, DP, RED, U, SH)                                    \
     do {                                                               \
         static unsigned char seen[64];                                 \
-        return launch(select_small_kernel<T, DP, RED, U>, seen);       \
+        return launch(select_small_kernel<T, DP, RED, U, SH>, seen);   \
     } while (0)
-#define TB_SMALL_U(DP, RED)                                            \
-    do {                                                               \
-        if (direct && alone) TB_SMALL(__nv_bfloat16, DP, RED, 4);      \
-        if (direct) TB_SMALL(__nv_bfloat16, DP, RED, 2);               \
-        TB_SMALL(float, DP, RED, 0);                                   \
+#define TB_SMALL_U(DP, RED)                                                 \
+    do {                                                                    \
+        if (direct && C > 1) TB_SMALL(__nv_bfloat16, DP, RED, 4, true);     \
+        if (direct && alone) TB_SMALL(__nv_bfloat16, DP, RED, 4, false);    \
+        if (direct) TB_SMALL(__nv_bfloat16, DP, RED, 2, false);             \
+        if (C > 1) TB_SMALL(float, DP, RED, 0, true);                       \
+        TB_SMALL(float, DP, RED, 0, false);                                 \
     } while (0)
     const bool max = a.reduce == TB_GROUP_MAX;
     if (gm.dp == 32) {
