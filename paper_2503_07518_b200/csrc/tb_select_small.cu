@@ -22,7 +22,7 @@ namespace {
 constexpr int kThreads = 512;
 constexpr int kWarps = kThreads / 32;
 constexpr int kHalf = 256;          // rows of a tile = threads that score it
-constexpr int kMaxCand = 8192;      // one bitmask half word per thread
+constexpr int kMaxCand = 16384;     // one bitmask word per thread
 constexpr int kBins = 2048;
 constexpr int kMaxShare = 4;        // blocks that stream one problem
 constexpr int kMaxRank = kThreads;  // keys of the threshold bin that are ranked pairwise
@@ -284,7 +284,7 @@ __global__ void __launch_bounds__(kThreads, kU == 2 ? 2 : 1) select_small_kernel
         }
         classify([&](uint32_t key) { return key > prefix ? 2 : 0; }, false);
         // the equal keys' bits, then as many of them as are wanted, lowest positions first
-        const int n_words = n_tiles * (kHalf / 32);    // <= 256 < kThreads
+        const int n_words = n_tiles * (kHalf / 32);    // <= kThreads
         uint32_t eq = 0u;
         if (tid < n_words)
             for (int e = 0; e < 32; ++e) eq |= (uint32_t)(tid * 32 + e < ncand && keys[tid * 32 + e] == prefix) << e;
@@ -310,16 +310,16 @@ size_t small_smem(int n_stages, int n_tiles, int tile_bytes) {
 }  // namespace
 
 // Launches of up to two blocks per SM.  Measured against the cluster kernel and the one-block-per-problem kernel, us per
-// launch at 32 dimensions, bf16 (this / the other): 32 problems of 1000 candidates 5.7 / 7.0, 2000 6.9 / 10.4, 4000 9.3 / 9.5,
-// 6000 level (its clusters bring four times the SMs to few problems; at 16 dimensions 8000 candidates 12.2 / 10.5);
-// 96 problems of 2000 7.5 / 10.2, 8000 16.1 / 21.8; 192 problems of 800 8.3 / 8.7, 2000 level, 4000 18.5 / 19.0, 8000 31.7 / 28.9;
-// 288 of 2000 12.1 / 16.1; 384 problems, a second wave: level or worse.  Neighbours and the caller's copy come for next to
-// nothing here and cost two more launches there (96 problems of 3000 with both: 8.3 / 18.4).
+// launch, bf16, 32 dimensions unless said (this / the other): 32 problems of 1000 candidates 5.6 / 7.0, 2000 6.7 / 10.4, 4000
+// 7.7 / 9.5, 8000 11.4 / 12.7, 12000 13.2 / 12.6 (eight blocks per problem bring more SMs there); 96 problems of 2000 7.3 /
+// 10.2, 9500 19.4 / 20.9, 16000 28.9 / 29.1, at 16 dimensions 14.9 / 17.3 and 23.4 / 24.5; two per SM: 192 of 2000 level, of
+// 6000 25.4 / 25.8 (16 dimensions 17.9 / 23.0), of 9500 level; 384 problems, a second wave: level or worse.  Neighbours and
+// the caller's copy come for next to nothing here and cost two more launches there (96 problems of 3000 with both: 8.3 / 18.4).
 bool select_small_takes(const tb_ctx* c, const UnitTable& ut, int max_cand, bool more) {
     if (c->drop_tile >= 0) return false;               // wait diagnostics: see select_kernel
     const int n_units = ut.layer_count * ut.n_seq * c->geom.Hl;
-    const bool alone = n_units <= c->sm_count;
-    return n_units <= 2 * c->sm_count && max_cand <= (more || alone ? kMaxCand : kMaxCand / 2);
+    const int most = more || (n_units <= c->sm_count && 2 * n_units > c->sm_count) ? kMaxCand : n_units <= c->sm_count ? 10 * 1024 : 8 * 1024;
+    return n_units <= 2 * c->sm_count && max_cand <= most;
 }
 
 cudaError_t launch_select_small(const tb_ctx* c, const UnitTable& ut, const SelectArgs& a, int max_cand, cudaStream_t s, bool dry) {

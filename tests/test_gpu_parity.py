@@ -657,7 +657,7 @@ def test_long_problem_cluster_kernel_unusual_distributions(H):
 
 @pytest.mark.parametrize("cfg,dp", [(2, 32), (2, 16), (1, 32), (1, 16)])
 @pytest.mark.parametrize("L,budget,sinks,recent", [(20, 1, 3, 2), (31, 7, 0, 0), (33, 32, 0, 0), (257, 100, 1, 0), (2055, 513, 4, 64), (4113, 2, 0, 17),
-                                                   (8192, 700, 0, 0)])
+                                                   (8192, 700, 0, 0), (16384, 1500, 0, 0), (10250, 900, 3, 3)])
 def test_small_selection_kernel_edges(H, cfg, dp, L, budget, sinks, recent):
     """One-block selection: sizes around the 32-row groups, the 256-row tiles and the largest it takes, both reductions and
     neighbour rules, with the caller's copy checked against the stored list through the attention that follows."""
