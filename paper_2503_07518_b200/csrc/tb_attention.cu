@@ -507,6 +507,8 @@ __global__ void __launch_bounds__(NW * 32) attn_mma_kernel(Geom gm, UnitTable ut
         }
     }
     attn_stamp(2);
+    // awaited before the first remote store: every block of the cluster runs, so its shared memory exists
+    if (a.cluster_merge && a.nsplit > 1) asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
 
     if (a.early_ok) pdl_wait();                        // the queries are this call's input
     attn_stamp(7);
@@ -775,6 +777,7 @@ __global__ void __launch_bounds__(NW * 32) attn_mma_kernel(Geom gm, UnitTable ut
             attn_stamp(6);
             return;
         }
+        asm volatile("barrier.cluster.wait.aligned;" ::: "memory");
         for (int slot = tid; slot < 256; slot += NW * 32) {
             const int mt = slot >> 5, ln = slot & 31;
             float4 acc, stat;

@@ -373,6 +373,7 @@ __global__ void __launch_bounds__(kPredThreads, 2) predictor_hidden_tile_kernel(
     const int n_chunk = (span + kChunk - 1) / kChunk;
     const uint4 zero = make_uint4(0u, 0u, 0u, 0u);
     pred_stamp(0, 0);
+    asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");    // awaited before the first remote write: the block runs
     // The states may come from the predecessor, and so may the weights: wait, then let the output kernel get ready.
     pdl_wait();
     pdl_launch_dependents();
@@ -463,6 +464,7 @@ __global__ void __launch_bounds__(kPredThreads, 2) predictor_hidden_tile_kernel(
         }
         __syncthreads();
         pred_stamp(0, 3);
+        if (group == 0) asm volatile("barrier.cluster.wait.aligned;" ::: "memory");
         for (int e = tid; e < kTileRows * kTileTok; e += kPredThreads) {
             const int row = e / kTileTok, tok = e % kTileTok;
             if (tok < n_here) *cluster.map_shared_rank(&s_p[group & 1][rank][row % kRows][tok], row / kRows) = get_sum<kN8>(s_sum, row, tok);
