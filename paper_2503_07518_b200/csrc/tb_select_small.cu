@@ -1,8 +1,9 @@
 // Selection of small problems: scoring, exact top-B, neighbour fetching and the copy of the list for the caller, one
 // block per (layer, sequence, list), one launch (paper Sec. 3.4, Sec. 4 "Token Selection Policy").
 //
-// A problem of a few thousand candidates is 32 to 512 KB of projected keys: one SM takes it in within 1 to 6 us, and
-// what a launch costs beyond that is latency.  So everything stays inside one block of 512 threads:
+// A problem of a few thousand candidates is 32 KB to 1 MB of projected keys: one SM takes it in within 1 to 10 us, and
+// what a launch costs beyond that is latency.  So everything stays inside one block of 512 threads; where a launch would
+// leave SMs idle, up to three more blocks of a cluster stream shares of the problem into that block's shared memory:
 //   stream   bf16 rows straight into tensor-core fragments (see RowStream), fp32 rows through 2-D TMA tiles of 256 rows, all
 //            requested at once when they fit; the order-preserving key goes to shared memory, score sums stay in registers
 //   digit    mean and deviation of all the scores place 2046 equal slices of score across mean +- 4.5 deviations (one
@@ -12,7 +13,7 @@
 //            on the bitmask, list
 // A crowded threshold bin (massive ties, a few huge outliers) goes through the key's own digits instead (11 + 11 + 10).
 //
-// The launch is a programmatic dependent: no clusters, so an early start cannot misplace anything.
+// The launch is a programmatic dependent: one block or a cluster of two or four, for which an early start finds room.
 #include "tb_select.cuh"
 
 namespace tb {
