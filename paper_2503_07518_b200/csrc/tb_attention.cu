@@ -368,6 +368,7 @@ __device__ __forceinline__ void f32_rows(const float* __restrict__ qbase, int g,
 
 // Shared memory behind the warps' stages for the merge inside a cluster of C blocks: the accumulator slices this
 // block owns from every block ([slices per owner][C][32 lanes] float4) and every block's (m, l) ([C][4] float4).
+constexpr size_t kFourWarpBytes = 76 * 1024;       // least shared memory of a 4-warp block (see launch_attention)
 static inline size_t cluster_merge_bytes(int C) { return (size_t)((8 + C - 1) / C) * C * 32 * 16 + (size_t)C * 4 * 16; }
 
 // NW warps per block.  With a.cluster_merge the blocks of one (sequence, KV head) form a thread-block
@@ -486,6 +487,8 @@ __global__ void __launch_bounds__(NW * 32) attn_mma_kernel(Geom gm, UnitTable ut
     };
     auto commit = [&]() { asm volatile("cp.async.commit_group;" ::: "memory"); };
     attn_stamp(1);
+    const bool split_cluster = a.cluster_merge && a.nsplit > 1;
+    if (split_cluster) asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
     // Lane i < kTok keeps, one bit per tile from the current one on, whether its row of that tile is a
     // bad list entry (outside the cached tokens): known when the tile's rows are issued, used when
     // the tile is consumed.  (Reading the entry a second time at consumption, as an earlier version did,
@@ -507,8 +510,9 @@ __global__ void __launch_bounds__(NW * 32) attn_mma_kernel(Geom gm, UnitTable ut
         }
     }
     attn_stamp(2);
-    // awaited before the first remote store: every block of the cluster runs, so its shared memory exists
-    if (a.cluster_merge && a.nsplit > 1) asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
+    // Every block of the cluster runs, so its shared memory exists for the merge's remote stores.  Awaited here, beside the
+    // gathers in flight: just before the stores it was 0.3 us of a small launch.
+    if (split_cluster) asm volatile("barrier.cluster.wait.aligned;" ::: "memory");
 
     if (a.early_ok) pdl_wait();                        // the queries are this call's input
     attn_stamp(7);
@@ -777,7 +781,6 @@ __global__ void __launch_bounds__(NW * 32) attn_mma_kernel(Geom gm, UnitTable ut
             attn_stamp(6);
             return;
         }
-        asm volatile("barrier.cluster.wait.aligned;" ::: "memory");
         for (int slot = tid; slot < 256; slot += NW * 32) {
             const int mt = slot >> 5, ln = slot & 31;
             float4 acc, stat;
@@ -894,25 +897,28 @@ cudaError_t launch_attention(const tb_ctx* c, const UnitTable& ut, const AttnArg
             if (e != cudaSuccess) return e;
             (void)cudaGetLastError();
         }
-        auto clusters_that_fit = [&](int csize) {     // how many clusters of `csize` 8-warp blocks run at once
-            if (max_active[csize] == 0) {
+        // how many clusters of `csize` blocks run at once: 8-warp blocks, one per SM, or 4-warp ones, two (at most 8 per cluster)
+        auto clusters_that_fit = [&](int csize, bool four = false) {
+            int& known = max_active[(four ? kAttnMaxCluster : 0) + csize];
+            if (known == 0) {
                 cudaLaunchConfig_t q = {};
-                q.gridDim = dim3(csize, 1, 1), q.blockDim = dim3(256, 1, 1);
+                q.gridDim = dim3(csize, 1, 1), q.blockDim = dim3(four ? 128 : 256, 1, 1);
                 const size_t mb = cluster_merge_bytes(csize);
                 const bool three = csize <= 8 && 8 * 3 * kStageBytes + mb <= 220 * 1024;
-                q.dynamicSmemBytes = 8 * (three ? 3 : 2) * kStageBytes + mb;
+                q.dynamicSmemBytes = four ? kFourWarpBytes : 8 * (three ? 3 : 2) * kStageBytes + mb;
                 cudaLaunchAttribute at[1];
                 at[0].id = cudaLaunchAttributeClusterDimension;
                 at[0].val.clusterDim.x = csize, at[0].val.clusterDim.y = 1, at[0].val.clusterDim.z = 1;
                 q.attrs = at, q.numAttrs = 1;
                 int n_clusters = 0;
-                cudaError_t qe = three ? cudaOccupancyMaxActiveClusters(&n_clusters, attn_mma_kernel<8, 3>, &q)
-                                       : cudaOccupancyMaxActiveClusters(&n_clusters, attn_mma_kernel<8, 2>, &q);
+                cudaError_t qe = four ? cudaOccupancyMaxActiveClusters(&n_clusters, attn_mma_kernel<4, 2>, &q)
+                                 : three ? cudaOccupancyMaxActiveClusters(&n_clusters, attn_mma_kernel<8, 3>, &q)
+                                         : cudaOccupancyMaxActiveClusters(&n_clusters, attn_mma_kernel<8, 2>, &q);
                 if (qe != cudaSuccess) n_clusters = 0;
                 (void)cudaGetLastError();
-                max_active[csize] = n_clusters > 0 ? n_clusters : -1;
+                known = n_clusters > 0 ? n_clusters : -1;
             }
-            return max_active[csize];
+            return known;
         };
         // Up to a block per SM: C blocks per problem, one cluster, merged inside it.  Measured over 4 to 192 problems of 64
         // to 20480 rows, 4, 8 and 12 warps, every cluster size and the global merge (figures: bf16, us per launch in a chain
@@ -926,9 +932,12 @@ cudaError_t launch_attention(const tb_ctx* c, const UnitTable& ut, const AttnArg
         //    x 4 warps and the global merge);
         //  - clusters of 3, 7 and 8 pack badly into the SMs of a GPC (3 is taken where the choice is 2), pairs fit everywhere; 9 fits when it takes half of the chip (non-portable:
         //    asked for);
-        //  - the global merge is left with what has too few problems for its rows (4 problems of 20480 rows: 12.6 with 32
-        //    blocks of 8 warps each, 15.3 with a cluster of 9), very long rows on a chip that clusters leave a third empty (96
-        //    of 10240: 76.6 with 3 x 4 warps, 82.0 with one block of 12), and more problems than SMs.
+        //  - up to five problems of 4K rows or more take 16 blocks each, half of the chip again (non-portable; 2 problems of 8000
+        //    rows: 8.6, 9.7 with 9 blocks each; 5 of 16000: 12.6, 14.3 with the global merge);
+        //  - the global merge is left with what has too few problems for its rows, that is, where clusters would leave part of
+        //    the chip empty and the rows outweigh the merge (4 problems of 20000 rows: 12.9 with 32 blocks of 8 warps each, 15.8
+        //    with a cluster of 12; 6 of 30000: 20.7, 22.2; 96 of 30000: 212 with 3 x 4 warps, 226 with one block of 12; fp32, whose
+        //    blocks take longer: 16 of 15000: 43, 54; 96 of 2500: 47, 59), and more problems than SMs.
         const int half = c->sm_count / 2, most = c->sm_count - c->sm_count / 8;
         const int small_block = f32 ? 64 : 256, large_block = f32 ? 192 : 384;
         auto allowed = [&](int C) { return C <= 2 || (C >= 4 && C <= 6) || (C == 9 && units * 9 <= half && clusters_that_fit(9) >= units); };
@@ -946,28 +955,35 @@ cudaError_t launch_attention(const tb_ctx* c, const UnitTable& ut, const AttnArg
             if (least == 3 && 4 * units <= most) least = 4;
             n = largest(want, half);
             if (n < want && n < least) n = largest(least, most);
+            if (!f32 && max_rows > 4096 && units * 16 <= half + half / 8 && clusters_that_fit(16) >= units) n = 16;
         }
 #ifdef TB_FORCE_ATTN_CLUSTER
         n = TB_FORCE_ATTN_CLUSTER;
 #endif
         const int rows_per_block = n ? (max_rows + n - 1) / n : 0;
+        // rows per block up to which the cluster merge is the better one, by the share of the chip that its blocks take
+        const int used = units * n, cluster_rows = f32 ? (used < half ? 420 : used < c->sm_count - c->sm_count / 4 ? 560 : 2000)
+                                                       : (n == 16 ? 1200 : used < 48 ? 1536 : used < 64 ? 3000 : 5 * used > 4 * c->sm_count ? 7680 : 10240);
         // fp32 rows keep an SM's warps busier: 4-warp blocks, two per SM, when they fill more of the chip
         const int n4 = f32 && units <= c->sm_count ? 2 * most / units : 0;
         if (n && n4 <= 8 && rows_per_block > large_block && 10 * n4 > 23 * n) {
             a.nsplit = n4, a.cluster_merge = 1;
-        } else if (n && !(units * n < (f32 ? half : 48) && rows_per_block > (f32 ? 700 : 1536)) && !(units * n < most && rows_per_block > 8192)) {
+        } else if (n && (units * n >= most || rows_per_block <= cluster_rows)) {
             a.nsplit = n, a.cluster_merge = 1;
             nw = rows_per_block <= (f32 ? 64 : 112) ? 4 : rows_per_block <= 256 || f32 ? 8 : 12;
         } else {
             a.nsplit = pick_nsplit(c, units, max_rows);
-            // few problems, one block of 8 warps per SM: as many rows in flight as two of 4, half the partials to merge
-            if (a.nsplit > 16) {
-                nw = 8;
-                if (f32) a.nsplit = c->sm_count / units < kMaxSplits ? c->sm_count / units : kMaxSplits;
-            }
-            // clusters only when the whole launch is resident at once: in multi-wave launches the
-            // co-scheduling constraint costs more than the global merge (measured on the batch-8 workload)
-            if (a.nsplit <= 8 && units * a.nsplit <= 2 * c->sm_count) a.cluster_merge = 1;
+            // Few problems, one block of 8 warps per SM: as many rows in flight as two of 4, half the partials to merge
+            // (8 problems of 131072 rows 82.9, with 32 blocks each, 1.7 waves of the chip, 88.9; 14 of 80000 86.8, 88.4 with
+            // 4-warp blocks).  At 17 problems that is 8 blocks each, a cluster, which packs badly: 148 against 104 with 17 x 4
+            // warps.
+            const int per_sm = c->sm_count / units < kMaxSplits ? c->sm_count / units : kMaxSplits;
+            if (a.nsplit > 16 && per_sm > 8) nw = 8, a.nsplit = per_sm;
+            // Clusters only when the whole launch is resident at once: otherwise the co-scheduling constraint costs more
+            // than the global merge.  How many clusters fit is asked, not computed: sizes that do not divide a GPC's
+            // blocks leave some of them empty (40 problems of 30000 rows, 7 blocks each: 126 in clusters, 94 without; 44, 6
+            // each, which fit: 99 and 103).  Without some room they land badly even so (fp32, 56 of 10000, 5 each: 102, 91).
+            if (a.nsplit <= 8 && units * a.nsplit <= 2 * c->sm_count - c->sm_count / 8 && clusters_that_fit(a.nsplit, true) >= units) a.cluster_merge = 1;
         }
     }
     dim3 grid(a.nsplit, gm.Ha, ut.layer_count * ut.n_seq);
@@ -980,7 +996,7 @@ cudaError_t launch_attention(const tb_ctx* c, const UnitTable& ut, const AttnArg
         // a third one in, and the block scheduler then loads some SMs with three blocks and leaves others with one
         // (batch 8 at 64K: 59 us per launch against 52.6).  Asking for a third of the SM's shared memory plus a
         // little keeps it at two.
-        if (nw == 4 && smem < 76 * 1024) smem = 76 * 1024;
+        if (nw == 4 && smem < kFourWarpBytes) smem = kFourWarpBytes;
         cudaLaunchConfig_t cfg = {};
         cfg.gridDim = grid;
         cfg.blockDim = dim3(nw * 32, 1, 1);

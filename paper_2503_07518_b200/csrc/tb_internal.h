@@ -138,7 +138,7 @@ struct tb_ctx {
     CUtensorMap kimp_map;                 // 2-D view of kimp: rows = all token slots, cols = d'
     int tile_rows;                        // rows per TMA box of the score pass
     int sm_count;
-    int attn_max_active[17];              // co-resident attention clusters per cluster size (0 = not asked yet)
+    int attn_max_active[25];              // co-resident attention clusters per cluster size, 8-warp blocks and (16 +) 4-warp ones (0 = not asked yet)
     void* res_rows;                       // resident sink + window rows (tb_bind_resident_rows), or NULL
     int res_sinks, res_window;
     void* imp_rows;                       // Important buffer (tb_bind_important_buffer), or NULL
