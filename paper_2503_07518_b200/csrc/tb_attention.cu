@@ -393,6 +393,10 @@ __global__ void __launch_bounds__(NW * 32) attn_mma_kernel(Geom gm, UnitTable ut
     __shared__ int sh_last;
 
     attn_stamp(0);
+    // Every block of the cluster has to run before the merge stores to its shared memory: arrive here, wait at the stores
+    // (8 problems of 3276 rows 5.5 us; waiting beside the gathers 5.7, behind the queries 6.0).
+    const bool split_cluster = a.cluster_merge && a.nsplit > 1;
+    if (split_cluster) asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
     // Dependency wait (see pdl_wait).  When the lists or cache rows may come from the predecessor: before the
     // first read of anything it may have written -- the list entries, or already the lengths and list counts when
     // those are read on the device; what comes from the kernel parameters alone (row map, split, addresses) runs
@@ -487,8 +491,6 @@ __global__ void __launch_bounds__(NW * 32) attn_mma_kernel(Geom gm, UnitTable ut
     };
     auto commit = [&]() { asm volatile("cp.async.commit_group;" ::: "memory"); };
     attn_stamp(1);
-    const bool split_cluster = a.cluster_merge && a.nsplit > 1;
-    if (split_cluster) asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
     // Lane i < kTok keeps, one bit per tile from the current one on, whether its row of that tile is a
     // bad list entry (outside the cached tokens): known when the tile's rows are issued, used when
     // the tile is consumed.  (Reading the entry a second time at consumption, as an earlier version did,
@@ -510,9 +512,6 @@ __global__ void __launch_bounds__(NW * 32) attn_mma_kernel(Geom gm, UnitTable ut
         }
     }
     attn_stamp(2);
-    // Every block of the cluster runs, so its shared memory exists for the merge's remote stores.  Awaited here, beside the
-    // gathers in flight: just before the stores it was 0.3 us of a small launch.
-    if (split_cluster) asm volatile("barrier.cluster.wait.aligned;" ::: "memory");
 
     if (a.early_ok) pdl_wait();                        // the queries are this call's input
     attn_stamp(7);
@@ -781,6 +780,7 @@ __global__ void __launch_bounds__(NW * 32) attn_mma_kernel(Geom gm, UnitTable ut
             attn_stamp(6);
             return;
         }
+    if (split_cluster) asm volatile("barrier.cluster.wait.aligned;" ::: "memory");
         for (int slot = tid; slot < 256; slot += NW * 32) {
             const int mt = slot >> 5, ln = slot & 31;
             float4 acc, stat;

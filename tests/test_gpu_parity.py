@@ -688,3 +688,22 @@ def test_fp32_attention_shapes(H, heads, budget):
     w = wl.workload(1, n_layers=1, n_q_heads=2 * heads, n_kv_heads=2, batch=2, lengths=[budget + 300, max(60, budget // 2)], budget=budget, sinks=3,
                     recent=5)
     full_pipeline_check(H, H.Case(w), tb().select_params(budget, 3, 5), dense_too=True)
+
+
+@pytest.mark.parametrize("config,batch,kv_heads,length", [
+    (2, 1, 2, 4097),      # 16 blocks per problem, fewest rows
+    (2, 1, 5, 19200),     # ... most rows
+    (2, 1, 5, 19201),     # one 8-warp block per SM through the workspace
+    (2, 7, 1, 27001),     # ... where clusters of nine take 63 SMs
+    (2, 17, 1, 61500),    # 17 splits of 4 warps: one block per SM would be eight
+    (2, 5, 8, 23050),     # seven splits that do not fit as clusters
+    (1, 2, 8, 3377),      # fp32, 96 blocks
+    (1, 17, 1, 3400),
+    (1, 12, 8, 577),      # fp32, one block per problem or three
+    (1, 7, 8, 4500),      # fp32, five splits that nearly fill the chip
+])
+def test_attention_blocks_per_problem_of_long_rows(H, config, batch, kv_heads, length):
+    """Each way that a launch of long rows is split (dense over the whole cache, sparse in the same context)."""
+    w = wl.workload(config, n_layers=1, n_q_heads=kv_heads, n_kv_heads=kv_heads, batch=batch, lengths=[length] + [max(1, length // 2)] * (batch - 1),
+                    budget=100, sinks=3, recent=5)
+    full_pipeline_check(H, H.Case(w), tb().select_params(100, 3, 5), dense_too=True)
