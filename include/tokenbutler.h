@@ -303,7 +303,8 @@ tb_status tb_bind_important_buffer(tb_ctx* ctx, void* buf_dev, size_t bytes);
  * growth_reserve = how many tokens a sequence may grow beyond its mirror while graphs are replayed: grids and
  * shared memory are sized for mirror + reserve.  While graphs replay the mirrors stand still; the checks
  * that need true lengths then happen on the device (an append past max_seq_len is skipped and reported as
- * TB_ERR_CAPACITY in the status word).  Call tb_sync_lengths before the next call that is not a replay. */
+ * TB_ERR_CAPACITY in the status word; so is a selection on a sequence that outgrew the reserve, which leaves out the
+ * candidates that its launch has no room for).  Call tb_sync_lengths before the next call that is not a replay. */
 tb_status tb_use_device_lengths(tb_ctx* ctx, int32_t on, int32_t growth_reserve);
 /* Synchronise `stream` and copy the device counters into the host mirrors (lengths and projected lengths). */
 tb_status tb_sync_lengths(tb_ctx* ctx, void* stream);

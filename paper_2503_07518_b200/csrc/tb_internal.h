@@ -59,6 +59,7 @@ struct SelectArgs {
     int radius, nmode;
     int32_t* idx_copy;    // [layer_count][n_seq][Hl][idx_cap] or NULL
     int32_t* cnt_copy;
+    int room;             // candidates that the launch's shared memory is sized for (whole groups of 256): see candidates_within
 };
 
 struct NeighborArgs {
@@ -98,7 +99,7 @@ struct AttnArgs {
     int known_cnt[kMaxLaunchUnits];
 };
 
-constexpr int kStatusCapacity = -3;      // device status: an append in a replayed graph ran past max_seq_len
+constexpr int kStatusCapacity = -3;      // device status: an append in a replayed graph ran past max_seq_len, or a sequence past its launch's room
 constexpr int kStatusUnprojected = -4;   // device status: a replayed selection found candidates that are not projected
 
 struct DevState {

@@ -133,6 +133,15 @@ __device__ __forceinline__ void check_candidates_projected(const Geom& gm, const
     }
 }
 
+// Candidates of a problem whose kernel keeps something per candidate in shared memory.  A replayed graph may find a sequence
+// longer than its launch was sized for (it outgrew the declared reserve): the candidates past `room` are left out and the
+// status word says so.
+__device__ __forceinline__ int candidates_within(const UnitTable& ut, int n, int room, int32_t* status) {
+    if (!ut.use_dev_len || n <= room) return n;
+    if (threadIdx.x == 0) atomicExch(status, kStatusCapacity);
+    return room;
+}
+
 // ---- bf16 rows straight into tensor-core fragments ------------------------------------------------------
 //
 // Over a 64-byte row (32 dimensions) thread tig of a row's four takes 16 contiguous bytes, so a warp's 16-byte load is

@@ -487,7 +487,7 @@ __global__ void __launch_bounds__(kThreads, 4)
     const int L = unit_len(gm, ut, ll, s);
     const int lo = min(a.sinks, L);
     const int hi = max(lo, L - a.recent);
-    const int ncand = hi - lo;
+    const int ncand = a.radius > 0 ? candidates_within(ut, hi - lo, a.room, status) : hi - lo;   // (the bitmasks of neighbour fetching)
     const int k = min(a.budget, ncand);
     check_candidates_projected(gm, ut, ll, s, hi, status);
     const size_t cu = list_unit(gm, ut, ll, s, h);
@@ -660,7 +660,8 @@ __global__ void __launch_bounds__(kThreads, 2)
     const int tid = threadIdx.x, lane = tid & 31, gid = lane >> 2, tig = lane & 3;
     const int pair = order.pair[blockIdx.x / gm.Hl], h = blockIdx.x % gm.Hl, rank = h % g;
     const int ll = pair / ut.n_seq, s = pair % ut.n_seq;
-    const int L = unit_len(gm, ut, ll, s), lo = min(a.sinks, L), hi = max(lo, L - a.recent), ncand = hi - lo, k = min(a.budget, ncand);
+    const int L = unit_len(gm, ut, ll, s), lo = min(a.sinks, L), hi = max(lo, L - a.recent);
+    const int ncand = a.radius > 0 ? candidates_within(ut, hi - lo, a.room, status) : hi - lo, k = min(a.budget, ncand);   // (the bitmasks)
     check_candidates_projected(gm, ut, ll, s, hi, status);
     const size_t cu = list_unit(gm, ut, ll, s, h);
     const ListOut out(gm, a, cu, pair * gm.Hl + h, state_idx, state_cnt);

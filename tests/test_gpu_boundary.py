@@ -282,3 +282,67 @@ def test_resident_rows_and_important_buffer_give_the_same_bits(H, on_host):
             for h in range(2):
                 ref, _ = base_case.oracle_attention(l, b, h, q[l, b], base[-1][0][l][b][h], p)
                 assert np.abs(base[-1][1][l, b, h * 4:(h + 1) * 4] - ref).max() <= 2e-3
+
+
+@pytest.mark.parametrize("heads,batch,length,scope,radius", [
+    ((2, 2), 1, 250, 0, 0),           # one block per list, keys and bitmask on chip
+    ((1, 1), 1, 2000, 0, 1),          # ... shared by a cluster
+    ((4, 2), 1, 10300, 1, 1),         # lists that share a key stream: the second bitmask
+    ((8, 8), 38, 250, 0, 2),          # more lists than fit at once: the same
+])
+def test_a_replay_that_outgrows_its_reserve_is_reported(H, heads, batch, length, scope, radius):
+    """A captured selection is replayed on sequences longer than the reserve it was sized for.  It selects among the
+    candidates there is room for -- ascending positions of the cache, no more than asked for -- and says TB_ERR_CAPACITY;
+    with the true lengths back in the mirrors the same context selects exactly again."""
+    b_ = tb()
+    hq, hkv = heads
+    n, budget, replays = 64, 40, 6
+    ctx = b_.Context(1, hq, hkv, 128, 32, b_.TB_BF16, batch, length + n * (replays + 1), budget, max_radius=radius, list_scope=scope)
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(5)
+    rand = lambda *s, **kw: torch.randn(*s, generator=gen, device="cuda", **kw)  # noqa: E731
+    ctx.set_projection(0, rand(hkv, 128, 32, dtype=torch.bfloat16))
+    rows = lambda m: rand(m * batch, hkv, 128, dtype=torch.bfloat16)  # noqa: E731
+    ctx.append_kv(0, 1, None, [length] * batch, rows(length), rows(length))
+    ctx.project_keys(0, 1, None, [0] * batch, [length] * batch)
+    ctx.use_device_lengths(True, growth_reserve=n)
+    qi = rand(1, batch, hq, 32)
+    lists = ctx.n_lists
+    idx = torch.zeros(1, batch, lists, ctx.index_capacity, dtype=torch.int32, device="cuda")
+    cnt = torch.zeros(1, batch, lists, dtype=torch.int32, device="cuda")
+    k, v = rows(n), rows(n)
+    p = b_.select_params(budget, 0, 0, radius)
+    stream = torch.cuda.Stream()
+    with torch.cuda.stream(stream):
+        g = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(g, stream=stream):
+            ctx.append_kv(0, 1, None, [n] * batch, k, v)
+            ctx.project_keys(0, 1, None, None, None, n_seq=batch)
+            ctx.select_topk(0, 1, None, batch, qi, p, idx, cnt)
+        ctx.sync_lengths(stream)
+        for t in range(replays):
+            g.replay()
+            got = ctx.get_status(stream)
+            now = length + n * (t + 1)
+            assert got in (0, b_.TB_ERR_CAPACITY) and (got == 0 or t > 0)
+            c, x = cnt.cpu().numpy(), idx.cpu().numpy()
+            assert ((c >= budget) & (c <= budget * (2 * radius + 1))).all()
+            for b in range(batch):
+                for h in range(lists):
+                    row = x[0, b, h, :c[0, b, h]]
+                    assert row[0] >= 0 and row[-1] < now and (np.diff(row) > 0).all()
+        assert got == b_.TB_ERR_CAPACITY               # 384 tokens past lengths with room for at most 64 + 64 + 255 more
+        ctx.sync_lengths(stream)
+    ctx.use_device_lengths(False)
+    L = length + n * replays
+    assert ctx.get_length(0, 0) == (L, L)
+    lists_now = torch.zeros_like(idx)
+    ctx.select_topk(0, 1, None, batch, qi, p, lists_now, cnt)
+    assert ctx.get_status() == 0
+    c, x = cnt.cpu().numpy(), lists_now.cpu().numpy()
+    for b in range(batch):
+        for h in range(lists):
+            kimp = H.to_host(ctx.kimp[0, b, h * hkv // lists, :L], b_.TB_BF16)
+            s = H.orc.score(qi[0, b, h * hq // lists:(h + 1) * hq // lists].cpu().numpy(), np.ascontiguousarray(kimp), b_.TB_BF16)
+            want = H.orc.neighbors(H.orc.select(s, 0, 0, budget), radius, 0, 0, L) if radius else H.orc.select(s, 0, 0, budget)
+            assert np.array_equal(x[0, b, h, :c[0, b, h]], want)
