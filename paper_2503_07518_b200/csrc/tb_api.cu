@@ -470,7 +470,7 @@ tb_status tb_select_topk(tb_ctx* c, int32_t lb, int32_t lc, const int32_t* seq_i
                 if (p->radius > 0 && !finished) {
                     NeighborArgs na;
                     na.idx_src = c->wk.sel_idx, na.cnt_src = c->wk.sel_cnt, na.src_stride = c->wk.sel_stride;
-                    na.radius = p->radius, na.nmode = p->nmode, na.sinks = p->sinks, na.recent = p->recent;
+                    na.radius = p->radius, na.nmode = p->nmode, na.sinks = p->sinks, na.recent = p->recent, na.room = max_cand;
                     e = launch_neighbors(c, ut, na, (cudaStream_t)stream, dry);
                     if (e != cudaSuccess) return dry ? TB_ERR_UNSUPPORTED : TB_ERR_CUDA;
                     if (!dry) c->last_list_write = (long long)c->launches, c->launches++;

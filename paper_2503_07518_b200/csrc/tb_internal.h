@@ -67,6 +67,7 @@ struct NeighborArgs {
     const int32_t* cnt_src;
     int src_stride;
     int radius, nmode, sinks, recent;
+    int room;                // candidates that the bitmask on chip is sized for: see candidates_within
 };
 
 // Where an attended row is read from: the K|V cache, or one of two optional copies in device memory.

@@ -52,15 +52,15 @@ cudaError_t launch_score(const tb_ctx* c, const UnitTable& ut, const float* q_im
 constexpr int kNbThreads = 256;
 
 __global__ void __launch_bounds__(kNbThreads) neighbor_kernel(Geom gm, UnitTable ut, NeighborArgs a, int32_t* __restrict__ state_idx,
-                                                              int32_t* __restrict__ state_cnt) {
+                                                              int32_t* __restrict__ state_cnt, int32_t* __restrict__ status) {
     extern __shared__ uint32_t mask[];               // one bit per candidate position
     __shared__ int warp_tot[kNbThreads / 32];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     int ll, s, h;
     decode_unit(gm, ut, blockIdx.x, ll, s, h);
     const int L = unit_len(gm, ut, ll, s);
-    const int lo = min(a.sinks, L), hi = max(lo, L - a.recent);
-    const int span = hi - lo;
+    const int lo = min(a.sinks, L);
+    const int span = candidates_within(ut, max(lo, L - a.recent) - lo, a.room, status), hi = lo + span;
     const int n_words = (span + 31) / 32;
     const int32_t* src = a.idx_src + (size_t)blockIdx.x * a.src_stride;
     const int cnt = a.cnt_src[blockIdx.x];
@@ -122,12 +122,7 @@ __global__ void __launch_bounds__(kNbThreads) neighbor_kernel(Geom gm, UnitTable
 
 cudaError_t launch_neighbors(const tb_ctx* c, const UnitTable& ut, const NeighborArgs& a, cudaStream_t s, bool dry) {
     const Geom& gm = c->geom;
-    int max_span = 0;
-    for (int i = 0; i < ut.layer_count * ut.n_seq; ++i) {
-        int L = ut.len[i], lo = a.sinks < L ? a.sinks : L, hi = L - a.recent > lo ? L - a.recent : lo;
-        if (hi - lo > max_span) max_span = hi - lo;
-    }
-    size_t smem = (size_t)((max_span + 31) / 32) * 4 + 16;
+    size_t smem = (size_t)((a.room + 31) / 32) * 4 + 16;
     if (smem > 200 * 1024) return cudaErrorInvalidConfiguration;   // one bit per candidate on chip: up to 1,638,272 candidates
     if (dry) return cudaSuccess;
     static unsigned char seen[64];
@@ -135,7 +130,7 @@ cudaError_t launch_neighbors(const tb_ctx* c, const UnitTable& ut, const Neighbo
         cudaError_t e = cudaFuncSetAttribute(neighbor_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
         if (e != cudaSuccess) return e;
     }
-    neighbor_kernel<<<ut.layer_count * ut.n_seq * gm.Hl, kNbThreads, smem, s>>>(gm, ut, a, c->st.idx, c->st.cnt);
+    neighbor_kernel<<<ut.layer_count * ut.n_seq * gm.Hl, kNbThreads, smem, s>>>(gm, ut, a, c->st.idx, c->st.cnt, c->st.status);
     return cudaGetLastError();
 }
 

@@ -289,6 +289,7 @@ def test_resident_rows_and_important_buffer_give_the_same_bits(H, on_host):
     ((1, 1), 1, 2000, 0, 1),          # ... shared by a cluster
     ((4, 2), 1, 10300, 1, 1),         # lists that share a key stream: the second bitmask
     ((8, 8), 38, 250, 0, 2),          # more lists than fit at once: the same
+    ((2, 2), 1, 20000, 0, 2),         # a cluster per list, the neighbour kernel's bitmask behind it
 ])
 def test_a_replay_that_outgrows_its_reserve_is_reported(H, heads, batch, length, scope, radius):
     """A captured selection is replayed on sequences longer than the reserve it was sized for.  It selects among the
