@@ -105,8 +105,11 @@ __global__ void __launch_bounds__(kThreads, kU == 2 ? 2 : 1) select_small_kernel
     const int unit = blockIdx.x / C;
     // What needs nothing from the predecessor runs beside its tail.
     if (tid == 0) sm->n_cand = 0;
-    if (!kDirect && tid == 0) prefetch_tmap(&tmap);
-    if (!kDirect && tid < n_stages) mbar_init(&sm->full[tid], 1), fence_mbar_init();
+    if (!kDirect && warp == 0) {
+        if (lane == 0) prefetch_tmap(&tmap);
+        if (lane < n_stages) mbar_init(&sm->full[lane], 1), fence_mbar_init();   // (14 stages at most: 16 KB tiles)
+        __syncwarp();                                  // thread 0 arms them and requests the first tiles before any block barrier
+    }
     reinterpret_cast<int4*>(sm->hist)[tid] = make_int4(0, 0, 0, 0);
     int ll, s, h;
     decode_unit(gm, ut, unit, ll, s, h);
