@@ -317,7 +317,8 @@ tb_status tb_sync_lengths(tb_ctx* ctx, void* stream);
  * 256 rows without requesting the copy, so that this wait runs out: the way to exercise the path without
  * a fault, a trap or an unbounded wait.  It is honoured only by a launch of one block (one sequence, one
  * list, at most 1023 candidates: nothing else is in flight and no other block waits); any other selection
- * call then returns TB_ERR_UNSUPPORTED and launches nothing.  One-shot; -1 = none. */
+ * call then returns TB_ERR_UNSUPPORTED and launches nothing.  (A bf16 selection of this size waits for no copy otherwise:
+ * with the hook armed it runs as the kernel of larger selections does.)  One-shot; -1 = none. */
 tb_status tb_set_wait_diagnostics(tb_ctx* ctx, int32_t poll_limit, int32_t drop_tile);
 
 /* Algorithmic bytes (projected keys scanned + K/V rows gathered, upper bound from host-known sizes)

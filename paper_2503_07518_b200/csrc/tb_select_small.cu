@@ -84,7 +84,7 @@ struct NoStream {
 template <typename T, int DP, int RED, int kU, bool kShared>
 __global__ void __launch_bounds__(kThreads, kU == 2 ? 2 : 1) select_small_kernel(const __grid_constant__ CUtensorMap tmap,
                                                                                  const unsigned char* __restrict__ kimp, Geom gm, UnitTable ut,
-                                                                                 SelectArgs a, int n_stages, int max_tiles, int share_tiles, uint32_t wait_limit,
+                                                                                 SelectArgs a, int n_stages, int max_tiles, int share_tiles, uint32_t wait_limit, int drop_tile,
                                                                                  int32_t* __restrict__ state_idx, int32_t* __restrict__ state_cnt,
                                                                                  int32_t* __restrict__ status) {
     constexpr int RB = DP * Elem<T>::kBytes, NCH = RB / 16;
@@ -135,7 +135,8 @@ __global__ void __launch_bounds__(kThreads, kU == 2 ? 2 : 1) select_small_kernel
     auto request = [&](int t) {                        // tile t, into its stage
         uint64_t* bar = &sm->full[t % n_stages];
         mbar_arrive_expect_tx(bar, kTileBytes);
-        tma_load_2d(ring + t % n_stages * kTileBytes, &tmap, 0, (int)(row0 + (long long)t * kHalf), bar);
+        // drop_tile: diagnostics only (see tb_set_wait_diagnostics): the barrier is armed and the copy left out
+        if (t != drop_tile) tma_load_2d(ring + t % n_stages * kTileBytes, &tmap, 0, (int)(row0 + (long long)t * kHalf), bar);
     };
     if (!kDirect && tid == 0)
         for (int t = 0; t < min(n_stages, my_tiles); ++t) request(t);
@@ -320,8 +321,9 @@ size_t small_smem(int n_stages, int n_tiles, int tile_bytes) {
 // 6000 25.4 / 25.8 (16 dimensions 17.9 / 23.0), of 9500 level; 384 problems, a second wave: level or worse.  Neighbours and
 // the caller's copy come for next to nothing here and cost two more launches there (96 problems of 3000 with both: 8.3 / 18.4).
 bool select_small_takes(const tb_ctx* c, const UnitTable& ut, int max_cand, bool more) {
-    if (c->drop_tile >= 0) return false;               // wait diagnostics: see select_kernel
     const int n_units = ut.layer_count * ut.n_seq * c->geom.Hl;
+    // wait diagnostics: launches of one block that wait for copies (the others: see launch_select)
+    if (c->drop_tile >= 0 && (c->geom.dtype == TB_BF16 || n_units > 1 || max_cand > 1023)) return false;
     const int most = more || (n_units <= c->sm_count && 2 * n_units > c->sm_count) ? kMaxCand : n_units <= c->sm_count ? 10 * 1024 : 8 * 1024;
     return n_units <= 2 * c->sm_count && max_cand <= most;
 }
@@ -333,6 +335,8 @@ cudaError_t launch_select_small(const tb_ctx* c, const UnitTable& ut, const Sele
     const int tile_bytes = kHalf * gm.dp * (gm.dtype == TB_BF16 ? 2 : 4);
     const int n_tiles = max_cand > kHalf ? (max_cand + kHalf - 1) / kHalf : 1;
     const uint32_t wait_limit = c->wait_poll_limit > 0 ? (uint32_t)c->wait_poll_limit : kWaitPollLimit;
+    const int drop_tile = c->drop_tile;                // one-shot
+    const_cast<tb_ctx*>(c)->drop_tile = -1;
 
     // fp32: all tiles in flight at once if an SM's share of shared memory holds them, all of it when every block has an SM
     // to itself, half otherwise.
@@ -362,7 +366,7 @@ cudaError_t launch_select_small(const tb_ctx* c, const UnitTable& ut, const Sele
             cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
             if (e != cudaSuccess) return e;
         }
-        return cudaLaunchKernelEx(&cfg, kernel, c->kimp_map, (const unsigned char*)c->kimp, gm, ut, a, n_stages, n_tiles, share_tiles, wait_limit,
+        return cudaLaunchKernelEx(&cfg, kernel, c->kimp_map, (const unsigned char*)c->kimp, gm, ut, a, n_stages, n_tiles, share_tiles, wait_limit, drop_tile,
                                   c->st.idx, c->st.cnt, c->st.status);
     };
     // a block alone on its SM keeps four groups of rows in flight per warp, two blocks two each (their registers)

@@ -40,6 +40,27 @@ def test_bounded_wait_runs_out_and_the_context_stays_usable(H):
     assert np.abs(out[0, 0] - ref).max() <= 2e-3
 
 
+@pytest.mark.parametrize("dp,length,tile", [(32, 900, 1), (16, 1023, 3), (32, 513, 0)])
+def test_bounded_wait_of_a_small_fp32_selection(H, dp, length, tile):
+    """The same on the kernel that fp32 selections of this size run with and without the hook: the rows that never arrive
+    rank last, everything else is exact, and the next call is clean."""
+    b_ = tb()
+    w = wl.workload(1, n_layers=1, n_q_heads=2, n_kv_heads=1, imp_dim=dp, lengths=[length], budget=200, outlier_channels=0)
+    case = H.Case(w)
+    _, qi = H.queries(w)
+    p = b_.select_params(w.budget)
+    _, full, s = case.oracle_select(0, 0, 0, qi[0, 0], p)
+    case.ctx.set_wait_diagnostics(poll_limit=2000, drop_tile=tile)
+    lost = H.gpu_select(case, qi, p)
+    assert case.ctx.get_status() == b_.TB_ERR_TIMEOUT
+    there = s.copy()
+    there[tile * 256:(tile + 1) * 256] = -np.inf
+    H.check_selection(lost[0][0][0], H.orc.select(there, 0, 0, w.budget), there)
+    case.ctx.set_wait_diagnostics(0, -1)
+    H.check_selection(H.gpu_select(case, qi, p)[0][0][0], full, s)
+    assert case.ctx.get_status() == 0
+
+
 def test_wait_diagnostics_are_refused_by_multi_block_launches(H):
     """The hook never reaches a launch in which another block could be left waiting: such a call returns
     TB_ERR_UNSUPPORTED and launches nothing."""
