@@ -456,7 +456,6 @@ tb_status tb_select_topk(tb_ctx* c, int32_t lb, int32_t lc, const int32_t* seq_i
                 a.idx_copy = idx_out ? idx_out + unit_off * c->geom.idx_cap : nullptr, a.cnt_copy = cnt_out ? cnt_out + unit_off : nullptr;
                 a.q_imp = q_imp + (size_t)(l0 - lb) * n_seq * c->geom.Hl * c->geom.gl * c->cfg.imp_dim;
                 a.budget = p->budget, a.sinks = p->sinks, a.recent = p->recent, a.reduce = reduce;
-                a.room = (max_cand + 255) & ~255;
                 if (p->radius == 0) {
                     a.idx_dst = nullptr, a.cnt_dst = nullptr, a.dst_is_state = 1, a.idx_stride = c->geom.idx_cap;
                 } else {

@@ -59,7 +59,6 @@ struct SelectArgs {
     int radius, nmode;
     int32_t* idx_copy;    // [layer_count][n_seq][Hl][idx_cap] or NULL
     int32_t* cnt_copy;
-    int room;             // candidates that the launch's shared memory is sized for (whole groups of 256): see candidates_within
 };
 
 struct NeighborArgs {
@@ -67,7 +66,7 @@ struct NeighborArgs {
     const int32_t* cnt_src;
     int src_stride;
     int radius, nmode, sinks, recent;
-    int room;                // candidates that the bitmask on chip is sized for: see candidates_within
+    int room;                // candidates that the bitmask is sized for: see candidates_within
 };
 
 // Where an attended row is read from: the K|V cache, or one of two optional copies in device memory.

@@ -136,8 +136,8 @@ __device__ __forceinline__ void check_candidates_projected(const Geom& gm, const
 // Candidates of a problem whose kernel keeps something per candidate in shared memory.  A replayed graph may find a sequence
 // longer than its launch was sized for (it outgrew the declared reserve): the candidates past `room` are left out and the
 // status word says so.
-__device__ __forceinline__ int candidates_within(const UnitTable& ut, int n, int room, int32_t* status) {
-    if (!ut.use_dev_len || n <= room) return n;
+__device__ __forceinline__ int candidates_within(int n, int room, int32_t* status) {
+    if (n <= room) return n;
     if (threadIdx.x == 0) atomicExch(status, kStatusCapacity);
     return room;
 }

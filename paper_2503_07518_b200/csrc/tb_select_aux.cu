@@ -60,7 +60,7 @@ __global__ void __launch_bounds__(kNbThreads) neighbor_kernel(Geom gm, UnitTable
     decode_unit(gm, ut, blockIdx.x, ll, s, h);
     const int L = unit_len(gm, ut, ll, s);
     const int lo = min(a.sinks, L);
-    const int span = candidates_within(ut, max(lo, L - a.recent) - lo, a.room, status), hi = lo + span;
+    const int span = candidates_within(max(lo, L - a.recent) - lo, a.room, status), hi = lo + span;
     const int n_words = (span + 31) / 32;
     const int32_t* src = a.idx_src + (size_t)blockIdx.x * a.src_stride;
     const int cnt = a.cnt_src[blockIdx.x];

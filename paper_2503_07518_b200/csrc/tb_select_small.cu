@@ -121,7 +121,7 @@ __global__ void __launch_bounds__(kThreads, kU == 2 ? 2 : 1) select_small_kernel
     if constexpr (kShared) asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");    // every block of the cluster runs
     const int L = unit_len(gm, ut, ll, s);
     const int lo = min(a.sinks, L), hi = max(lo, L - a.recent);
-    const int ncand = candidates_within(ut, hi - lo, a.room, status), k = min(a.budget, ncand);
+    const int ncand = candidates_within(hi - lo, max_tiles * kHalf, status), k = min(a.budget, ncand);
     check_candidates_projected(gm, ut, ll, s, hi, status);
     if (k <= 0 || k == ncand) {                        // nothing to rank: none, or all (neighbours add nothing then)
         if (rank == 0) out.all<kThreads>(lo, k);

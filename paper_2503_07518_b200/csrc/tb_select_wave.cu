@@ -186,8 +186,8 @@ __device__ __forceinline__ bool wave_finish_mask(int* hist, WaveSmem* sm, const 
     const int mask_bytes = (n_words * 4 + 15) & ~15;
     uint32_t* mask = reinterpret_cast<uint32_t*>(scratch);
     uint2* list = reinterpret_cast<uint2*>(scratch + mask_bytes);
-    // bin 0 (everything below the sampled range) is too crowded to list
-    if (mask_bytes > scratch_bytes || (!exact && (bc > (scratch_bytes - mask_bytes) / 8 || bin == 0))) return false;
+    // bin 0 (everything below the sampled range) is too crowded to list; neighbours need a second mask
+    if ((out.radius > 0 ? 2 * mask_bytes : mask_bytes) > scratch_bytes || (!exact && (bc > (scratch_bytes - mask_bytes) / 8 || bin == 0))) return false;
     const uint32_t bin_base = dg.base + ((uint32_t)(bin - 1) << dg.shift);       // lowest key of the threshold bin
     const int bin_bits = bin == 2047 ? 32 : dg.shift;  // bits of (key - bin_base) inside the bin; the top bin is open-ended
     // Keys of the threshold bin: [bin_from, above_from); keys of the bins above it: [above_from, 2^32), if any.
@@ -310,7 +310,7 @@ __device__ __forceinline__ bool wave_finish_mask(int* hist, WaveSmem* sm, const 
     }
 
     FIN_MARK(2);
-    // (the list of the bin's keys is done with: neighbours are fetched into its place; the launcher has made room)
+    // (the list of the bin's keys is done with: neighbours are fetched into its place)
     finish_mask_list<kThreads>(mask, reinterpret_cast<uint32_t*>(scratch + mask_bytes), ncand, lo, out, sm->warp_a);
     FIN_MARK(3);
     return true;
@@ -444,21 +444,21 @@ __device__ __forceinline__ void wave_general(int* hist, WaveSmem* sm, const uint
 
 // The general path, then what is left to do with the list it wrote: neighbours (on a bitmask in `scratch`) and the copy.
 __device__ __forceinline__ void wave_general_finish(int* hist, WaveSmem* sm, const uint32_t* __restrict__ keys_unit, unsigned char* scratch,
-                                                    int scratch_bytes, int ncand, int k, int lo, const ListOut& out) {
+                                                    int scratch_bytes, int ncand, int k, int lo, const ListOut& out, int32_t* status) {
     wave_general(hist, sm, keys_unit, reinterpret_cast<uint4*>(scratch), scratch_bytes / 16, ncand, k, lo, out.idx, out.cnt);
     if (out.radius == 0 && !out.idx_copy && !out.cnt_copy) return;
     __syncthreads();                                   // the block sees its own list
     if (out.radius > 0) {
-        const int n_words = (ncand + 31) / 32;
+        const int n = candidates_within(ncand, scratch_bytes / 64 * 256, status), n_words = (n + 31) / 32;    // two bitmasks
         uint32_t* mask = reinterpret_cast<uint32_t*>(scratch);
         for (int i = threadIdx.x; i < n_words; i += kThreads) mask[i] = 0u;
         __syncthreads();
         for (int i = threadIdx.x; i < k; i += kThreads) {
             const int p = out.idx[i] - lo;
-            atomicOr(&mask[p >> 5], 1u << (p & 31));
+            if (p < n) atomicOr(&mask[p >> 5], 1u << (p & 31));
         }
         __syncthreads();
-        finish_mask_list<kThreads>(mask, mask + ((n_words + 3) & ~3), ncand, lo, out, sm->warp_a);
+        finish_mask_list<kThreads>(mask, mask + ((n_words + 3) & ~3), n, lo, out, sm->warp_a);
         return;
     }
     for (int i = threadIdx.x; i < k; i += kThreads)
@@ -487,7 +487,7 @@ __global__ void __launch_bounds__(kThreads, 4)
     const int L = unit_len(gm, ut, ll, s);
     const int lo = min(a.sinks, L);
     const int hi = max(lo, L - a.recent);
-    const int ncand = a.radius > 0 ? candidates_within(ut, hi - lo, a.room, status) : hi - lo;   // (the bitmasks of neighbour fetching)
+    const int ncand = hi - lo;
     const int k = min(a.budget, ncand);
     check_candidates_projected(gm, ut, ll, s, hi, status);
     const size_t cu = list_unit(gm, ut, ll, s, h);
@@ -617,7 +617,7 @@ __global__ void __launch_bounds__(kThreads, 4)
 
     // ---- finish -----------------------------------------------------------------------------------
     if (!wave_finish_mask(hist, sm, dg, keys_unit, stage_base, n_stages * (int)kTileBytes, ncand, k, lo, out))
-        wave_general_finish(hist, sm, keys_unit, stage_base, n_stages * (int)kTileBytes, ncand, k, lo, out);
+        wave_general_finish(hist, sm, keys_unit, stage_base, n_stages * (int)kTileBytes, ncand, k, lo, out, status);
     wave_stamp(3);
 }
 
@@ -660,8 +660,7 @@ __global__ void __launch_bounds__(kThreads, 2)
     const int tid = threadIdx.x, lane = tid & 31, gid = lane >> 2, tig = lane & 3;
     const int pair = order.pair[blockIdx.x / gm.Hl], h = blockIdx.x % gm.Hl, rank = h % g;
     const int ll = pair / ut.n_seq, s = pair % ut.n_seq;
-    const int L = unit_len(gm, ut, ll, s), lo = min(a.sinks, L), hi = max(lo, L - a.recent);
-    const int ncand = a.radius > 0 ? candidates_within(ut, hi - lo, a.room, status) : hi - lo, k = min(a.budget, ncand);   // (the bitmasks)
+    const int L = unit_len(gm, ut, ll, s), lo = min(a.sinks, L), hi = max(lo, L - a.recent), ncand = hi - lo, k = min(a.budget, ncand);
     check_candidates_projected(gm, ut, ll, s, hi, status);
     const size_t cu = list_unit(gm, ut, ll, s, h);
     const ListOut out(gm, a, cu, pair * gm.Hl + h, state_idx, state_cnt);
@@ -799,7 +798,7 @@ __global__ void __launch_bounds__(kThreads, 2)
     const uint32_t* keys_unit = keys0 + rank * key_pitch;
     const Digit dg = sm->digit[rank];
     if (!wave_finish_mask(mine, &sm->w, dg, keys_unit, scratch, scratch_bytes, ncand, k, lo, out))
-        wave_general_finish(mine, &sm->w, keys_unit, scratch, scratch_bytes, ncand, k, lo, out);
+        wave_general_finish(mine, &sm->w, keys_unit, scratch, scratch_bytes, ncand, k, lo, out, status);
     asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");            // this block's histograms stay until they have been read
 }
 
