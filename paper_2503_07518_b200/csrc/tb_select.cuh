@@ -151,13 +151,44 @@ __device__ __forceinline__ int candidates_within(int n, int room, int32_t* statu
 // all 24 bits of the fp32 query, lowest term first, so every product is exact and only the fp32 sums round (against fp64:
 // rms error 1.4e-8 of sum |q k|, where the FMA chains above have 2.0e-8).  TB_GROUP_SUM: all eight columns hold the summed
 // query and a lane keeps the value that belongs to its row; TB_GROUP_MAX: column = head, a row's score is the largest over
-// the columns.  A row's score depends only on its bytes, never on where it sits.
+// the columns.  A row's score depends only on its bytes, never on where it sits.  Infinities do not survive the split (a
+// query's lower terms are zero or of either sign: inf * 0, inf - inf): rows with an infinite score are scored again, by the
+// FMA chains, behind the stream (rescore).  The kernels look for them only where a sum over the scores, or a query, is not
+// finite.
 constexpr int kQueryFrags = 3 * 2 * 32;   // a query's B fragments: terms x steps x lanes
 
 __device__ __forceinline__ void mma_16816(float (&d)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0, uint32_t b1) {
     asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
                  : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
                  : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
+}
+
+__device__ __forceinline__ bool is_finite(float s) { return fabsf(s) <= 3.402823466e38f; }
+// row_score / row_score_max of one bf16 row in global memory, from the staged queries: kept small, it hardly ever runs.
+template <int DP, int RED>
+__device__ __forceinline__ float rescore(const unsigned char* row, const float* qs, int g) {
+    float best = -INFINITY;
+    const int n = RED == TB_GROUP_MAX ? g : 1, per = RED == TB_GROUP_MAX ? 1 : g;   // scores of a row, queries summed for each
+#pragma unroll 1
+    for (int u = 0; u < n; ++u) {
+        float acc = 0.f, other = 0.f;                  // this chunk's chain and the other one's
+#pragma unroll 1
+        for (int c = 0; c < DP / 8; ++c) {
+            float f[8];
+            Elem<__nv_bfloat16>::unpack16(__ldcg(reinterpret_cast<const uint4*>(row) + c), f);
+#pragma unroll
+            for (int e = 0; e < 8; ++e) {
+                float q = 0.f;
+#pragma unroll 1
+                for (int i = 0; i < per; ++i) q += qs[(u + i) * DP + c * 8 + e];
+                acc = fmaf(q, f[e], acc);
+            }
+            const float t = acc;
+            acc = other, other = t;
+        }
+        best = RED == TB_GROUP_MAX ? fmaxf(best, acc + other) : acc + other;
+    }
+    return best;
 }
 
 template <int DP, int RED>
@@ -187,7 +218,9 @@ struct FragScorer {
                 }
 #pragma unroll
                 for (int t = 0; t < kTerms; ++t) {
-                    const __nv_bfloat162 v = __floats2bfloat162_rn(x, y);
+                    // (a finite value does not become an infinity: above the largest bf16 it takes that one first)
+                    const float top = 3.38953139e38f;
+                    const __nv_bfloat162 v = __floats2bfloat162_rn(is_finite(x) ? fminf(fmaxf(x, -top), top) : x, is_finite(y) ? fminf(fmaxf(y, -top), top) : y);
                     b[t][half] = *reinterpret_cast<const uint32_t*>(&v);
                     x -= __low2float(v), y -= __high2float(v);
                 }
@@ -270,6 +303,13 @@ struct RowStream {
             const float sc = scorer.score(piece, row0, slot);
             return [=, &consume] { if (slot < n) consume(slot, sc); };
         });
+    }
+    // f(slot) for every row that run() gives to this thread
+    template <typename F>
+    __device__ __forceinline__ void own_rows(F&& f) const {
+        const int lane = threadIdx.x & 31;
+#pragma unroll 1
+        for (int slot = warp * 32 + (lane >> 2) + 8 * (lane & 3); slot < n; slot += n_warps * 32) f(slot);
     }
     // f(pieces, first row) for every group of 32; what it returns is called once the group's successor has been requested
     template <typename F>

@@ -143,7 +143,7 @@ __global__ void __launch_bounds__(kThreads, kU == 2 ? 2 : 1) select_small_kernel
     if (tid < gm.gl * DP) sm->qs[tid] = a.q_imp[query_row(gm, ut, ll, s, h) * DP + tid];
     typename std::conditional<kDirect, RowStream<DP, RED, kDirect ? kU : 1>, NoStream>::type rs;
     rs.start(kimp + row0 * RB, n_local);
-    __syncthreads();
+    const bool odd_query = __syncthreads_or(kDirect && tid < gm.gl * DP && !is_finite(sm->qs[tid]));   // (its own element)
 
     // ---- stream ------------------------------------------------------------------------------------
     float s1 = 0.f, s2 = 0.f;
@@ -164,6 +164,11 @@ __global__ void __launch_bounds__(kThreads, kU == 2 ? 2 : 1) select_small_kernel
         FragScorer<DP, RED> scorer;
         scorer.load_staged(sm->qs, gm.gl, sm->frags);
         rs.run(scorer, keep);
+        if (odd_query || !is_finite(s1))               // infinite scores, or scores dropped beside an infinite query (see FragScorer)
+            rs.own_rows([&](int slot) {
+                const float sc = rescore<DP, RED>(rs.rows + (size_t)slot * RB, sm->qs, gm.gl);
+                if (!is_finite(sc)) put_key(slot, order_key(sc));
+            });
     } else {
         // The two halves of the block take tiles in turn; the number of stages is even when stages are used again, so that
         // a stage belongs to one half (its barrier's phases are then waited for in order).  A wait that runs out

@@ -646,6 +646,28 @@ struct __align__(16) SharedSmem {
     alignas(16) unsigned char rows[kSampleRows * 64];
 };
 
+// The rows of a thread that have an infinite score for some list, by the FMA chains (see FragScorer): the keys parked and the
+// histograms counted for them are put right.
+template <int DP>
+__device__ __noinline__ void shared_rescore(SharedSmem* sm, int* hist, const unsigned char* rows, uint32_t* keys, int g, int n_local, size_t key_pitch) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, gid = lane >> 2, tig = lane & 3;
+    const bool halves = g <= 4;                        // the rows and lists of a lane: see the stream
+    const int u0 = 2 * (halves ? tig & 1 : tig);
+    for (int i = 0; i < (n_local + kThreads - 1) / kThreads * 4; ++i) {        // a warp's groups of 32 rows, in quarters
+        const int in = 8 * (i & 3) + gid, slot = ((i >> 2) * kWarps + warp) * 32 + in;
+        if (slot >= n_local || (halves && (in >> 4) != tig >> 1)) continue;
+        for (int u = u0; u < min(u0 + 2, g); ++u) {
+            const float sc = rescore<DP, TB_GROUP_SUM>(rows + (size_t)slot * DP * 2, sm->qs + u * DP, 1);
+            if (is_finite(sc)) continue;
+            uint32_t* at = keys + u * key_pitch + slot;                        // (this thread's own store)
+            const uint32_t key = order_key(sc);
+            atomicAdd(hist + u * kDigitBins + sm->digit[u].bin(__ldcg(at)), -1);
+            atomicAdd(hist + u * kDigitBins + sm->digit[u].bin(key), 1);
+            *at = key;
+        }
+    }
+}
+
 template <int DP>
 __global__ void __launch_bounds__(kThreads, 2)
     select_shared_kernel(const unsigned char* __restrict__ kimp, Geom gm, UnitTable ut, WaveOrder order, SelectArgs a, int scratch_bytes, int keep_in_l2,
@@ -687,7 +709,7 @@ __global__ void __launch_bounds__(kThreads, 2)
     Stream rs;
     rs.start(stream + (size_t)slot0 * RB, n_local);
     for (int i = tid; i < g * kDigitBins; i += kThreads) hist[i] = 0;
-    __syncthreads();
+    const bool odd_query = __syncthreads_or(tid < g * DP && !is_finite(sm->qs[tid]));   // (its own element)
     typename Stream::Scorer scorer;
     scorer.load_staged(sm->qs, g, sm->frags);
 
@@ -741,6 +763,7 @@ __global__ void __launch_bounds__(kThreads, 2)
         uint32_t* keys[2];
         int* bins[2];
         DigitCounter counter[2];
+        float sum = 0.f;                               // of a list's scores of every row: an infinite key is infinite to all lists
 #pragma unroll
         for (int e = 0; e < 2; ++e) {
             const int u = min(u0 + e, g - 1);
@@ -757,6 +780,7 @@ __global__ void __launch_bounds__(kThreads, 2)
             struct { float d[2][4]; } x;
             scorer.columns(v, x.d);
             return [&, x, row0] {
+                sum += (x.d[0][0] + x.d[0][2]) + (x.d[1][0] + x.d[1][2]);
                 if (halves) {
                     const int base = row0 + 16 * (tig >> 1) + gid;
 #pragma unroll
@@ -775,6 +799,7 @@ __global__ void __launch_bounds__(kThreads, 2)
 #pragma unroll
         for (int e = 0; e < 2; ++e)                    // (lanes of a warp count for different lists)
             if (u0 + e < g && counter[e].below) atomicAdd(bins[e], counter[e].below);
+        if (odd_query || !is_finite(sum)) shared_rescore<DP>(sm, hist, rs.rows, keys0 + slot0, g, n_local, key_pitch);
     }
     asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
 

@@ -125,3 +125,40 @@ def test_lists_that_share_a_key_stream(H, q_heads, kv_heads, dp):
                 for h in range(q_heads):
                     _, full, _ = case.oracle_select(0, b, h, ties[0, b], p)
                     assert np.array_equal(lists[0][b][h], full)
+
+
+@pytest.mark.parametrize("dp", [16, 32])
+@pytest.mark.parametrize("scope,reduce,lengths", [(0, 0, [700, 40]), (0, 1, [700, 300]), (0, 0, [3000]), (1, 0, [700]), (1, 0, [12001, 700])])
+def test_infinite_scores_rank_as_infinities(H, scope, reduce, lengths, dp):
+    """A projected key or a query that overflowed to an infinity gives infinite scores: last or first in the ranking, equal
+    ones by position, whichever kernel ranks them.  (No term of a score is inf * 0 here, no sum inf - inf.)"""
+    w = wl.workload(2, n_layers=1, n_q_heads=8, n_kv_heads=2, imp_dim=dp, batch=len(lengths), lengths=lengths, budget=max(lengths) - 30)
+    case = H.Case(w, list_scope=scope)
+    _, qi = H.queries(w)
+    qi = np.abs(qi) + np.float32(0.01)                 # the key's sign is the infinity's; three bf16 terms, some of them negative
+    r = np.random.Generator(np.random.PCG64(3))
+    for b, L in enumerate(lengths):
+        x = wl.storage_to_f32(case.Kimp[0][b][:, :L], w.dtype).copy()
+        x[x == 0] = 1.0
+        for h in range(2):
+            rows = r.permutation(L)[:L // 5 + 2]
+            x[h, rows, r.integers(0, dp, rows.size)] = np.where(np.arange(rows.size) % 7 == 0, np.inf, -np.inf)
+        case.Kimp[0][b][:, :L] = wl.to_storage(x.astype(np.float32), w.dtype)
+        case.ctx.kimp[0, b, :, :L] = H.to_dev(case.Kimp[0][b][:, :L], w.dtype)
+    heads = np.arange(8) % 4 == 2                      # one head of a group asks for an infinity in a channel of its own
+    for queries in (qi, np.where(heads[None, None, :, None] & (np.arange(dp) == 3), np.float32(np.inf), qi)):
+        if not np.isfinite(queries).all():             # ... of keys that are finite and not zero
+            for b, L in enumerate(lengths):
+                x = r.standard_normal((2, L, dp)).astype(np.float32)
+                x[np.abs(x) < 0.01] = 1.0
+                case.Kimp[0][b][:, :L] = wl.to_storage(x, w.dtype)
+                case.ctx.kimp[0, b, :, :L] = H.to_dev(case.Kimp[0][b][:, :L], w.dtype)
+        for budget in (5, min(lengths) // 2, w.budget):
+            p = tb().select_params(budget, reduce=reduce)
+            lists = H.gpu_select(case, queries, p)
+            assert case.ctx.get_status() == 0
+            for b in range(w.batch):
+                for h in range(case.Hl):
+                    _, full, s = case.oracle_select(0, b, h, queries[0, b], p)
+                    assert not np.isnan(s).any()
+                    H.check_selection(lists[0][b][h], full, s)
