@@ -227,7 +227,8 @@ __global__ void __launch_bounds__(kPredThreads) predictor_out_kernel(const T* __
 // ---- bf16: both linears on the tensor cores, weights as the left operand ------------------------------
 // D[32 weight rows x tokens] += W[32 x K] . X[K x tokens] with mma.sync.m16n8k16: the weights are exact in bf16, and
 // the fp32 right operand (scaled hidden states, resp. hidden units) is split into bf16 terms, one MMA each, accumulated
-// in fp32: three terms, which hold all 24 bits of it, for up to four tokens, two (16 bits) for more.  A block's work is 32 weight rows x 512 channels -- 32 KB of
+// in fp32: three terms, which hold all 24 bits of it, for up to four tokens and for odd shapes (in groups of eight tokens),
+// two (16 bits) for the rest.  A block's work is 32 weight rows x 512 channels -- 32 KB of
 // weights, about what an SM receives in a memory latency, so that an 8B-shaped linear (8 MB) is 128 blocks that
 // request everything they need at once -- against all tokens of the call.  The tensor pipe is idle most of the time
 // and latency is what there is to save: every thread's weights are in flight before it looks at the tokens.
@@ -652,7 +653,9 @@ extern "C" tb_status tb_predict_importance_queries(const tb_predictor* p, const 
         };
         const int groups = (n_tokens + kTileTokMax - 1) / kTileTokMax, n8 = ((n_tokens + groups - 1) / groups + 7) / 8;
         using std::integral_constant;
-        if (n_tokens < 5) e = launch(integral_constant<int, 3>{}, integral_constant<int, 1>{});
+        // 24 bits of both right operands for up to four tokens, and for shapes off the 32-channel runs (always computed so)
+        const bool whole = n_tokens < 5 || p->model_dim % 32 || p->hidden_dim % 32 || n_out % 8;
+        if (whole) e = launch(integral_constant<int, 3>{}, integral_constant<int, 1>{});
         else if (n8 == 1) e = launch(integral_constant<int, 2>{}, integral_constant<int, 1>{});
         else if (n8 == 2) e = launch(integral_constant<int, 2>{}, integral_constant<int, 2>{});
         else if (n8 == 3) e = launch(integral_constant<int, 2>{}, integral_constant<int, 3>{});

@@ -512,6 +512,23 @@ def test_predictor_tile_edges(H, tokens):
         assert np.abs(q.cpu().numpy() - want).max() <= 4e-5, (E, hid, np.abs(q.cpu().numpy() - want).max())
 
 
+@pytest.mark.parametrize("E,hid,slots,heads,dp", [(72, 8, 1, 1, 16), (4872, 512, 1, 3, 32), (1024, 1032, 2, 1, 16), (520, 24, 3, 3, 12)])
+def test_predictor_odd_shapes_keep_all_bits_of_many_tokens(H, E, hid, slots, heads, dp):
+    """bf16 channel or unit counts off the 32-wide runs: every token of a batch as accurate as it is alone -- the same bits."""
+    tokens = 21
+    w = wl.workload(2, batch=tokens, n_q_heads=heads, n_kv_heads=1, imp_dim=dp)
+    dev = [H.to_dev(a, w.dtype) for a in wl.gen_predictor(w, 1, model_dim=E, hidden_dim=hid, slots=slots)]
+    scratch = torch.empty(tokens * hid, dtype=torch.float32, device="cuda")
+    q = torch.full((slots, tokens, heads, dp), float("nan"), dtype=torch.float32, device="cuda")
+    one = torch.full((slots, 1, heads, dp), float("nan"), dtype=torch.float32, device="cuda")
+    for n in (5, 8, 9, tokens):
+        out = q.view(-1)[:slots * n * heads * dp].view(slots, n, heads, dp)
+        assert tb().predict_importance_queries(dev[0][:n], *dev[1:], w.dtype, heads, slots, dp, scratch, out) == tb().TB_OK
+        for t in range(n):
+            assert tb().predict_importance_queries(dev[0][t:t + 1].clone(), *dev[1:], w.dtype, heads, slots, dp, scratch, one) == tb().TB_OK
+            assert torch.equal(out[:, t], one[:, 0]), (n, t)
+
+
 def test_predictor_output_feeds_selection(H):
     """The predictor's output block is the q_imp argument of tb_select_topk for its consumer layers:
     selecting with it on the GPU equals selecting with the oracle's queries in the oracle."""
