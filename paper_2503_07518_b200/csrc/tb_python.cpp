@@ -13,6 +13,7 @@
 
 #include <ATen/core/Tensor.h>
 #include <c10/cuda/CUDAStream.h>
+#include <torch/csrc/Exceptions.h>
 #include <torch/csrc/autograd/python_variable.h>
 
 #include <cstdint>
@@ -25,7 +26,8 @@ namespace {
 PyObject* g_data_ptr;        // "data_ptr"
 PyObject* g_cuda_stream;     // "cuda_stream"
 
-// Each reader returns false with a Python exception set.
+// Each reader returns false with a Python exception set, or throws what torch throws (a tensor without storage, no
+// device): guarded() makes that a Python exception.
 
 bool read_pointer(PyObject* o, void** out) {      // a tensor, or None
     *out = nullptr;
@@ -211,7 +213,14 @@ PyObject* predict_importance_queries(PyObject*, PyObject* const* a, Py_ssize_t n
     return call([&] { return tb_predict_importance_queries(&p, hidden, n_tok, (float*)scratch, (float*)q_imp, stream); });
 }
 
-#define TB_METHOD(name) {#name, (PyCFunction)(void (*)(void))name, METH_FASTCALL, nullptr}
+template <PyObject* (*f)(PyObject*, PyObject* const*, Py_ssize_t)>
+PyObject* guarded(PyObject* self, PyObject* const* a, Py_ssize_t n) {
+    HANDLE_TH_ERRORS
+    return f(self, a, n);
+    END_HANDLE_TH_ERRORS
+}
+
+#define TB_METHOD(name) {#name, (PyCFunction)(void (*)(void))guarded<name>, METH_FASTCALL, nullptr}
 PyMethodDef methods[] = {TB_METHOD(append_kv), TB_METHOD(project_keys), TB_METHOD(select_topk), TB_METHOD(sparse_decode_attention),
                          TB_METHOD(predict_importance_queries), {nullptr, nullptr, 0, nullptr}};
 PyModuleDef module = {PyModuleDef_HEAD_INIT, "_tokenbutler", nullptr, -1, methods, nullptr, nullptr, nullptr, nullptr};

@@ -3,6 +3,7 @@ public header declares (no compute calls here)."""
 import ctypes
 import os
 import re
+import sys
 
 import pytest
 
@@ -84,3 +85,20 @@ def test_extension_module_unpacks_like_ctypes(libpath):
                 (None, "0", 1, None, 1, None, p, None, None, s), (None, 0, 1, None, 1, None, p, None, None)):
         with pytest.raises((TypeError, ValueError)):
             b._calls.select_topk(*bad)
+
+
+@pytest.mark.parametrize("call", [
+    "append_kv(None, 0, 1, None, [1], sparse, None, s)",
+    "select_topk(None, 0, 1, None, 1, sparse, p, None, None, s)",
+    "project_keys(None, 0, 1, None, [0], [1], 1, None)",                       # the current stream of no device
+    "predict_importance_queries(0, 1, 1, 16, 0, 1e-5, sparse, None, m, None, m, None, None, s)",
+    "predict_importance_queries(0, 1, 1, 16, 0, 1e-5, None, None, m, None, m[0], None, None, s)",   # no second size
+])
+def test_what_torch_throws_is_a_python_exception(libpath, call):
+    import subprocess
+    code = ("import torch\nfrom paper_2503_07518_b200 import binding as b\nb.lib()\n"
+            "sparse, m = torch.eye(3).to_sparse(), torch.zeros(4, 8)\n"
+            "p, s = b.select_params(4), type('Stream', (), {'cuda_stream': 0})()\n"
+            "try:\n    b._calls.%s\nexcept Exception as e:\n    print('raised', type(e).__name__)" % call)
+    r = subprocess.run([sys.executable, "-c", code], cwd=ROOT, env=dict(os.environ, CUDA_VISIBLE_DEVICES=""), capture_output=True, text=True)
+    assert r.returncode == 0 and "raised" in r.stdout, (r.returncode, r.stdout, r.stderr[-300:])
