@@ -25,6 +25,7 @@ namespace {
 
 PyObject* g_data_ptr;        // "data_ptr"
 PyObject* g_cuda_stream;     // "cuda_stream"
+PyObject* g_shape;           // "shape"
 
 // Each reader returns false with a Python exception set, or throws what torch throws (a tensor without storage, no
 // device): guarded() makes that a Python exception.
@@ -184,27 +185,38 @@ PyObject* sparse_decode_attention(PyObject*, PyObject* const* a, Py_ssize_t n) {
     });
 }
 
+// A tensor (or whatever else has a shape and says where it is) and its leading sizes; `cols` may be null.
 bool read_matrix(PyObject* o, void** out, int32_t* rows, int32_t* cols) {
-    if (!THPVariable_Check(o) || THPVariable_Unpack(o).dim() != 2) {
-        PyErr_SetString(PyExc_TypeError, "a two-dimensional tensor is expected");
-        return false;
+    int32_t* sizes[2] = {rows, cols};
+    if (THPVariable_Check(o) && THPVariable_Unpack(o).dim() >= (cols ? 2 : 1)) {
+        const at::Tensor& t = THPVariable_Unpack(o);
+        *out = t.data_ptr();
+        for (int i = 0; i < (cols ? 2 : 1); ++i) *sizes[i] = (int32_t)t.size(i);
+        return true;
     }
-    const at::Tensor& t = THPVariable_Unpack(o);
-    *out = t.data_ptr(), *rows = (int32_t)t.size(0), *cols = (int32_t)t.size(1);
-    return true;
+    PyObject* shape = PyObject_GetAttr(o, g_shape);
+    if (!shape) return false;
+    bool ok = true;
+    for (int i = 0; i < (cols ? 2 : 1) && ok; ++i) {
+        PyObject* n = PySequence_GetItem(shape, i);    // (an IndexError where there are fewer)
+        ok = n && read_int(n, sizes[i]);
+        Py_XDECREF(n);
+    }
+    Py_DECREF(shape);
+    return ok && o != Py_None && read_pointer(o, out);
 }
 
 // (dtype, n_q_heads, n_slots, imp_dim, activation, ln_eps, ln_weight, ln_bias, w1, w2, hidden, scratch, q_imp, stream)
 PyObject* predict_importance_queries(PyObject*, PyObject* const* a, Py_ssize_t n) {
     tb_predictor p;
     void *lw, *lb, *w1, *w2, *hidden, *scratch, *q_imp, *stream;
-    int32_t n_tok, w1_cols;
+    int32_t n_tok;
     if (!want(n, 14) || !read_int(a[0], &p.dtype) || !read_int(a[1], &p.n_q_heads) || !read_int(a[2], &p.n_slots) ||
         !read_int(a[3], &p.imp_dim) || !read_int(a[4], &p.activation))
         return nullptr;
     const double eps = PyFloat_AsDouble(a[5]);
     if (eps == -1.0 && PyErr_Occurred()) return nullptr;
-    if (!read_pointer(a[6], &lw) || !read_pointer(a[7], &lb) || !read_matrix(a[8], &w1, &p.hidden_dim, &w1_cols) || !read_pointer(a[9], &w2) ||
+    if (!read_pointer(a[6], &lw) || !read_pointer(a[7], &lb) || !read_matrix(a[8], &w1, &p.hidden_dim, nullptr) || !read_pointer(a[9], &w2) ||
         !read_matrix(a[10], &hidden, &n_tok, &p.model_dim) || !read_pointer(a[11], &scratch) || !read_pointer(a[12], &q_imp) ||
         !read_stream(a[13], &stream))
         return nullptr;
@@ -230,6 +242,7 @@ PyModuleDef module = {PyModuleDef_HEAD_INIT, "_tokenbutler", nullptr, -1, method
 PyMODINIT_FUNC PyInit__tokenbutler(void) {
     g_data_ptr = PyUnicode_InternFromString("data_ptr");
     g_cuda_stream = PyUnicode_InternFromString("cuda_stream");
-    if (!g_data_ptr || !g_cuda_stream) return nullptr;
+    g_shape = PyUnicode_InternFromString("shape");
+    if (!g_data_ptr || !g_cuda_stream || !g_shape) return nullptr;
     return PyModule_Create(&module);
 }

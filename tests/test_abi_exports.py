@@ -102,3 +102,22 @@ def test_what_torch_throws_is_a_python_exception(libpath, call):
             "try:\n    b._calls.%s\nexcept Exception as e:\n    print('raised', type(e).__name__)" % call)
     r = subprocess.run([sys.executable, "-c", code], cwd=ROOT, env=dict(os.environ, CUDA_VISIBLE_DEVICES=""), capture_output=True, text=True)
     assert r.returncode == 0 and "raised" in r.stdout, (r.returncode, r.stdout, r.stderr[-300:])
+
+
+def test_predictor_binding_takes_what_has_a_shape(libpath):
+    """Sizes are read from the leading dimensions of tensors of any rank, and of other objects with a shape and a data_ptr()."""
+    import torch
+    from paper_2503_07518_b200 import binding as b
+
+    class Where:
+        def __init__(self, t):
+            self.shape, self.data_ptr = t.shape, t.data_ptr
+
+    t = torch.zeros(64, 64)
+    s = type("Stream", (), {"cuda_stream": 0})()
+    call = lambda hidden, w1: b.predict_importance_queries(hidden, t, t, w1, t, b.TB_F32, 1, 1, 16, t, t, ln_eps=-1.0, stream=s)  # noqa: E731
+    for hidden, w1 in ((t, t), (t.view(64, 64, 1), t.view(64, 8, 8)), (t, t.view(-1)), (Where(t), Where(t))):
+        assert call(hidden, w1) == b.TB_ERR_INVALID_ARG            # the library's answer to a negative epsilon
+    for hidden in (t.view(-1), None, 3):
+        with pytest.raises((IndexError, AttributeError, TypeError)):
+            call(hidden, t)
