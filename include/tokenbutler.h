@@ -172,7 +172,10 @@ tb_status tb_score_tokens(tb_ctx* ctx, int32_t layer, const int32_t* seq_ids, in
  * the stored lists stay (stale reuse).  Otherwise, per (layer, sequence, list): candidates are
  * positions [min(S,L), max(min(S,L), L-W)); the `budget` highest scores are kept (all candidates if
  * fewer), equal scores resolved toward the LOWER position, -0.0 == +0.0; the list is expanded by the
- * neighbour rule, clipped to the candidates, and stored ascending in the context.
+ * neighbour rule, clipped to the candidates, and stored ascending in the context.  Scores are fp32 sums of exact (bf16) or
+ * fp32 products; the order of summation depends on the sizes of the call (candidates, lists, radius), so tokens whose scores
+ * agree to fp32 rounding may rank either way between calls of other sizes, or than tb_score_tokens' values would; tokens with
+ * the same key bytes always tie.  Whether the copies below are asked for changes nothing.
  * q_imp_dev: [layer_count][n_seq][Hq][d'] fp32 ([..][1][d'] under TB_SCOPE_LAYER).  idx_out_dev /
  * cnt_out_dev (optional, may be NULL): copies of the stored lists, [layer_count][n_seq][Hl][tb_index_capacity()]
  * and [..][Hl].

@@ -324,12 +324,14 @@ size_t small_smem(int n_stages, int n_tiles, int tile_bytes) {
 // 7.7 / 9.5, 8000 11.4 / 12.7, 12000 13.2 / 12.6 (eight blocks per problem bring more SMs there); 96 problems of 2000 7.3 /
 // 10.2, 9500 19.4 / 20.9, 16000 28.9 / 29.1, at 16 dimensions 14.9 / 17.3 and 23.4 / 24.5; two per SM: 192 of 2000 level, of
 // 6000 25.4 / 25.8 (16 dimensions 17.9 / 23.0), of 9500 level; 384 problems, a second wave: level or worse.  Neighbours and
-// the caller's copy come for next to nothing here and cost two more launches there (96 problems of 3000 with both: 8.3 / 18.4).
-bool select_small_takes(const tb_ctx* c, const UnitTable& ut, int max_cand, bool more) {
+// the caller's copy come for next to nothing here and cost two more launches there (96 problems of 3000 with both: 8.3 / 18.4),
+// so neighbours raise the limit.  A copy does not: the scores are summed in another order here, and an output that the caller
+// may leave out must not decide which of two tokens within fp32 rounding of one another is stored.
+bool select_small_takes(const tb_ctx* c, const UnitTable& ut, int max_cand, bool neighbours) {
     const int n_units = ut.layer_count * ut.n_seq * c->geom.Hl;
     // wait diagnostics: launches of one block that wait for copies (the others: see launch_select)
     if (c->drop_tile >= 0 && (c->geom.dtype == TB_BF16 || n_units > 1 || max_cand > 1023)) return false;
-    const int most = more || (n_units <= c->sm_count && 2 * n_units > c->sm_count) ? kMaxCand : n_units <= c->sm_count ? 10 * 1024 : 8 * 1024;
+    const int most = neighbours || (n_units <= c->sm_count && 2 * n_units > c->sm_count) ? kMaxCand : n_units <= c->sm_count ? 10 * 1024 : 8 * 1024;
     return n_units <= 2 * c->sm_count && max_cand <= most;
 }
 

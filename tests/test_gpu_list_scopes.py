@@ -162,3 +162,29 @@ def test_infinite_scores_rank_as_infinities(H, scope, reduce, lengths, dp):
                     _, full, s = case.oracle_select(0, b, h, queries[0, b], p)
                     assert not np.isnan(s).any()
                     H.check_selection(lists[0][b][h], full, s)
+
+
+@pytest.mark.parametrize("n_heads,batch,length", [(4, 1, 12000), (8, 2, 10300), (8, 20, 9000), (8, 10, 12000), (2, 1, 3000)])
+def test_asking_for_the_lists_does_not_change_them(H, n_heads, batch, length):
+    """Keys that are permutations of one another under a query of equal entries: exact scores tie, fp32 sums differ in their
+    last bits by the order of summation.  The stored list has to be the same whether a copy is asked for or not."""
+    dp = 32
+    ctx = tb().Context(1, n_heads, n_heads, 128, dp, tb().TB_BF16, batch, length, 500)
+    zeros = torch.zeros(batch * length, n_heads, 128, dtype=torch.bfloat16, device="cuda")
+    ctx.append_kv(0, 1, None, [length] * batch, zeros, zeros)
+    ctx.project_keys(0, 1, None, [0] * batch, [length] * batch)
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(11)
+    row = torch.randn(dp, generator=gen, device="cuda").to(torch.bfloat16)
+    perm = torch.rand(ctx.kimp.shape, generator=gen, device="cuda").argsort(-1)
+    ctx.kimp.copy_(row[perm])
+    q = torch.full((1, batch, n_heads, dp), 1.0 / 3.0, device="cuda")
+    idx = torch.zeros(2, 1, batch, n_heads, ctx.index_capacity, dtype=torch.int32, device="cuda")
+    cnt = torch.zeros(2, 1, batch, n_heads, dtype=torch.int32, device="cuda")
+    refresh, stored = tb().select_params(500, interval=2), tb().select_params(500, interval=2, step=1)
+    ctx.select_topk(0, 1, None, batch, q, refresh)
+    ctx.select_topk(0, 1, None, batch, q, stored, idx[0], cnt[0])
+    ctx.select_topk(0, 1, None, batch, q, refresh, idx[1], cnt[1])
+    assert ctx.get_status() == 0 and (cnt == 500).all()
+    assert torch.equal(idx[0], idx[1])
+    assert not torch.equal(idx[0][..., :500], torch.arange(500, device="cuda", dtype=torch.int32).expand(1, batch, n_heads, 500))

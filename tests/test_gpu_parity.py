@@ -161,7 +161,8 @@ def test_scores_match_oracle_and_selection_is_exact_topk_of_them(H):
             _, _, s = case.oracle_select(0, b, h, qi[0, b], p)
             assert np.allclose(sc[b, h, :L], 0.5 * s, rtol=1e-5, atol=1e-5)
             assert np.all(np.isnan(sc[b, h, L:]))                       # tail untouched
-            # the fused kernel ranks by these very fp32 values: exact top-k, ties to the lower index
+            # the fused kernel ranks by these values to fp32 rounding, and no two of this data's straddle the threshold that
+            # closely: exact top-k, ties to the lower index
             lo, hi = H.orc.candidate_range(L, p.sinks, p.recent)
             cand = np.arange(lo, hi)
             order = np.lexsort((cand, -sc[b, h, lo:hi].astype(np.float64)))
