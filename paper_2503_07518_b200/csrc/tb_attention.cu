@@ -983,7 +983,9 @@ cudaError_t launch_attention(const tb_ctx* c, const UnitTable& ut, const AttnArg
             // than the global merge.  How many clusters fit is asked, not computed: sizes that do not divide a GPC's
             // blocks leave some of them empty (40 problems of 30000 rows, 7 blocks each: 126 in clusters, 94 without; 44, 6
             // each, which fit: 99 and 103).  Without some room they land badly even so (fp32, 56 of 10000, 5 each: 102, 91).
-            if (a.nsplit <= 8 && units * a.nsplit <= 2 * c->sm_count - c->sm_count / 8 && clusters_that_fit(a.nsplit, true) >= units) a.cluster_merge = 1;
+            // One block per problem needs no room: its result is the problem's, and it writes that itself.
+            if (a.nsplit == 1) a.cluster_merge = 1;
+            else if (a.nsplit <= 8 && units * a.nsplit <= 2 * c->sm_count - c->sm_count / 8 && clusters_that_fit(a.nsplit, true) >= units) a.cluster_merge = 1;
         }
     }
     dim3 grid(a.nsplit, gm.Ha, ut.layer_count * ut.n_seq);

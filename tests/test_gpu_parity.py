@@ -725,3 +725,18 @@ def test_attention_blocks_per_problem_of_long_rows(H, config, batch, kv_heads, l
     w = wl.workload(config, n_layers=1, n_q_heads=kv_heads, n_kv_heads=kv_heads, batch=batch, lengths=[length] + [max(1, length // 2)] * (batch - 1),
                     budget=100, sinks=3, recent=5)
     full_pipeline_check(H, H.Case(w), tb().select_params(100, 3, 5), dense_too=True)
+
+
+@pytest.mark.parametrize("batch,heads", [(35, 8), (37, 8), (40, 8)])
+def test_one_block_per_problem_writes_its_result_itself(H, batch, heads):
+    """More problems than the two blocks per SM that a split would take: no partials go through the workspace."""
+    w = wl.workload(2, n_layers=1, n_q_heads=heads, n_kv_heads=heads, batch=batch, lengths=[900 - 7 * b for b in range(batch)], budget=60, sinks=3, recent=5)
+    case = H.Case(w)
+    p = tb().select_params(60, 3, 5)
+    full_pipeline_check(H, case, p, dense_too=True)
+    partials = case.ctx.workspace[:batch * heads * 32 * 130 * 4]
+    partials.fill_(0xA5)
+    q, _ = H.queries(w)
+    H.gpu_attention(case, q, p)
+    H.gpu_attention(case, q, tb().select_params(-1))
+    assert case.ctx.get_status() == 0 and (partials == 0xA5).all()
