@@ -930,13 +930,16 @@ cudaError_t launch_attention(const tb_ctx* c, const UnitTable& ut, const AttnArg
         //    blocks go (32 problems of 640 rows: 3.9 with 2 x 12 warps, 5.2 with 4 x 8; 24 of 1280: 5.3 with 4 blocks each, 8.9
         //    with 6; 96 of 2560: 23.1 with one, 38.8 with 3 x 4 warps and the global merge; 16 of 15000: 23 with 6, 25 with 18
         //    x 4 warps and the global merge);
-        //  - clusters of 3, 7 and 8 pack badly into the SMs of a GPC (3 is taken where the choice is 2), pairs fit everywhere; 9 fits when it takes half of the chip (non-portable:
-        //    asked for);
+        //  - clusters of 3, 7 and 8 pack badly into the SMs of a GPC (3 is taken where the choice is 2), pairs fit everywhere; 9
+        //    fits when it takes half of the chip (non-portable: asked for).  Up to five sixths of the chip 8 do fit (16 problems
+        //    of 2500 rows, 128 blocks: 8.9, 6.4 with 6 each), and where 6 would leave a warp more than its two stages they win (9
+        //    problems of 2500 rows 4.8 / 5.2; 14 of 2500 5.5 / 6.1, of 30000 34.0 / 35.4; 12 of 5000 8.5 / 9.4; below, 6 do: 11
+        //    of 2100 4.3, 5.0 with 8);
         //  - up to five problems of 4K rows or more take 16 blocks each, half of the chip again (non-portable; 2 problems of 8000
         //    rows: 8.6, 9.7 with 9 blocks each; 5 of 16000: 12.6, 14.3 with the global merge);
         //  - the global merge is left with what has too few problems for its rows, that is, where clusters would leave part of
         //    the chip empty and the rows outweigh the merge (4 problems of 20000 rows: 12.9 with 32 blocks of 8 warps each, 15.8
-        //    with a cluster of 12; 6 of 30000: 20.7, 22.2; 96 of 30000: 212 with 3 x 4 warps, 226 with one block of 12; fp32, whose
+        //    with a cluster of 12; 6 of 30000: 20.7, 22.2; fp32, whose
         //    blocks take longer: 16 of 15000: 43, 54; 96 of 2500: 47, 59), and more problems than SMs.
         const int half = c->sm_count / 2, most = c->sm_count - c->sm_count / 8;
         const int small_block = f32 ? 64 : 256, large_block = f32 ? 192 : 384;
@@ -956,6 +959,7 @@ cudaError_t launch_attention(const tb_ctx* c, const UnitTable& ut, const AttnArg
             n = largest(want, half);
             if (n < want && n < least) n = largest(least, most);
             if (!f32 && max_rows > 4096 && units * 16 <= half + half / 8 && clusters_that_fit(16) >= units) n = 16;
+            if (!f32 && n < 8 && max_rows > n * large_block && max_rows > 6 * large_block && 48 * units <= 5 * c->sm_count && clusters_that_fit(8) >= units) n = 8;
         }
 #ifdef TB_FORCE_ATTN_CLUSTER
         n = TB_FORCE_ATTN_CLUSTER;
@@ -966,11 +970,22 @@ cudaError_t launch_attention(const tb_ctx* c, const UnitTable& ut, const AttnArg
                                                        : (n == 16 ? 1200 : used < 48 ? 1536 : used < 64 ? 3000 : 5 * used > 4 * c->sm_count ? 7680 : 10240);
         // fp32 rows keep an SM's warps busier: 4-warp blocks, two per SM, when they fill more of the chip
         const int n4 = f32 && units <= c->sm_count ? 2 * most / units : 0;
+        // One block of 12 warps each, more than half of the SMs: the rest idles.  Blocks of 4 warps, two per SM and three in a
+        // cluster, are the better as long as these fit with room (one / three: 80 problems of 3000 rows 23.2 / 21.0, 88 of 2100
+        // 17.4 / 16.8, of 8000 62.1 / 55.4, 76 of 8000 level; 92, which fill the chip but for ten SMs, of 2100 17.9 / 20.6).
+        // Beyond, pairs are from 12 times two tiles per warp on (one / two: 112 of 8000 73.1 / 68.4; 144 of 4500 49.7 / 50.0, of
+        // 4800 53.2 / 52.7, of 30000 328 / 307).
+        int fours = 1;
+        if (!f32 && n == 1 && units > half) {
+            if (max_rows > 3 * large_block && 3 * units <= 2 * c->sm_count - c->sm_count / 5 && clusters_that_fit(3, true) >= units) fours = 3;
+            else if (max_rows > 12 * large_block && units > half + half / 8 && clusters_that_fit(2, true) >= units) fours = 2;
+        }
         if (n && n4 <= 8 && rows_per_block > large_block && 10 * n4 > 23 * n) {
             a.nsplit = n4, a.cluster_merge = 1;
         } else if (n && (units * n >= most || rows_per_block <= cluster_rows)) {
             a.nsplit = n, a.cluster_merge = 1;
             nw = rows_per_block <= (f32 ? 64 : 112) ? 4 : rows_per_block <= 256 || f32 ? 8 : 12;
+            if (fours > 1) a.nsplit = fours, nw = kAttnWarps;
         } else {
             a.nsplit = pick_nsplit(c, units, max_rows);
             // Few problems, one block of 8 warps per SM: as many rows in flight as two of 4, half the partials to merge

@@ -719,6 +719,10 @@ def test_fp32_attention_shapes(H, heads, budget):
     (1, 17, 1, 3400),
     (1, 12, 8, 577),      # fp32, one block per problem or three
     (1, 7, 8, 4500),      # fp32, five splits that nearly fill the chip
+    (2, 9, 1, 2400),      # eight blocks where six leave a warp a third tile
+    (2, 15, 1, 2305),     # ... as many as fit
+    (2, 14, 8, 4700),     # two 4-warp blocks instead of one of 12
+    (2, 11, 8, 1153),     # three
 ])
 def test_attention_blocks_per_problem_of_long_rows(H, config, batch, kv_heads, length):
     """Each way that a launch of long rows is split (dense over the whole cache, sparse in the same context)."""
