@@ -10,6 +10,8 @@ import os
 
 import torch
 
+from .build import calls_abi, calls_match
+
 TB_OK = 0
 TB_ERR_INVALID_ARG, TB_ERR_UNSUPPORTED, TB_ERR_CAPACITY, TB_ERR_UNPROJECTED = -1, -2, -3, -4
 TB_ERR_STATE, TB_ERR_CUDA, TB_ERR_TIMEOUT, TB_ERR_BAD_INDEX = -5, -6, -7, -8
@@ -64,6 +66,8 @@ def lib():
             if not os.path.exists(path):
                 raise RuntimeError("%s has not been built: run `python -m paper_2503_07518_b200.build` "
                                    "(there is no fallback path)" % os.path.basename(path))
+        if not calls_match():
+            raise RuntimeError("%s was not %s: run `python -m paper_2503_07518_b200.build`" % (os.path.basename(CALLS_PATH), calls_abi()))
         L = C.CDLL(LIB_PATH)
         L.tb_status_string.restype = C.c_char_p
         L.tb_last_step_bytes.restype = C.c_uint64

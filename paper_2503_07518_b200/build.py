@@ -16,8 +16,20 @@ NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", 
               "--expt-relaxed-constexpr", "--expt-extended-lambda"]
 
 
+def calls_abi() -> str:
+    """What the extension module is compiled against and cannot be loaded without: torch's and CPython's C++ interfaces."""
+    import importlib.metadata
+    return "built for torch %s, %s" % (importlib.metadata.version("torch"), sysconfig.get_config_var("SOABI"))
+
+
+def calls_match() -> bool:
+    """Whether the extension module was built for the torch and Python that are running (it carries their names)."""
+    with open(CALLS, "rb") as f:
+        return calls_abi().encode() + b"\0" in f.read()
+
+
 def _stale() -> bool:
-    if not os.path.exists(LIB) or not os.path.exists(CALLS):
+    if not os.path.exists(LIB) or not os.path.exists(CALLS) or not calls_match():
         return True
     t = min(os.path.getmtime(LIB), os.path.getmtime(CALLS))
     deps = [os.path.join(CSRC, f) for f in os.listdir(CSRC)] + [os.path.join(HERE, "..", "include", "tokenbutler.h")]
@@ -47,7 +59,7 @@ def _build_locked(verbose: bool) -> str:
     cxx = os.environ.get("CXX", "g++")
     torch_dir = os.path.dirname(torch.__file__)
     calls_obj = os.path.join(CSRC, "tb_python.o")
-    calls = subprocess.Popen([cxx, "-O2", "-std=c++17", "-fPIC", "-D_GLIBCXX_USE_CXX11_ABI=%d" % torch._C._GLIBCXX_USE_CXX11_ABI,
+    calls = subprocess.Popen([cxx, "-O2", "-std=c++17", "-fPIC", '-DTB_CALLS_ABI="%s"' % calls_abi(), "-D_GLIBCXX_USE_CXX11_ABI=%d" % torch._C._GLIBCXX_USE_CXX11_ABI,
                               "-I" + sysconfig.get_paths()["include"], "-I" + os.path.join(torch_dir, "include"),
                               "-I" + os.path.join(torch_dir, "include", "torch", "csrc", "api", "include"),
                               "-I" + os.path.join(os.path.dirname(os.path.dirname(nvcc)), "include"), "-c", os.path.join(CSRC, "tb_python.cpp"),

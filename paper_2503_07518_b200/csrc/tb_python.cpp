@@ -21,6 +21,9 @@
 
 #include "../../include/tokenbutler.h"
 
+// Read from the file by build.py and binding.py: another torch or Python needs another build.
+extern "C" __attribute__((used, visibility("default"))) const char tb_calls_abi[] = TB_CALLS_ABI;
+
 namespace {
 
 PyObject* g_data_ptr;        // "data_ptr"

@@ -121,3 +121,17 @@ def test_predictor_binding_takes_what_has_a_shape(libpath):
     for hidden in (t.view(-1), None, 3):
         with pytest.raises((IndexError, AttributeError, TypeError)):
             call(hidden, t)
+
+
+def test_a_module_built_for_another_torch_is_not_loaded(libpath, monkeypatch):
+    """It is rebuilt by the build and refused by the binding: its symbols are those of the torch and Python it was built for."""
+    from paper_2503_07518_b200 import binding as b
+    from paper_2503_07518_b200 import build
+    import importlib.metadata
+    assert build.calls_match() and not build._stale()
+    real = importlib.metadata.version
+    monkeypatch.setattr(importlib.metadata, "version", lambda name: real(name) + "1" if name == "torch" else real(name))
+    assert build._stale()
+    monkeypatch.setattr(b, "_lib", None)
+    with pytest.raises(RuntimeError, match="built for torch"):
+        b.lib()
