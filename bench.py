@@ -42,7 +42,7 @@ NCU_TRAFFIC_BYTES = {
     ("cfg2_llama8b_32k", "attn_kernel"): 13_598_208,               # profiles/attn_mma_kernel_cfg2_32k.md
     ("cfg3_batched_serving", "select_kernel"): 398_907_392 + 5_187_840,   # profiles/select_wave_kernel_cfg3_batched.md
     ("cfg4_long_context_128k", "select_kernel"): 268_011_264 + 3_980_544,  # profiles/select_cw_kernel_cfg4_128k.md
-    ("cfg5_interval_neighbors", "attn_kernel"): 309_490_432 + 4_711_680,   # profiles/attn_mma_kernel_cfg5_interval.md
+    ("cfg5_interval_neighbors", "attn_kernel"): 309_490_432 + 4_711_680,   # profiles/attn_mma_kernel_cfg5_interval.md (the rows' bytes; captured with other splits)
 }
 
 
@@ -728,8 +728,8 @@ def measure_trajectory(args, w):
         "e2e": {"value": tokens / (ms_e2e * 1e-3), "unit": UNIT, "us_per_step": ms_e2e * 1e3,
                 "h2d_bytes_per_step": sum(h.numel() * h.element_size() for h in host), "d2h_bytes_per_step": out_host.numel() * 4,
                 "how": "copies on two copy streams, two sets of device buffers: a step's copies overlap its neighbours' compute"},
-        "kernels": {"select_kernel+neighbor_kernel": {"us_per_launch": sel_ms * 1e3, "bytes_per_launch": sel_bytes,
-                                                      "gbs": sel_bytes / (sel_ms * 1e-3) / 1e9, "launches_per_refresh": len(groups)},
+        "kernels": {"selection with neighbours": {"us_per_launch": sel_ms * 1e3, "bytes_per_launch": sel_bytes,
+                                                  "gbs": sel_bytes / (sel_ms * 1e-3) / 1e9, "launches_per_refresh": len(groups)},
                     "attn_kernel": {"us_per_launch": att_ms * 1e3, "bytes_per_launch": att_bytes,
                                     "gbs": att_bytes / (att_ms * 1e-3) / 1e9, "launches_per_step": w.n_layers}},
         "roofline": {"bound": "hbm", "kernel": "attn_mma_kernel", "achieved": att_bytes / (att_ms * 1e-3) / 1e9,
