@@ -780,7 +780,7 @@ __global__ void __launch_bounds__(NW * 32) attn_mma_kernel(Geom gm, UnitTable ut
             attn_stamp(6);
             return;
         }
-    if (split_cluster) asm volatile("barrier.cluster.wait.aligned;" ::: "memory");
+        if (split_cluster) asm volatile("barrier.cluster.wait.aligned;" ::: "memory");
         for (int slot = tid; slot < 256; slot += NW * 32) {
             const int mt = slot >> 5, ln = slot & 31;
             float4 acc, stat;
@@ -845,8 +845,8 @@ __global__ void __launch_bounds__(NW * 32) attn_mma_kernel(Geom gm, UnitTable ut
 }
 
 static int pick_nsplit(const tb_ctx* c, int units, int max_rows) {
-    // about two blocks per SM and never a thin second wave: with 64 problems of 9.8K rows, 4 splits
-    // (256 blocks) ran at 58.5 us, 5 at 63.6, 6 at 61.5, 7 (448 blocks, four more than fit at once) at 75.7,
+    // about two blocks per SM and never a thin second wave: with 64 problems of 9.8K rows (which now take two 12-warp
+    // blocks each, see launch_attention), 4 splits (256 blocks) ran at 58.5 us, 5 at 63.6, 6 at 61.5, 7 (448 blocks, four more than fit at once) at 75.7,
     // 10 at 65.0
     int n = 2 * c->sm_count / units;
 #ifdef TB_FORCE_NSPLIT

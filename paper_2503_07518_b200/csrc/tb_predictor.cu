@@ -236,7 +236,7 @@ __global__ void __launch_bounds__(kPredThreads) predictor_out_kernel(const T* __
 // 24, 31 with 64, of which 1.3 are the weights at the copy bandwidth.  (Before: 8.8 with a warp pair per hidden unit and
 // 18.7, 31.9, 61 with 16-token left tiles whose blocks each normalised every token.)  The weights go through shared
 // memory because their copies then cost no registers: with the fragments loaded straight into registers the kernels
-// spilled and ran at 11.3 us.  Two blocks must fit an SM: the output kernel's blocks sit beside the hidden kernel's and
+// spilled and ran at 11.3 us.  Two blocks must fit an SM (they do up to 24 staged tokens; with 32 staged one does): the output kernel's blocks sit beside the hidden kernel's and
 // have their weights before the hidden units exist, and at one block per SM only 15 of the 16 clusters start at once.
 //
 // The 16 k-indices of an MMA step are mapped to channels so that every thread's operands are 16 contiguous bytes:
