@@ -235,6 +235,7 @@ tb_status tb_create(const tb_config* cfg, void* kv, void* kimp, void* state, voi
     c->last_cache_write = c->last_list_write = -4;
     c->tile_rows = 256;
     for (int& known : c->attn_max_active) known = 0;
+    for (int& known : c->stream_max_active) known = 0;
     if (cudaDeviceGetAttribute(&c->sm_count, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) { delete c; return TB_ERR_CUDA; }
     // only the small control parts need defined contents; the index lists and partials are always
     // written before they are read
@@ -449,7 +450,7 @@ tb_status tb_select_topk(tb_ctx* c, int32_t lb, int32_t lc, const int32_t* seq_i
                     cand_range(ut.len[i], p->sinks, p->recent, &lo, &hi);
                     if (hi - lo > max_cand) max_cand = hi - lo;
                 }
-                const bool small = select_small_takes(c, ut, max_cand, p->radius > 0);
+                const bool small = select_small_takes(c, ut, max_cand);
                 finished = small;
                 SelectArgs a;
                 a.radius = p->radius, a.nmode = p->nmode;

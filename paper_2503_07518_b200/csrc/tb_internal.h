@@ -140,6 +140,7 @@ struct tb_ctx {
     int tile_rows;                        // rows per TMA box of the score pass
     int sm_count;
     int attn_max_active[25];              // co-resident attention clusters per cluster size, 8-warp blocks and (16 +) 4-warp ones (0 = not asked yet)
+    int stream_max_active[17];            // co-resident clusters of the streaming selection per cluster size (0 = not asked yet)
     void* res_rows;                       // resident sink + window rows (tb_bind_resident_rows), or NULL
     int res_sinks, res_window;
     void* imp_rows;                       // Important buffer (tb_bind_important_buffer), or NULL
@@ -208,10 +209,12 @@ cudaError_t launch_select_wave(const tb_ctx* c, const UnitTable& ut, const Selec
 cudaError_t launch_select_shared(const tb_ctx* c, const UnitTable& ut, const SelectArgs& a, cudaStream_t s, bool dry, bool* finished);
 // small problems: one block each, neighbours and the caller's copy of the list included; whether a launch whose longest
 // problem has max_cand candidates is its kind (not whether the caller wants copies: they must not change the lists)
-bool select_small_takes(const tb_ctx* c, const UnitTable& ut, int max_cand, bool neighbours);
+bool select_small_takes(const tb_ctx* c, const UnitTable& ut, int max_cand);
 cudaError_t launch_select_small(const tb_ctx* c, const UnitTable& ut, const SelectArgs& a, int max_cand, cudaStream_t s, bool dry = false);
 // few, long problems: a cluster per problem on parked keys
 cudaError_t launch_select_cw(const tb_ctx* c, const UnitTable& ut, const SelectArgs& a, cudaStream_t s, bool dry = false);
+// long problems: a cluster of blocks each, neighbours and the caller's copy included; *taken = false: not its kind
+cudaError_t launch_select_stream(const tb_ctx* c, const UnitTable& ut, const SelectArgs& a, cudaStream_t s, bool dry, bool* taken);
 cudaError_t launch_neighbors(const tb_ctx* c, const UnitTable& ut, const NeighborArgs& a, cudaStream_t s, bool dry = false);
 // copies the rows of the stored lists into the Important buffer (after a refresh)
 cudaError_t launch_migrate(const tb_ctx* c, const UnitTable& ut, cudaStream_t s);

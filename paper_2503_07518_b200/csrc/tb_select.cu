@@ -727,6 +727,11 @@ cudaError_t launch_select(const tb_ctx* c, const UnitTable& ut, const SelectArgs
     if (c->drop_tile >= 0 && (to_wave || to_cw)) return cudaErrorInvalidConfiguration;   // wait diagnostics: single-block launches of this kernel only
     // Lists that share a key stream read it once.
     if (gm.dtype == TB_BF16 && gm.Hl > gm.Hi && c->drop_tile < 0) return launch_select_shared(c, ut, a, s, dry, finished);
+    if (c->drop_tile < 0) {
+        bool taken;
+        cudaError_t e = launch_select_stream(c, ut, a, s, dry, &taken);
+        if (taken) return *finished = true, e;
+    }
     if (to_wave) return launch_select_wave(c, ut, a, s, dry, finished);
     if (to_cw) return launch_select_cw(c, ut, a, s, dry);
     const int n_tiles = (max_cand + kTileRows - 1) / kTileRows;

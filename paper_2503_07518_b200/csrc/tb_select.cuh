@@ -2,6 +2,7 @@
 // cores, with exact products and fp32 sums in another order), launch-unit decoding, neighbours and lists.
 #pragma once
 
+#include <algorithm>
 #include <type_traits>
 
 #include "tb_common.cuh"
@@ -133,6 +134,23 @@ __device__ __forceinline__ void check_candidates_projected(const Geom& gm, const
     }
 }
 
+// Launch order of the (layer, sequence) pairs: longest first, so that the blocks still running when
+// the grid drains are the short ones.
+struct WaveOrder {
+    uint16_t pair[kMaxLaunchUnits];
+};
+
+// The pairs of a launch, longest first, and their candidates; returns the most.
+inline int longest_first(const UnitTable& ut, const SelectArgs& a, WaveOrder& order, int (&cand)[kMaxLaunchUnits]) {
+    const int n_pairs = ut.layer_count * ut.n_seq;
+    for (int i = 0; i < n_pairs; ++i) {
+        const int L = ut.len[i], lo = a.sinks < L ? a.sinks : L, hi = L - a.recent > lo ? L - a.recent : lo;
+        cand[i] = hi - lo, order.pair[i] = (uint16_t)i;
+    }
+    std::stable_sort(order.pair, order.pair + n_pairs, [&](uint16_t x, uint16_t y) { return cand[x] > cand[y]; });
+    return cand[order.pair[0]];
+}
+
 // Candidates of a problem whose kernel keeps something per candidate in shared memory.  A replayed graph may find a sequence
 // longer than its launch was sized for (it outgrew the declared reserve): the candidates past `room` are left out and the
 // status word says so.
@@ -148,14 +166,17 @@ __device__ __forceinline__ int candidates_within(int n, int room, int32_t* statu
 // eight whole rows, and with the query's dimensions permuted the same way the four 4-byte words are the A operand of two
 // m16n8k16 steps (8 bytes and one step for 16 dimensions).  No shared memory, no barrier; every warp keeps kU groups of 32
 // rows in flight.   D[16 rows x 8] += K[16 x 16] . Q[16 x 8], fp32 accumulators; Q is split into three bf16 terms that hold
-// all 24 bits of the fp32 query, lowest term first, so every product is exact and only the fp32 sums round (against fp64:
-// rms error 1.4e-8 of sum |q k|, where the FMA chains above have 2.0e-8).  TB_GROUP_SUM: all eight columns hold the summed
-// query and a lane keeps the value that belongs to its row; TB_GROUP_MAX: column = head, a row's score is the largest over
-// the columns.  A row's score depends only on its bytes, never on where it sits.  Infinities do not survive the split (a
-// query's lower terms are zero or of either sign: inf * 0, inf - inf): rows with an infinite score are scored again, by the
-// FMA chains, behind the stream (rescore).  The kernels look for them only where a sum over the scores, or a query, is not
-// finite.
-constexpr int kQueryFrags = 3 * 2 * 32;   // a query's B fragments: terms x steps x lanes
+// all 24 bits of the fp32 query, so every product is exact and only the fp32 sums round (against fp64, 32 dimensions, four
+// heads: rms error 1.7e-8 of sum |q k|, where the FMA chains above have 2.5e-8; 16 dimensions 1.9e-8 and 2.5e-8).
+// TB_GROUP_SUM: the columns are the terms of the summed query, (high, middle, low, 0) twice, so a group takes four MMAs and
+// its operands four registers; a lane adds two terms, its neighbour the other two, one shuffle brings them together at the lane
+// that owns the row.  (All eight columns the summed query, the terms one after the other: 12 MMAs at 8.7 cycles each in chains
+// of six, operands from shared memory.)  TB_GROUP_MAX: column = head, the terms one after the other, lowest first; a row's
+// score is the largest over the columns.  A row's score depends only on its bytes, never on where it sits.  Infinities do not
+// survive the split (a query's lower terms are zero or of either sign: inf * 0, inf - inf): rows with an infinite score are
+// scored again, by the FMA chains, behind the stream (rescore).  The kernels look for them only where a sum over the scores, or
+// a query, is not finite.
+constexpr int kQueryFrags = 3 * 2 * 32;   // TB_GROUP_MAX, a query's B fragments: terms x steps x lanes
 
 __device__ __forceinline__ void mma_16816(float (&d)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0, uint32_t b1) {
     asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
@@ -195,40 +216,56 @@ template <int DP, int RED>
 struct FragScorer {
     static constexpr int kSteps = DP / 16, kTerms = 3, kRowBytes = DP * 2;
     typedef typename std::conditional<DP == 32, uint4, uint2>::type Piece;    // a thread's quarter of a row
-    const uint2* frag;                                 // this lane's B fragments, [term][step][lane], in shared memory
-    // Called by all threads of the block with the queries staged and visible; `frags` holds kQueryFrags entries.
+    uint2 b[RED == TB_GROUP_SUM ? kSteps : 1];         // this lane's B fragments, per step
+    const uint2* frag;                                 // ... or where they are in shared memory, [term][step][lane]
+    // The largest bf16 term of (x, y), taken off them.  (The first one: a finite value does not become an infinity, above the
+    // largest bf16 it takes that one.)
+    __device__ __forceinline__ static uint32_t split(float& x, float& y, bool first = false) {
+        const float top = 3.38953139e38f;
+        const __nv_bfloat162 v = first ? __floats2bfloat162_rn(is_finite(x) ? fminf(fmaxf(x, -top), top) : x, is_finite(y) ? fminf(fmaxf(y, -top), top) : y)
+                                       : __floats2bfloat162_rn(x, y);
+        x -= __low2float(v), y -= __high2float(v);
+        return *reinterpret_cast<const uint32_t*>(&v);
+    }
+    // Called by all threads of the block.  TB_GROUP_SUM: `qs` in shared or global memory; TB_GROUP_MAX: staged and visible,
+    // `frags` holds kQueryFrags entries, one barrier.
     __device__ __forceinline__ void load_staged(const float* qs, int g, uint2* frags) {
-        const int lane = threadIdx.x & 31, st = threadIdx.x >> 5, gid = lane >> 2, tig = lane & 3;
-        frag = frags + lane;
-        if (st < kSteps) {
-            uint32_t b[kTerms][2];
+        const int lane = threadIdx.x & 31, gid = lane >> 2, tig = lane & 3;
+        // dimensions of word 2 st + half of the piece: tig * (DP / 4) + st * 4 + half * 2
+        if constexpr (RED == TB_GROUP_SUM) {
+            float x[kSteps * 2], y[kSteps * 2];
 #pragma unroll
-            for (int half = 0; half < 2; ++half) {
-                const int k = tig * (DP / 4) + st * 4 + half * 2;             // the dimensions of word 2 st + half of the piece
-                float x, y;
-                if constexpr (RED == TB_GROUP_SUM) {
-                    x = y = 0.f;
-                    for (int u = 0; u < g; ++u) {      // in head order
-                        const float2 v = *reinterpret_cast<const float2*>(qs + u * DP + k);
-                        x += v.x, y += v.y;
-                    }
-                } else {
-                    const float2 v = *reinterpret_cast<const float2*>(qs + min(gid, g - 1) * DP + k);
-                    x = v.x, y = v.y;
+            for (int i = 0; i < kSteps * 2; ++i) x[i] = y[i] = 0.f;
+#pragma unroll 4
+            for (int u = 0; u < g; ++u)                // in head order
+#pragma unroll
+                for (int i = 0; i < kSteps; ++i) {
+                    const float4 v = *reinterpret_cast<const float4*>(qs + u * DP + tig * (DP / 4) + i * 4);
+                    x[2 * i] += v.x, y[2 * i] += v.y, x[2 * i + 1] += v.z, y[2 * i + 1] += v.w;
                 }
 #pragma unroll
-                for (int t = 0; t < kTerms; ++t) {
-                    // (a finite value does not become an infinity: above the largest bf16 it takes that one first)
-                    const float top = 3.38953139e38f;
-                    const __nv_bfloat162 v = __floats2bfloat162_rn(is_finite(x) ? fminf(fmaxf(x, -top), top) : x, is_finite(y) ? fminf(fmaxf(y, -top), top) : y);
-                    b[t][half] = *reinterpret_cast<const uint32_t*>(&v);
-                    x -= __low2float(v), y -= __high2float(v);
-                }
+            for (int i = 0; i < kSteps * 2; ++i) {
+                const uint32_t high = split(x[i], y[i], true), middle = split(x[i], y[i]), low = split(x[i], y[i]);
+                const uint32_t mine = (gid & 3) == 0 ? high : (gid & 3) == 1 ? middle : (gid & 3) == 2 ? low : 0u;
+                if (i & 1) b[i >> 1].y = mine;
+                else b[i >> 1].x = mine;
             }
+        } else {
+            const int st = threadIdx.x >> 5;
+            frag = frags + lane;
+            if (st < kSteps) {
+                uint32_t t[kTerms][2];
 #pragma unroll
-            for (int t = 0; t < kTerms; ++t) frags[(t * kSteps + st) * 32 + lane] = make_uint2(b[t][0], b[t][1]);
+                for (int half = 0; half < 2; ++half) {
+                    float2 v = *reinterpret_cast<const float2*>(qs + min(gid, g - 1) * DP + tig * (DP / 4) + st * 4 + half * 2);
+#pragma unroll
+                    for (int i = 0; i < kTerms; ++i) t[i][half] = split(v.x, v.y, i == 0);
+                }
+#pragma unroll
+                for (int i = 0; i < kTerms; ++i) frags[(i * kSteps + st) * 32 + lane] = make_uint2(t[i][0], t[i][1]);
+            }
+            __syncthreads();
         }
-        __syncthreads();
     }
     // v[m]: this thread's piece of row 8 m + gid of the 32; d[m][2 i + e]: row 16 m + 8 i + gid, column 2 tig + e
     __device__ __forceinline__ void columns(const Piece (&v)[4], float (&d)[2][4]) const {
@@ -249,51 +286,126 @@ struct FragScorer {
     // returns the score of the row this lane looks after (my_row)
     __device__ __forceinline__ float score(const Piece (&v)[4], int row0, int& my_row) const {
         const int lane = threadIdx.x & 31, gid = lane >> 2, tig = lane & 3;
-        float d[2][4];
-        columns(v, d);
-        // lane (gid, tig) takes row gid + 8 tig: accumulator 0 / 2 of the first 16 rows, then of the second
+        // lane (gid, tig) takes row gid + 8 tig: accumulator pair 0 / 1 of the first 16 rows, then of the second
         my_row = row0 + gid + 8 * tig;
-        float r[4] = {d[0][0], d[0][2], d[1][0], d[1][2]};
-        if constexpr (RED == TB_GROUP_MAX) {
-            r[0] = fmaxf(r[0], d[0][1]), r[1] = fmaxf(r[1], d[0][3]), r[2] = fmaxf(r[2], d[1][1]), r[3] = fmaxf(r[3], d[1][3]);
+        float d[2][4], r[4];
+        if constexpr (RED == TB_GROUP_SUM) {
 #pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                r[i] = fmaxf(r[i], __shfl_xor_sync(0xffffffffu, r[i], 1));
-                r[i] = fmaxf(r[i], __shfl_xor_sync(0xffffffffu, r[i], 2));
+            for (int m = 0; m < 2; ++m) {
+                d[m][0] = d[m][1] = d[m][2] = d[m][3] = 0.f;
+                mma_16816(d[m], v[2 * m].x, v[2 * m + 1].x, v[2 * m].y, v[2 * m + 1].y, b[0].x, b[0].y);
+                if constexpr (DP == 32) mma_16816(d[m], v[2 * m].z, v[2 * m + 1].z, v[2 * m].w, v[2 * m + 1].w, b[kSteps - 1].x, b[kSteps - 1].y);
+                r[2 * m] = d[m][0] + d[m][1], r[2 * m + 1] = d[m][2] + d[m][3];
+            }
+        } else {
+            columns(v, d);
+            r[0] = fmaxf(d[0][0], d[0][1]), r[1] = fmaxf(d[0][2], d[0][3]), r[2] = fmaxf(d[1][0], d[1][1]), r[3] = fmaxf(d[1][2], d[1][3]);
+#pragma unroll
+            for (int i = 0; i < 4; ++i) r[i] = fmaxf(r[i], __shfl_xor_sync(0xffffffffu, r[i], 2));
+        }
+        const float lo = tig & 2 ? r[2] : r[0], hi = tig & 2 ? r[3] : r[1];
+        const float mine = tig & 1 ? hi : lo, other = __shfl_xor_sync(0xffffffffu, tig & 1 ? lo : hi, 1);
+        return RED == TB_GROUP_SUM ? mine + other : fmaxf(mine, other);
+    }
+    __device__ __forceinline__ static void load_piece(Piece& v, const unsigned char* quarter) { v = __ldcg(reinterpret_cast<const Piece*>(quarter)); }
+};
+
+// fp32 rows the same way: thread tig of a row's four takes a quarter of it, 32 rows per group, one FMA chain per quarter; three
+// shuffles per four rows add the quarters and leave each lane the score of one row.  A row's score depends only on its bytes,
+// and its sums are shorter than the two chains of row_score (rms error 2.1e-8 of sum |q k| for 2.5e-8).
+template <int DP, int RED>
+struct QuarterScorer {
+    static constexpr int kRowBytes = DP * 4, kPer = DP / 16;                  // 16-byte pieces of a quarter
+    struct Piece { uint4 w[kPer]; };
+    float qr[RED == TB_GROUP_SUM ? DP / 4 : 1];
+    const float* qs;
+    int g;
+    __device__ __forceinline__ void load_staged(const float* qs_, int g_, uint2*) {
+        const int tig = threadIdx.x & 3;
+        qs = qs_ + tig * (DP / 4), g = g_;
+        if constexpr (RED == TB_GROUP_SUM) {
+#pragma unroll
+            for (int j = 0; j < DP / 4; ++j) qr[j] = 0.f;
+#pragma unroll 4
+            for (int u = 0; u < g_; ++u)               // in head order
+#pragma unroll
+                for (int j = 0; j < DP / 4; j += 4) {
+                    const float4 v = *reinterpret_cast<const float4*>(qs + u * DP + j);
+                    qr[j] += v.x, qr[j + 1] += v.y, qr[j + 2] += v.z, qr[j + 3] += v.w;
+                }
+        }
+    }
+    __device__ __forceinline__ float reduce(const Piece (&v)[4], const float* q) const {
+        const int tig = threadIdx.x & 3;
+        float r[4];
+#pragma unroll
+        for (int m = 0; m < 4; ++m) {
+            r[m] = 0.f;
+#pragma unroll
+            for (int c = 0; c < kPer; ++c) {
+                float f[4];
+                Elem<float>::unpack16(v[m].w[c], f);
+#pragma unroll
+                for (int e = 0; e < 4; ++e) r[m] = fmaf(q[c * 4 + e], f[e], r[m]);
             }
         }
-        const float lo = tig & 1 ? r[1] : r[0], hi = tig & 1 ? r[3] : r[2];
-        return tig & 2 ? hi : lo;
+        const float a0 = (tig & 2 ? r[2] : r[0]) + __shfl_xor_sync(0xffffffffu, tig & 2 ? r[0] : r[2], 2);
+        const float a1 = (tig & 2 ? r[3] : r[1]) + __shfl_xor_sync(0xffffffffu, tig & 2 ? r[1] : r[3], 2);
+        return (tig & 1 ? a1 : a0) + __shfl_xor_sync(0xffffffffu, tig & 1 ? a0 : a1, 1);
     }
-    // rows at `rows` (the first of the 32), n of them exist
-    __device__ __forceinline__ static void load(Piece (&v)[4], const unsigned char* rows, int n) {
-        const int lane = threadIdx.x & 31, gid = lane >> 2, tig = lane & 3;
-        const unsigned char* p = rows + gid * kRowBytes + tig * (kRowBytes / 4);
+    __device__ __forceinline__ float score(const Piece (&v)[4], int row0, int& my_row) const {
+        const int lane = threadIdx.x & 31;
+        my_row = row0 + (lane >> 2) + 8 * (lane & 3);
+        if constexpr (RED == TB_GROUP_SUM) return reduce(v, qr);
+        float best = -INFINITY;
+        for (int u = 0; u < g; ++u) best = fmaxf(best, reduce(v, qs + u * DP));
+        return best;
+    }
+    __device__ __forceinline__ static void load_piece(Piece& v, const unsigned char* quarter) {
 #pragma unroll
-        for (int m = 0; m < 4; ++m)
-            if (8 * m + gid < n) v[m] = __ldcg(reinterpret_cast<const Piece*>(p + 8 * m * kRowBytes));
+        for (int c = 0; c < kPer; ++c) v.w[c] = __ldcg(reinterpret_cast<const uint4*>(quarter) + c);
     }
 };
 
-// The bf16 stream of a block: rows [0, n) from `rows`, in groups of 32 dealt to the warps in turn, kU groups per warp in
-// flight.
-template <int DP, int RED, int kU>
+// A group of 32 rows into a warp's registers: v[m] = this thread's quarter of row 8 m + gid; row(i) = address of row i < n.
+template <typename Scorer, typename F>
+__device__ __forceinline__ void load_rows(typename Scorer::Piece (&v)[4], int n, F&& row) {
+    const int lane = threadIdx.x & 31, gid = lane >> 2, tig = lane & 3;
+#pragma unroll
+    for (int m = 0; m < 4; ++m)
+        if (8 * m + gid < n) Scorer::load_piece(v[m], row(8 * m + gid) + tig * (Scorer::kRowBytes / 4));
+}
+
+// The stream of a block of kW warps: rows [0, n) from `rows`, in groups of 32 dealt to the warps in turn, kU groups per warp in
+// flight.  kWhole: n is a multiple of 32 (less code).  (Groups claimed from a counter as they are requested even out the warps, 1 us apart after 0.5 MB, but the claim is
+// in every group's way: 32 problems of 32768 rows 20.1 -> 20.8 us.)
+template <typename S, int kU, int kW, bool kWhole = false>
 struct RowStream {
-    typedef FragScorer<DP, RED> Scorer;
+    typedef S Scorer;
+    static constexpr int kGroupBytes = 32 * Scorer::kRowBytes;
     typename Scorer::Piece v[kU][4];
     const unsigned char* rows;
-    int n, warp, n_warps;
+    int n, warp;
     __device__ __forceinline__ void load(int u, int g) {
-        if (g * 32 < n) Scorer::load(v[u], rows + (size_t)g * 32 * Scorer::kRowBytes, n - g * 32);
-    }
-    __device__ __forceinline__ void start(const unsigned char* rows_, int n_) {
-        rows = rows_, n = n_, warp = threadIdx.x >> 5, n_warps = blockDim.x >> 5;
+        const unsigned char* first = rows + (size_t)g * kGroupBytes;
+        if (kWhole ? g * 32 < n : g * 32 + 32 <= n) {  // warp-uniform
+            const int lane = threadIdx.x & 31;
 #pragma unroll
-        for (int u = 0; u < kU; ++u) {
-#pragma unroll
-            for (int m = 0; m < 4; ++m) v[u][m] = {};
-            load(u, u * n_warps + warp);
+            for (int m = 0; m < 4; ++m) Scorer::load_piece(v[u][m], first + (8 * m + (lane >> 2)) * Scorer::kRowBytes + (lane & 3) * (Scorer::kRowBytes / 4));
+        } else if (!kWhole && g * 32 < n) {            // the last one
+            load_rows<Scorer>(v[u], n - g * 32, [&](int i) { return first + i * Scorer::kRowBytes; });
         }
+    }
+    // requests the groups [u0, u1) of every warp
+    __device__ __forceinline__ void start(const unsigned char* rows_, int n_, int u0 = 0, int u1 = kU) {
+        rows = rows_, n = n_, warp = threadIdx.x >> 5;
+#pragma unroll
+        for (int u = 0; u < kU; ++u)
+            if (u >= u0 && u < u1) {
+#pragma unroll
+                for (int m = 0; m < 4; ++m) v[u][m] = {};
+                load(u, u * kW + warp);
+            }
     }
     // consume(slot, score) for every row
     template <typename F>
@@ -301,7 +413,7 @@ struct RowStream {
         run_groups([&](const typename Scorer::Piece (&piece)[4], int row0) {
             int slot;
             const float sc = scorer.score(piece, row0, slot);
-            return [=, &consume] { if (slot < n) consume(slot, sc); };
+            return [=, &consume] { if (kWhole || slot < n) consume(slot, sc); };
         });
     }
     // f(slot) for every row that run() gives to this thread
@@ -309,18 +421,19 @@ struct RowStream {
     __device__ __forceinline__ void own_rows(F&& f) const {
         const int lane = threadIdx.x & 31;
 #pragma unroll 1
-        for (int slot = warp * 32 + (lane >> 2) + 8 * (lane & 3); slot < n; slot += n_warps * 32) f(slot);
+        for (int slot = warp * 32 + (lane >> 2) + 8 * (lane & 3); slot < n; slot += kW * 32) f(slot);
     }
     // f(pieces, first row) for every group of 32; what it returns is called once the group's successor has been requested
     template <typename F>
     __device__ __forceinline__ void run_groups(F&& f) {
-        for (int g0 = warp; g0 * 32 < n; g0 += kU * n_warps) {
+#pragma unroll 1
+        for (int g0 = warp; g0 * 32 < n; g0 += kU * kW) {
 #pragma unroll
             for (int u = 0; u < kU; ++u) {
-                const int g = g0 + u * n_warps;
+                const int g = g0 + u * kW;
                 if (g * 32 >= n) break;                // warp-uniform
                 auto rest = f(v[u], g * 32);
-                load(u, g + kU * n_warps);
+                load(u, g + kU * kW);
                 rest();
             }
         }
@@ -340,6 +453,23 @@ struct DigitCounter {
         below = warp_sum_int(below);
         if ((threadIdx.x & 31) == 0 && below) atomicAdd(hist, below);
         below = 0;
+    }
+};
+
+// The same for keys that are mostly in the first or the last bin (a bin that is cut again): both are counted in a register, at
+// most 65535 of each per thread.
+template <int kLast>
+struct EdgeCounter {
+    uint32_t edges = 0;                                // below | above << 16
+    __device__ __forceinline__ void add(int* hist, uint32_t bin) {
+        if (bin - 1u < kLast - 1u) asm volatile("red.shared.add.s32 [%0], 1;" ::"r"(smem_u32(hist + bin)) : "memory");
+        else edges += bin ? 0x10000u : 1u;
+    }
+    __device__ __forceinline__ void flush(int* hist) {   // whole warps; followed by a barrier
+        const int below = warp_sum_int((int)(edges & 0xffffu)), above = warp_sum_int((int)(edges >> 16));
+        if ((threadIdx.x & 31) == 0 && below) atomicAdd(hist, below);
+        if ((threadIdx.x & 31) == 0 && above) atomicAdd(hist + kLast, above);
+        edges = 0;
     }
 };
 

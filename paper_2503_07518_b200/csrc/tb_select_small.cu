@@ -141,7 +141,7 @@ __global__ void __launch_bounds__(kThreads, kU == 2 ? 2 : 1) select_small_kernel
     if (!kDirect && tid == 0)
         for (int t = 0; t < min(n_stages, my_tiles); ++t) request(t);
     if (tid < gm.gl * DP) sm->qs[tid] = a.q_imp[query_row(gm, ut, ll, s, h) * DP + tid];
-    typename std::conditional<kDirect, RowStream<DP, RED, kDirect ? kU : 1>, NoStream>::type rs;
+    typename std::conditional<kDirect, RowStream<FragScorer<DP, RED>, kDirect ? kU : 1, kWarps>, NoStream>::type rs;
     rs.start(kimp + row0 * RB, n_local);
     const bool odd_query = __syncthreads_or(kDirect && tid < gm.gl * DP && !is_finite(sm->qs[tid]));   // (its own element)
 
@@ -319,19 +319,20 @@ size_t small_smem(int n_stages, int n_tiles, int tile_bytes) {
 
 }  // namespace
 
-// Launches of up to two blocks per SM.  Measured against the cluster kernel and the one-block-per-problem kernel, us per
-// launch, bf16, 32 dimensions unless said (this / the other): 32 problems of 1000 candidates 5.6 / 7.0, 2000 6.7 / 10.4, 4000
-// 7.7 / 9.5, 8000 11.4 / 12.7, 12000 13.2 / 12.6 (eight blocks per problem bring more SMs there); 96 problems of 2000 7.3 /
-// 10.2, 9500 19.4 / 20.9, 16000 28.9 / 29.1, at 16 dimensions 14.9 / 17.3 and 23.4 / 24.5; two per SM: 192 of 2000 level, of
-// 6000 25.4 / 25.8 (16 dimensions 17.9 / 23.0), of 9500 level; 384 problems, a second wave: level or worse.  Neighbours and
-// the caller's copy come for next to nothing here and cost two more launches there (96 problems of 3000 with both: 8.3 / 18.4),
-// so neighbours raise the limit.  A copy does not: the scores are summed in another order here, and an output that the caller
+// Launches of up to two blocks per SM, as long as one block's finish is cheaper than a cluster's.  Against the streaming kernel,
+// us per launch, bf16, 32 dimensions unless said (this / the other): 8 problems of 4000 candidates 7.6 / 9.8, 10000 11.1 / 11.1, 32
+// of 8000 11.1 / 12.1, with neighbours 14.3 / 15.3 and 16000 20.9 / 18.5; more problems than half of the SMs leave the other
+// one block each too: 96 of 8000 15.8 / 16.8, 16000 26.6 / 26.8, fp32 42.1 / 44.1; two per SM: 192 of 6000 20.6 / 21.7, 8000
+// 25.4 / 26.3, with neighbours 160 of 12000 51 / 40; fp32, whose rows do not go straight into registers here, 160 of 4000 32 /
+// 25, 2000 20 / 15.6.  384 problems, a second wave: level with one block of 256 threads each, or worse.
+// Whether the caller wants copies does not matter: the scores are summed in another order here, and an output that the caller
 // may leave out must not decide which of two tokens within fp32 rounding of one another is stored.
-bool select_small_takes(const tb_ctx* c, const UnitTable& ut, int max_cand, bool neighbours) {
+bool select_small_takes(const tb_ctx* c, const UnitTable& ut, int max_cand) {
     const int n_units = ut.layer_count * ut.n_seq * c->geom.Hl;
     // wait diagnostics: launches of one block that wait for copies (the others: see launch_select)
     if (c->drop_tile >= 0 && (c->geom.dtype == TB_BF16 || n_units > 1 || max_cand > 1023)) return false;
-    const int most = neighbours || (n_units <= c->sm_count && 2 * n_units > c->sm_count) ? kMaxCand : n_units <= c->sm_count ? 10 * 1024 : 8 * 1024;
+    if (n_units > c->sm_count && c->geom.dtype != TB_BF16 && c->drop_tile < 0) return max_cand <= 1500;
+    const int most = n_units <= c->sm_count ? (2 * n_units > c->sm_count ? kMaxCand : 10 * 1024) : 8 * 1024;
     return n_units <= 2 * c->sm_count && max_cand <= most;
 }
 

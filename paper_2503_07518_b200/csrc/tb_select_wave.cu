@@ -43,12 +43,6 @@ constexpr int kSampleRows = 64;     // rows scored up front to place the first d
 constexpr int kMinSampled = 2048;   // smaller problems use the key's top bits as first digit
 constexpr int kBatch = 8;           // 16-byte key loads a thread keeps in flight
 
-// Launch order of the (layer, sequence) pairs: longest first, so that the blocks still running when
-// the grid drains are the short ones.
-struct WaveOrder {
-    uint16_t pair[kMaxLaunchUnits];
-};
-
 #ifdef TB_PHASE_TIMING
 __device__ unsigned long long g_fin_ns[8];
 __device__ unsigned long long g_cw_ns[8];
@@ -672,7 +666,7 @@ template <int DP>
 __global__ void __launch_bounds__(kThreads, 2)
     select_shared_kernel(const unsigned char* __restrict__ kimp, Geom gm, UnitTable ut, WaveOrder order, SelectArgs a, int scratch_bytes, int keep_in_l2,
                          int32_t* __restrict__ state_idx, int32_t* __restrict__ state_cnt, int32_t* __restrict__ status, uint32_t* __restrict__ keys_g) {
-    typedef RowStream<DP, TB_GROUP_MAX, kSharedU> Stream;
+    typedef RowStream<FragScorer<DP, TB_GROUP_MAX>, kSharedU, kWarps> Stream;
     constexpr int RB = DP * 2;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     int* hist = reinterpret_cast<int*>(smem_raw);                                 // [g][kDigitBins]
@@ -828,17 +822,6 @@ __global__ void __launch_bounds__(kThreads, 2)
 }
 
 namespace {
-
-// The pairs of a launch, longest first, and their candidates; returns the most.
-int longest_first(const UnitTable& ut, const SelectArgs& a, WaveOrder& order, int (&cand)[kMaxLaunchUnits]) {
-    const int n_pairs = ut.layer_count * ut.n_seq;
-    for (int i = 0; i < n_pairs; ++i) {
-        const int L = ut.len[i], lo = a.sinks < L ? a.sinks : L, hi = L - a.recent > lo ? L - a.recent : lo;
-        cand[i] = hi - lo, order.pair[i] = (uint16_t)i;
-    }
-    std::stable_sort(order.pair, order.pair + n_pairs, [&](uint16_t x, uint16_t y) { return cand[x] > cand[y]; });
-    return cand[order.pair[0]];
-}
 
 // The arguments of a launch that can fetch neighbours (`room` bytes on chip for two bitmasks) and copy the lists itself, or
 // that leaves both to the kernels after it.

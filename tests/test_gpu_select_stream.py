@@ -1,0 +1,84 @@
+"""The streaming selection kernel at the sizes where it can go wrong: shares of a cluster, rows past the last whole group of
+32, ragged batches with problems that have nothing to rank, blocks that keep digits instead of scores, the two block sizes,
+crowded bins, ties and infinities.  Keys and queries are small whole numbers, so every score is exact and every list is the
+oracle's, whatever the order of the sums."""
+import numpy as np
+import pytest
+import torch
+
+pytestmark = pytest.mark.gpu
+
+from test_gpu_parity import H, tb  # noqa: E402,F401
+
+# heads, group, lengths, d', dtype, reduce, budget, sinks, recent, radius, mode, data
+CASES = [
+    (1, 1, [10241], 32, "bf16", "sum", 700, 0, 0, 0, 0, "int"),                    # ten blocks, one row past a group
+    (2, 4, [12345, 10500, 3, 700], 32, "bf16", "sum", 900, 4, 16, 0, 0, "int"),    # ragged: everything, and less than a block's share
+    (8, 4, [32768], 32, "bf16", "max", 3276, 0, 0, 0, 0, "int"),
+    (8, 1, [16411, 16384], 16, "bf16", "sum", 300, 16, 64, 1, 0, "int"),           # neighbours across the blocks' borders
+    (4, 2, [20000, 11111], 32, "fp32", "sum", 2000, 3, 5, 2, 1, "int"),
+    (4, 8, [15001], 16, "fp32", "max", 7000, 0, 0, 0, 0, "int"),                   # threshold near zero score
+    (8, 4, [11000] * 20, 32, "bf16", "sum", 1100, 0, 0, 1, 1, "int"),              # 160 problems: blocks of 256 threads
+    (8, 1, [21003] + [17000] * 19, 32, "bf16", "sum", 3000, 0, 0, 0, 0, "int"),    # ... that keep digits
+    (8, 1, [2050] * 20, 32, "fp32", "sum", 200, 0, 0, 0, 0, "int"),
+    (8, 1, [47009] * 10, 32, "bf16", "sum", 5000, 0, 0, 0, 0, "int"),              # one block of 512 threads, digits
+    (2, 4, [40000], 32, "bf16", "sum", 1234, 0, 0, 0, 0, "ties"),
+    (8, 1, [47000] * 10, 16, "bf16", "max", 2345, 0, 0, 0, 0, "ties"),             # ... from the rows again
+    (2, 1, [30000], 32, "fp32", "sum", 29990, 0, 0, 0, 0, "ties"),
+    (2, 2, [30000], 32, "bf16", "sum", 40, 0, 0, 0, 0, "outliers"),                # the sampled bracket ends far below the threshold
+    (8, 1, [47000] * 10, 32, "bf16", "sum", 100, 0, 0, 0, 0, "outliers"),
+    (2, 2, [20000], 32, "bf16", "sum", 50, 0, 0, 0, 0, "inf"),
+    (2, 2, [20000], 16, "bf16", "max", 50, 0, 0, 0, 0, "inf"),
+]
+
+
+@pytest.mark.parametrize("ci", range(len(CASES)))
+def test_lists_are_the_oracles(H, ci):
+    b_ = tb()
+    heads, g, lens, dp, dt, reduce, budget, sinks, recent, radius, mode, data = CASES[ci]
+    dtype = b_.TB_BF16 if dt == "bf16" else b_.TB_F32
+    store = b_.torch_dtype(dtype)
+    red = b_.TB_GROUP_SUM if reduce == "sum" else b_.TB_GROUP_MAX
+    B = len(lens)
+    ctx = b_.Context(1, heads * g, heads, 128, dp, dtype, B, -(-max(lens) // 64) * 64, budget, radius)
+    ctx.set_projection(0, torch.zeros(heads, 128, dp, dtype=store, device="cuda"))
+    rows = torch.zeros(sum(lens), heads, 128, dtype=store, device="cuda")
+    ctx.append_kv(0, 1, None, lens, rows, rows)
+    ctx.project_keys(0, 1, None, [0] * B, lens)
+    del rows
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(ci)
+    x = torch.randn(ctx.kimp.shape, generator=gen, device="cuda")
+    x = (x.mul_(1.0).round_() if data == "ties" else x.mul_(40).round_()).clamp_(-120, 120)
+    q = torch.randn(1, B, heads * g, dp, generator=gen, device="cuda").mul_(20).round_().clamp_(-60, 60)
+    if data == "ties":                                   # whole numbers below 2 dp: thousands share a score
+        q = q.sign()
+    if data == "outliers":                               # more rows than are wanted score far above all others, close together
+        for b, L in enumerate(lens):
+            at = torch.randint(0, L, (budget + 800,), generator=gen, device="cuda")
+            up = q[0, b].view(heads, g, dp).sum(1).sign().unsqueeze(1) * 120
+            x[0, b][:, at] = up + torch.randint(-3, 4, (heads, len(at), dp), generator=gen, device="cuda")
+    if data == "inf":
+        x[0, 0, :, 1000:20000:997, 3] = float("inf")     # of either sign once multiplied: every row's other products are finite
+        q[..., 3] = q[..., 3].abs() + 1
+    ctx.kimp.copy_(x.to(store))
+    idx = torch.zeros(1, B, heads, ctx.index_capacity, dtype=torch.int32, device="cuda")
+    cnt = torch.zeros(1, B, heads, dtype=torch.int32, device="cuda")
+    for copied in (True, False):                         # the caller's copy, and the stored lists
+        p = b_.select_params(budget, sinks, recent, radius, mode, 2, 0 if copied else 1, red)
+        if copied:
+            ctx.select_topk(0, 1, None, B, q, p, idx, cnt)
+        else:
+            idx.zero_(), cnt.zero_()
+            ctx.select_topk(0, 1, None, B, None, p, idx, cnt)
+        assert ctx.get_status() == 0
+        got_n, got = cnt.cpu().numpy(), idx.cpu().numpy()
+        for b in range(0, B, 1 if copied else max(1, B - 1)):
+            for h in range(heads):
+                s = (ctx.kimp[0, b, h, :lens[b]].double() @ q[0, b, h * g:(h + 1) * g].double().T)
+                s = (s.sum(1) if reduce == "sum" else s.max(1).values).cpu().numpy()
+                want = H.orc.select(s, sinks, recent, budget)
+                lo, hi = H.orc.candidate_range(lens[b], sinks, recent)
+                if radius and len(want) < hi - lo:
+                    want = H.orc.neighbors(want, radius, mode, lo, hi)
+                assert np.array_equal(got[0, b, h, :got_n[0, b, h]], want), (b, h)
