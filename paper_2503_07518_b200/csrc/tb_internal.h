@@ -205,7 +205,7 @@ cudaError_t launch_score(const tb_ctx* c, const UnitTable& ut, const float* q_im
 cudaError_t launch_select(const tb_ctx* c, const UnitTable& ut, const SelectArgs& a, cudaStream_t s, bool dry, bool* finished);
 // one block per problem; launch_select hands over to it when a launch holds at least two problems per SM
 cudaError_t launch_select_wave(const tb_ctx* c, const UnitTable& ut, const SelectArgs& a, cudaStream_t s, bool dry, bool* finished);
-// several lists per key stream (bf16, one list per query head): a cluster per stream
+// several lists per key stream (bf16, one list per query head), many and long: a cluster per stream
 cudaError_t launch_select_shared(const tb_ctx* c, const UnitTable& ut, const SelectArgs& a, cudaStream_t s, bool dry, bool* finished);
 // small problems: one block each, neighbours and the caller's copy of the list included; whether a launch whose longest
 // problem has max_cand candidates is its kind (not whether the caller wants copies: they must not change the lists)

@@ -725,9 +725,14 @@ cudaError_t launch_select(const tb_ctx* c, const UnitTable& ut, const SelectArgs
     const bool to_wave = 2 * n_units >= 3 * c->sm_count || (n_units > c->sm_count && max_cand <= 20 * 1024) || max_cand > kCwLimit;
     const bool to_cw = max_cand > cw_from && max_cand <= kCwLimit;
     if (c->drop_tile >= 0 && (to_wave || to_cw)) return cudaErrorInvalidConfiguration;   // wait diagnostics: single-block launches of this kernel only
-    // Lists that share a key stream read it once.
-    if (gm.dtype == TB_BF16 && gm.Hl > gm.Hi && c->drop_tile < 0) return launch_select_shared(c, ut, a, s, dry, finished);
-    if (c->drop_tile < 0) {
+    // Lists that share a key stream read it once where there are many and they are long.  Otherwise the others' reads are L2 hits
+    // and a block per list is done earlier (us, four lists per stream, this / one problem per list: 512 lists of 1000 24 / 9.7, 8000
+    // 47 / 41, 16000 65 / 71; 32 of 16000 27 / 12; seven lists: 448 of 10000 59 / 51, 16000 71 / 75).
+    const bool many = n_units > c->sm_count;
+    if (gm.dtype == TB_BF16 && gm.Hl > gm.Hi && c->drop_tile < 0 && (ut.use_dev_len || (many && max_cand > (gm.Hl > 4 * gm.Hi ? 14000 : 10000))))
+        return launch_select_shared(c, ut, a, s, dry, finished);
+    // (Replayed graphs in which many sequences grow keep the kernels whose room is the workspace's.)
+    if (c->drop_tile < 0 && !(many && ut.use_dev_len)) {
         bool taken;
         cudaError_t e = launch_select_stream(c, ut, a, s, dry, &taken);
         if (taken) return *finished = true, e;

@@ -20,15 +20,14 @@ namespace tb {
 
 namespace {
 
-constexpr int kThreads = 512;
-constexpr int kWarps = kThreads / 32;
 constexpr int kHalf = 256;          // rows of a tile = threads that score it
-constexpr int kMaxCand = 16384;     // one bitmask word per thread
 constexpr int kBins = 2048;
 constexpr int kMaxShare = 4;        // blocks that stream one problem
-constexpr int kMaxRank = kThreads;  // keys of the threshold bin that are ranked pairwise
 
+template <int kThreads>
 struct __align__(16) SmallSmem {
+    static constexpr int kWarps = kThreads / 32, kMaxCand = 32 * kThreads;   // one bitmask word per thread
+    static constexpr int kMaxRank = kThreads;   // keys of the threshold bin that are ranked pairwise
     int hist[kBins];
     uint32_t mask[kMaxCand / 32], mask_out[kMaxCand / 32];
     uint2 cand[kMaxRank];           // (key, candidate) of the threshold bin
@@ -44,14 +43,17 @@ __device__ __forceinline__ float key_score(uint32_t key) { return __uint_as_floa
 
 // The bin that holds the k-th largest of the histogrammed keys: all threads get it, with k' = k - keys in higher bins
 // and the bin's population.  1 <= k <= total.
-__device__ __forceinline__ void find_bin(SmallSmem* sm, int nbins, int k, int& bin, int& krem, int& count) {
+template <int kThreads>
+__device__ __forceinline__ void find_bin(SmallSmem<kThreads>* sm, int nbins, int k, int& bin, int& krem, int& count) {
+    constexpr int kPer = kBins / kThreads, kWarps = kThreads / 32;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    int b[4] = {0, 0, 0, 0};
-    if (tid * 4 < nbins) {
-        const int4 x = reinterpret_cast<const int4*>(sm->hist)[tid];
-        b[0] = x.x, b[1] = x.y, b[2] = x.z, b[3] = x.w;
+    int b[kPer], mine = 0;
+#pragma unroll
+    for (int i = 0; i < kPer; i += 4) {
+        const int4 x = tid * kPer < nbins ? reinterpret_cast<const int4*>(sm->hist + tid * kPer)[i / 4] : make_int4(0, 0, 0, 0);
+        b[i] = x.x, b[i + 1] = x.y, b[i + 2] = x.z, b[i + 3] = x.w;
+        mine += (x.x + x.y) + (x.z + x.w);
     }
-    const int mine = (b[0] + b[1]) + (b[2] + b[3]);
     const int incl = warp_incl_scan(mine, lane);
     if (lane == 31) sm->slots[warp] = incl;
     __syncthreads();
@@ -65,8 +67,8 @@ __device__ __forceinline__ void find_bin(SmallSmem* sm, int nbins, int k, int& b
     int run = total - below - mine;                    // keys in bins above this thread's
     if (run < k && k <= run + mine) {                  // exactly one thread
 #pragma unroll
-        for (int i = 3; i >= 0; --i) {
-            if (run < k && k <= run + b[i]) sm->bin = tid * 4 + i, sm->krem = k - run, sm->count = b[i];
+        for (int i = kPer - 1; i >= 0; --i) {
+            if (run < k && k <= run + b[i]) sm->bin = tid * kPer + i, sm->krem = k - run, sm->count = b[i];
             run += b[i];
         }
     }
@@ -81,8 +83,8 @@ struct NoStream {
 // bf16 rows: kU groups of 32 rows in flight per warp (see RowStream); fp32 rows (kU = 0): through a ring of n_stages tiles.
 // kShared: a cluster of blocks per problem streams it, block r the r-th run of share_tiles tiles, with keys and sums going
 // to block 0's shared memory; behind one cluster barrier block 0 finishes alone.
-template <typename T, int DP, int RED, int kU, bool kShared>
-__global__ void __launch_bounds__(kThreads, kU == 2 ? 2 : 1) select_small_kernel(const __grid_constant__ CUtensorMap tmap,
+template <typename T, int DP, int RED, int kU, bool kShared, int kThreads>
+__global__ void __launch_bounds__(kThreads, kU == 2 ? 1024 / kThreads : 1) select_small_kernel(const __grid_constant__ CUtensorMap tmap,
                                                                                  const unsigned char* __restrict__ kimp, Geom gm, UnitTable ut,
                                                                                  SelectArgs a, int n_stages, int max_tiles, int share_tiles, uint32_t wait_limit, int drop_tile,
                                                                                  int32_t* __restrict__ state_idx, int32_t* __restrict__ state_cnt,
@@ -93,7 +95,9 @@ __global__ void __launch_bounds__(kThreads, kU == 2 ? 2 : 1) select_small_kernel
     extern __shared__ unsigned char smem_raw[];
     unsigned char* ring = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);   // swizzled boxes start on the swizzle period
     uint32_t* keys = reinterpret_cast<uint32_t*>(ring + n_stages * kTileBytes);          // max_tiles * 256
-    SmallSmem* sm = reinterpret_cast<SmallSmem*>(keys + max_tiles * kHalf);
+    typedef SmallSmem<kThreads> Smem;
+    constexpr int kWarps = Smem::kWarps, kMaxRank = Smem::kMaxRank;
+    Smem* sm = reinterpret_cast<Smem*>(keys + max_tiles * kHalf);
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
 
     uint32_t C = 1, rank = 0;
@@ -110,7 +114,7 @@ __global__ void __launch_bounds__(kThreads, kU == 2 ? 2 : 1) select_small_kernel
         if (lane < n_stages) mbar_init(&sm->full[lane], 1), fence_mbar_init();   // (14 stages at most: 16 KB tiles)
         __syncwarp();                                  // thread 0 arms them and requests the first tiles before any block barrier
     }
-    reinterpret_cast<int4*>(sm->hist)[tid] = make_int4(0, 0, 0, 0);
+    for (int i = tid; i < kBins / 4; i += kThreads) reinterpret_cast<int4*>(sm->hist)[i] = make_int4(0, 0, 0, 0);
     int ll, s, h;
     decode_unit(gm, ut, unit, ll, s, h);
     const size_t cu = list_unit(gm, ut, ll, s, h);
@@ -282,7 +286,7 @@ __global__ void __launch_bounds__(kThreads, kU == 2 ? 2 : 1) select_small_kernel
 #pragma unroll 1
         for (int pass = 0; pass < 3; ++pass) {
             const int bits = pass == 2 ? 10 : 11, shift = low_bits - bits;
-            reinterpret_cast<int4*>(sm->hist)[tid] = make_int4(0, 0, 0, 0);
+            for (int i = tid; i < kBins / 4; i += kThreads) reinterpret_cast<int4*>(sm->hist)[i] = make_int4(0, 0, 0, 0);
             __syncthreads();
             for (int i = tid; i < ncand; i += kThreads) {
                 const uint32_t key = keys[i];
@@ -313,18 +317,20 @@ __global__ void __launch_bounds__(kThreads, kU == 2 ? 2 : 1) select_small_kernel
     finish_mask_list<kThreads>(sm->mask, sm->mask_out, ncand, lo, out, sm->slots);
 }
 
-size_t small_smem(int n_stages, int n_tiles, int tile_bytes) {
-    return 1024 + (size_t)n_stages * tile_bytes + (size_t)n_tiles * kHalf * 4 + sizeof(SmallSmem);
+size_t small_smem(int n_stages, int n_tiles, int tile_bytes, int threads = 512) {
+    return 1024 + (size_t)n_stages * tile_bytes + (size_t)n_tiles * kHalf * 4 + (threads == 512 ? sizeof(SmallSmem<512>) : sizeof(SmallSmem<256>));
 }
 
 }  // namespace
 
-// Launches of up to two blocks per SM, as long as one block's finish is cheaper than a cluster's.  Against the streaming kernel,
+// As long as one block's finish is cheaper than a cluster's.  Against the streaming kernel,
 // us per launch, bf16, 32 dimensions unless said (this / the other): 8 problems of 4000 candidates 7.6 / 9.8, 10000 11.1 / 11.1, 32
 // of 8000 11.1 / 12.1, with neighbours 14.3 / 15.3 and 16000 20.9 / 18.5; more problems than half of the SMs leave the other
 // one block each too: 96 of 8000 15.8 / 16.8, 16000 26.6 / 26.8, fp32 42.1 / 44.1; two per SM: 192 of 6000 20.6 / 21.7, 8000
 // 25.4 / 26.3, with neighbours 160 of 12000 51 / 40; fp32, whose rows do not go straight into registers here, 160 of 4000 32 /
-// 25, 2000 20 / 15.6.  384 problems, a second wave: level with one block of 256 threads each, or worse.
+// 25, 2000 20 / 15.6.  More than two problems per SM: against the kernel of one 256-thread block each that parks its keys in memory,
+// 512 of 300 8.2 / 11.6, 1000 11.6 / 15.5, 4900 36.7 / 38.8, ragged to 4900 30.7 / 32.3, 6000 42.6 / 44.1, 8000 61 / 58; 2048 of 1000 36
+// / 46; lists that share a key stream, whose rows are L2 hits for all but one, 512 of 8000 41 / 47.
 // Whether the caller wants copies does not matter: the scores are summed in another order here, and an output that the caller
 // may leave out must not decide which of two tokens within fp32 rounding of one another is stored.
 bool select_small_takes(const tb_ctx* c, const UnitTable& ut, int max_cand) {
@@ -332,8 +338,10 @@ bool select_small_takes(const tb_ctx* c, const UnitTable& ut, int max_cand) {
     // wait diagnostics: launches of one block that wait for copies (the others: see launch_select)
     if (c->drop_tile >= 0 && (c->geom.dtype == TB_BF16 || n_units > 1 || max_cand > 1023)) return false;
     if (n_units > c->sm_count && c->geom.dtype != TB_BF16 && c->drop_tile < 0) return max_cand <= 1500;
-    const int most = n_units <= c->sm_count ? (2 * n_units > c->sm_count ? kMaxCand : 10 * 1024) : 8 * 1024;
-    return n_units <= 2 * c->sm_count && max_cand <= most;
+    const int most = n_units <= c->sm_count ? (2 * n_units > c->sm_count ? SmallSmem<512>::kMaxCand : 10 * 1024) : 8 * 1024;
+    if (n_units > 2 * c->sm_count)                     // (replayed graphs in which these sequences grow: the kernel whose room is the workspace's)
+        return c->drop_tile < 0 && !ut.use_dev_len && max_cand <= (c->geom.Hl > c->geom.Hi ? SmallSmem<256>::kMaxCand : 5000);
+    return max_cand <= most;
 }
 
 cudaError_t launch_select_small(const tb_ctx* c, const UnitTable& ut, const SelectArgs& a, int max_cand, cudaStream_t s, bool dry) {
@@ -354,6 +362,9 @@ cudaError_t launch_select_small(const tb_ctx* c, const UnitTable& ut, const Sele
     int C = 1;
     while (2 * C <= kMaxShare && 2 * C * n_units <= c->sm_count && n_tiles >= 2 * C * 4) C *= 2;
     const int share_tiles = (n_tiles + C - 1) / C;
+    // Short lists, or more than fit the chip with 512 threads each: blocks of 256, four per SM (160 problems of 1000 candidates
+    // 7.6 us, 8.6 with 512 threads, 2000 level, 4000 15.6 / 14.7; 512 of 1000 11.5 / 17.1).
+    const int threads = direct && (n_units > 2 * c->sm_count || (!alone && max_cand <= 2048)) ? 256 : 512;
     int n_stages = direct ? 0 : share_tiles;
     if (small_smem(n_stages, n_tiles, tile_bytes) > room) {
         n_stages &= ~1;                                // even: see the stream loop
@@ -361,8 +372,8 @@ cudaError_t launch_select_small(const tb_ctx* c, const UnitTable& ut, const Sele
     }
 
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(n_units * C, 1, 1), cfg.blockDim = dim3(kThreads, 1, 1), cfg.stream = s;
-    cfg.dynamicSmemBytes = small_smem(n_stages, n_tiles, tile_bytes);
+    cfg.gridDim = dim3(n_units * C, 1, 1), cfg.blockDim = dim3(threads, 1, 1), cfg.stream = s;
+    cfg.dynamicSmemBytes = small_smem(n_stages, n_tiles, tile_bytes, threads);
     cudaLaunchAttribute attr[2];
     attr[1].id = cudaLaunchAttributeClusterDimension;
     attr[1].val.clusterDim.x = C, attr[1].val.clusterDim.y = 1, attr[1].val.clusterDim.z = 1;
@@ -378,18 +389,19 @@ cudaError_t launch_select_small(const tb_ctx* c, const UnitTable& ut, const Sele
                                   c->st.idx, c->st.cnt, c->st.status);
     };
     // a block alone on its SM keeps four groups of rows in flight per warp, two blocks two each (their registers)
-#define TB_SMALL(T, DP, RED, U, SH)                                    \
-    do {                                                               \
-        static unsigned char seen[64];                                 \
-        return launch(select_small_kernel<T, DP, RED, U, SH>, seen);   \
+#define TB_SMALL(T, DP, RED, U, SH, NT)                                    \
+    do {                                                                   \
+        static unsigned char seen[64];                                     \
+        return launch(select_small_kernel<T, DP, RED, U, SH, NT>, seen);   \
     } while (0)
-#define TB_SMALL_U(DP, RED)                                                 \
-    do {                                                                    \
-        if (direct && C > 1) TB_SMALL(__nv_bfloat16, DP, RED, 4, true);     \
-        if (direct && alone) TB_SMALL(__nv_bfloat16, DP, RED, 4, false);    \
-        if (direct) TB_SMALL(__nv_bfloat16, DP, RED, 2, false);             \
-        if (C > 1) TB_SMALL(float, DP, RED, 0, true);                       \
-        TB_SMALL(float, DP, RED, 0, false);                                 \
+#define TB_SMALL_U(DP, RED)                                                      \
+    do {                                                                         \
+        if (direct && C > 1) TB_SMALL(__nv_bfloat16, DP, RED, 4, true, 512);     \
+        if (direct && alone) TB_SMALL(__nv_bfloat16, DP, RED, 4, false, 512);    \
+        if (direct && threads == 256) TB_SMALL(__nv_bfloat16, DP, RED, 2, false, 256); \
+        if (direct) TB_SMALL(__nv_bfloat16, DP, RED, 2, false, 512);             \
+        if (C > 1) TB_SMALL(float, DP, RED, 0, true, 512);                       \
+        TB_SMALL(float, DP, RED, 0, false, 512);                                 \
     } while (0)
     const bool max = a.reduce == TB_GROUP_MAX;
     if (gm.dp == 32) {

@@ -599,8 +599,9 @@ cudaError_t launch_select_stream(const tb_ctx* c, const UnitTable& ut, const Sel
         else take = !f32 && (max || narrow) && max_cand >= 16000;
         if (!take) return cudaSuccess;
     }
-    l.room = ((max_cand + C - 1) / C + 127) / 128 * 128;
-    l.most = a.radius > 0 ? max_cand : C * l.room;     // (a replayed graph may find more)
+    const int spare = ut.use_dev_len && a.radius == 0 ? 2048 : 0;   // a replayed graph may find more than it declared
+    l.room = ((max_cand + spare + C - 1) / C + 127) / 128 * 128;
+    l.most = a.radius > 0 ? max_cand : C * l.room;
     const int per_sm = 512 / threads;
     auto smem = [&](bool scores) { return stream_smem(threads, C, l.room, a.radius > 0, scores); };
     if ((C > 1 && l.room > kMaxShare) || smem(false) > 226 * 1024 / per_sm) return cudaSuccess;
