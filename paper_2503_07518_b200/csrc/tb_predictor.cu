@@ -232,11 +232,11 @@ __global__ void __launch_bounds__(kPredThreads) predictor_out_kernel(const T* __
 // weights, about what an SM receives in a memory latency, so that an 8B-shaped linear (8 MB) is 128 blocks that
 // request everything they need at once -- against all tokens of the call.  The tensor pipe is idle most of the time
 // and latency is what there is to save: every thread's weights are in flight before it looks at the tokens.
-// Measured, one call of a 4096 -> 512 -> 4096 predictor in a chain of them: 7.2 us with 1 token, 7.2 with 8, 11.9 with
-// 24, 31 with 64, of which 1.3 are the weights at the copy bandwidth.  (Before: 8.8 with a warp pair per hidden unit and
-// 18.7, 31.9, 61 with 16-token left tiles whose blocks each normalised every token.)  The weights go through shared
+// Measured, one call of a 4096 -> 512 -> 4096 predictor in a chain of them: 7.2 us with 1 token, 7.0 with 8, 7.7 with 16, 10.7
+// with 24, 13.3 with 47, 22 with 64, of which 1.3 are the weights at the copy bandwidth.  (With the token groups one after the
+// other in the same blocks, as large as 32: 9.5 with 16, 12.0 with 24, 20.6 with 47, 31 with 64.)  The weights go through shared
 // memory because their copies then cost no registers: with the fragments loaded straight into registers the kernels
-// spilled and ran at 11.3 us.  Two blocks must fit an SM (they do up to 24 staged tokens; with 32 staged one does): the output kernel's blocks sit beside the hidden kernel's and
+// spilled and ran at 11.3 us.  Two blocks must fit an SM (they do up to 24 tokens): the output kernel's blocks sit beside the hidden kernel's and
 // have their weights before the hidden units exist, and at one block per SM only 15 of the 16 clusters start at once.
 //
 // The 16 k-indices of an MMA step are mapped to channels so that every thread's operands are 16 contiguous bytes:
@@ -245,7 +245,8 @@ __global__ void __launch_bounds__(kPredThreads) predictor_out_kernel(const T* __
 // same mapping, so the sum over channels is unchanged.
 constexpr int kTileRows = 32;        // weight rows of a block
 constexpr int kChunk = 512;          // channels of a block's tile: 4 warps x 4 runs of 32, for each of two 16-row halves
-constexpr int kTileTokMax = 32;      // tokens staged at once; a kernel instance stages 8 * kN8 of them
+constexpr int kTileTokMax = 24;      // tokens of a group; a kernel instance takes 8 * kN8 of them
+constexpr int kTwoPerSm = 76 * 1024; // shared memory of which two blocks' worth fits an SM and three do not
 constexpr int kXPitch = kChunk * 2 + 64;   // bytes per (term, token) row: eight rows' 64-byte pieces hit all banks twice
 constexpr int kClusterK = 8;         // blocks (one cluster) that share the channels of a hidden-unit tile
 
@@ -345,7 +346,7 @@ __device__ __forceinline__ float get_sum(const TileSums<kN8>& s, int row, int to
 //     sum = rstd * sum_b (P_b - (mean - s_b) G_b) + sum_b B_b
 // where mean - s_b is small against the spread, so nothing cancels.  Blocks are summed in rank order.
 template <int kTerms, int kN8>
-__global__ void __launch_bounds__(kPredThreads, 2) predictor_hidden_tile_kernel(const __nv_bfloat16* __restrict__ H,
+__global__ void __launch_bounds__(kPredThreads, kN8 == 1 ? 3 : 2) predictor_hidden_tile_kernel(const __nv_bfloat16* __restrict__ H,
                                                                                 const __nv_bfloat16* __restrict__ ln_w,
                                                                                 const __nv_bfloat16* __restrict__ ln_b,
                                                                                 const __nv_bfloat16* __restrict__ W1,
@@ -362,11 +363,10 @@ __global__ void __launch_bounds__(kPredThreads, 2) predictor_hidden_tile_kernel(
     unsigned char* xs = ws + kWBytes;
     __shared__ TileSums<kN8> s_sum;
     __shared__ float2 s_gb[4][kTileRows];              // (G, B) of the block's rows, per channel quarter
-    // from every block of the cluster (a buffer per token group): P and (G, B) of this block's rows, and every token's
-    // (shift, shifted sum, shifted sum of squares)
-    __shared__ float s_p[2][kClusterK][kRows][kTileTok];
+    // from every block of the cluster: P and (G, B) of this block's rows, and every token's (shift, shifted sum, shifted sum of squares)
+    __shared__ float s_p[kClusterK][kRows][kTileTok];
     __shared__ float2 s_gb_all[kClusterK][kRows];
-    __shared__ float4 s_stat[2][kClusterK][kTileTok];
+    __shared__ float4 s_stat[kClusterK][kTileTok];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, gid = lane >> 2, tig = lane & 3;
     const int j0 = blockIdx.y * kTileRows;
     const int span = (((E + 31) / 32 + kClusterK - 1) / kClusterK) * 32;     // channels of a block
@@ -380,18 +380,16 @@ __global__ void __launch_bounds__(kPredThreads, 2) predictor_hidden_tile_kernel(
     pdl_launch_dependents();
     pred_stamp(0, 1);
 
-    for (int t0 = 0, group = 0; t0 < n_tok; t0 += kTileTok, ++group) {
-        const int n_here = min(kTileTok, n_tok - t0);
+    const int t0 = blockIdx.z * kTileTok, n_here = min(kTileTok, n_tok - t0);   // this cluster's tokens
+    {
         float acc[kAccs<kN8>][4] = {}, gb[4] = {};
         float shift[kOwn], s1[kOwn], s2[kOwn];
 #pragma unroll
         for (int i = 0; i < kOwn; ++i) shift[i] = s1[i] = s2[i] = 0.f;
         for (int kc = 0; kc < n_chunk; ++kc) {
             const int c0 = c_begin + kc * kChunk;
-            if (n_chunk > 1 || group == 0) {
-                if (kc + group) __syncthreads();       // the previous chunk's operands have been read
-                request_weights(ws, W1, hid, E, j0, c0, c_end);
-            }
+            if (kc) __syncthreads();                   // the previous chunk's operands have been read
+            request_weights(ws, W1, hid, E, j0, c0, c_end);
             // A warp looks after tokens warp, warp + 8, ... of the group, a lane after channels 8 lane .. + 7 and
             // 256 + 8 lane .. + 7 of the chunk.
             uint4 hv[kOwn][2], gv[2];
@@ -409,13 +407,11 @@ __global__ void __launch_bounds__(kPredThreads, 2) predictor_hidden_tile_kernel(
             }
             // right operand of the G, B product: column 0 = layer-norm weights, column 1 = biases
             uint4 gbx[4];
-            if (group == 0) {
-                const __nv_bfloat16* src = gid == 0 ? ln_w : ln_b;
+            const __nv_bfloat16* src = gid == 0 ? ln_w : ln_b;
 #pragma unroll
-                for (int r = 0; r < 4; ++r) {
-                    const int c = c0 + ((warp & 3) * 4 + r) * 32 + 8 * tig;
-                    gbx[r] = gid < 2 && c < c_end ? __ldg(reinterpret_cast<const uint4*>(src + c)) : zero;
-                }
+            for (int r = 0; r < 4; ++r) {
+                const int c = c0 + ((warp & 3) * 4 + r) * 32 + 8 * tig;
+                gbx[r] = gid < 2 && c < c_end ? __ldg(reinterpret_cast<const uint4*>(src + c)) : zero;
             }
             if (kc == 0) {
                 const int n = min(kChunk, c_end - c0);
@@ -455,22 +451,21 @@ __global__ void __launch_bounds__(kPredThreads, 2) predictor_hidden_tile_kernel(
             wait_weights();
             __syncthreads();
             pred_stamp(0, 2);
-            if (group == 0) mma_tile<kTerms, kN8, true>(acc, ws, xs, gb, gbx);
-            else mma_tile<kTerms, kN8, false>(acc, ws, xs, nullptr, nullptr);
+            mma_tile<kTerms, kN8, true>(acc, ws, xs, gb, gbx);
         }
         put_sums<kN8>(s_sum, acc);
-        if (group == 0 && tig == 0) {
+        if (tig == 0) {
             s_gb[warp & 3][(warp >> 2) * 16 + gid] = make_float2(gb[0], gb[1]);
             s_gb[warp & 3][(warp >> 2) * 16 + gid + 8] = make_float2(gb[2], gb[3]);
         }
         __syncthreads();
         pred_stamp(0, 3);
-        if (group == 0) asm volatile("barrier.cluster.wait.aligned;" ::: "memory");
+        asm volatile("barrier.cluster.wait.aligned;" ::: "memory");
         for (int e = tid; e < kTileRows * kTileTok; e += kPredThreads) {
             const int row = e / kTileTok, tok = e % kTileTok;
-            if (tok < n_here) *cluster.map_shared_rank(&s_p[group & 1][rank][row % kRows][tok], row / kRows) = get_sum<kN8>(s_sum, row, tok);
+            if (tok < n_here) *cluster.map_shared_rank(&s_p[rank][row % kRows][tok], row / kRows) = get_sum<kN8>(s_sum, row, tok);
         }
-        if (group == 0 && tid < kTileRows) {
+        if (tid < kTileRows) {
             const float2 a = s_gb[0][tid], b = s_gb[1][tid], c = s_gb[2][tid], d = s_gb[3][tid];
             *cluster.map_shared_rank(&s_gb_all[rank][tid % kRows], tid / kRows) = make_float2((a.x + b.x) + (c.x + d.x), (a.y + b.y) + (c.y + d.y));
         }
@@ -479,7 +474,7 @@ __global__ void __launch_bounds__(kPredThreads, 2) predictor_hidden_tile_kernel(
             const int tl = i * kPredWarps + warp;
             if (tl >= n_here) break;                   // warp-uniform
             const float a = warp_sum(s1[i]), b = warp_sum(s2[i]);
-            if (lane < kClusterK) *cluster.map_shared_rank(&s_stat[group & 1][rank][tl], lane) = make_float4(shift[i], a, b, 0.f);   // lane r tells block r
+            if (lane < kClusterK) *cluster.map_shared_rank(&s_stat[rank][tl], lane) = make_float4(shift[i], a, b, 0.f);   // lane r tells block r
         }
         pred_stamp(0, 4);
         cluster.sync();
@@ -491,7 +486,7 @@ __global__ void __launch_bounds__(kPredThreads, 2) predictor_hidden_tile_kernel(
                 float mean = 0.f;
 #pragma unroll
                 for (int r = 0; r < kClusterK; ++r) {
-                    st[r] = s_stat[group & 1][r][tok];
+                    st[r] = s_stat[r][tok];
                     const float n = (float)max(0, min(span, E - r * span));
                     mean += fmaf(n, st[r].x, st[r].y);
                 }
@@ -503,7 +498,7 @@ __global__ void __launch_bounds__(kPredThreads, 2) predictor_hidden_tile_kernel(
                     const float n = (float)max(0, min(span, E - r * span)), u = mean - st[r].x;
                     const float2 w = s_gb_all[r][row];
                     var += fmaf(u, fmaf(n, u, -2.f * st[r].y), st[r].z);
-                    sum += fmaf(-u, w.x, s_p[group & 1][r][row][tok]);
+                    sum += fmaf(-u, w.x, s_p[r][row][tok]);
                     bias += w.y;
                 }
                 const float rstd = rsqrtf(fmaxf(var / (float)E, 0.f) + eps);
@@ -523,7 +518,7 @@ __global__ void __launch_bounds__(kPredThreads, 2) predictor_hidden_tile_kernel(
 
 // q_imp for 32 output rows per block, all hidden units.
 template <int kTerms, int kN8>
-__global__ void __launch_bounds__(kPredThreads, 2) predictor_out_tile_kernel(const __nv_bfloat16* __restrict__ W2, const float* __restrict__ hidden,
+__global__ void __launch_bounds__(kPredThreads, kN8 == 1 ? 3 : 2) predictor_out_tile_kernel(const __nv_bfloat16* __restrict__ W2, const float* __restrict__ hidden,
                                                                           float* __restrict__ q_imp, int n_tok, int hid, int n_out,
                                                                           int per_slot) {
     extern __shared__ __align__(128) unsigned char ws[];   // weights [32 rows][kXPitch], then hidden units [term][token][kXPitch]
@@ -540,18 +535,17 @@ __global__ void __launch_bounds__(kPredThreads, 2) predictor_out_tile_kernel(con
     pdl_wait();
     pdl_launch_dependents();
     pred_stamp(1, 1);
-    for (int t0 = 0; t0 < n_tok; t0 += kTileTok) {
-        const int n_here = min(kTileTok, n_tok - t0);
+    const int t0 = blockIdx.y * kTileTok, n_here = min(kTileTok, n_tok - t0);   // this block's tokens
+    {
         float acc[kAccs<kN8>][4] = {};
         for (int kc = 0; kc < n_chunk; ++kc) {
-            if (n_chunk > 1 && t0 + kc) {
+            if (kc) {
                 __syncthreads();                       // the previous chunk's operands have been read
                 request_weights(ws, W2, n_out, hid, o0, kc * kChunk, hid);
             }
             constexpr int kVec = kChunk / 8, kStep = kPredThreads / kVec;      // 8 values at a time, four tokens per round
             const int c = kc * kChunk + tid % kVec * 8;
             if constexpr (kTerms == 2) {               // the hidden-unit kernel has split them
-                if (t0 + kc) __syncthreads();          // the previous operands have been read
 #pragma unroll
                 for (int i = 0; i < kTerms * kTileTok / kStep; ++i) {
                     const int row = i * kStep + tid / kVec, tl = row % kTileTok;
@@ -574,7 +568,6 @@ __global__ void __launch_bounds__(kPredThreads, 2) predictor_out_tile_kernel(con
                     x[i][0] = in ? __ldcg(src) : make_float4(0.f, 0.f, 0.f, 0.f);
                     x[i][1] = in ? __ldcg(src + 1) : make_float4(0.f, 0.f, 0.f, 0.f);
                 }
-                if (kc) __syncthreads();
 #pragma unroll
                 for (int i = 0; i < kTileTok / kStep; ++i) {
                     float v[8] = {x[i][0].x, x[i][0].y, x[i][0].z, x[i][0].w, x[i][1].x, x[i][1].y, x[i][1].z, x[i][1].w};
@@ -630,36 +623,57 @@ extern "C" tb_status tb_predict_importance_queries(const tb_predictor* p, const 
     cfg.attrs = attr;
     cudaError_t e;
     if (p->dtype == TB_BF16) {
-        // eights of tokens staged at once: all of the call's, or equal shares of at most 32
+        // The tokens go to the clusters (blocks) of grid layers in groups of 8, 16 or 24, the smallest for which the hidden kernel
+        // still runs at once: the preparation of a group is what its blocks' time grows with, and more groups read the weights
+        // from L2.  Otherwise as few groups as hold 24.  us per call, 4096 -> 512 -> 4096, groups of 8 / 16 / 24: 16 tokens 7.8 /
+        // 9.5 / 9.5, 24 10.7 / 11.8 / 11.8, 32 15 / 10.8 / 13.3, 47 19 / 18.4 / 13.3; with 1024 hidden units, twice the blocks, 32
+        // tokens 27 / 21.4 / 23.3, 64 48 / 38.6 / 33.9.
+        int n8 = 1;
+        bool two_per_sm = true;
+        if (n_tokens > 8) {
+            static int sm_counts[64];
+            int dev = 0, sms = 0;
+            if (cudaGetDevice(&dev) != cudaSuccess) return TB_ERR_CUDA;
+            if (dev < 64) sms = sm_counts[dev];
+            if (!sms && cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return TB_ERR_CUDA;
+            if (dev < 64) sm_counts[dev] = sms;
+            const int tiles = kClusterK * ((p->hidden_dim + kTileRows - 1) / kTileRows);
+            auto blocks = [&](int eights) { return tiles * ((n_tokens + 8 * eights - 1) / (8 * eights)); };
+            n8 = blocks(1) <= 3 * sms ? 1 : blocks(2) <= 2 * sms ? 2 : 3;
+            if (n8 == 3 && blocks(3) > 2 * sms) {
+                const int groups = (n_tokens + kTileTokMax - 1) / kTileTokMax;
+                n8 = ((n_tokens + groups - 1) / groups + 7) / 8;
+            }
+            two_per_sm = blocks(n8) <= 2 * sms;
+        }
         auto launch = [&](auto terms, auto eights) {
             constexpr int kTerms = decltype(terms)::value, kN8 = decltype(eights)::value;
-            constexpr int smem = kWBytes + kTerms * kN8 * 8 * kXPitch;
+            constexpr int used = kWBytes + kTerms * kN8 * 8 * kXPitch, smem = used > kTwoPerSm ? used : kTwoPerSm;
             static unsigned char seen[64];
             if (first_use_on_this_device(seen)) {
                 cudaError_t r = cudaFuncSetAttribute(predictor_hidden_tile_kernel<kTerms, kN8>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
                 if (r == cudaSuccess) r = cudaFuncSetAttribute(predictor_out_tile_kernel<kTerms, kN8>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
                 if (r != cudaSuccess) return r;
             }
-            cfg.dynamicSmemBytes = smem;
-            cfg.gridDim = dim3(kClusterK, (p->hidden_dim + kTileRows - 1) / kTileRows, 1), cfg.numAttrs = 2;
+            cfg.dynamicSmemBytes = two_per_sm ? smem : used;   // (blocks of eight tokens fit three times: uneven where two would do)
+            const unsigned n_groups = (unsigned)((n_tokens + kN8 * 8 - 1) / (kN8 * 8));
+            cfg.gridDim = dim3(kClusterK, (p->hidden_dim + kTileRows - 1) / kTileRows, n_groups), cfg.numAttrs = 2;
             cudaError_t r = cudaLaunchKernelEx(&cfg, predictor_hidden_tile_kernel<kTerms, kN8>, (const __nv_bfloat16*)hidden_dev,
                                                (const __nv_bfloat16*)p->ln_weight, (const __nv_bfloat16*)p->ln_bias,
                                                (const __nv_bfloat16*)p->w1, scratch_dev, (int)n_tokens, (int)p->model_dim,
                                                (int)p->hidden_dim, p->ln_eps, (int)p->activation);
             if (r != cudaSuccess) return r;
-            cfg.gridDim = dim3((unsigned)((n_out + kTileRows - 1) / kTileRows), 1, 1), cfg.numAttrs = 1;
+            cfg.gridDim = dim3((unsigned)((n_out + kTileRows - 1) / kTileRows), n_groups, 1), cfg.numAttrs = 1;
             return cudaLaunchKernelEx(&cfg, predictor_out_tile_kernel<kTerms, kN8>, (const __nv_bfloat16*)p->w2, (const float*)scratch_dev,
                                       q_imp_dev, (int)n_tokens, (int)p->hidden_dim, n_out_i, per_slot);
         };
-        const int groups = (n_tokens + kTileTokMax - 1) / kTileTokMax, n8 = ((n_tokens + groups - 1) / groups + 7) / 8;
         using std::integral_constant;
         // 24 bits of both right operands for up to four tokens, and for shapes off the 32-channel runs (always computed so)
         const bool whole = n_tokens < 5 || p->model_dim % 32 || p->hidden_dim % 32 || n_out % 8;
         if (whole) e = launch(integral_constant<int, 3>{}, integral_constant<int, 1>{});
         else if (n8 == 1) e = launch(integral_constant<int, 2>{}, integral_constant<int, 1>{});
         else if (n8 == 2) e = launch(integral_constant<int, 2>{}, integral_constant<int, 2>{});
-        else if (n8 == 3) e = launch(integral_constant<int, 2>{}, integral_constant<int, 3>{});
-        else e = launch(integral_constant<int, 2>{}, integral_constant<int, 4>{});
+        else e = launch(integral_constant<int, 2>{}, integral_constant<int, 3>{});
     } else {
         const int g1 = (p->hidden_dim + kPredWarps / 2 - 1) / (kPredWarps / 2), g2 = (int)((n_out + kPredWarps - 1) / kPredWarps);
         int stage_tok = (int)(48 * 1024 / (p->hidden_dim * sizeof(float))) / kTokChunk * kTokChunk;   // hidden_dim <= 1536 gives >= 8
