@@ -79,11 +79,11 @@ struct Slices {
     __device__ __forceinline__ uint32_t linear_bin(float score) const { return __float2uint_rz(place(score)); }   // (below 0 becomes 0)
     __device__ __forceinline__ uint32_t key_bin(uint32_t key) const { return min((max(key, base) - base) >> shift, (uint32_t)(kBins - 1)); }
     __device__ __forceinline__ uint32_t bin(float score) const { return linear() ? linear_bin(score) : key_bin(order_key(score)); }
-    // from the keys of the sample scores that bracket the threshold: twice as much again above the highest, since of 64 rows
+    // from the keys of the sample scores that bracket the threshold; `reach` times as far up as they are apart, since of 64 rows
     // none may be in the upper 2 %
-    __device__ __forceinline__ void bracket(uint32_t s_lo, uint32_t s_hi) {
+    __device__ __forceinline__ void bracket(uint32_t s_lo, uint32_t s_hi, float reach) {
         const float lo = key_score(s_lo), width = key_score(s_hi) - lo;
-        scale = (float)(kBins - 2) / (3.f * width), off = 1.f - lo * scale;
+        scale = (float)(kBins - 2) / (reach * width), off = 1.f - lo * scale;
         if (!(scale > 0.f && is_finite(scale) && is_finite(off))) scale = 1.f, off = 0.f;   // equal, infinite: any slices will do
         shift = -1;
     }
@@ -95,9 +95,15 @@ struct Slices {
         base = from - min(from, 1u << shift);
     }
     __device__ __forceinline__ bool one_key(int b) const { return shift == 0 && b < kBins - 1 && (b > 0 || base == 0u); }
-    // finer slices for bin b (not one_key).  A slice of score ends at about these keys; should the threshold be beyond, the next
-    // cut finds it in the open bin there.
+    // Finer slices for bin b (not one_key).  Above or below the bracket: first twice the bracket, further on, which is where the
+    // threshold will be.  A slice of score ends at about these keys; should the threshold be beyond, the next cut finds it in the
+    // open bin there.
     __device__ __forceinline__ void cut(int b) {
+        const float next = b == 0 ? off * 0.5f + (float)(kBins - 2) : off * 0.5f - (float)(kBins - 4) * 0.5f;
+        if (shift == -1 && (b == 0 || b == kBins - 1) && is_finite(next)) {
+            scale *= 0.5f, off = next, shift = -2;
+            return;
+        }
         uint32_t from = base + ((uint32_t)b << (shift & 31)), last = from + ((1u << (shift & 31)) - 1u);
         if (linear()) from = order_key(((float)b - 0.01f - off) / scale), last = max(from, order_key(((float)b + 1.01f - off) / scale));
         cover(b == 0 ? 0u : from, b == kBins - 1 ? 0xffffffffu : last);
@@ -266,7 +272,7 @@ __global__ void __launch_bounds__(kThreads, 512 / kThreads) select_stream_kernel
         }
     }
     __syncthreads();
-    sl.bracket(sm->s_lo, sm->s_hi);
+    sl.bracket(sm->s_lo, sm->s_hi, mean < 3.f ? 4.5f : 3.f);
 
     // ---- rounds: one, hardly ever more ---------------------------------------------------------------------------------
     DigitCounter counter;
