@@ -38,10 +38,10 @@ UNIT = "tokens/s"
 # dram__bytes_read.sum + dram__bytes_write.sum per launch of the dominant kernel, from the ncu
 # captures summarised under profiles/ (None until a capture exists for that workload).
 NCU_TRAFFIC_BYTES = {
-    ("cfg2_llama8b_32k", "select_kernel"): 67_221_760 + 848_896,   # profiles/select_kernel_cfg2_32k.md
+    ("cfg2_llama8b_32k", "select_kernel"): 67_198_464 + 216_576,   # profiles/select_stream_kernel.md
     ("cfg2_llama8b_32k", "attn_kernel"): 13_598_208,               # profiles/attn_mma_kernel_cfg2_32k.md
-    ("cfg3_batched_serving", "select_kernel"): 398_907_392 + 5_187_840,   # profiles/select_wave_kernel_cfg3_batched.md
-    ("cfg4_long_context_128k", "select_kernel"): 268_011_264 + 3_980_544,  # profiles/select_cw_kernel_cfg4_128k.md
+    ("cfg3_batched_serving", "select_kernel"): 396_212_480 + 4_382_208,   # profiles/select_stream_kernel.md
+    ("cfg4_long_context_128k", "select_kernel"): 268_140_032 + 3_217_664,  # profiles/select_stream_kernel.md
     ("cfg5_interval_neighbors", "attn_kernel"): 309_490_432 + 4_711_680,   # profiles/attn_mma_kernel_cfg5_interval.md (the rows' bytes; captured with other splits)
 }
 

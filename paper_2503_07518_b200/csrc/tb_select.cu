@@ -712,6 +712,7 @@ cudaError_t launch_select(const tb_ctx* c, const UnitTable& ut, const SelectArgs
         int L = ut.len[i], lo = a.sinks < L ? a.sinks : L, hi = L - a.recent > lo ? L - a.recent : lo;
         if (hi - lo > max_cand) max_cand = hi - lo;
     }
+    // What neither the small nor the streaming kernel takes:
     // Many problems (one and a half per SM or more; measured crossover between 32 and 256 on 148 SMs)
     // fill the GPU by themselves: one block each, no clusters.  So do more problems than SMs as long as they are short (160
     // of 9500 candidates: 34.3 us against 36.7 in clusters, 192 of 16000: 47.6 / 54.5), and problems beyond what the
