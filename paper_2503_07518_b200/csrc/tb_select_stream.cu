@@ -248,9 +248,11 @@ __global__ void __launch_bounds__(kThreads, 512 / kThreads) select_stream_kernel
         scorer.load_staged(sm->qs, gm.gl, sm->frags);
     }
 
-    // about p * kSampleRows sample keys lie above the threshold (p = k / candidates): +- 4 standard deviations of that rank
+    // about p * kSampleRows sample keys lie above the threshold (p = k / candidates): +- 4 standard deviations of that rank, one
+    // more down and a longer reach up where a second look costs the rows again (eight 64K
+    // sequences, a step of four layers: 261 us, 348 with the narrow bracket)
     const float p = (float)k / (float)ncand, mean = p * kSampleRows, sd = sqrtf(mean * (1.f - p));
-    const int r_hi = max(0, (int)floorf(mean - 4.f * sd) - 1), r_lo = min(kSampleRows - 1, (int)ceilf(mean + 4.f * sd) + 1);
+    const int r_hi = max(0, (int)floorf(mean - 4.f * sd) - 1), r_lo = min(kSampleRows - 1, (int)ceilf(mean + (keep_scores ? 4.f : 5.f) * sd) + 1);
     Slices<kBins> sl;
     if (warp < kSampleRows / 32) {
         int at;
@@ -272,7 +274,7 @@ __global__ void __launch_bounds__(kThreads, 512 / kThreads) select_stream_kernel
         }
     }
     __syncthreads();
-    sl.bracket(sm->s_lo, sm->s_hi, mean < 3.f ? 4.5f : 3.f);
+    sl.bracket(sm->s_lo, sm->s_hi, !keep_scores ? 6.f : mean < 3.f ? 4.5f : 3.f);
 
     // ---- rounds: one, hardly ever more ---------------------------------------------------------------------------------
     DigitCounter counter;
@@ -589,7 +591,8 @@ cudaError_t launch_select_stream(const tb_ctx* c, const UnitTable& ut, const Sel
     // problems' worth of rows per line (16 dimensions) is what the other spends its time on.  fp32 rows: 256 of 8000 53 / 62, 512
     // of 12000 137 / 153, but 160 of 12000 59 / 50 and 160 of 40000 219 / 210.
     int C = 1;
-    const int sms = c->sm_count, threads = n_units <= sms ? 512 : 256;
+    const int sms = c->sm_count;
+    int threads = n_units <= sms ? 512 : 256;
     if (n_units <= sms) {
         const int sizes[] = {16, 12, 10, 9, 8, 6, 5, 4, 3, 2, 1};
         for (int x : sizes) {
@@ -605,11 +608,15 @@ cudaError_t launch_select_stream(const tb_ctx* c, const UnitTable& ut, const Sel
         else take = !f32 && (max || narrow) && max_cand >= 16000;
         if (!take) return cudaSuccess;
     }
-    const int spare = ut.use_dev_len && a.radius == 0 ? 2048 : 0;   // a replayed graph may find more than it declared
+    // a replayed graph may find more than it declared
+    const int spare = ut.use_dev_len && a.radius == 0 ? 2048 : 0;
     l.room = ((max_cand + spare + C - 1) / C + 127) / 128 * 128;
     l.most = a.radius > 0 ? max_cand : C * l.room;
-    const int per_sm = 512 / threads;
     auto smem = [&](bool scores) { return stream_smem(threads, C, l.room, a.radius > 0, scores); };
+    // Two blocks of digits do not fit an SM: one of 512 threads, if two waves of them fill most of the chip (256 problems of 65536
+    // 184 us, 230 in the kernel that parks its keys, ragged from 32768 on 144 / 187; of 50000 145 / 175).
+    if (threads == 256 && smem(false) > 113 * 1024 && n_units <= 2 * sms && 4 * n_units >= 5 * sms) threads = 512;
+    const int per_sm = 512 / threads;
     if ((C > 1 && l.room > kMaxShare) || smem(false) > 226 * 1024 / per_sm) return cudaSuccess;
     *taken = true;
     if (dry) return cudaSuccess;

@@ -22,6 +22,7 @@ CASES = [
     (8, 1, [21003] + [17000] * 19, 32, "bf16", "sum", 3000, 0, 0, 0, 0, "int"),    # ... that keep digits
     (8, 1, [2050] * 20, 32, "fp32", "sum", 200, 0, 0, 0, 0, "int"),
     (8, 1, [47009] * 10, 32, "bf16", "sum", 5000, 0, 0, 0, 0, "int"),              # one block of 512 threads, digits
+    (8, 1, [50000, 49999] * 14, 16, "bf16", "sum", 5000, 0, 0, 1, 0, "int"),       # two waves of those
     (2, 4, [40000], 32, "bf16", "sum", 1234, 0, 0, 0, 0, "ties"),
     (8, 1, [47000] * 10, 16, "bf16", "max", 2345, 0, 0, 0, 0, "ties"),             # ... from the rows again
     (2, 1, [30000], 32, "fp32", "sum", 29990, 0, 0, 0, 0, "ties"),
