@@ -235,7 +235,6 @@ tb_status tb_create(const tb_config* cfg, void* kv, void* kimp, void* state, voi
     c->last_cache_write = c->last_list_write = -4;
     c->tile_rows = 256;
     for (int& known : c->attn_max_active) known = 0;
-    for (int& known : c->stream_max_active) known = 0;
     if (cudaDeviceGetAttribute(&c->sm_count, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) { delete c; return TB_ERR_CUDA; }
     // only the small control parts need defined contents; the index lists and partials are always
     // written before they are read

@@ -140,7 +140,6 @@ struct tb_ctx {
     int tile_rows;                        // rows per TMA box of the score pass
     int sm_count;
     int attn_max_active[25];              // co-resident attention clusters per cluster size, 8-warp blocks and (16 +) 4-warp ones (0 = not asked yet)
-    int stream_max_active[17];            // co-resident clusters of the streaming selection per cluster size (0 = not asked yet)
     void* res_rows;                       // resident sink + window rows (tb_bind_resident_rows), or NULL
     int res_sinks, res_window;
     void* imp_rows;                       // Important buffer (tb_bind_important_buffer), or NULL

@@ -17,6 +17,8 @@
 // order-preserving 32-bit key, from the scores on chip or, where only the digits fit, from the rows, until it is small or one
 // key wide: a few rounds at most, each a thousand times finer.
 // Nothing waits for anything but cluster barriers and the block's own loads.
+#include <atomic>
+
 #include "tb_select.cuh"
 
 namespace tb {
@@ -569,7 +571,10 @@ cudaError_t launch_select_stream(const tb_ctx* c, const UnitTable& ut, const Sel
     // how many clusters of C blocks run at once: one block per SM, whatever its shared memory
     auto fits = [&](int C) {
         if (C == 1) return c->sm_count;
-        int& known = const_cast<tb_ctx*>(c)->stream_max_active[C];
+        static std::atomic<int> of_device[64][kMaxBlocks + 1];   // 0 = not asked yet
+        int dev = 0;
+        if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return -1;
+        int known = of_device[dev][C].load(std::memory_order_relaxed);
         if (known == 0) {
             attr[0].val.clusterDim.x = C;
             int n = 0;
@@ -577,6 +582,7 @@ cudaError_t launch_select_stream(const tb_ctx* c, const UnitTable& ut, const Sel
             if (launch_any<512>(c, ut, order, a, l) != cudaSuccess) n = 0;
             l.fit = nullptr;
             known = n > 0 ? n : -1;
+            of_device[dev][C].store(known, std::memory_order_relaxed);
         }
         return known;
     };
