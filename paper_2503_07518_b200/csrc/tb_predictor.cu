@@ -246,7 +246,6 @@ __global__ void __launch_bounds__(kPredThreads) predictor_out_kernel(const T* __
 constexpr int kTileRows = 32;        // weight rows of a block
 constexpr int kChunk = 512;          // channels of a block's tile: 4 warps x 4 runs of 32, for each of two 16-row halves
 constexpr int kTileTokMax = 24;      // tokens of a group; a kernel instance takes 8 * kN8 of them
-constexpr int kTwoPerSm = 76 * 1024; // shared memory of which two blocks' worth fits an SM and three do not
 constexpr int kXPitch = kChunk * 2 + 64;   // bytes per (term, token) row: eight rows' 64-byte pieces hit all banks twice
 constexpr int kClusterK = 8;         // blocks (one cluster) that share the channels of a hidden-unit tile
 
@@ -345,8 +344,8 @@ __device__ __forceinline__ float get_sum(const TileSums<kN8>& s, int row, int to
 // and the shifted sums of h and h^2 over its channels; behind one exchange through distributed shared memory
 //     sum = rstd * sum_b (P_b - (mean - s_b) G_b) + sum_b B_b
 // where mean - s_b is small against the spread, so nothing cancels.  Blocks are summed in rank order.
-template <int kTerms, int kN8>
-__global__ void __launch_bounds__(kPredThreads, kN8 == 1 ? 3 : 2) predictor_hidden_tile_kernel(const __nv_bfloat16* __restrict__ H,
+template <int kTerms, int kN8, int kPerSm>
+__global__ void __launch_bounds__(kPredThreads, kPerSm) predictor_hidden_tile_kernel(const __nv_bfloat16* __restrict__ H,
                                                                                 const __nv_bfloat16* __restrict__ ln_w,
                                                                                 const __nv_bfloat16* __restrict__ ln_b,
                                                                                 const __nv_bfloat16* __restrict__ W1,
@@ -517,8 +516,8 @@ __global__ void __launch_bounds__(kPredThreads, kN8 == 1 ? 3 : 2) predictor_hidd
 }
 
 // q_imp for 32 output rows per block, all hidden units.
-template <int kTerms, int kN8>
-__global__ void __launch_bounds__(kPredThreads, kN8 == 1 ? 3 : 2) predictor_out_tile_kernel(const __nv_bfloat16* __restrict__ W2, const float* __restrict__ hidden,
+template <int kTerms, int kN8, int kPerSm>
+__global__ void __launch_bounds__(kPredThreads, kPerSm) predictor_out_tile_kernel(const __nv_bfloat16* __restrict__ W2, const float* __restrict__ hidden,
                                                                           float* __restrict__ q_imp, int n_tok, int hid, int n_out,
                                                                           int per_slot) {
     extern __shared__ __align__(128) unsigned char ws[];   // weights [32 rows][kXPitch], then hidden units [term][token][kXPitch]
@@ -628,6 +627,8 @@ extern "C" tb_status tb_predict_importance_queries(const tb_predictor* p, const 
         // from L2.  Otherwise as few groups as hold 24.  us per call, 4096 -> 512 -> 4096, groups of 8 / 16 / 24: 16 tokens 7.8 /
         // 9.5 / 9.5, 24 10.7 / 11.8 / 11.8, 32 15 / 10.8 / 13.3, 47 19 / 18.4 / 13.3; with 1024 hidden units, twice the blocks, 32
         // tokens 27 / 21.4 / 23.3, 64 48 / 38.6 / 33.9.
+        // Groups of eight come compiled for two and for three blocks per SM.  The third costs registers (80 a thread) and is taken
+        // only where two per SM do not hold the grid: 5120 -> 512, 9 to 16 tokens 10.1-10.4 us with two, 12.1 as one group of 16.
         int n8 = 1;
         bool two_per_sm = true;
         if (n_tokens > 8) {
@@ -646,34 +647,37 @@ extern "C" tb_status tb_predict_importance_queries(const tb_predictor* p, const 
             }
             two_per_sm = blocks(n8) <= 2 * sms;
         }
-        auto launch = [&](auto terms, auto eights) {
-            constexpr int kTerms = decltype(terms)::value, kN8 = decltype(eights)::value;
-            constexpr int used = kWBytes + kTerms * kN8 * 8 * kXPitch, smem = used > kTwoPerSm ? used : kTwoPerSm;
+        auto launch = [&](auto terms, auto eights, auto per_sm) {
+            constexpr int kTerms = decltype(terms)::value, kN8 = decltype(eights)::value, kPerSm = decltype(per_sm)::value;
+            constexpr int smem = kWBytes + kTerms * kN8 * 8 * kXPitch;
             static unsigned char seen[64];
             if (first_use_on_this_device(seen)) {
-                cudaError_t r = cudaFuncSetAttribute(predictor_hidden_tile_kernel<kTerms, kN8>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-                if (r == cudaSuccess) r = cudaFuncSetAttribute(predictor_out_tile_kernel<kTerms, kN8>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+                cudaError_t r = cudaFuncSetAttribute(predictor_hidden_tile_kernel<kTerms, kN8, kPerSm>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+                if (r == cudaSuccess) r = cudaFuncSetAttribute(predictor_out_tile_kernel<kTerms, kN8, kPerSm>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
                 if (r != cudaSuccess) return r;
             }
-            cfg.dynamicSmemBytes = two_per_sm ? smem : used;   // (blocks of eight tokens fit three times: uneven where two would do)
+            cfg.dynamicSmemBytes = smem;
             const unsigned n_groups = (unsigned)((n_tokens + kN8 * 8 - 1) / (kN8 * 8));
             cfg.gridDim = dim3(kClusterK, (p->hidden_dim + kTileRows - 1) / kTileRows, n_groups), cfg.numAttrs = 2;
-            cudaError_t r = cudaLaunchKernelEx(&cfg, predictor_hidden_tile_kernel<kTerms, kN8>, (const __nv_bfloat16*)hidden_dev,
+            cudaError_t r = cudaLaunchKernelEx(&cfg, predictor_hidden_tile_kernel<kTerms, kN8, kPerSm>, (const __nv_bfloat16*)hidden_dev,
                                                (const __nv_bfloat16*)p->ln_weight, (const __nv_bfloat16*)p->ln_bias,
                                                (const __nv_bfloat16*)p->w1, scratch_dev, (int)n_tokens, (int)p->model_dim,
                                                (int)p->hidden_dim, p->ln_eps, (int)p->activation);
             if (r != cudaSuccess) return r;
             cfg.gridDim = dim3((unsigned)((n_out + kTileRows - 1) / kTileRows), n_groups, 1), cfg.numAttrs = 1;
-            return cudaLaunchKernelEx(&cfg, predictor_out_tile_kernel<kTerms, kN8>, (const __nv_bfloat16*)p->w2, (const float*)scratch_dev,
+            return cudaLaunchKernelEx(&cfg, predictor_out_tile_kernel<kTerms, kN8, kPerSm>, (const __nv_bfloat16*)p->w2, (const float*)scratch_dev,
                                       q_imp_dev, (int)n_tokens, (int)p->hidden_dim, n_out_i, per_slot);
         };
         using std::integral_constant;
         // 24 bits of both right operands for up to four tokens, and for shapes off the 32-channel runs (always computed so)
         const bool whole = n_tokens < 5 || p->model_dim % 32 || p->hidden_dim % 32 || n_out % 8;
-        if (whole) e = launch(integral_constant<int, 3>{}, integral_constant<int, 1>{});
-        else if (n8 == 1) e = launch(integral_constant<int, 2>{}, integral_constant<int, 1>{});
-        else if (n8 == 2) e = launch(integral_constant<int, 2>{}, integral_constant<int, 2>{});
-        else e = launch(integral_constant<int, 2>{}, integral_constant<int, 3>{});
+        using I1 = integral_constant<int, 1>;
+        using I2 = integral_constant<int, 2>;
+        using I3 = integral_constant<int, 3>;
+        if (whole) e = launch(I3{}, I1{}, I2{});
+        else if (n8 == 1) e = two_per_sm ? launch(I2{}, I1{}, I2{}) : launch(I2{}, I1{}, I3{});
+        else if (n8 == 2) e = launch(I2{}, I2{}, I2{});
+        else e = launch(I2{}, I3{}, I2{});
     } else {
         const int g1 = (p->hidden_dim + kPredWarps / 2 - 1) / (kPredWarps / 2), g2 = (int)((n_out + kPredWarps - 1) / kPredWarps);
         int stage_tok = (int)(48 * 1024 / (p->hidden_dim * sizeof(float))) / kTokChunk * kTokChunk;   // hidden_dim <= 1536 gives >= 8
