@@ -212,6 +212,21 @@ __device__ __forceinline__ float rescore(const unsigned char* row, const float* 
     return best;
 }
 
+// f(j, elements j .. j + 3) for every four of a thread's quarter of a query, of each of the g queries in head order.  `quarter` may
+// be the caller's memory: 16 bytes at a time where that is aligned (`wide`), else 4.  (Staged in shared memory first, behind a
+// barrier, the eight selections of a decode step over 32768 tokens take 7.5 us longer.)
+template <int DP, typename F>
+__device__ __forceinline__ void each_piece(const float* quarter, int g, bool wide, F&& f) {
+    auto all = [&](auto load) {
+#pragma unroll 4
+        for (int u = 0; u < g; ++u)
+#pragma unroll
+            for (int j = 0; j < DP / 4; j += 4) f(j, load(quarter + u * DP + j));
+    };
+    if (wide) all([](const float* p) { return *reinterpret_cast<const float4*>(p); });
+    else all([](const float* p) { return make_float4(p[0], p[1], p[2], p[3]); });
+}
+
 template <int DP, int RED>
 struct FragScorer {
     static constexpr int kSteps = DP / 16, kTerms = 3, kRowBytes = DP * 2;
@@ -227,22 +242,18 @@ struct FragScorer {
         x -= __low2float(v), y -= __high2float(v);
         return *reinterpret_cast<const uint32_t*>(&v);
     }
-    // Called by all threads of the block.  TB_GROUP_SUM: `qs` in shared or global memory; TB_GROUP_MAX: staged and visible,
-    // `frags` holds kQueryFrags entries, one barrier.
-    __device__ __forceinline__ void load_staged(const float* qs, int g, uint2* frags) {
+    // Called by all threads of the block.  TB_GROUP_SUM: `qs` in shared or global memory, `wide` if 16-byte aligned;
+    // TB_GROUP_MAX: staged and visible, `frags` holds kQueryFrags entries, one barrier.
+    __device__ __forceinline__ void load_staged(const float* qs, int g, uint2* frags, bool wide = true) {
         const int lane = threadIdx.x & 31, gid = lane >> 2, tig = lane & 3;
         // dimensions of word 2 st + half of the piece: tig * (DP / 4) + st * 4 + half * 2
         if constexpr (RED == TB_GROUP_SUM) {
             float x[kSteps * 2], y[kSteps * 2];
 #pragma unroll
             for (int i = 0; i < kSteps * 2; ++i) x[i] = y[i] = 0.f;
-#pragma unroll 4
-            for (int u = 0; u < g; ++u)                // in head order
-#pragma unroll
-                for (int i = 0; i < kSteps; ++i) {
-                    const float4 v = *reinterpret_cast<const float4*>(qs + u * DP + tig * (DP / 4) + i * 4);
-                    x[2 * i] += v.x, y[2 * i] += v.y, x[2 * i + 1] += v.z, y[2 * i + 1] += v.w;
-                }
+            each_piece<DP>(qs + tig * (DP / 4), g, wide, [&](int j, float4 v) {
+                x[j / 2] += v.x, y[j / 2] += v.y, x[j / 2 + 1] += v.z, y[j / 2 + 1] += v.w;
+            });
 #pragma unroll
             for (int i = 0; i < kSteps * 2; ++i) {
                 const uint32_t high = split(x[i], y[i], true), middle = split(x[i], y[i]), low = split(x[i], y[i]);
@@ -320,19 +331,13 @@ struct QuarterScorer {
     float qr[RED == TB_GROUP_SUM ? DP / 4 : 1];
     const float* qs;
     int g;
-    __device__ __forceinline__ void load_staged(const float* qs_, int g_, uint2*) {
+    __device__ __forceinline__ void load_staged(const float* qs_, int g_, uint2*, bool wide = true) {
         const int tig = threadIdx.x & 3;
         qs = qs_ + tig * (DP / 4), g = g_;
         if constexpr (RED == TB_GROUP_SUM) {
 #pragma unroll
             for (int j = 0; j < DP / 4; ++j) qr[j] = 0.f;
-#pragma unroll 4
-            for (int u = 0; u < g_; ++u)               // in head order
-#pragma unroll
-                for (int j = 0; j < DP / 4; j += 4) {
-                    const float4 v = *reinterpret_cast<const float4*>(qs + u * DP + j);
-                    qr[j] += v.x, qr[j + 1] += v.y, qr[j + 2] += v.z, qr[j + 3] += v.w;
-                }
+            each_piece<DP>(qs, g_, wide, [&](int j, float4 v) { qr[j] += v.x, qr[j + 1] += v.y, qr[j + 2] += v.z, qr[j + 3] += v.w; });
         }
     }
     __device__ __forceinline__ float reduce(const Piece (&v)[4], const float* q) const {

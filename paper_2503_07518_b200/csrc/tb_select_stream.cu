@@ -244,7 +244,7 @@ __global__ void __launch_bounds__(kThreads, 512 / kThreads) select_stream_kernel
     Scorer scorer;
     bool odd_query = false;                            // (a summed query that is not finite shows in every score)
     if constexpr (RED == TB_GROUP_SUM) {
-        scorer.load_staged(q_unit, gm.gl, nullptr);
+        scorer.load_staged(q_unit, gm.gl, nullptr, (reinterpret_cast<uintptr_t>(a.q_imp) & 15u) == 0u);   // (queries start at any float)
     } else {
         odd_query = __syncthreads_or(kMma && !is_finite(q_elem));
         scorer.load_staged(sm->qs, gm.gl, sm->frags);

@@ -46,8 +46,31 @@ CASES = [
 
 @pytest.mark.parametrize("ci", range(len(CASES)))
 def test_lists_are_the_oracles(H, ci):
+    check_lists(H, CASES[ci], ci)
+
+
+# one per kernel that selects; their queries are read in different ways
+@pytest.mark.parametrize("case", [
+    (2, 4, [700, 333], 32, "bf16", "sum", 90, 0, 0, 0, 0, "int"),
+    (2, 4, [700, 333], 16, "fp32", "sum", 90, 0, 0, 0, 0, "int"),
+    (2, 4, [12345, 10500], 32, "bf16", "sum", 900, 4, 16, 0, 0, "int"),
+    (2, 4, [12345, 10500], 16, "bf16", "sum", 900, 4, 16, 1, 0, "int"),
+    (2, 4, [12345, 10500], 32, "bf16", "max", 900, 4, 16, 0, 0, "int"),
+    (2, 4, [12345, 10500], 32, "fp32", "sum", 900, 4, 16, 0, 0, "int"),
+    (2, 8, [12345, 10500], 16, "fp32", "max", 900, 4, 16, 0, 0, "int"),
+    (8, 4, [11000] * 20, 32, "bf16", "sum", 1100, 0, 0, 0, 0, "int"),
+    (8, 4, [2050] * 20, 32, "fp32", "sum", 200, 0, 0, 0, 0, "int"),
+    (8, 1, [9000] * 48, 32, "bf16", "sum", 400, 0, 0, 0, 0, "int"),
+    (4, 4, [15000] * 10, 32, "bf16", "per head", 800, 0, 0, 0, 0, "int"),
+])
+def test_queries_may_start_at_any_float(H, case):
+    """The importance queries are floats: a view that starts one float into its storage gives the same lists."""
+    check_lists(H, case, 5, q_offset=1)
+
+
+def check_lists(H, case, seed, q_offset=0):
     b_ = tb()
-    heads, g, lens, dp, dt, reduce, budget, sinks, recent, radius, mode, data = CASES[ci]
+    heads, g, lens, dp, dt, reduce, budget, sinks, recent, radius, mode, data = case
     dtype = b_.TB_BF16 if dt == "bf16" else b_.TB_F32
     store = b_.torch_dtype(dtype)
     red = b_.TB_GROUP_MAX if reduce == "max" else b_.TB_GROUP_SUM
@@ -62,7 +85,7 @@ def test_lists_are_the_oracles(H, ci):
     ctx.project_keys(0, 1, None, [0] * B, lens)
     del rows
     gen = torch.Generator(device="cuda")
-    gen.manual_seed(ci)
+    gen.manual_seed(seed)
     x = torch.randn(ctx.kimp.shape, generator=gen, device="cuda")
     x = (x.mul_(1.0).round_() if data == "ties" else x.mul_(40).round_()).clamp_(-120, 120)
     q = torch.randn(1, B, heads * g, dp, generator=gen, device="cuda").mul_(20).round_().clamp_(-60, 60)
@@ -77,12 +100,14 @@ def test_lists_are_the_oracles(H, ci):
         x[0, 0, :, 1000:lens[0]:97, 3] = float("inf")    # of either sign once multiplied: every row's other products are finite
         q[..., 3] = q[..., 3].abs() + 1
     ctx.kimp.copy_(x.to(store))
+    q_mem = torch.empty(q.numel() + q_offset, device="cuda")
+    q_at = q_mem[q_offset:].view(q.shape).copy_(q)
     idx = torch.zeros(1, B, lists, ctx.index_capacity, dtype=torch.int32, device="cuda")
     cnt = torch.zeros(1, B, lists, dtype=torch.int32, device="cuda")
     for copied in (True, False):                         # the caller's copy, and the stored lists
         p = b_.select_params(budget, sinks, recent, radius, mode, 2, 0 if copied else 1, red)
         if copied:
-            ctx.select_topk(0, 1, None, B, q, p, idx, cnt)
+            ctx.select_topk(0, 1, None, B, q_at, p, idx, cnt)
         else:
             idx.zero_(), cnt.zero_()
             ctx.select_topk(0, 1, None, B, None, p, idx, cnt)
