@@ -337,10 +337,11 @@ bool select_small_takes(const tb_ctx* c, const UnitTable& ut, int max_cand) {
     const int n_units = ut.layer_count * ut.n_seq * c->geom.Hl;
     // wait diagnostics: launches of one block that wait for copies (the others: see launch_select)
     if (c->drop_tile >= 0 && (c->geom.dtype == TB_BF16 || n_units > 1 || max_cand > 1023)) return false;
-    if (n_units > c->sm_count && c->geom.dtype != TB_BF16 && c->drop_tile < 0) return max_cand <= 1500;
+    // (Replayed graphs in which this many sequences grow: the kernel whose room is the workspace's.)
+    if (n_units > 2 * c->sm_count && ut.use_dev_len) return false;
+    if (n_units > c->sm_count && c->geom.dtype != TB_BF16) return max_cand <= 1500;
+    if (n_units > 2 * c->sm_count) return max_cand <= (c->geom.Hl > c->geom.Hi ? SmallSmem<256>::kMaxCand : 5000);
     const int most = n_units <= c->sm_count ? (2 * n_units > c->sm_count ? SmallSmem<512>::kMaxCand : 10 * 1024) : 8 * 1024;
-    if (n_units > 2 * c->sm_count)                     // (replayed graphs in which these sequences grow: the kernel whose room is the workspace's)
-        return c->drop_tile < 0 && !ut.use_dev_len && max_cand <= (c->geom.Hl > c->geom.Hi ? SmallSmem<256>::kMaxCand : 5000);
     return max_cand <= most;
 }
 

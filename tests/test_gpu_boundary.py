@@ -305,27 +305,30 @@ def test_resident_rows_and_important_buffer_give_the_same_bits(H, on_host):
                 assert np.abs(base[-1][1][l, b, h * 4:(h + 1) * 4] - ref).max() <= 2e-3
 
 
-@pytest.mark.parametrize("heads,batch,length,scope,radius,n,reported", [
-    ((2, 2), 1, 250, 0, 0, 64, True),           # one block per list, keys and bitmask on chip
-    ((1, 1), 1, 2000, 0, 1, 64, True),          # ... shared by a cluster
-    ((4, 2), 1, 10300, 1, 1, 16384, True),      # lists that share a key stream: the second bitmask
-    ((4, 2), 1, 20000, 1, 1, 1024, False),      # ... which has room to spare
-    ((8, 8), 38, 250, 0, 2, 64, False),         # more lists than fit at once: the same
-    ((2, 2), 1, 20000, 0, 2, 64, True),         # a cluster per list, the neighbour kernel's bitmask behind it
+@pytest.mark.parametrize("heads,batch,length,scope,radius,n,reported,dtype", [
+    ((2, 2), 1, 250, 0, 0, 64, True, "bf16"),           # one block per list, keys and bitmask on chip
+    ((1, 1), 1, 2000, 0, 1, 64, True, "bf16"),          # ... shared by a cluster
+    ((4, 2), 1, 10300, 1, 1, 16384, True, "bf16"),      # lists that share a key stream: the second bitmask
+    ((4, 2), 1, 20000, 1, 1, 1024, False, "bf16"),      # ... which has room to spare
+    ((8, 8), 38, 250, 0, 2, 64, False, "bf16"),         # more lists than fit at once: the same
+    ((8, 8), 38, 250, 0, 0, 64, False, "fp32"),
+    ((2, 2), 1, 20000, 0, 2, 64, True, "bf16"),         # a cluster per list, the neighbour kernel's bitmask behind it
 ])
-def test_a_replay_that_outgrows_its_reserve_is_reported(H, heads, batch, length, scope, radius, n, reported):
+def test_a_replay_that_outgrows_its_reserve_is_reported(H, heads, batch, length, scope, radius, n, reported, dtype):
     """A captured selection is replayed on sequences longer than the reserve it was sized for.  It selects among the
     candidates there is room for -- ascending positions of the cache, no more than asked for -- and says TB_ERR_CAPACITY if
     that leaves any out; with the true lengths back in the mirrors the same context selects exactly again."""
     b_ = tb()
+    dt = b_.TB_BF16 if dtype == "bf16" else b_.TB_F32
+    store = b_.torch_dtype(dt)
     hq, hkv = heads
     budget, replays = 40, 6
-    ctx = b_.Context(1, hq, hkv, 128, 32, b_.TB_BF16, batch, length + n * (replays + 1), budget, max_radius=radius, list_scope=scope)
+    ctx = b_.Context(1, hq, hkv, 128, 32, dt, batch, length + n * (replays + 1), budget, max_radius=radius, list_scope=scope)
     gen = torch.Generator(device="cuda")
     gen.manual_seed(5)
     rand = lambda *s, **kw: torch.randn(*s, generator=gen, device="cuda", **kw)  # noqa: E731
-    ctx.set_projection(0, rand(hkv, 128, 32, dtype=torch.bfloat16))
-    rows = lambda m: rand(m * batch, hkv, 128, dtype=torch.bfloat16)  # noqa: E731
+    ctx.set_projection(0, rand(hkv, 128, 32, dtype=store))
+    rows = lambda m: rand(m * batch, hkv, 128, dtype=store)  # noqa: E731
     ctx.append_kv(0, 1, None, [length] * batch, rows(length), rows(length))
     ctx.project_keys(0, 1, None, [0] * batch, [length] * batch)
     ctx.use_device_lengths(True, growth_reserve=n)
@@ -365,7 +368,7 @@ def test_a_replay_that_outgrows_its_reserve_is_reported(H, heads, batch, length,
     c, x = cnt.cpu().numpy(), lists_now.cpu().numpy()
     for b in range(batch):
         for h in range(lists):
-            kimp = H.to_host(ctx.kimp[0, b, h * hkv // lists, :L], b_.TB_BF16)
-            s = H.orc.score(qi[0, b, h * hq // lists:(h + 1) * hq // lists].cpu().numpy(), np.ascontiguousarray(kimp), b_.TB_BF16)
+            kimp = H.to_host(ctx.kimp[0, b, h * hkv // lists, :L], dt)
+            s = H.orc.score(qi[0, b, h * hq // lists:(h + 1) * hq // lists].cpu().numpy(), np.ascontiguousarray(kimp), dt)
             want = H.orc.neighbors(H.orc.select(s, 0, 0, budget), radius, 0, 0, L) if radius else H.orc.select(s, 0, 0, budget)
             assert np.array_equal(x[0, b, h, :c[0, b, h]], want)
