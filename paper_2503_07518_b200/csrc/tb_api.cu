@@ -449,7 +449,7 @@ tb_status tb_select_topk(tb_ctx* c, int32_t lb, int32_t lc, const int32_t* seq_i
                     cand_range(ut.len[i], p->sinks, p->recent, &lo, &hi);
                     if (hi - lo > max_cand) max_cand = hi - lo;
                 }
-                const bool small = select_small_takes(c, ut, max_cand);
+                const bool small = select_small_takes(c, ut, max_cand, p->radius > 0);
                 finished = small;
                 SelectArgs a;
                 a.radius = p->radius, a.nmode = p->nmode;

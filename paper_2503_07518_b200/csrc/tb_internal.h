@@ -208,7 +208,7 @@ cudaError_t launch_select_wave(const tb_ctx* c, const UnitTable& ut, const Selec
 cudaError_t launch_select_shared(const tb_ctx* c, const UnitTable& ut, const SelectArgs& a, cudaStream_t s, bool dry, bool* finished);
 // small problems: one block each, neighbours and the caller's copy of the list included; whether a launch whose longest
 // problem has max_cand candidates is its kind (not whether the caller wants copies: they must not change the lists)
-bool select_small_takes(const tb_ctx* c, const UnitTable& ut, int max_cand);
+bool select_small_takes(const tb_ctx* c, const UnitTable& ut, int max_cand, bool neighbours);
 cudaError_t launch_select_small(const tb_ctx* c, const UnitTable& ut, const SelectArgs& a, int max_cand, cudaStream_t s, bool dry = false);
 // few, long problems: a cluster per problem on parked keys
 cudaError_t launch_select_cw(const tb_ctx* c, const UnitTable& ut, const SelectArgs& a, cudaStream_t s, bool dry = false);

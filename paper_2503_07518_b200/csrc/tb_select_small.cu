@@ -331,17 +331,23 @@ size_t small_smem(int n_stages, int n_tiles, int tile_bytes, int threads = 512) 
 // 25, 2000 20 / 15.6.  More than two problems per SM: against the kernel of one 256-thread block each that parks its keys in memory,
 // 512 of 300 8.2 / 11.6, 1000 11.6 / 15.5, 4900 36.7 / 38.8, ragged to 4900 30.7 / 32.3, 6000 42.6 / 44.1, 8000 61 / 58; 2048 of 1000 36
 // / 46; lists that share a key stream, whose rows are L2 hits for all but one, 512 of 8000 41 / 47.
+// Under device lengths the streaming kernel takes neither more lists than SMs nor lists that share a key stream; with neighbours,
+// against the kernels that do: 160 of 9000 32 / 38, 16000 50 / 55, 296 of 16000 65 / 72, at 16 dimensions 45 / 50; one list per query
+// head, four per stream, 32 of 11000 14.9 / 22.3, 16000 17.1 / 26, 160 of 9000 26.0 / 28.3, 12000 30.5 / 30.7, 16000 37 / 34.
 // Whether the caller wants copies does not matter: the scores are summed in another order here, and an output that the caller
 // may leave out must not decide which of two tokens within fp32 rounding of one another is stored.
-bool select_small_takes(const tb_ctx* c, const UnitTable& ut, int max_cand) {
+bool select_small_takes(const tb_ctx* c, const UnitTable& ut, int max_cand, bool neighbours) {
     const int n_units = ut.layer_count * ut.n_seq * c->geom.Hl;
+    const bool many = n_units > c->sm_count, per_head = c->geom.Hl > c->geom.Hi;
     // wait diagnostics: launches of one block that wait for copies (the others: see launch_select)
     if (c->drop_tile >= 0 && (c->geom.dtype == TB_BF16 || n_units > 1 || max_cand > 1023)) return false;
     // (Replayed graphs in which this many sequences grow: the kernel whose room is the workspace's.)
     if (n_units > 2 * c->sm_count && ut.use_dev_len) return false;
-    if (n_units > c->sm_count && c->geom.dtype != TB_BF16) return max_cand <= 1500;
-    if (n_units > 2 * c->sm_count) return max_cand <= (c->geom.Hl > c->geom.Hi ? SmallSmem<256>::kMaxCand : 5000);
-    const int most = n_units <= c->sm_count ? (2 * n_units > c->sm_count ? SmallSmem<512>::kMaxCand : 10 * 1024) : 8 * 1024;
+    if (many && c->geom.dtype != TB_BF16) return max_cand <= 1500;
+    if (n_units > 2 * c->sm_count) return max_cand <= (per_head ? SmallSmem<256>::kMaxCand : 5000);
+    if (ut.use_dev_len && neighbours && c->geom.dtype == TB_BF16 && (many || per_head))
+        return max_cand <= (many && per_head ? 12 * 1024 : SmallSmem<512>::kMaxCand);
+    const int most = !many ? (2 * n_units > c->sm_count ? SmallSmem<512>::kMaxCand : 10 * 1024) : 8 * 1024;
     return max_cand <= most;
 }
 

@@ -222,3 +222,26 @@ def queries(w: wl.Workload, step=0, layers=None):
         qs.append(np.stack([p[0] for p in pairs]))
         qis.append(np.stack([p[1] for p in pairs]))
     return np.stack(qs), np.stack(qis)
+
+
+def launched_kernels(call) -> list:
+    """The (mangled) names of the kernels that call() launches, in order: it is captured, not run."""
+    from cuda.bindings import driver
+    graph = torch.cuda.CUDAGraph(keep_graph=True)
+    with torch.cuda.graph(graph):
+        call()
+    names = []
+    err, nodes, n = driver.cuGraphGetNodes(driver.CUgraph(graph.raw_cuda_graph()))
+    if n:
+        err, nodes, n = driver.cuGraphGetNodes(driver.CUgraph(graph.raw_cuda_graph()), n)
+    assert err == driver.CUresult.CUDA_SUCCESS, err
+    for node in nodes[:n]:
+        err, kind = driver.cuGraphNodeGetType(node)
+        if kind != driver.CUgraphNodeType.CU_GRAPH_NODE_TYPE_KERNEL:
+            continue
+        err, params = driver.cuGraphKernelNodeGetParams(node)
+        assert err == driver.CUresult.CUDA_SUCCESS, err
+        err, name = driver.cuFuncGetName(params.func) if int(params.func) else driver.cuKernelGetName(params.kern)
+        assert err == driver.CUresult.CUDA_SUCCESS, err
+        names.append(name.decode())
+    return names

@@ -68,7 +68,8 @@ def test_queries_may_start_at_any_float(H, case):
     check_lists(H, case, 5, q_offset=1)
 
 
-def check_lists(H, case, seed, q_offset=0):
+def check_lists(H, case, seed, q_offset=0, kernel=None, dev_lengths=False):
+    """The lists of one call, and of the stored lists after it, are the oracle's; `kernel`: the one that has to select."""
     b_ = tb()
     heads, g, lens, dp, dt, reduce, budget, sinks, recent, radius, mode, data = case
     dtype = b_.TB_BF16 if dt == "bf16" else b_.TB_F32
@@ -104,6 +105,11 @@ def check_lists(H, case, seed, q_offset=0):
     q_at = q_mem[q_offset:].view(q.shape).copy_(q)
     idx = torch.zeros(1, B, lists, ctx.index_capacity, dtype=torch.int32, device="cuda")
     cnt = torch.zeros(1, B, lists, dtype=torch.int32, device="cuda")
+    if dev_lengths:
+        ctx.use_device_lengths(True)
+    if kernel:
+        p = b_.select_params(budget, sinks, recent, radius, mode, reduce=red)
+        assert kernel in H.launched_kernels(lambda: ctx.select_topk(0, 1, None, B, q_at, p, idx, cnt))[0]
     for copied in (True, False):                         # the caller's copy, and the stored lists
         p = b_.select_params(budget, sinks, recent, radius, mode, 2, 0 if copied else 1, red)
         if copied:
