@@ -874,9 +874,9 @@ cudaError_t launch_attention(const tb_ctx* c, const UnitTable& ut, const AttnArg
     int nw = kAttnWarps;
     const bool f32 = gm.dtype != TB_BF16;
     {
-        static unsigned char seen[64];
+        static DeviceFlags done;
         int* max_active = const_cast<tb_ctx*>(c)->attn_max_active;
-        if (first_use_on_this_device(seen)) {
+        const cudaError_t configured = once_per_device(done, [&] {
             cudaError_t e = cudaSuccess;
             auto prepare = [&](auto kernel, int max_kb, bool required) {
                 cudaError_t r = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, max_kb * 1024);
@@ -894,9 +894,10 @@ cudaError_t launch_attention(const tb_ctx* c, const UnitTable& ut, const AttnArg
             };
             prepare_f32(std::integral_constant<int, 1>{}), prepare_f32(std::integral_constant<int, 2>{});
             prepare_f32(std::integral_constant<int, 4>{}), prepare_f32(std::integral_constant<int, 8>{});
-            if (e != cudaSuccess) return e;
             (void)cudaGetLastError();
-        }
+            return e;
+        });
+        if (configured != cudaSuccess) return configured;
         // how many clusters of `csize` blocks run at once: 8-warp blocks, one per SM, or 4-warp ones, two (at most 8 per cluster)
         auto clusters_that_fit = [&](int csize, bool four = false) {
             int& known = max_active[(four ? kAttnMaxCluster : 0) + csize];

@@ -382,35 +382,29 @@ cudaError_t launch_project(const tb_ctx* c, const UnitTable& ut, const int* pos_
         const __nv_bfloat16* wp = (const __nv_bfloat16*)c->st.W;
         if (gm.dp == 32) {
             const size_t smem = kPmTokens * kPmKPitch + 128 * (32 * 2 + 16);
-            static unsigned char seen[64];
-            if (first_use_on_this_device(seen)) {
-                cudaError_t e = cudaFuncSetAttribute(project_mma_kernel<32>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-                if (e != cudaSuccess) return e;
-            }
+            static DeviceFlags done;
+            const cudaError_t e = allow_shared_memory(done, project_mma_kernel<32>, (int)smem);
+            if (e != cudaSuccess) return e;
             project_mma_kernel<32><<<grid_mma, kPmThreads, smem, s>>>(gm, ut, pt, kvp, wp, (__nv_bfloat16*)c->kimp, c->st.len_proj, c->st.misc_counter + 1);
         } else {
             const size_t smem = kPmTokens * kPmKPitch + 128 * (16 * 2 + 16);
-            static unsigned char seen[64];
-            if (first_use_on_this_device(seen)) {
-                cudaError_t e = cudaFuncSetAttribute(project_mma_kernel<16>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-                if (e != cudaSuccess) return e;
-            }
+            static DeviceFlags done;
+            const cudaError_t e = allow_shared_memory(done, project_mma_kernel<16>, (int)smem);
+            if (e != cudaSuccess) return e;
             project_mma_kernel<16><<<grid_mma, kPmThreads, smem, s>>>(gm, ut, pt, kvp, wp, (__nv_bfloat16*)c->kimp, c->st.len_proj, c->st.misc_counter + 1);
         }
         return cudaGetLastError();
     }
     dim3 grid((max_range + kProjTokens - 1) / kProjTokens, gm.Hi, ut.layer_count * ut.n_seq);
-    auto launch = [&](auto kernel, unsigned char (&seen)[64]) {
+    auto launch = [&](auto kernel, DeviceFlags& done) {
         const int smem = (128 * gm.dp + kProjTokens * (128 + 4)) * 4;
-        if (first_use_on_this_device(seen)) {
-            cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-            if (e != cudaSuccess) return e;
-        }
+        const cudaError_t e = allow_shared_memory(done, kernel, smem);
+        if (e != cudaSuccess) return e;
         kernel<<<grid, kProjThreads, smem, s>>>(gm, ut, pt, (const float*)c->kv, (const float*)c->st.W, (float*)c->kimp, c->st.len_proj, c->st.misc_counter + 1);
         return cudaGetLastError();
     };
-    static unsigned char seen32[64], seen16[64];
-    return gm.dp == 32 ? launch(project_kernel<32>, seen32) : launch(project_kernel<16>, seen16);
+    static DeviceFlags done32, done16;
+    return gm.dp == 32 ? launch(project_kernel<32>, done32) : launch(project_kernel<16>, done16);
 }
 
 }  // namespace tb

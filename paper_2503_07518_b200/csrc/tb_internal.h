@@ -5,6 +5,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <atomic>
 #include <vector>
 
 #include "../../include/tokenbutler.h"
@@ -179,13 +180,22 @@ __device__ __forceinline__ bool last_block_arrives(uint32_t* counter, unsigned n
 #endif
 
 // Kernel attributes (dynamic shared-memory limit, non-portable cluster sizes) belong to a device's
-// context, so each launcher configures its kernels on first use per device.
-inline bool first_use_on_this_device(unsigned char (&seen)[64]) {
+// context, so each launcher configures its kernels on first use per device: nobody goes on to a launch before `configure`
+// has succeeded there.  Threads that arrive meanwhile do the same themselves; setting an attribute twice changes nothing.
+typedef std::atomic<unsigned char> DeviceFlags[64];
+template <typename F>
+cudaError_t once_per_device(DeviceFlags& done, F&& configure) {
     int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return true;
-    if (seen[dev]) return false;
-    seen[dev] = 1;
-    return true;
+    const bool known = cudaGetDevice(&dev) == cudaSuccess && dev >= 0 && dev < 64;
+    if (known && done[dev].load(std::memory_order_acquire)) return cudaSuccess;
+    const cudaError_t e = configure();
+    if (known && e == cudaSuccess) done[dev].store(1, std::memory_order_release);
+    return e;
+}
+// ... where all there is to set is the dynamic shared memory that a launch may ask for
+template <typename K>
+cudaError_t allow_shared_memory(DeviceFlags& done, K kernel, int bytes) {
+    return once_per_device(done, [&] { return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes); });
 }
 
 // tb_cache.cu

@@ -650,16 +650,14 @@ extern "C" tb_status tb_predict_importance_queries(const tb_predictor* p, const 
         auto launch = [&](auto terms, auto eights, auto per_sm) {
             constexpr int kTerms = decltype(terms)::value, kN8 = decltype(eights)::value, kPerSm = decltype(per_sm)::value;
             constexpr int smem = kWBytes + kTerms * kN8 * 8 * kXPitch;
-            static unsigned char seen[64];
-            if (first_use_on_this_device(seen)) {
-                cudaError_t r = cudaFuncSetAttribute(predictor_hidden_tile_kernel<kTerms, kN8, kPerSm>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-                if (r == cudaSuccess) r = cudaFuncSetAttribute(predictor_out_tile_kernel<kTerms, kN8, kPerSm>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-                if (r != cudaSuccess) return r;
-            }
+            static DeviceFlags hidden_done, out_done;
+            cudaError_t r = allow_shared_memory(hidden_done, predictor_hidden_tile_kernel<kTerms, kN8, kPerSm>, smem);
+            if (r == cudaSuccess) r = allow_shared_memory(out_done, predictor_out_tile_kernel<kTerms, kN8, kPerSm>, smem);
+            if (r != cudaSuccess) return r;
             cfg.dynamicSmemBytes = smem;
             const unsigned n_groups = (unsigned)((n_tokens + kN8 * 8 - 1) / (kN8 * 8));
             cfg.gridDim = dim3(kClusterK, (p->hidden_dim + kTileRows - 1) / kTileRows, n_groups), cfg.numAttrs = 2;
-            cudaError_t r = cudaLaunchKernelEx(&cfg, predictor_hidden_tile_kernel<kTerms, kN8, kPerSm>, (const __nv_bfloat16*)hidden_dev,
+            r = cudaLaunchKernelEx(&cfg, predictor_hidden_tile_kernel<kTerms, kN8, kPerSm>, (const __nv_bfloat16*)hidden_dev,
                                                (const __nv_bfloat16*)p->ln_weight, (const __nv_bfloat16*)p->ln_bias,
                                                (const __nv_bfloat16*)p->w1, scratch_dev, (int)n_tokens, (int)p->model_dim,
                                                (int)p->hidden_dim, p->ln_eps, (int)p->activation);

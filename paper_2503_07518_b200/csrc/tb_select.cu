@@ -794,12 +794,9 @@ cudaError_t launch_select(const tb_ctx* c, const UnitTable& ut, const SelectArgs
 
 #define TB_SEL_R(T, DP, RED)                                                                                       \
     do {                                                                                                           \
-        static unsigned char seen[64];                                                                            \
-        if (first_use_on_this_device(seen)) {                                                                                         \
-            cudaError_t e = cudaFuncSetAttribute(select_kernel<T, DP, RED>, cudaFuncAttributeMaxDynamicSharedMemorySize, \
-                                                 227 * 1024);                                                      \
-            if (e != cudaSuccess) return e;                                                                        \
-        }                                                                                                          \
+        static DeviceFlags done;                                                                                   \
+        const cudaError_t e = allow_shared_memory(done, select_kernel<T, DP, RED>, 227 * 1024);                    \
+        if (e != cudaSuccess) return e;                                                                            \
         return cudaLaunchKernelEx(&cfg, select_kernel<T, DP, RED>, c->kimp_map, (const unsigned char*)c->kimp, gm, ut, a, \
                                   tiles_per_cta, n_stages, wait_limit, drop_tile, c->st.idx, c->st.cnt, c->st.status); \
     } while (0)

@@ -125,11 +125,9 @@ cudaError_t launch_neighbors(const tb_ctx* c, const UnitTable& ut, const Neighbo
     size_t smem = (size_t)((a.room + 31) / 32) * 4 + 16;
     if (smem > 200 * 1024) return cudaErrorInvalidConfiguration;   // one bit per candidate on chip: up to 1,638,272 candidates
     if (dry) return cudaSuccess;
-    static unsigned char seen[64];
-    if (first_use_on_this_device(seen)) {
-        cudaError_t e = cudaFuncSetAttribute(neighbor_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
-        if (e != cudaSuccess) return e;
-    }
+    static DeviceFlags done;
+    const cudaError_t e = allow_shared_memory(done, neighbor_kernel, 200 * 1024);
+    if (e != cudaSuccess) return e;
     neighbor_kernel<<<ut.layer_count * ut.n_seq * gm.Hl, kNbThreads, smem, s>>>(gm, ut, a, c->st.idx, c->st.cnt, c->st.status);
     return cudaGetLastError();
 }

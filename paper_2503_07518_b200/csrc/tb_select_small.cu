@@ -387,19 +387,17 @@ cudaError_t launch_select_small(const tb_ctx* c, const UnitTable& ut, const Sele
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;   // see pdl_wait()
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr, cfg.numAttrs = C > 1 ? 2 : 1;
-    auto launch = [&](auto kernel, unsigned char (&seen)[64]) {
-        if (first_use_on_this_device(seen)) {
-            cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
-            if (e != cudaSuccess) return e;
-        }
+    auto launch = [&](auto kernel, DeviceFlags& done) {
+        const cudaError_t e = allow_shared_memory(done, kernel, 227 * 1024);
+        if (e != cudaSuccess) return e;
         return cudaLaunchKernelEx(&cfg, kernel, c->kimp_map, (const unsigned char*)c->kimp, gm, ut, a, n_stages, n_tiles, share_tiles, wait_limit, drop_tile,
                                   c->st.idx, c->st.cnt, c->st.status);
     };
     // a block alone on its SM keeps four groups of rows in flight per warp, two blocks two each (their registers)
 #define TB_SMALL(T, DP, RED, U, SH, NT)                                    \
     do {                                                                   \
-        static unsigned char seen[64];                                     \
-        return launch(select_small_kernel<T, DP, RED, U, SH, NT>, seen);   \
+        static DeviceFlags done;                                           \
+        return launch(select_small_kernel<T, DP, RED, U, SH, NT>, done);   \
     } while (0)
 #define TB_SMALL_U(DP, RED)                                                      \
     do {                                                                         \

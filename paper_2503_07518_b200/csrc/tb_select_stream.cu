@@ -523,13 +523,15 @@ struct StreamLaunch {
 template <typename T, int DP, int RED, int kThreads>
 cudaError_t launch(const tb_ctx* c, const UnitTable& ut, const StreamOrder& order, const SelectArgs& a, const StreamLaunch& l) {
     const auto kernel = select_stream_kernel<T, DP, RED, kThreads>;
-    static unsigned char seen[64];
-    if (first_use_on_this_device(seen)) {
-        cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 226 * 1024);
+    static DeviceFlags done;
+    const cudaError_t configured = once_per_device(done, [&] {
+        const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 226 * 1024);
         if (e != cudaSuccess) return e;
         (void)cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
         (void)cudaGetLastError();
-    }
+        return e;
+    });
+    if (configured != cudaSuccess) return configured;
     if (l.fit) {
         if (cudaOccupancyMaxActiveClusters(l.fit, kernel, &l.cfg) != cudaSuccess) *l.fit = 0;
         (void)cudaGetLastError();

@@ -857,16 +857,14 @@ cudaError_t launch_select_shared(const tb_ctx* c, const UnitTable& ut, const Sel
     attr[0].id = cudaLaunchAttributeClusterDimension;
     attr[0].val.clusterDim.x = g, attr[0].val.clusterDim.y = 1, attr[0].val.clusterDim.z = 1;
     cfg.attrs = attr, cfg.numAttrs = 1;
-    auto launch = [&](auto kernel, unsigned char (&seen)[64]) {
-        if (first_use_on_this_device(seen)) {
-            cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 224 * 1024);
-            if (e != cudaSuccess) return e;
-        }
+    auto launch = [&](auto kernel, DeviceFlags& done) {
+        const cudaError_t e = allow_shared_memory(done, kernel, 224 * 1024);
+        if (e != cudaSuccess) return e;
         return cudaLaunchKernelEx(&cfg, kernel, (const unsigned char*)c->kimp, gm, ut, order, a, (int)scratch, keep_in_l2, c->st.idx, c->st.cnt, c->st.status,
                                   c->wk.sel_keys);
     };
-    static unsigned char seen32[64], seen16[64];
-    return gm.dp == 32 ? launch(select_shared_kernel<32>, seen32) : launch(select_shared_kernel<16>, seen16);
+    static DeviceFlags done32, done16;
+    return gm.dp == 32 ? launch(select_shared_kernel<32>, done32) : launch(select_shared_kernel<16>, done16);
 }
 
 cudaError_t launch_select_wave(const tb_ctx* c, const UnitTable& ut, const SelectArgs& a_in, cudaStream_t s, bool dry, bool* finished) {
@@ -897,12 +895,9 @@ cudaError_t launch_select_wave(const tb_ctx* c, const UnitTable& ut, const Selec
 
 #define TB_SEL_R(T, DP, RED)                                                                                                   \
     do {                                                                                                                \
-        static unsigned char seen[64];                                                                                  \
-        if (first_use_on_this_device(seen)) {                                                                           \
-            cudaError_t e = cudaFuncSetAttribute(select_wave_kernel<T, DP, RED>, cudaFuncAttributeMaxDynamicSharedMemorySize, \
-                                                 226 * 1024);                                                            \
-            if (e != cudaSuccess) return e;                                                                             \
-        }                                                                                                               \
+        static DeviceFlags done;                                                                                        \
+        const cudaError_t e = allow_shared_memory(done, select_wave_kernel<T, DP, RED>, 226 * 1024);                    \
+        if (e != cudaSuccess) return e;                                                                                 \
         select_wave_kernel<T, DP, RED><<<n_units, kThreads, smem, s>>>(c->kimp_map, (const unsigned char*)c->kimp, gm, ut, order, a, n_stages, keep_in_l2, c->st.idx, c->st.cnt, \
                                                                   c->st.status, c->wk.sel_keys);                        \
         return cudaGetLastError();                                                                                      \
@@ -1391,12 +1386,9 @@ cudaError_t launch_select_cw(const tb_ctx* c, const UnitTable& ut, const SelectA
     cfg.attrs = attr, cfg.numAttrs = 1;
 #define TB_CW_R(T, DP, RED)                                                                                              \
     do {                                                                                                                 \
-        static unsigned char seen[64];                                                                                   \
-        if (first_use_on_this_device(seen)) {                                                                            \
-            cudaError_t e = cudaFuncSetAttribute(select_cw_kernel<T, DP, RED>, cudaFuncAttributeMaxDynamicSharedMemorySize, \
-                                                 226 * 1024);                                                            \
-            if (e != cudaSuccess) return e;                                                                              \
-        }                                                                                                                \
+        static DeviceFlags done;                                                                                         \
+        const cudaError_t e = allow_shared_memory(done, select_cw_kernel<T, DP, RED>, 226 * 1024);                       \
+        if (e != cudaSuccess) return e;                                                                                  \
         return cudaLaunchKernelEx(&cfg, select_cw_kernel<T, DP, RED>, c->kimp_map, (const unsigned char*)c->kimp, gm, ut, a, \
                                   tiles_per_cta, n_stages, c->st.idx, c->st.cnt, c->st.status, c->wk.sel_keys,           \
                                   digits_on_chip ? (uint16_t*)nullptr : c->wk.sel_bins, keep_in_l2);                    \
