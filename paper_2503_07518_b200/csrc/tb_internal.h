@@ -198,6 +198,34 @@ cudaError_t allow_shared_memory(DeviceFlags& done, K kernel, int bytes) {
     return once_per_device(done, [&] { return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes); });
 }
 
+// How many clusters of `blocks` blocks (2 .. 16) run at once: ask() says, or that it cannot (< 0).  Asked once per context, since a green
+// context or a client with a share of the SMs has fewer than its device; the context that asked last on a device is remembered.
+// A failed query is not, nor where the driver does not number its contexts.
+inline bool current_context_id(unsigned long long* id) {
+    typedef CUresult (*GetId)(CUcontext, unsigned long long*);
+    static const GetId get = [] {
+        void* fn = nullptr;
+        cudaDriverEntryPointQueryResult found;
+        const bool ok = cudaGetDriverEntryPoint("cuCtxGetId", &fn, cudaEnableDefault, &found) == cudaSuccess && found == cudaDriverEntryPointSuccess;
+        return ok ? reinterpret_cast<GetId>(fn) : (GetId) nullptr;
+    }();
+    return get && get(nullptr, id) == CUDA_SUCCESS;
+}
+template <typename F>
+int clusters_that_fit(int blocks, F&& ask) {
+    static std::atomic<uint64_t> known[64][17];        // context << 16 | answer + 1
+    unsigned long long id = 0;
+    int dev = 0;
+    const bool keep = current_context_id(&id) && cudaGetDevice(&dev) == cudaSuccess && dev >= 0 && dev < 64 && blocks <= 16;
+    if (keep) {
+        const uint64_t k = known[dev][blocks].load(std::memory_order_relaxed);
+        if ((k & 0xffffu) && k >> 16 == (id & 0xffffffffffffull)) return (int)(k & 0xffffu) - 1;
+    }
+    const int n = ask();
+    if (keep && n >= 0 && n < 0xffff) known[dev][blocks].store((uint64_t)id << 16 | (uint64_t)(n + 1), std::memory_order_relaxed);
+    return n;
+}
+
 // tb_cache.cu
 cudaError_t launch_append(const tb_ctx* c, const UnitTable& ut, const int* n_new, const int* tok_off, int total_new,
                           const void* k, const void* v, cudaStream_t s);

@@ -17,8 +17,6 @@
 // order-preserving 32-bit key, from the scores on chip or, where only the digits fit, from the rows, until it is small or one
 // key wide: a few rounds at most, each a thousand times finer.
 // Nothing waits for anything but cluster barriers and the block's own loads.
-#include <atomic>
-
 #include "tb_select.cuh"
 
 namespace tb {
@@ -533,7 +531,7 @@ cudaError_t launch(const tb_ctx* c, const UnitTable& ut, const StreamOrder& orde
     });
     if (configured != cudaSuccess) return configured;
     if (l.fit) {
-        if (cudaOccupancyMaxActiveClusters(l.fit, kernel, &l.cfg) != cudaSuccess) *l.fit = 0;
+        if (cudaOccupancyMaxActiveClusters(l.fit, kernel, &l.cfg) != cudaSuccess) *l.fit = -1;
         (void)cudaGetLastError();
         return cudaSuccess;
     }
@@ -573,20 +571,14 @@ cudaError_t launch_select_stream(const tb_ctx* c, const UnitTable& ut, const Sel
     // how many clusters of C blocks run at once: one block per SM, whatever its shared memory
     auto fits = [&](int C) {
         if (C == 1) return c->sm_count;
-        static std::atomic<int> of_device[64][kMaxBlocks + 1];   // 0 = not asked yet
-        int dev = 0;
-        if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return -1;
-        int known = of_device[dev][C].load(std::memory_order_relaxed);
-        if (known == 0) {
+        return clusters_that_fit(C, [&] {
             attr[0].val.clusterDim.x = C;
-            int n = 0;
+            int n = -1;
             l.cfg.gridDim = dim3(C, 1, 1), l.cfg.dynamicSmemBytes = 100 * 1024, l.fit = &n;
-            if (launch_any<512>(c, ut, order, a, l) != cudaSuccess) n = 0;
+            if (launch_any<512>(c, ut, order, a, l) != cudaSuccess) n = -1;
             l.fit = nullptr;
-            known = n > 0 ? n : -1;
-            of_device[dev][C].store(known, std::memory_order_relaxed);
-        }
-        return known;
+            return n;
+        });
     };
     // Up to a problem per SM: blocks of 512 threads, as many per problem as run at once, each with at least 1024 rows.  us per
     // launch, bf16, 32 dimensions, a tenth selected, against the kernels before (clusters on TMA rings): 8 problems of 131072
