@@ -217,14 +217,20 @@ __device__ __forceinline__ float rescore(const unsigned char* row, const float* 
 // barrier, the eight selections of a decode step over 32768 tokens take 7.5 us longer.)
 template <int DP, typename F>
 __device__ __forceinline__ void each_piece(const float* quarter, int g, bool wide, F&& f) {
-    auto all = [&](auto load) {
+    if (wide) {
 #pragma unroll 4
         for (int u = 0; u < g; ++u)
 #pragma unroll
-            for (int j = 0; j < DP / 4; j += 4) f(j, load(quarter + u * DP + j));
-    };
-    if (wide) all([](const float* p) { return *reinterpret_cast<const float4*>(p); });
-    else all([](const float* p) { return make_float4(p[0], p[1], p[2], p[3]); });
+            for (int j = 0; j < DP / 4; j += 4) f(j, *reinterpret_cast<const float4*>(quarter + u * DP + j));
+    } else {
+#pragma unroll 1
+        for (int u = 0; u < g; ++u)
+#pragma unroll
+            for (int j = 0; j < DP / 4; j += 4) {
+                const float* p = quarter + u * DP + j;
+                f(j, make_float4(p[0], p[1], p[2], p[3]));
+            }
+    }
 }
 
 template <int DP, int RED>
