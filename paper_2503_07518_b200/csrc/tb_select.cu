@@ -214,7 +214,7 @@ __global__ void __launch_bounds__(kSelThreads) select_kernel(const __grid_consta
     const int L = unit_len(gm, ut, ll, s);
     const int lo = min(a.sinks, L);
     const int hi = max(lo, L - a.recent);
-    const int ncand = hi - lo;
+    const int ncand = candidates_within(hi - lo, C * tiles_per_cta * kTileRows, status);
     const int k = min(a.budget, ncand);
     check_candidates_projected(gm, ut, ll, s, hi, status);
     const size_t cu = list_unit(gm, ut, ll, s, h);

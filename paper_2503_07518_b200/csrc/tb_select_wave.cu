@@ -979,8 +979,9 @@ __global__ void __launch_bounds__(kThreads, 2)
     int ll, s, h;
     decode_unit(gm, ut, blockIdx.y, ll, s, h);
     const int L = unit_len(gm, ut, ll, s);
-    const int lo = min(a.sinks, L), ncand = max(lo, L - a.recent) - lo, k = min(a.budget, ncand);
-    check_candidates_projected(gm, ut, ll, s, lo + ncand, status);
+    const int lo = min(a.sinks, L), hi = max(lo, L - a.recent);
+    const int ncand = candidates_within(hi - lo, (int)C * tiles_per_cta * kRows, status), k = min(a.budget, ncand);
+    check_candidates_projected(gm, ut, ll, s, hi, status);
     const size_t cu = list_unit(gm, ut, ll, s, h);
     const size_t dst_row = a.dst_is_state ? cu : (size_t)blockIdx.y;
     int32_t* idx_dst = (a.dst_is_state ? state_idx : a.idx_dst) + dst_row * a.idx_stride;

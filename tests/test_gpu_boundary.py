@@ -312,7 +312,9 @@ def test_resident_rows_and_important_buffer_give_the_same_bits(H, on_host):
     ((4, 2), 1, 20000, 1, 1, 1024, False, "bf16"),      # ... which has room to spare
     ((8, 8), 38, 250, 0, 2, 64, False, "bf16"),         # more lists than fit at once: the same
     ((8, 8), 38, 250, 0, 0, 64, False, "fp32"),
-    ((2, 2), 1, 20000, 0, 2, 64, True, "bf16"),         # a cluster per list, the neighbour kernel's bitmask behind it
+    ((2, 2), 1, 20000, 0, 2, 64, True, "bf16"),         # a cluster per list
+    ((8, 8), 19, 20600, 0, 0, 512, True, "bf16"),       # ... on TMA rings
+    ((1, 1), 1, 1060000, 0, 0, 1024, True, "bf16"),     # ... with the keys in the workspace
 ])
 def test_a_replay_that_outgrows_its_reserve_is_reported(H, heads, batch, length, scope, radius, n, reported, dtype):
     """A captured selection is replayed on sequences longer than the reserve it was sized for.  It selects among the
