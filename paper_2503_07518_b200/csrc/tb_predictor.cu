@@ -632,12 +632,12 @@ extern "C" tb_status tb_predict_importance_queries(const tb_predictor* p, const 
         int n8 = 1;
         bool two_per_sm = true;
         if (n_tokens > 8) {
-            static int sm_counts[64];
+            static std::atomic<int> sm_counts[64];
             int dev = 0, sms = 0;
             if (cudaGetDevice(&dev) != cudaSuccess) return TB_ERR_CUDA;
-            if (dev < 64) sms = sm_counts[dev];
+            if (dev < 64) sms = sm_counts[dev].load(std::memory_order_relaxed);
             if (!sms && cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return TB_ERR_CUDA;
-            if (dev < 64) sm_counts[dev] = sms;
+            if (dev < 64) sm_counts[dev].store(sms, std::memory_order_relaxed);
             const int tiles = kClusterK * ((p->hidden_dim + kTileRows - 1) / kTileRows);
             auto blocks = [&](int eights) { return tiles * ((n_tokens + 8 * eights - 1) / (8 * eights)); };
             n8 = blocks(1) <= 3 * sms ? 1 : blocks(2) <= 2 * sms ? 2 : 3;
