@@ -650,9 +650,11 @@ extern "C" tb_status tb_predict_importance_queries(const tb_predictor* p, const 
         auto launch = [&](auto terms, auto eights, auto per_sm) {
             constexpr int kTerms = decltype(terms)::value, kN8 = decltype(eights)::value, kPerSm = decltype(per_sm)::value;
             constexpr int smem = kWBytes + kTerms * kN8 * 8 * kXPitch;
-            static DeviceFlags hidden_done, out_done;
-            cudaError_t r = allow_shared_memory(hidden_done, predictor_hidden_tile_kernel<kTerms, kN8, kPerSm>, smem);
-            if (r == cudaSuccess) r = allow_shared_memory(out_done, predictor_out_tile_kernel<kTerms, kN8, kPerSm>, smem);
+            static DeviceFlags done;
+            cudaError_t r = once_per_device(done, [&] {
+                const cudaError_t e = cudaFuncSetAttribute(predictor_hidden_tile_kernel<kTerms, kN8, kPerSm>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+                return e != cudaSuccess ? e : cudaFuncSetAttribute(predictor_out_tile_kernel<kTerms, kN8, kPerSm>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+            });
             if (r != cudaSuccess) return r;
             cfg.dynamicSmemBytes = smem;
             const unsigned n_groups = (unsigned)((n_tokens + kN8 * 8 - 1) / (kN8 * 8));
