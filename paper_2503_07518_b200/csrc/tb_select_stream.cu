@@ -611,7 +611,8 @@ cudaError_t launch_select_stream(const tb_ctx* c, const UnitTable& ut, const Sel
     // a replayed graph may find more than it declared
     const int spare = ut.use_dev_len && a.radius == 0 ? 2048 : 0;
     l.room = ((max_cand + spare + C - 1) / C + 127) / 128 * 128;
-    l.most = a.radius > 0 ? max_cand : C * l.room;
+    // (neighbours: whole tiles of 256, as in the kernel of one block per list)
+    l.most = a.radius > 0 ? std::min(C * l.room, (max_cand + 255) / 256 * 256) : C * l.room;
     auto smem = [&](bool scores) { return stream_smem(threads, C, l.room, a.radius > 0, scores); };
     // Two blocks of digits do not fit an SM: one of 512 threads, if two waves of them fill most of the chip (256 problems of 65536
     // 184 us, 230 in the kernel that parks its keys, ragged from 32768 on 144 / 187; of 50000 145 / 175).
