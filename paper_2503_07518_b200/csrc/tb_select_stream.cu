@@ -65,6 +65,13 @@ __device__ __forceinline__ uint32_t push_ge(uint32_t bits, uint32_t x, uint32_t 
     return r;
 }
 
+// NaN stays: what is not a number goes to the lowest bin and takes no number's place.
+__device__ __forceinline__ float min_or_nan(float x, float y) {
+    float r;
+    asm("min.NaN.f32 %0, %1, %2;" : "=f"(r) : "f"(x), "f"(y));
+    return r;
+}
+
 __device__ __forceinline__ float key_score(uint32_t key) { return __uint_as_float(key & 0x80000000u ? key & 0x7fffffffu : ~key); }
 
 // Bins, monotone in the score: equal slices of score or, once one of these was too full, slices of 2^shift keys from base up; the
@@ -75,8 +82,8 @@ struct Slices {
     uint32_t base;                  // slices of keys
     int shift;
     __device__ __forceinline__ bool linear() const { return shift < 0; }
-    __device__ __forceinline__ float place(float score) const { return fminf(fmaf(score, scale, off), (float)(kBins - 1)); }
-    __device__ __forceinline__ uint32_t linear_bin(float score) const { return __float2uint_rz(place(score)); }   // (below 0 becomes 0)
+    __device__ __forceinline__ float place(float score) const { return min_or_nan(fmaf(score, scale, off), (float)(kBins - 1)); }
+    __device__ __forceinline__ uint32_t linear_bin(float score) const { return __float2uint_rz(place(score)); }   // (below 0, and NaN, becomes 0)
     __device__ __forceinline__ uint32_t key_bin(uint32_t key) const { return min((max(key, base) - base) >> shift, (uint32_t)(kBins - 1)); }
     __device__ __forceinline__ uint32_t bin(float score) const { return linear() ? linear_bin(score) : key_bin(order_key(score)); }
     // from the keys of the sample scores that bracket the threshold; `reach` times as far up as they are apart, since of 64 rows

@@ -30,7 +30,7 @@ CASES = [
     (8, 1, [47000] * 10, 32, "bf16", "sum", 100, 0, 0, 0, 0, "outliers"),
     (2, 2, [20000], 32, "bf16", "sum", 50, 0, 0, 0, 0, "inf"),
     (2, 2, [20000], 16, "bf16", "max", 50, 0, 0, 0, 0, "inf"),
-    # short lists, blocks of 256 threads: two per SM and more
+    # short lists, blocks of 256 threads: two per SM and more (and, with one of 5003, the kernel that parks its keys)
     (8, 2, [2048, 33, 1000, 64] * 5, 32, "bf16", "sum", 100, 2, 3, 1, 0, "int"),
     (8, 1, [5003, 4000, 1, 31, 257] * 8, 32, "bf16", "sum", 400, 0, 0, 0, 0, "int"),
     (8, 4, [1300] * 38, 16, "bf16", "max", 600, 0, 16, 2, 1, "int"),
@@ -41,6 +41,21 @@ CASES = [
     (4, 7, [8200] * 11, 32, "bf16", "per head", 500, 4, 0, 1, 1, "int"),
     (8, 4, [15000], 32, "bf16", "per head", 900, 0, 0, 0, 0, "int"),
     (4, 4, [11000, 10500] * 5, 16, "bf16", "per head", 800, 0, 0, 0, 0, "int"),
+    # infinities of either sign, an infinite query, NaN: where scores are kept, and where digits are
+    (2, 2, [20000], 32, "bf16", "sum", 900, 0, 0, 0, 0, "infs"),
+    (2, 2, [20000], 16, "bf16", "max", 19900, 0, 0, 0, 0, "infs"),
+    (2, 4, [20000], 32, "bf16", "max", 9000, 0, 0, 0, 0, "infinite query"),
+    (2, 4, [20000], 32, "fp32", "max", 15000, 0, 0, 0, 0, "infinite query"),
+    (2, 2, [20000], 32, "fp32", "sum", 19900, 0, 0, 0, 0, "infs"),
+    (2, 2, [20000], 32, "bf16", "sum", 900, 0, 0, 0, 0, "nan"),
+    (8, 1, [47000] * 10, 32, "bf16", "sum", 700, 0, 0, 0, 0, "infs"),
+    (8, 1, [47000] * 10, 16, "bf16", "sum", 46800, 0, 0, 0, 0, "infs"),
+    (8, 1, [47000] * 10, 16, "bf16", "max", 5000, 0, 0, 0, 0, "infs"),
+    (8, 2, [47000] * 10, 32, "bf16", "max", 12000, 0, 0, 0, 0, "infinite query"),
+    (8, 1, [47000] * 10, 32, "bf16", "sum", 700, 0, 0, 0, 0, "nan"),
+    (8, 1, [23000] * 10, 32, "fp32", "sum", 700, 0, 0, 0, 0, "infs"),
+    (8, 1, [47000] * 10, 32, "bf16", "sum", 30000, 0, 0, 0, 0, "below"),
+    (2, 1, [30000], 32, "bf16", "sum", 9000, 0, 0, 0, 0, "binades"),
 ]
 
 
@@ -97,6 +112,27 @@ def check_lists(H, case, seed, q_offset=0, kernel=None, dev_lengths=False):
             at = torch.randint(0, L, (budget + min(800, L // 4),), generator=gen, device="cuda")
             up = q[0, b].view(heads, g, dp).sum(1).sign().unsqueeze(1) * 120
             x[0, b][:, at] = up + torch.randint(-3, 4, (heads, len(at), dp), generator=gen, device="cuda")
+    lo = min(sinks, min(lens))
+    if data in ("binades", "below"):                     # one channel carries the score, one head of a group asks for it
+        x[..., 1:], x[..., 0] = 0, x[..., 0].bfloat16().float()
+        q.view(1, B, lists, gl, dp).copy_((torch.arange(gl * dp, device="cuda") == 0).view(gl, dp))
+    if data == "binades":                                # 400 of them, both signs
+        x[..., 0] = torch.exp2(torch.randint(-100, 101, x.shape[:-1], generator=gen, device="cuda").float()) * x[..., 0].sign().add(0.5).sign()
+    if data == "below":                                  # the rows that are looked at first score highest, the wanted ones do not
+        for b, L in enumerate(lens):
+            at = lo + torch.arange(64, device="cuda") * max(L - sinks - recent, 1) // 64
+            x[0, b, :, at, 0] = 1000 + 8 * torch.arange(64, device="cuda", dtype=torch.float32)
+    if data == "infs":                                   # of either sign
+        for b, L in enumerate(lens):
+            x[0, b, :, 50:L:97, 3] = float("inf")
+            x[0, b, :, 90:L:97, 3] = float("-inf")
+        q[..., 3] = q[..., 3].abs() + 1
+    if data == "infinite query":                         # one head's, of keys that are not zero
+        x[..., 3] = torch.where(x[..., 3] == 0, 7, x[..., 3])
+        q[:, :, ::gl, 3] = float("inf")
+    if data == "nan":                                    # takes no number's place
+        for b, L in enumerate(lens):
+            x[0, b, :, 50:L:97, 3] = float("nan")
     if data == "inf":
         x[0, 0, :, 1000:lens[0]:97, 3] = float("inf")    # of either sign once multiplied: every row's other products are finite
         q[..., 3] = q[..., 3].abs() + 1
@@ -123,6 +159,7 @@ def check_lists(H, case, seed, q_offset=0, kernel=None, dev_lengths=False):
             for h in range(lists):
                 s = (ctx.kimp[0, b, h * heads // lists, :lens[b]].double() @ q[0, b, h * gl:(h + 1) * gl].double().T)
                 s = (s.max(1).values if reduce == "max" else s.sum(1)).cpu().numpy()
+                s = np.where(np.isnan(s), -np.inf, s)
                 want = H.orc.select(s, sinks, recent, budget)
                 lo, hi = H.orc.candidate_range(lens[b], sinks, recent)
                 if radius and len(want) < hi - lo:
