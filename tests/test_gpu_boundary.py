@@ -314,6 +314,7 @@ def test_resident_rows_and_important_buffer_give_the_same_bits(H, on_host):
     ((8, 8), 38, 250, 0, 0, 64, False, "fp32"),
     ((2, 2), 1, 20000, 0, 2, 64, True, "bf16"),         # a cluster per list
     ((2, 2), 1, 11900, 0, 1, 16, False, "bf16"),        # ... whose last 256 candidates are not all declared
+    ((2, 2), 1, 20000, 0, 0, 1024, True, "bf16"),
     ((8, 8), 19, 20600, 0, 0, 512, True, "bf16"),       # ... on TMA rings
     ((1, 1), 1, 1060000, 0, 0, 1024, True, "bf16"),     # ... with the keys in the workspace
 ])
