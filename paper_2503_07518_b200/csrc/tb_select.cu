@@ -741,28 +741,11 @@ cudaError_t launch_select(const tb_ctx* c, const UnitTable& ut, const SelectArgs
     if (to_wave) return launch_select_wave(c, ut, a, s, dry, finished);
     if (to_cw) return launch_select_cw(c, ut, a, s, dry);
     const int n_tiles = (max_cand + kTileRows - 1) / kTileRows;
-    // Cluster size: enough blocks to cover the GPU about twice, at least 4 tiles per block, and a
-    // key array per block of at most 32 KB where the cluster limit allows (64 KB otherwise).
+    if (c->drop_tile >= 0 && (n_units > 1 || n_tiles > 7)) return cudaErrorInvalidConfiguration;   // ... one block that holds it all
+    // Cluster size: several waves of blocks, so the key array stays small enough for two per SM, and one block's selection phase
+    // overlaps the other's streaming.  (Fewer lists than half of the SMs come here with the diagnostic only.)
     int C = 1;
-    if (2 * n_units > c->sm_count) {
-        // several waves of blocks: keep the key array small enough for two blocks per SM, so one
-        // block's selection phase overlaps the other's streaming
-        while (C < kMaxCluster && (n_tiles + C - 1) / C * kTileRows > 8192) C *= 2;
-    } else {
-        // few problems: one wave.  Two blocks per SM when their key arrays leave room for two rings
-        // (more bytes in flight), otherwise one block per SM.
-        const int tile_b = kTileRows * gm.dp * (gm.dtype == TB_BF16 ? 2 : 4);
-        C = 2 * c->sm_count / n_units;
-        if (C > kMaxCluster) C = kMaxCluster;
-        while (C > 1 && n_tiles / C < 4) --C;
-        const int tpc = (n_tiles + C - 1) / C;
-        if (select_fixed_smem(tpc, tile_b) + 3 * (size_t)tile_b > 113 * 1024) {
-            C = c->sm_count / n_units;
-            if (C > kMaxCluster) C = kMaxCluster;
-            while (C > 1 && n_tiles / C < 4) --C;
-        }
-    }
-    while (C < kMaxCluster && (n_tiles + C - 1) / C * kTileRows > kMaxKeysPerBlock) ++C;
+    while (C < kMaxCluster && (n_tiles + C - 1) / C * kTileRows > 8192) C *= 2;
     int tiles_per_cta = (n_tiles + C - 1) / C;
     if (tiles_per_cta < 1) tiles_per_cta = 1;
     if (tiles_per_cta * kTileRows > kMaxKeysPerBlock) return cudaErrorInvalidConfiguration;
@@ -772,8 +755,7 @@ cudaError_t launch_select(const tb_ctx* c, const UnitTable& ut, const SelectArgs
 
     // diagnostics of the bounded waits (tb_set_wait_diagnostics): one-shot, single-block launches only
     const uint32_t wait_limit = c->wait_poll_limit > 0 ? (uint32_t)c->wait_poll_limit : kWaitPollLimit;
-    const int drop_tile = C == 1 && n_units == 1 ? c->drop_tile : -1;
-    if (c->drop_tile >= 0 && drop_tile < 0) return cudaErrorInvalidConfiguration;
+    const int drop_tile = c->drop_tile;
     if (dry) return cudaSuccess;
     const_cast<tb_ctx*>(c)->drop_tile = -1;
 
