@@ -240,15 +240,15 @@ cudaError_t launch_score(const tb_ctx* c, const UnitTable& ut, const float* q_im
 // (the entry points check every chunk of a call this way before the first real launch)
 // *finished: the launch fetches neighbours and fills the caller's copies itself
 cudaError_t launch_select(const tb_ctx* c, const UnitTable& ut, const SelectArgs& a, cudaStream_t s, bool dry, bool* finished);
-// one block per problem; launch_select hands over to it when a launch holds at least two problems per SM
+// one block per problem on parked keys: many problems that the small and the streaming kernel leave
 cudaError_t launch_select_wave(const tb_ctx* c, const UnitTable& ut, const SelectArgs& a, cudaStream_t s, bool dry, bool* finished);
-// several lists per key stream (bf16, one list per query head), many and long: a cluster per stream
+// several lists per key stream (bf16, one list per query head), many and long or under device lengths: a cluster per stream
 cudaError_t launch_select_shared(const tb_ctx* c, const UnitTable& ut, const SelectArgs& a, cudaStream_t s, bool dry, bool* finished);
 // small problems: one block each, neighbours and the caller's copy of the list included; whether a launch whose longest
 // problem has max_cand candidates is its kind (not whether the caller wants copies: they must not change the lists)
 bool select_small_takes(const tb_ctx* c, const UnitTable& ut, int max_cand, bool neighbours);
 cudaError_t launch_select_small(const tb_ctx* c, const UnitTable& ut, const SelectArgs& a, int max_cand, cudaStream_t s, bool dry = false);
-// few, long problems: a cluster per problem on parked keys
+// problems too long for the streaming kernel: a cluster per problem on parked keys
 cudaError_t launch_select_cw(const tb_ctx* c, const UnitTable& ut, const SelectArgs& a, cudaStream_t s, bool dry = false);
 // long problems: a cluster of blocks each, neighbours and the caller's copy included; *taken = false: not its kind
 cudaError_t launch_select_stream(const tb_ctx* c, const UnitTable& ut, const SelectArgs& a, cudaStream_t s, bool dry, bool* taken);

@@ -717,6 +717,8 @@ cudaError_t launch_select(const tb_ctx* c, const UnitTable& ut, const SelectArgs
     // fill the GPU by themselves: one block each, no clusters.  So do more problems than SMs as long as they are short (160
     // of 9500 candidates: 34.3 us against 36.7 in clusters, 192 of 16000: 47.6 / 54.5), and problems beyond what the
     // parked-key cluster kernel takes.
+    // This kernel is left with 149 to 221 problems: fp32 ones and, under device lengths, bf16 ones of 20K to 96K candidates, bf16
+    // ones of 50K to 96K whose digits do not fit an SM twice (149 to 184 of them: 160 of 65536 160 us, 103 of it bytes).
     // Long problems go to the cluster kernel that parks the keys in memory and keeps 2 bytes per row on chip: two blocks per
     // SM where this one, with 4 bytes per row, has room for one.  Where the line lies depends on the blocks per problem that
     // leaves it: eight to four (128K tokens: 70.1 -> 59.1 us per launch; at 32K the two are level), two (128 problems of
@@ -730,6 +732,7 @@ cudaError_t launch_select(const tb_ctx* c, const UnitTable& ut, const SelectArgs
     // and a block per list is done earlier (us, four lists per stream, this / one problem per list: 512 lists of 1000 24 / 9.7, 8000
     // 47 / 41, 16000 65 / 71; 32 of 16000 27 / 12; seven lists: 448 of 10000 59 / 51, 16000 71 / 75).
     const bool many = n_units > c->sm_count;
+    // (Under device lengths always: its room is the workspace's.)
     if (gm.dtype == TB_BF16 && gm.Hl > gm.Hi && c->drop_tile < 0 && (ut.use_dev_len || (many && max_cand > (gm.Hl > 4 * gm.Hi ? 14000 : 10000))))
         return launch_select_shared(c, ut, a, s, dry, finished);
     // (Replayed graphs in which many sequences grow keep the kernels whose room is the workspace's.)

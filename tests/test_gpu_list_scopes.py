@@ -16,7 +16,7 @@ from test_gpu_parity import H, full_pipeline_check, tb  # noqa: E402,F401
 
 
 CASES = [
-    # cluster kernel (few problems), bf16 tensor-core attention with a group of one / of four
+    # a block per list, or a small cluster; bf16 tensor-core attention with a group of one / of four
     (2, dict(n_layers=2, batch=2, lengths=[5000, 777], budget=200, sinks=3, recent=9)),
     # fp32 storage, d' = 16, g = 2
     (1, dict(n_layers=1, n_q_heads=8, n_kv_heads=4, imp_dim=16, batch=3, lengths=[1500, 260, 2049], budget=100, sinks=1, recent=4)),
@@ -53,7 +53,7 @@ def test_scope_pipeline_matches_oracle(H, scope, ci):
 
 def test_per_query_head_lists_many_problems(H):
     """One list per query head turns 24 sequences x 32 query heads into 768 problems of one launch:
-    the one-block-per-problem selection kernel, then attention with a group of one."""
+    a block of 256 threads per list, then attention with a group of one."""
     b_ = tb()
     w = wl.workload(2, n_layers=1, batch=24, lengths=[1800 + 53 * i for i in range(24)], budget=96)
     case = H.Case(w, list_scope=b_.TB_SCOPE_Q_HEAD)
@@ -104,8 +104,9 @@ def test_scope_argument_checks(H):
 
 @pytest.mark.parametrize("q_heads,kv_heads,dp", [(4, 2, 32), (8, 2, 16), (7, 1, 32), (8, 1, 32), (3, 1, 16)])
 def test_lists_that_share_a_key_stream(H, q_heads, kv_heads, dp):
-    """Per-query-head lists beyond the one-block kernel: shares of the stream that end off a 32-row group, a sequence short
-    enough to be unsampled beside a long one, both neighbour rules, and thresholds in crowded bins (massive ties)."""
+    """Few per-query-head lists: lengths off a 32-row group, a sequence short enough to be unsampled beside a long one, both
+    neighbour rules, and thresholds in crowded bins (massive ties).  Each list streams its keys itself at this number; the kernel
+    that reads a stream once for all its lists is in test_gpu_select_routes.py."""
     for lengths, budget, sinks, recent, radius, nmode in (([9001, 700], 300, 2, 5, 0, 0), ([12345, 8300], 1000, 0, 0, 1, 1), ([40007], 5, 0, 16, 2, 0)):
         w = wl.workload(2, n_layers=1, n_q_heads=q_heads, n_kv_heads=kv_heads, imp_dim=dp, batch=len(lengths), lengths=lengths, budget=budget,
                         sinks=sinks, recent=recent, radius=radius, nmode=nmode)

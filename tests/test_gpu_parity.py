@@ -96,7 +96,7 @@ def test_bf16_gqa_ragged_batch(H):
 
 
 def test_cluster_path_long_sequence(H):
-    # one sequence, two KV heads: the selection is spread over a thread-block cluster of 8
+    # one sequence, two KV heads: each list is spread over a thread-block cluster
     w = wl.workload(4, n_layers=1, n_q_heads=8, n_kv_heads=2, lengths=[20011], budget=777, sinks=16, recent=256, planted=0)
     case = H.Case(w)
     p = tb().select_params(w.budget, w.sinks, w.recent)
@@ -376,7 +376,8 @@ def _crafted_scores_case(H, scores_per_head, budget, sinks=0, recent=0):
 
 
 def test_cluster_selection_unusual_distributions(H):
-    """Paths of the cluster radix select that ordinary data never takes (20011 tokens, 2 heads: a cluster of 8)."""
+    """Paths of the streaming kernel that ordinary data never takes (20011 tokens, 2 heads: a cluster per list; the same for the
+    other kernels in test_gpu_select_routes.py)."""
     r = np.random.Generator(np.random.PCG64(77))
     L = 20011
     # every score equal: the threshold bin holds everything, the lowest positions win
@@ -428,9 +429,8 @@ def _bf16_exact(x):
 
 
 def test_many_problem_selection_kernel(H):
-    """Launches with hundreds of problems take the one-block-per-problem kernel (40 sequences x 8 heads
-    here).  Its first digit is placed from a sample of each problem's scores; these cases put the
-    threshold in every kind of bin that digit has, and on the general path behind it."""
+    """Launches with hundreds of problems (40 sequences x 8 heads here: one block of 256 threads each, four per SM).
+    These cases put the threshold in every kind of bin that the first digit has, and on the general path behind it."""
     r = np.random.Generator(np.random.PCG64(78))
     n_seq, n_heads = 40, 8
     # ordinary data, long enough to be sampled, ending mid-tile; and too short to be sampled
@@ -460,10 +460,9 @@ def test_many_problem_selection_kernel(H):
 
 
 def test_selection_of_very_long_problems(H):
-    """A single problem of 270K candidates: the parked-key cluster kernel with its rows' first digits on
-    chip.  One of 700K: more rows per block than shared memory holds digits for, so they live in the
-    workspace; ordinary scores, and a few distinct values (crowded threshold bins: the bin is cut again from
-    the parked keys, then the general path)."""
+    """A single problem of 270K and one of 700K candidates on sixteen blocks: with their scores and with only their digits
+    on chip; ordinary scores, and a few distinct values (crowded threshold bins are cut again, from the rows).  Beyond a
+    million candidates: test_gpu_select_routes.py."""
     r = np.random.Generator(np.random.PCG64(79))
     _crafted_scores_case(H, _bf16_exact(r.standard_normal((1, 270001))), budget=5000, sinks=4, recent=64)
     _crafted_scores_case(H, _bf16_exact(r.standard_normal((1, 700001))), budget=9000, sinks=4, recent=64)
@@ -593,9 +592,9 @@ def test_kv_cache_in_pinned_host_memory(H):
 def test_group_max_reduction(H):
     """TB_GROUP_MAX (a token's score is the largest of its group's g head scores): materialised scores
     against the oracle, the fused selection = exact top-k of those very fp32 values, on the cluster
-    kernel (one long sequence), on the many-problem kernel (40 sequences) and through the whole pipeline."""
+    kernel (one long sequence), on a block per list (40 sequences) and through the whole pipeline."""
     b_ = tb()
-    # cluster kernel + score kernel, g = 4
+    # streaming kernel + score kernel, g = 4
     w = wl.workload(2, n_layers=1, batch=2, lengths=[9000, 700], budget=300, sinks=2, recent=5)
     case = H.Case(w)
     q, qi = H.queries(w)
@@ -616,7 +615,7 @@ def test_group_max_reduction(H):
             order = np.lexsort((cand, -sc[b, h, lo:hi].astype(np.float64)))
             assert np.array_equal(lists[0][b][h], np.sort(cand[order[:w.budget]]))
     full_pipeline_check(H, case, p)
-    # many-problem kernel: 40 sequences x 8 KV heads in one launch, fp32 storage and d' = 16 as well
+    # a block per list: 40 sequences x 8 KV heads in one launch, fp32 storage and d' = 16 as well
     for cfg, over in ((2, dict(n_layers=1, batch=40, lengths=[2300 + 37 * i for i in range(40)], budget=128)),
                       (1, dict(n_layers=1, n_q_heads=16, n_kv_heads=8, imp_dim=16, batch=40, lengths=[2100 + 11 * i for i in range(40)],
                                budget=64, sinks=1, recent=3))):
@@ -634,8 +633,8 @@ def test_group_max_reduction(H):
 
 @pytest.mark.parametrize("nmode", [0, 1])
 def test_many_problem_selection_with_neighbours_and_attention(H, nmode):
-    """The one-block-per-problem selection kernel in the full pipeline: 32 sequences x 8 KV heads per
-    launch, neighbour expansion from its pre-expansion lists, attention from the stored lists."""
+    """Many short lists in the full pipeline: 32 sequences x 8 KV heads per launch, a block per list that expands its
+    neighbours itself, attention from the stored lists."""
     w = wl.workload(5, n_layers=1, batch=32, lengths=[2100 + 29 * i for i in range(32)], budget=120, sinks=2, recent=16, radius=1)
     case = H.Case(w)
     p = tb().select_params(w.budget, w.sinks, w.recent, radius=1, nmode=nmode)
@@ -643,9 +642,8 @@ def test_many_problem_selection_with_neighbours_and_attention(H, nmode):
 
 
 def test_long_problem_cluster_kernel_unusual_distributions(H):
-    """Problems beyond 48K candidates take the cluster kernel that parks its keys (70001 tokens, 2 heads
-    here).  Cases for each way its threshold search can go: a bin cut again, the open bin above the
-    sampled bracket, the open bin below it and massive ties (general path on the parked keys)."""
+    """70001 tokens, 2 heads, a cluster of sixteen blocks each.  Cases for each way the threshold search can go: a bin
+    cut again, the open bin above the sampled bracket, the open bin below it and massive ties."""
     r = np.random.Generator(np.random.PCG64(80))
     L = 70001
     _crafted_scores_case(H, _bf16_exact(r.standard_normal((2, L))), budget=3000, sinks=3, recent=40)
