@@ -313,13 +313,21 @@ __global__ void __launch_bounds__(kThreads, 512 / kThreads) select_stream_kernel
             if (keep_scores) {
                 for (int i = tid; i < n_local; i += kThreads) recount.add(sm->hist, sl.bin(scores[i]));
             } else {
+                // Rows outside the bin stay above or below it: only a group of 32 with one inside is read again.  256 lists of 65536 of
+                // which a few per launch have 250 or 350 equal keys at their threshold: 242 and 304 us, with all rows read again 288
+                // and 367, without such lists 197.  (Not scoring the other groups either: 222 and 260, but the code is in the way of
+                // launches that never come here, 337.5 -> 339.8 us per decode step at 32K.)
 #pragma unroll 1
                 for (int g0 = warp * 32; g0 < n_local; g0 += kThreads) {
-                    load_rows<Scorer>(few, n_local - g0, [&](int i) { return rows + (size_t)(g0 + i) * RB; });
+                    if (__any_sync(0xffffffffu, g0 + lane < n_local && digits[g0 + lane] == bin))
+                        load_rows<Scorer>(few, n_local - g0, [&](int i) { return rows + (size_t)(g0 + i) * RB; });
                     int slot;
-                    const float sc = scorer.score(few, g0, slot);
-                    if (slot < n_local) recount.add(sm->hist, put(slot, sc, sl.bin(sc)));
-                    if (kMma) odd = odd || odd_query || !is_finite(sc);
+                    const float sc = scorer.score(few, g0, slot);   // (of rows that are not there, or of others: not used)
+                    if (slot < n_local) {
+                        const int d = digits[slot];
+                        recount.add(sm->hist, put(slot, sc, d == bin ? sl.bin(sc) : d > bin ? kBins - 1 : 0));
+                        if (kMma) odd = odd || (d == bin && (odd_query || !is_finite(sc)));
+                    }
                 }
             }
             __syncwarp();

@@ -56,6 +56,11 @@ CASES = [
     (8, 1, [23000] * 10, 32, "fp32", "sum", 700, 0, 0, 0, 0, "infs"),
     (8, 1, [47000] * 10, 32, "bf16", "sum", 30000, 0, 0, 0, 0, "below"),
     (2, 1, [30000], 32, "bf16", "sum", 9000, 0, 0, 0, 0, "binades"),
+    # more equal rows at the threshold than are ranked, where digits are kept: one block, two waves of them, a cluster
+    (8, 1, [47000, 46001] * 5, 32, "bf16", "sum", 5000, 0, 0, 0, 0, "equal"),
+    (8, 1, [50000, 49999] * 14, 16, "bf16", "sum", 5000, 0, 0, 1, 0, "equal"),
+    (1, 2, [900001], 32, "bf16", "sum", 50000, 0, 0, 0, 0, "equal"),
+    (8, 1, [47000] * 10, 16, "fp32", "sum", 4000, 0, 0, 0, 0, "equal"),
 ]
 
 
@@ -130,6 +135,12 @@ def check_lists(H, case, seed, q_offset=0, kernel=None, dev_lengths=False):
     if data == "infinite query":                         # one head's, of keys that are not zero
         x[..., 3] = torch.where(x[..., 3] == 0, 7, x[..., 3])
         q[:, :, ::gl, 3] = float("inf")
+    if data == "equal":                                  # some hundred equal rows at the threshold, in one block's share and all over
+        for b, L in enumerate(lens):
+            at = torch.cat([torch.arange(L - 400, L, device="cuda"), torch.randint(0, L, (300,), generator=gen, device="cuda")])
+            for h in range(heads):
+                kth = (x[0, b, h, :L] @ q[0, b, h * g:(h + 1) * g].sum(0)).topk(budget).indices[-1]
+                x[0, b, h, at] = x[0, b, h, kth].clone()
     if data == "nan":                                    # takes no number's place
         for b, L in enumerate(lens):
             x[0, b, :, 50:L:97, 3] = float("nan")
