@@ -232,8 +232,8 @@ __global__ void __launch_bounds__(kPredThreads) predictor_out_kernel(const T* __
 // weights, about what an SM receives in a memory latency, so that an 8B-shaped linear (8 MB) is 128 blocks that
 // request everything they need at once -- against all tokens of the call.  The tensor pipe is idle most of the time
 // and latency is what there is to save: every thread's weights are in flight before it looks at the tokens.
-// Measured, one call of a 4096 -> 512 -> 4096 predictor in a chain of them: 7.2 us with 1 token, 7.0 with 8, 7.7 with 16, 10.7
-// with 24, 13.3 with 47, 22 with 64, of which 1.3 are the weights at the copy bandwidth.  (With the token groups one after the
+// Measured, one call of a 4096 -> 512 -> 4096 predictor in a chain of them: 7.2 us with 1 token, 7.2 with 8, 8.0 with 16, 11.0
+// with 24, 14.1 with 47, 23 with 64, of which 1.3 are the weights at the copy bandwidth.  (With the token groups one after the
 // other in the same blocks, as large as 32: 9.5 with 16, 12.0 with 24, 20.6 with 47, 31 with 64.)  The weights go through shared
 // memory because their copies then cost no registers: with the fragments loaded straight into registers the kernels
 // spilled and ran at 11.3 us.  Two blocks must fit an SM (they do up to 24 tokens): the output kernel's blocks sit beside the hidden kernel's and

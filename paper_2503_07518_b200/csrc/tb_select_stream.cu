@@ -630,7 +630,7 @@ cudaError_t launch_select_stream(const tb_ctx* c, const UnitTable& ut, const Sel
     l.most = a.radius > 0 ? std::min(C * l.room, (max_cand + 255) / 256 * 256) : C * l.room;
     auto smem = [&](bool scores) { return stream_smem(threads, C, l.room, a.radius > 0, scores); };
     // Two blocks of digits do not fit an SM: one of 512 threads, if two waves of them fill most of the chip (256 problems of 65536
-    // 184 us, 230 in the kernel that parks its keys, ragged from 32768 on 144 / 187; of 50000 145 / 175).
+    // 182 us, with neighbours 204, 230 in the kernel that parks its keys, ragged from 32768 on 144 / 187; of 50000 145 / 175).
     if (threads == 256 && smem(false) > 113 * 1024 && n_units <= 2 * sms && 4 * n_units >= 5 * sms) threads = 512;
     const int per_sm = 512 / threads;
     if ((C > 1 && l.room > kMaxShare) || smem(false) > 226 * 1024 / per_sm) return cudaSuccess;
